@@ -170,7 +170,7 @@ void apply_fmm(fmmpc_handle &H, int part, const double *r, double *out, int nrhs
 void apply_fmm_eager(fmmpc_handle &H, int part, const double *r, double *out, int nrhs);
 void clear_solve_graphs(fmmpc_handle &H);
 void precond_op(fmmpc_handle &H, const double *r, double *z, double *scratch, int nrhs, bool in_capture);
-void q1_mass_solve(fmmpc_handle &H, const double *r, double *c, int nrhs);
+void q1_mass_solve(fmmpc_handle &H, const double *r, double *tmp, double *c, int nrhs);
 int solve_graphed(fmmpc_handle &H, const double *f, const double *g, double *u, int nrhs, const fmmpc_solve_opts &o,
                   fmmpc_solve_info &info);
 cudaGraphExec_t solve_graph(std::vector<fmmpc_handle *> &hs, int method, int m, int nrhs, bool has_g);

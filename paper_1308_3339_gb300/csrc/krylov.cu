@@ -123,26 +123,77 @@ __global__ void k_fold_rhs(OpDev o, int64_t total, const double *__restrict__ f,
   b[t] = v;
 }
 
-// Solves with (1/6) tridiag(1, 4, 1) along every row (cols = 0) or column (cols = 1) of every
-// right-hand side: dst = scale * src on the way (src may alias dst).  cp[k], iden[k]: the
-// Thomas coefficients of the constant matrix, formed once on the host.
-__global__ void k_mass_sweep(int n, int nrhs, int cols, double scale, const double *__restrict__ src,
-                             double *__restrict__ dst, const double *__restrict__ cp,
-                             const double *__restrict__ iden) {
-  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= (int64_t)nrhs * n) return;
+// Solves with (1/6) tridiag(1, 4, 1) along every row (COLS = false) or column (true) of every
+// right-hand side: dst = scale * solution; src and dst distinct.  cp[k], iden[k]: the Thomas
+// coefficients of the constant matrix, formed once on the host (cp[k] = iden[k] / 6).
+//
+// A thread per line would run two serial recurrences over the whole line (n = 512: 279 us a
+// sweep on 512 threads, the row sweep uncoalesced).  Both recurrences forget their start by a
+// factor cp -> 0.268 a step, 0.268^32 = 5e-19, below half an ulp: a recurrence started from zero
+// MS_WARM = 32 steps early is the whole line's to FP64 rounding.  So a block takes 32 lines x
+// MS_SEG outputs with a halo of 32 on both sides in shared memory, and each warp one chunk of 32
+// outputs (lane = line) after 32 warm-up steps: forward for the segment's chunks and the right
+// halo's, then backward from 32 past each chunk.  Bound by the chain's latency and FP64 issue
+// (about 8 operations an output); 512 x 512: 13 us a sweep.
+constexpr int MS_WARM = 32, MS_SEG = 64, MS_LEN = MS_SEG + 2 * MS_WARM, MS_THREADS = MS_SEG + 32;
+template <bool COLS>
+__global__ void __launch_bounds__(MS_THREADS) k_mass_sweep(int n, int64_t lines, double scale,
+                                                           const double *__restrict__ src, double *__restrict__ dst,
+                                                           const double *__restrict__ cp,
+                                                           const double *__restrict__ iden) {
+  // element k of line l at [k][l] (columns) or [l][k] (rows), odd pitch
+  constexpr int PK = COLS ? 33 : 1, PL = COLS ? 1 : MS_LEN + 1;
+  __shared__ double sb[COLS ? MS_LEN * 33 : 32 * (MS_LEN + 1)], scp[MS_LEN], sid[MS_LEN];
+  const int lane = threadIdx.x & 31, c0 = MS_WARM + (threadIdx.x & ~31);  // chunk: elements [c0, c0 + 32)
   const int64_t N = (int64_t)n * n;
   const int lgn = __ffs(n) - 1;
-  const int64_t rhs = t >> lgn, line = t & (n - 1);
-  const int64_t base = rhs * N + (cols ? line : line * n), st = cols ? n : 1;
-  double y = 0.0;
-  for (int k = 0; k < n; ++k) {
-    y = (scale * src[base + k * st] - (1.0 / 6.0) * y) * iden[k];
-    dst[base + k * st] = y;
+  const int k0 = (int)blockIdx.y * MS_SEG - MS_WARM;  // position of element 0 of the window
+  const int64_t l0 = (int64_t)blockIdx.x * 32;
+  // global index of element k of line l (lines over all right-hand sides; n is a power of two)
+  auto at = [&](int64_t l, int k) -> int64_t {
+    const int64_t rhs = l >> lgn, line = l & (n - 1);
+    return rhs * N + (COLS ? (int64_t)k * n + line : line * n + k);
+  };
+  for (int i = threadIdx.x; i < 32 * MS_LEN; i += MS_THREADS) {
+    const int k = COLS ? i >> 5 : i % MS_LEN, l = COLS ? i & 31 : i / MS_LEN;
+    const bool in = k0 + k >= 0 && k0 + k < n && l0 + l < lines;
+    sb[k * PK + l * PL] = in ? src[at(l0 + l, k0 + k)] : 0.0;
   }
-  for (int k = n - 2; k >= 0; --k) {
-    y = dst[base + k * st] - cp[k] * y;
-    dst[base + k * st] = y;
+  for (int k = threadIdx.x; k < MS_LEN; k += MS_THREADS) {
+    const bool in = k0 + k >= 0 && k0 + k < n;
+    scp[k] = in ? cp[k0 + k] : 0.0;  // zero outside the line: the recurrences stay at zero there
+    sid[k] = in ? iden[k0 + k] * scale : 0.0;
+  }
+  __syncthreads();
+  double *const col = sb + lane * PL;
+  double y[32], x = 0.0;
+  // forward, y_k = b_k / pivot_k - cp_k y_{k-1}
+#pragma unroll 8
+  for (int k = c0 - MS_WARM; k < c0; ++k) x = fma(-scp[k], x, col[k * PK] * sid[k]);
+#pragma unroll
+  for (int k = 0; k < 32; ++k) y[k] = x = fma(-scp[c0 + k], x, col[(c0 + k) * PK] * sid[c0 + k]);
+  __syncthreads();
+#pragma unroll
+  for (int k = 0; k < 32; ++k) col[(c0 + k) * PK] = y[k];
+  __syncthreads();
+  // backward, x_k = y_k - cp_k x_{k+1}, from 32 past the chunk; the halo's warp has no output
+  const bool outputs = c0 < MS_WARM + MS_SEG;
+  if (outputs) {
+    x = 0.0;
+#pragma unroll 8
+    for (int k = c0 + 63; k >= c0 + 32; --k) x = fma(-scp[k], x, col[k * PK]);
+#pragma unroll
+    for (int k = 31; k >= 0; --k) y[k] = x = fma(-scp[c0 + k], x, y[k]);
+  }
+  __syncthreads();
+  if (outputs) {
+#pragma unroll
+    for (int k = 0; k < 32; ++k) col[(c0 + k) * PK] = y[k];
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < 32 * MS_SEG; i += MS_THREADS) {
+    const int k = MS_WARM + (COLS ? i >> 5 : i % MS_SEG), l = COLS ? i & 31 : i / MS_SEG;
+    if (k0 + k < n && l0 + l < lines) dst[at(l0 + l, k0 + k)] = sb[k * PK + l * PL];
   }
 }
 
@@ -369,22 +420,25 @@ __global__ void k_cg_p(int64_t N, int nrhs, const double *__restrict__ beta, con
 }  // namespace
 
 // c = M^{-1} r for the consistent Q1 mass matrix M = h^2 (M1 (x) M1) of the interior nodes:
-// tridiagonal solves along every row, then every column (the preconditioner of the Q1
-// operator acts on the finite-element function of the residual, Sec. 6.1).
-void q1_mass_solve(fmmpc_handle &H, const double *r, double *c, int nrhs) {
+// tridiagonal solves along every row into tmp, then along every column into c (the
+// preconditioner of the Q1 operator acts on the finite-element function of the residual,
+// Sec. 6.1).  tmp is distinct from r and c; c may alias r.
+void q1_mass_solve(fmmpc_handle &H, const double *r, double *tmp, double *c, int nrhs) {
   const int n = H.g.n;
   const double h = H.g.h;
-  k_mass_sweep<<<nblk((int64_t)nrhs * n), 256, 0, H.stream>>>(n, nrhs, 0, 1.0 / (h * h), r, c, H.q1tab, H.q1tab + n);
-  k_mass_sweep<<<nblk((int64_t)nrhs * n), 256, 0, H.stream>>>(n, nrhs, 1, 1.0, c, c, H.q1tab, H.q1tab + n);
+  const int64_t lines = (int64_t)nrhs * n;
+  const dim3 grid(nblk(lines, 32), nblk(n, MS_SEG));
+  k_mass_sweep<false><<<grid, MS_THREADS, 0, H.stream>>>(n, lines, 1.0 / (h * h), r, tmp, H.q1tab, H.q1tab + n);
+  k_mass_sweep<true><<<grid, MS_THREADS, 0, H.stream>>>(n, lines, 1.0, tmp, c, H.q1tab, H.q1tab + n);
   FMMPC_LAUNCH_CHECK();
 }
 
 // z = P^{-1} r; with the Q1 operator, P^{-1} M^{-1} r through scratch (which may alias r when
-// r is not needed afterwards).  in_capture: the apply's kernels go into the stream being
+// r is not needed afterwards) and z itself (distinct from both).  in_capture: the apply's kernels go into the stream being
 // captured instead of its own graph.
 void precond_op(fmmpc_handle &H, const double *r, double *z, double *scratch, int nrhs, bool in_capture) {
   if (H.op == 2) {
-    q1_mass_solve(H, r, scratch, nrhs);
+    q1_mass_solve(H, r, z, scratch, nrhs);
     r = scratch;
   }
   if (in_capture) apply_fmm_eager(H, PART_FULL, r, z, nrhs);
