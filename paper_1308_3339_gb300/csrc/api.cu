@@ -268,6 +268,8 @@ int fmmpc_apply_bc(fmmpc_handle *h, const double *f_dev, const double *g_dev, do
     } restore{h, h->bem_form};
     h->bem_form = 0;
     h->bc_g = g_dev;
+    init_bem_bc(*h);
+    init_bnd_dl(*h);
     apply_fmm(*h, PART_BC, f_dev, u_dev, n_rhs);
     return FMMPC_OK;
   });
@@ -281,6 +283,7 @@ int fmmpc_apply_transpose(fmmpc_handle *h, const double *zb_dev, double *rb_dev,
     if (h->bem_form != FMMPC_BEM_SINGLE_LAYER)
       throw Error(FMMPC_ERR_UNSUPPORTED, "apply_transpose: the single-layer correction only");
     init_bem_transpose(*h);
+    init_fmm_transpose(*h);
     struct Restore {
       fmmpc_handle *h;
       ~Restore() { h->trans_pass = false; }
@@ -295,7 +298,10 @@ int fmmpc_set_bem_form(fmmpc_handle *h, int32_t form) {
   if (!h) return FMMPC_ERR_INVALID;
   return guarded(h, [&] {
     require(form == FMMPC_BEM_SINGLE_LAYER || form == FMMPC_BEM_DOUBLE_LAYER, "set_bem_form: unknown form");
-    if (form == FMMPC_BEM_DOUBLE_LAYER) init_bem_dl(*h);
+    if (form == FMMPC_BEM_DOUBLE_LAYER) {
+      init_bem_dl(*h);
+      if (!init_bnd_dl(*h)) throw Error(FMMPC_ERR_OOM, "set_bem_form: no memory for the near double layer");
+    }
     if (form != h->bem_form) {
       for (auto &e : h->gcache) cudaGraphExecDestroy(e.exec);  // captured with the other form
       h->gcache.clear();

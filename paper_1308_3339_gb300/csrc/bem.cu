@@ -66,10 +66,11 @@ __global__ void k_bem_S(int n, double h, double lnh, double *__restrict__ S) {
   S[t] = -(h / (2.0 * PI)) * (I + ell * lnh);
 }
 
-// First block row of -1/2 I + K, K_mk = int_k dG/dn_y(y_m, y) dGamma = (1/2pi) atan2(l d,
+// First block row of diag I + K, K_mk = int_k dG/dn_y(y_m, y) dGamma = (1/2pi) atan2(l d,
 // d^2 + s1 s2) with d the signed normal offset of y_m from element k's line (zero on the
-// same side): the system (-1/2 I + K) mu = -(V r)|_Gamma of the double-layer correction.
-__global__ void k_bem_Kdl(int n, double *__restrict__ A) {
+// same side): diag = -1/2 the system (-1/2 I + K) mu = -(V r)|_Gamma of the double-layer
+// correction, diag = 1/2 the boundary data term of Eq. e:ubound.
+__global__ void k_bem_Kdl(int n, double diag, double *__restrict__ A) {
   const int NG = 4 * n;
   int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= (int64_t)n * NG) return;
@@ -79,7 +80,7 @@ __global__ void k_bem_Kdl(int n, double *__restrict__ A) {
   const int sk = k / n, kk = k % n;
   double v = 0.0;
   if (sk == 0) {
-    v = (k == mrow) ? -0.5 : 0.0;
+    v = (k == mrow) ? diag : 0.0;
   } else {
     double u, d;
     side_coords_d(sk, np1, x, y, u, d);
@@ -117,6 +118,19 @@ __global__ void k_bem_pack(int n, const double *__restrict__ B0, const double *_
   o[n + k] = B2[m * n + k];
   o[2 * n + k] = C1[2 * (m * n + k)];
   o[3 * n + k] = C1[2 * (m * n + k) + 1];
+}
+
+// In place, row m of a first block row [S0 | S1 | S2 | S3] to its side-DFT form
+// [S0+S1+S2+S3 | S0-S1+S2-S3 | S0-S2 | S1-S3] (the blocks that k_bem_apply multiplies by).
+__global__ void k_bem_dft(int n, double *__restrict__ A) {
+  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= (int64_t)n * n) return;
+  double *o = A + (t / n) * 4 * n + t % n;
+  const double s0 = o[0], s1 = o[n], s2 = o[2 * n], s3 = o[3 * n];
+  o[0] = (s0 + s2) + (s1 + s3);
+  o[n] = (s0 + s2) - (s1 + s3);
+  o[2 * n] = s0 - s2;
+  o[3 * n] = s1 - s3;
 }
 
 __global__ void k_identity(int N, double *__restrict__ B, int cplx) {
@@ -282,7 +296,7 @@ void init_bem_dl(fmmpc_handle &H) {
   DevPool tmp;
   try {
     double *A = tmp.get<double>((size_t)n * N);
-    k_bem_Kdl<<<nblk((int64_t)n * N), 256, 0, s>>>(n, A);
+    k_bem_Kdl<<<nblk((int64_t)n * N), 256, 0, s>>>(n, -0.5, A);
     FMMPC_LAUNCH_CHECK();
     double *B0 = tmp.get<double>((size_t)n * n), *B2 = tmp.get<double>((size_t)n * n);
     double *C1 = tmp.get<double>((size_t)2 * n * n);
@@ -309,6 +323,34 @@ void init_bem_dl(fmmpc_handle &H) {
     cudaStreamSynchronize(s);
     throw;
   }
+}
+
+// 1/2 I + K in the side-DFT form, the boundary data term of Eq. e:ubound, for apply_bc; formed
+// on its first call.  Summing the 16 n^2 atan2 of K g directly took 1160 us at n = 1024; the
+// 6 n^2 multiply-adds of the block-circulant form take 15 us.  Not formed (false) while the
+// handle's stream is being captured, or without memory for it: the caller sums directly.
+bool init_bem_bc(fmmpc_handle &H) {
+  if (H.Kbc) return true;
+  cudaStreamCaptureStatus cap{};
+  if (cudaStreamIsCapturing(H.stream, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
+    cudaGetLastError();
+    return false;
+  }
+  const int n = H.g.n;
+  const size_t nv = (size_t)H.g.NG * H.nrhs_max;
+  double *A = nullptr;
+  try {
+    if (!H.bc_vt) H.bc_vt = H.pool.get<double>(nv);
+    if (!H.bc_kg) H.bc_kg = H.pool.get<double>(nv);
+    A = H.pool.get<double>((size_t)n * H.g.NG);
+  } catch (const Error &) {
+    return false;
+  }
+  k_bem_Kdl<<<nblk((int64_t)n * H.g.NG), 256, 0, H.stream>>>(n, 0.5, A);
+  k_bem_dft<<<nblk((int64_t)n * n), 256, 0, H.stream>>>(n, A);
+  FMMPC_LAUNCH_CHECK();
+  H.Kbc = A;
+  return true;
 }
 
 }  // namespace fmmpc

@@ -734,11 +734,26 @@ inline int64_t bup_blocks(int n, int L) {
 
 
 // ------------------------------------------------------------------ collocation points
-// Set-up for the single-precision forms: the near-field log kernel between each collocation
-// point and the nodes of its near volume leaves, formed in FP64 and stored FP32.  Warp per
-// point; layout [boundary leaf: pfirst m m^2][point in leaf][near leaf][node].
+// int over an element of ln|x - y| ds (node units), stable closed form:
+// with s1 = (a - x).t, s2 = s1 + l, d = (x - a).n, A_i = s_i^2 + d^2,
+// = 1/2 [ l ln A2 + s1 log1p(l (s1 + s2) / A1) ] - l + d atan2(l d, d^2 + s1 s2).
+template <typename R>
+__device__ __forceinline__ R seg_log_int(R s1, R ell, R d) {
+  const R s2 = s1 + ell;
+  const R A1 = s1 * s1 + d * d, A2 = s2 * s2 + d * d;
+  R v = R(0.5) * (ell * dev_log<R>(A2) + s1 * log1p(ell * (s1 + s2) / A1)) - ell;
+  if (d != R(0)) v += d * atan2(ell * d, d * d + s1 * s2);
+  return v;
+}
+
+// Near-field operators of the collocation points, formed once in FP64 and stored as T: between
+// each boundary element and the nodes of its near volume leaves, the log kernel at the element's
+// midpoint (INTEGRAL false: V r at the collocation points) or its integral over the element
+// (true: the transpose pass).  Warp per element; layout [boundary leaf: pfirst m m^2][element in
+// leaf][near leaf][node].
+template <typename T, bool INTEGRAL>
 __global__ void k_colloc_mat(Geo g, const int32_t *__restrict__ pfirst, const int32_t *__restrict__ psrc,
-                             float *__restrict__ Kc) {
+                             T *__restrict__ Kc) {
   const int64_t wid = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (wid >= (int64_t)g.NG) return;
@@ -751,26 +766,32 @@ __global__ void k_colloc_mat(Geo g, const int32_t *__restrict__ pfirst, const in
   for (int e0 = pfirst[bl]; e0 < pfirst[bl + 1]; ++e0) {
     int a, b;
     morton_decode((uint32_t)psrc[e0], a, b);
-    float *kr = Kc + kbase + (int64_t)(e0 - pfirst[bl]) * (m * m);
+    T *kr = Kc + kbase + (int64_t)(e0 - pfirst[bl]) * (m * m);
     for (int t = lane; t < m * m; t += 32) {
       const int i = a * m + t % m, j = b * m + t / m;
       int u, d;
       side_coords(side, n + 1, i + 1, j + 1, u, d);
-      const double ds = (double)(numc - 2 * (int64_t)u * n) / (2.0 * n);
-      kr[t] = (float)(0.5 * log(ds * ds + (double)d * (double)d));
+      if (INTEGRAL) {
+        const int64_t num = along * (int64_t)(n + 1) - (int64_t)u * n;  // element start minus node, over n
+        kr[t] = (T)seg_log_int<double>((double)num / n, (n + 1.0) / n, (double)d);
+      } else {
+        const double ds = (double)(numc - 2 * (int64_t)u * n) / (2.0 * n);
+        kr[t] = (T)(0.5 * log(ds * ds + (double)d * (double)d));
+      }
     }
   }
 }
 
-
 // (V r)(y_m) = -(1/2pi)[ Re sum_n Lt_n zt^n  +  sum_{near nodes} w_j ln|y_m - x_j| ].
 // Warp per (collocation point, rhs); requires L < 32.  mode 0: both sums; mode 1: the near
 // sum alone, into vnear (it needs only the weights, so it can run beside the volume
-// upward pass); mode 2: the far sum, added to the near sum read from vnear.
+// upward pass); mode 2: the far sum, added to the near sum read from vnear.  Kc: the near-field
+// log kernel of k_colloc_mat, read 16 bytes a lane (a leaf row's nodes are consecutive in the
+// table and in the weight image, whose rows and halo are multiples of 4 nodes).
 template <typename R>
 __global__ void k_colloc(Geo g, int nrhs, const R *__restrict__ wpad, const cpx<R> *__restrict__ Lb,
                          const int32_t *__restrict__ pfirst, const int32_t *__restrict__ psrc,
-                         double *__restrict__ vcol, const float *__restrict__ Kc, float *__restrict__ vt_hi,
+                         double *__restrict__ vcol, const R *__restrict__ Kc, float *__restrict__ vt_hi,
                          float *__restrict__ vt_lo, int mode, R *__restrict__ vnear) {
   // block (rhs, along): warp w takes the collocation point `along` of side w
   __shared__ double sv[4];
@@ -780,48 +801,26 @@ __global__ void k_colloc(Geo g, int nrhs, const R *__restrict__ wpad, const cpx<
   const int ge = side * n + along;
   const int64_t bl = ((int64_t)side << L) + along / m;
   const R *W = wpad + (int64_t)rhs * g.npad * g.npad;
-  const R inv2n = R(1) / (R)(2 * n);
-  const int64_t numc = (2 * (int64_t)along + 1) * (n + 1);
   R acc = 0;
-  // precomputed (single-precision forms): Kc[(pfirst m + ip c) m^2 + el m^2 + t] = ln|y - x_t|
-  const int c_near = pfirst[bl + 1] - pfirst[bl];
-  const int64_t kbase = ((int64_t)pfirst[bl] * m + (int64_t)(along % m) * c_near) * (m * m);
-  bool done_near = mode == 2;
-  if (mode == 2) acc = vnear[(int64_t)rhs * g.NG + ge];
-  if constexpr (std::is_same<R, float>::value) {
-    if (!done_near && Kc && m == 8 && (g.pad & 3) == 0 && (g.npad & 3) == 0) {
-      // 16 lanes per near leaf, 4 consecutive nodes of a leaf row per lane (float4)
-      const float4 *k4 = reinterpret_cast<const float4 *>(Kc + kbase);
+  if (mode == 2) {
+    acc = vnear[(int64_t)rhs * g.NG + ge];
+  } else {
+    constexpr int V = 16 / sizeof(R);
+    const int e0 = pfirst[bl], c_near = pfirst[bl + 1] - e0, lgv = 2 * (31 - __clz(m)) - (V == 4 ? 2 : 1);
+    const R *kr = Kc + ((int64_t)e0 * m + (int64_t)(along % m) * c_near) * (m * m);
 #pragma unroll 4
-      for (int it = lane; it < c_near * 16; it += 32) {
-        const int el = it >> 4, t4 = it & 15;
-        int a, b;
-        morton_decode((uint32_t)psrc[pfirst[bl] + el], a, b);
-        const int row = b * 8 + (t4 >> 1), col = a * 8 + (t4 & 1) * 4;
-        const float4 wv = *reinterpret_cast<const float4 *>(W + (int64_t)(row + g.pad) * g.npad + col + g.pad);
-        const float4 kv = k4[it];
+    for (int it = lane; it < c_near << lgv; it += 32) {
+      const int el = it >> lgv, t = (it & ((1 << lgv) - 1)) * V;
+      int a, b;
+      morton_decode((uint32_t)psrc[e0 + el], a, b);
+      const R *wr = W + (int64_t)(b * m + t / m + g.pad) * g.npad + a * m + t % m + g.pad;
+      if constexpr (V == 4) {
+        const float4 wv = *reinterpret_cast<const float4 *>(wr), kv = reinterpret_cast<const float4 *>(kr)[it];
         acc += wv.x * kv.x + wv.y * kv.y + wv.z * kv.z + wv.w * kv.w;
+      } else {
+        const double2 wv = *reinterpret_cast<const double2 *>(wr), kv = reinterpret_cast<const double2 *>(kr)[it];
+        acc = fma(wv.x, kv.x, fma(wv.y, kv.y, acc));
       }
-      done_near = true;
-    }
-  }
-  if (!done_near)
-  for (int e0 = pfirst[bl]; e0 < pfirst[bl + 1]; ++e0) {
-    int a, b;
-    morton_decode((uint32_t)psrc[e0], a, b);
-    if (Kc) {
-      const float *kr = Kc + kbase + (int64_t)(e0 - pfirst[bl]) * (m * m);
-      for (int t = lane; t < m * m; t += 32)
-        acc += W[(int64_t)(b * m + t / m + g.pad) * g.npad + a * m + t % m + g.pad] * (R)kr[t];
-      continue;
-    }
-    for (int t = lane; t < m * m; t += 32) {
-      const int i = a * m + t % m, j = b * m + t / m;
-      int u, d;
-      side_coords(side, n + 1, i + 1, j + 1, u, d);
-      // (y_e - x) along the side = ((2 along + 1)(n + 1) - 2 u n) / (2n), exact numerator
-      const R ds = (R)(numc - 2 * (int64_t)u * n) * inv2n;
-      acc += W[(int64_t)(j + g.pad) * g.npad + i + g.pad] * (R(0.5) * dev_log<R>(ds * ds + (R)d * (R)d));
     }
   }
   if (mode != 2) acc = warp_sum(acc);
@@ -880,7 +879,8 @@ __global__ void k_colloc(Geo g, int nrhs, const R *__restrict__ wpad, const cpx<
 // The boundary data term of Eq. e:ubound moved to the left: vcol_m -= (1/2 g_m + (K g)_m)
 // at every collocation point, K_mk = int_k dG/dn_y(y_m, y) dGamma = (1/2pi) atan2(l d,
 // d^2 + s1 s2) (zero on the point's own side), so that the BEM solve q = S^{-1}(-vcol) gives
-// S q = (1/2 I + K) g - (V f)|_Gamma.  Block per (collocation point, rhs), FP64.
+// S q = (1/2 I + K) g - (V f)|_Gamma.  Block per (collocation point, rhs), FP64.  The direct sum:
+// for a first apply_bc whose table of 1/2 I + K cannot be formed (init_bem_bc).
 __global__ void __launch_bounds__(256) k_dl_colloc(int n, int nrhs, const double *__restrict__ gdat,
                                                    double *__restrict__ vcol) {
   __shared__ double red[8];
@@ -920,14 +920,19 @@ __global__ void __launch_bounds__(256) k_dl_colloc(int n, int nrhs, const double
   }
 }
 
-// vt[rhs] = [v^0 | v^2 | a | b] from vcol[rhs] = [v0 | v1 | v2 | v3]
-__global__ void k_bem_vt(int n, int nrhs, const double *__restrict__ vcol, double *__restrict__ vt) {
+// vt[rhs] = [v^0 | v^2 | a | b] from vcol[rhs] = [v0 | v1 | v2 | v3], add (if given) added to it
+__global__ void k_bem_vt(int n, int nrhs, const double *__restrict__ vcol, const double *__restrict__ add,
+                         double *__restrict__ vt) {
   const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= (int64_t)nrhs * n) return;
   const int64_t rr = t / n;
   const int k = (int)(t % n);
   const double *v = vcol + rr * 4 * n;
-  const double v0 = v[k], v1 = v[n + k], v2 = v[2 * n + k], v3 = v[3 * n + k];
+  double v0 = v[k], v1 = v[n + k], v2 = v[2 * n + k], v3 = v[3 * n + k];
+  if (add) {
+    const double *a = add + rr * 4 * n;
+    v0 += a[k], v1 += a[n + k], v2 += a[2 * n + k], v3 += a[3 * n + k];
+  }
   double *o = vt + rr * 4 * n;
   o[k] = (v0 + v2) + (v1 + v3);
   o[n + k] = (v0 + v2) - (v1 + v3);
@@ -935,44 +940,48 @@ __global__ void k_bem_vt(int n, int nrhs, const double *__restrict__ vcol, doubl
   o[3 * n + k] = v1 - v3;
 }
 
-// Block per row m of the transformed first block row T[m] = [C^0 | C^2 | A | B][m].
-__global__ void __launch_bounds__(256) k_bem_apply(int n, int nrhs, const double *__restrict__ T,
-                                                   const double *__restrict__ vt, double *__restrict__ q) {
-  __shared__ double red[8][4];
-  const int mrow = blockIdx.x, tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
-  const int NG = 4 * n;
-  const double *Tr = T + (int64_t)mrow * NG;
+// Rows m of the transformed first block row T[m] = [C^0 | C^2 | A | B][m], two warps a row (half
+// of its columns each), four rows a block, 16-byte loads.  Bound by FP64 issue: 6 n^2 multiply-adds
+// a right-hand side, 11 us at n = 1024.  The lanes meet by a transposing butterfly, 6 FP64 adds a
+// warp for the four sums: with a warp tree each (20) on eight warps a row the cross-lane adds
+// were as many as the products, and the pass took 27 us.
+constexpr int BEM64_ROWS = 4;
+__global__ void __launch_bounds__(64 * BEM64_ROWS) k_bem_apply(int n, int nrhs, const double *__restrict__ T,
+                                                              const double *__restrict__ vt, double *__restrict__ q) {
+  __shared__ double red[BEM64_ROWS][2][4];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, rb = w >> 1, hw = w & 1;
+  const int mrow = blockIdx.x * BEM64_ROWS + rb;  // n is a multiple of 4
+  const int NG = 4 * n, n2 = n >> 1, kend = (hw + 1) * (n2 >> 1);
+  const double2 *t2 = reinterpret_cast<const double2 *>(T + (int64_t)mrow * NG);
   for (int rr = 0; rr < nrhs; ++rr) {
-    const double *v = vt + (int64_t)rr * NG;
+    const double2 *v = reinterpret_cast<const double2 *>(vt + (int64_t)rr * NG);
     double p0 = 0.0, p2 = 0.0, re = 0.0, im = 0.0;
-    for (int k = tid; k < n; k += 256) {
-      const double c0 = Tr[k], c2 = Tr[n + k], ca = Tr[2 * n + k], cb = Tr[3 * n + k];
-      const double a = v[2 * n + k], b = v[3 * n + k];
-      p0 = fma(c0, v[k], p0);
-      p2 = fma(c2, v[n + k], p2);
-      re = fma(ca, a, fma(cb, b, re));
-      im = fma(cb, a, fma(-ca, b, im));
+#pragma unroll 2
+    for (int k = hw * (n2 >> 1) + lane; k < kend; k += 32) {
+      const double2 c0 = t2[k], c2 = t2[n2 + k], ca = t2[2 * n2 + k], cb = t2[3 * n2 + k];
+      const double2 x0 = v[k], x2 = v[n2 + k], a = v[2 * n2 + k], b = v[3 * n2 + k];
+      p0 = fma(c0.x, x0.x, fma(c0.y, x0.y, p0));
+      p2 = fma(c2.x, x2.x, fma(c2.y, x2.y, p2));
+      re = fma(ca.x, a.x, fma(cb.x, b.x, fma(ca.y, a.y, fma(cb.y, b.y, re))));
+      im = fma(cb.x, a.x, fma(-ca.x, b.x, fma(cb.y, a.y, fma(-ca.y, b.y, im))));
     }
-    double acc[4] = {p0, p2, re, im};
+    // lane 8 g ends with the warp's sum of value g of (p0, p2, re, im)
+    const bool u4 = (lane & 16) != 0, u3 = (lane & 8) != 0;
+    const double b0 = (u4 ? re : p0) + __shfl_xor_sync(0xffffffffu, u4 ? p0 : re, 16);
+    const double b1 = (u4 ? im : p2) + __shfl_xor_sync(0xffffffffu, u4 ? p2 : im, 16);
+    double d = (u3 ? b1 : b0) + __shfl_xor_sync(0xffffffffu, u3 ? b0 : b1, 8);
 #pragma unroll
-    for (int sg = 0; sg < 4; ++sg) {
-      const double x = warp_sum(acc[sg]);
-      if (lane == 0) red[w][sg] = x;
-    }
+    for (int o = 4; o > 0; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
+    if ((lane & 7) == 0) red[rb][hw][lane >> 3] = d;
     __syncthreads();
-    if (tid == 0) {
-      double P0 = 0.0, P2 = 0.0, R = 0.0, I = 0.0;
-      for (int ww = 0; ww < 8; ++ww) {
-        P0 += red[ww][0];
-        P2 += red[ww][1];
-        R += red[ww][2];
-        I += red[ww][3];
-      }
-      double *qr = q + (int64_t)rr * NG;
-      qr[mrow] = -0.25 * (P0 + P2 + 2.0 * R);
-      qr[n + mrow] = -0.25 * (P0 - P2 - 2.0 * I);
-      qr[2 * n + mrow] = -0.25 * (P0 + P2 - 2.0 * R);
-      qr[3 * n + mrow] = -0.25 * (P0 - P2 + 2.0 * I);
+    if (threadIdx.x < BEM64_ROWS) {
+      const double(*x)[4] = red[threadIdx.x];
+      const double P0 = x[0][0] + x[1][0], P2 = x[0][1] + x[1][1], R = x[0][2] + x[1][2], I = x[0][3] + x[1][3];
+      double *qr = q + (int64_t)rr * NG + blockIdx.x * BEM64_ROWS + threadIdx.x;
+      qr[0] = -0.25 * (P0 + P2 + 2.0 * R);
+      qr[n] = -0.25 * (P0 - P2 - 2.0 * I);
+      qr[2 * n] = -0.25 * (P0 + P2 - 2.0 * R);
+      qr[3 * n] = -0.25 * (P0 - P2 + 2.0 * I);
     }
     __syncthreads();
   }
@@ -1092,65 +1101,15 @@ __global__ void __launch_bounds__(64 * BEM_ROWS) k_bem_apply_f2(int n, int nrhs,
 }
 
 // ------------------------------------------------------------------ near boundary field
-// int over an element of ln|x - y| ds (node units), stable closed form:
-// with s1 = (a - x).t, s2 = s1 + l, d = (x - a).n, A_i = s_i^2 + d^2,
-// = 1/2 [ l ln A2 + s1 log1p(l (s1 + s2) / A1) ] - l + d atan2(l d, d^2 + s1 s2).
-template <typename R>
-__device__ __forceinline__ R seg_log_int(R s1, R ell, R d) {
-  const R s2 = s1 + ell;
-  const R A1 = s1 * s1 + d * d, A2 = s2 * s2 + d * d;
-  R v = R(0.5) * (ell * dev_log<R>(A2) + s1 * log1p(ell * (s1 + s2) / A1)) - ell;
-  if (d != R(0)) v += d * atan2(ell * d, d * d + s1 * s2);
-  return v;
-}
-
-// Block of 256 per (volume leaf next to the boundary, rhs): each thread takes one node and
-// a strided share of the element list; partial sums meet in shared memory.
-template <typename R>
-__global__ void __launch_bounds__(256) k_bnd_near(Geo g, int64_t nbnear, int nrhs, const int32_t *__restrict__ leaf,
-                                                  const int32_t *__restrict__ first, const int32_t *__restrict__ src,
-                                                  const double *__restrict__ q, R *__restrict__ phib) {
-  __shared__ R red[256];
-  const int slot = blockIdx.x, rhs = blockIdx.y;
-  const int n = g.n, m = g.m, L = g.L, mm = m * m;
-  const int ngrp = blockDim.x / mm;
-  const int t = threadIdx.x % mm, grp = threadIdx.x / mm;
-  int a, b;
-  morton_decode((uint32_t)leaf[slot], a, b);
-  const R ell = (R)((n + 1.0) / n), invn = R(1) / (R)n, hR = (R)g.h;
-  const double *qr = q + (int64_t)rhs * g.NG;
-  const int x = a * m + t % m + 1, y = b * m + t / m + 1;
-  const int f0 = first[slot], cnt = (first[slot + 1] - f0) * m;
-  R acc = 0;
-  if (grp < ngrp)
-    for (int idx = grp; idx < cnt; idx += ngrp) {
-      const int bl = src[f0 + idx / m], e = idx % m;
-      const int side = bl >> L;
-      const int64_t kk = bl & ((int64_t(1) << L) - 1);
-      int u, d;
-      side_coords(side, n + 1, x, y, u, d);
-      // s1 = t_a - u with t_a = (k m + e)(n + 1)/n: exact integer numerator over n
-      const int64_t num = (kk * m + e) * (int64_t)(n + 1) - (int64_t)u * n;
-      acc += (R)qr[side * n + kk * m + e] * hR * seg_log_int<R>((R)num * invn, ell, (R)d);
-    }
-  red[threadIdx.x] = acc;
-  __syncthreads();
-  if (threadIdx.x < mm) {
-    R s = 0;
-    for (int q2 = 0; q2 < ngrp; ++q2) s += red[q2 * mm + threadIdx.x];
-    phib[((int64_t)rhs * nbnear + slot) * mm + threadIdx.x] = s;
-  }
-}
-
-// Double layer near the boundary: phib[slot][t] (+)= dsgn sum_e dens_e theta_e(x_t), theta_e =
+// Double layer near the boundary: phib[slot][t] += dsgn sum_e dens_e theta_e(x_t), theta_e =
 // int_e d/dn_y ln|x - y| ds = -atan2(l d, d^2 + s1 s2) (the signed angle element e subtends at
-// the node, outward normal; node units, so no factor h).  Same blocks and element lists as
-// k_bnd_near.  accumulate = 0 writes instead of adding (no single layer in that apply).
+// the node, outward normal; node units, so no factor h).  Block of 256 per (volume leaf next to
+// the boundary, rhs): each thread takes one node and a strided share of the element list; partial
+// sums meet in shared memory.  The direct sum: for a first apply_bc whose table cannot be formed.
 template <typename R>
-__global__ void __launch_bounds__(256) k_dl_near(Geo g, int64_t nbnear, int nrhs, const int32_t *__restrict__ leaf,
+__global__ void __launch_bounds__(256) k_dl_near(Geo g, int64_t nbnear, const int32_t *__restrict__ leaf,
                                                  const int32_t *__restrict__ first, const int32_t *__restrict__ src,
-                                                 const double *__restrict__ dens, R dsgn, int accumulate,
-                                                 R *__restrict__ phib) {
+                                                 const double *__restrict__ dens, R dsgn, R *__restrict__ phib) {
   __shared__ R red[256];
   const int slot = blockIdx.x, rhs = blockIdx.y;
   const int n = g.n, m = g.m, L = g.L, mm = m * m;
@@ -1180,120 +1139,93 @@ __global__ void __launch_bounds__(256) k_dl_near(Geo g, int64_t nbnear, int nrhs
     R sacc = 0;
     for (int q2 = 0; q2 < ngrp; ++q2) sacc += red[q2 * mm + threadIdx.x];
     R *o = phib + ((int64_t)rhs * nbnear + slot) * mm + threadIdx.x;
-    *o = (accumulate ? *o : R(0)) + dsgn * sacc;
+    *o += dsgn * sacc;
   }
 }
 
-// Point sources at the collocation points next to the boundary (the transpose pass):
-// phib[slot][t] = sum_e c_e h^2 ln|x_t - y_e| (node units) over the elements of the leaf's
-// near boundary runs; y_e the element midpoint.  Same blocks and lists as k_bnd_near.
-template <typename R>
-__global__ void __launch_bounds__(256) k_pt_near(Geo g, int64_t nbnear, int nrhs, const int32_t *__restrict__ leaf,
-                                                 const int32_t *__restrict__ first, const int32_t *__restrict__ src,
-                                                 const double *__restrict__ c, R *__restrict__ phib) {
-  __shared__ double red[256];
-  const int slot = blockIdx.x, rhs = blockIdx.y;
-  const int n = g.n, m = g.m, L = g.L, mm = m * m;
-  const int ngrp = blockDim.x / mm;
-  const int t = threadIdx.x % mm, grp = threadIdx.x / mm;
-  int a, b;
-  morton_decode((uint32_t)leaf[slot], a, b);
-  const double h2 = g.h * g.h;
-  const double *cr = c + (int64_t)rhs * g.NG;
-  const int x = a * m + t % m + 1, y = b * m + t / m + 1;
-  const int f0 = first[slot], cnt = (first[slot + 1] - f0) * m;
-  double acc = 0;
-  if (grp < ngrp)
-    for (int idx = grp; idx < cnt; idx += ngrp) {
-      const int bl = src[f0 + idx / m], e = idx % m;
-      const int side = bl >> L;
-      const int64_t kk = bl & ((int64_t(1) << L) - 1);
-      int u, d;
-      side_coords(side, n + 1, x, y, u, d);
-      // midpoint minus node along the side: ((2(k m + e) + 1)(n + 1) - 2 u n) / (2n)
-      const double ds = (double)((2 * (kk * m + e) + 1) * (int64_t)(n + 1) - 2 * (int64_t)u * n) / (2.0 * n);
-      acc += cr[side * n + kk * m + e] * h2 * 0.5 * log(ds * ds + (double)d * (double)d);
-    }
-  red[threadIdx.x] = acc;
-  __syncthreads();
-  if (threadIdx.x < mm) {
-    double sacc = 0;
-    for (int q2 = 0; q2 < ngrp; ++q2) sacc += red[q2 * mm + threadIdx.x];
-    phib[((int64_t)rhs * nbnear + slot) * mm + threadIdx.x] = (R)sacc;
+// The far weights of the transpose pass: for a boundary run of level l (nl = n >> l elements) and
+// its element a, wt[..][k] = int over the element of z^k ds without the side's direction,
+// nl (o2^{k+1} - o1^{k+1}) / (k + 1), o1 and o2 the element's ends from the run's centre in run
+// units; level l at offset p (2n - 2 nl), then [element of the run][k].
+__global__ void k_colloc_T_far(Geo g, double *__restrict__ wt) {
+  const int t = blockIdx.x * blockDim.x + threadIdx.x;
+  int l = 0, a = t;
+  while (l <= g.L && a >= g.n >> l) a -= g.n >> l++;
+  if (l > g.L) return;
+  const int nl = g.n >> l;
+  const double ell = (g.n + 1.0) / g.n, o1 = ell * (a - 0.5 * nl) / nl, o2 = o1 + ell / nl;
+  double p1 = o1, p2 = o2;
+  for (int k = 0; k < g.p; ++k) {
+    wt[(int64_t)t * g.p + k] = nl * (p2 - p1) / (k + 1);
+    p1 *= o1;
+    p2 *= o2;
   }
 }
 
 // The transpose pass's boundary values: t_k = int_{element k} Phi(y) dGamma_y / h^2 for the
 // volume potential Phi of the weights (h^2 zb) whose local expansions Lb and near nodes the
-// collocation pass uses, i.e. (S_OG^T zb)_k = sum_i zb_i int_k G(x_i, y) dGamma.  Far part:
-// int_e Re sum_k Lt_k z^k over the element, z the offset from each ancestor run's centre in
-// run units, in closed form; near part: the closed-form element integrals of ln|y - x_j|.
-// Block per (boundary leaf run, rhs); FP64 arithmetic.
+// collocation pass uses, i.e. (S_OG^T zb)_k = sum_i zb_i int_k G(x_i, y) dGamma.  Near part: the
+// element integrals of ln|y - x_j| from the table Kt (k_colloc_mat); far part: int_e Re sum_k
+// Lt_k z^k over the element for each ancestor run, the integrals of z^k from the table wt, z's
+// direction e^k one of 1, i, -1, -i.  FP64 arithmetic.  Blocks and warps as in k_colloc.
+//
+// Evaluating the closed-form integrals in every pass cost 5e6 FP64 log, log1p and atan2 and a
+// serial far sum per element: 1484 us at 1024^2; from the tables it is 5e6 FP64 multiply-adds
+// (8.7 us of the FP64 pipe, 40 MB of table).
 template <typename R>
-__global__ void __launch_bounds__(256) k_colloc_T(Geo g, int nrhs, const R *__restrict__ wpad,
-                                                  const cpx<R> *__restrict__ Lb, const int32_t *__restrict__ pfirst,
-                                                  const int32_t *__restrict__ psrc, double *__restrict__ tout) {
-  __shared__ double red[8][16];
-  const int n = g.n, m = g.m, L = g.L, p = g.p, mm = m * m;
-  const int64_t bl = blockIdx.x;
-  const int rhs = blockIdx.y;
-  const int side = (int)(bl >> L);
-  const int64_t kk = bl & ((int64_t(1) << L) - 1);
+__global__ void __launch_bounds__(128) k_colloc_T(Geo g, const R *__restrict__ wpad, const cpx<R> *__restrict__ Lb,
+                                                  const int32_t *__restrict__ pfirst, const int32_t *__restrict__ psrc,
+                                                  const double *__restrict__ Kt, const double *__restrict__ wt,
+                                                  double *__restrict__ tout) {
+  const int lane = threadIdx.x & 31;
+  const int rhs = (int)(blockIdx.x / g.n), along = (int)(blockIdx.x % g.n), side = threadIdx.x >> 5;
+  const int n = g.n, m = g.m, L = g.L, p = g.p;
+  const int64_t bl = ((int64_t)side << L) + along / m;
   const R *W = wpad + (int64_t)rhs * g.npad * g.npad;
-  const double ell = (n + 1.0) / n;
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  const int c_near = pfirst[bl + 1] - pfirst[bl];
-  for (int e = 0; e < m; ++e) {
-    double acc = 0.0;
-    for (int it = threadIdx.x; it < c_near * mm; it += blockDim.x) {
-      const int el = it / mm, t = it % mm;
-      int a, b;
-      morton_decode((uint32_t)psrc[pfirst[bl] + el], a, b);
-      const int i = a * m + t % m, j = b * m + t / m;
-      int u, d;
-      side_coords(side, n + 1, i + 1, j + 1, u, d);
-      const int64_t num = (kk * m + e) * (int64_t)(n + 1) - (int64_t)u * n;
-      acc += (double)W[(int64_t)(j + g.pad) * g.npad + i + g.pad] * seg_log_int<double>((double)num / n, ell, (double)d);
+  double acc = 0.0;
+  const int e0 = pfirst[bl], c_near = pfirst[bl + 1] - e0, lgv = 2 * (31 - __clz(m)) - 1;
+  const double2 *kr =
+      reinterpret_cast<const double2 *>(Kt + ((int64_t)e0 * m + (int64_t)(along % m) * c_near) * (m * m));
+#pragma unroll 4
+  for (int it = lane; it < c_near << lgv; it += 32) {
+    const int el = it >> lgv, t = (it & ((1 << lgv) - 1)) * 2;
+    int a, b;
+    morton_decode((uint32_t)psrc[e0 + el], a, b);
+    const R *wr = W + (int64_t)(b * m + t / m + g.pad) * g.npad + a * m + t % m + g.pad;
+    const double2 kv = kr[it];
+    double w0, w1;
+    if constexpr (sizeof(R) == 4) {
+      const float2 wv = *reinterpret_cast<const float2 *>(wr);
+      w0 = f32_to_f64_bits(wv.x);
+      w1 = f32_to_f64_bits(wv.y);
+    } else {
+      const double2 wv = *reinterpret_cast<const double2 *>(wr);
+      w0 = wv.x;
+      w1 = wv.y;
     }
-    acc = warp_sum(acc);
-    if (lane == 0) red[wid][e] = acc;
+    acc = fma(w0, kv.x, fma(w1, kv.y, acc));
   }
-  __syncthreads();
-  if (threadIdx.x < m) {
-    const int e = threadIdx.x;
-    double near = 0.0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) near += red[w][e];
-    const int along = (int)(kk * m + e);  // element index along the side
-    const double ex = (side == 0) ? 1.0 : (side == 2 ? -1.0 : 0.0);
-    const double ey = (side == 1) ? 1.0 : (side == 3 ? -1.0 : 0.0);
-    double far = 0.0;
-    for (int l = 0; l <= L; ++l) {
-      const int nl = n >> l;
-      const int64_t id = ((int64_t)side << l) + along / nl;
-      const double o1 = ell * ((double)(along % nl) - 0.5 * nl) / nl, o2 = o1 + ell / nl;
-      const cpx<R> *Lc = Lb + (int64_t)rhs * g.nbcell * p + (blevel_offset(l) + id) * p;
-      // sum_k Lt_k e^k nl (o2^{k+1} - o1^{k+1}) / (k + 1)
-      double pr = 1.0, pi = 0.0, p1 = o1, p2 = o2;  // e^k; o^{k+1}
-      for (int k = 0; k < p; ++k) {
-        const double w = nl * (p2 - p1) / (k + 1);
-        far += w * ((double)Lc[k].re * pr - (double)Lc[k].im * pi);
-        const double nr = pr * ex - pi * ey, ni = pr * ey + pi * ex;
-        pr = nr;
-        pi = ni;
-        p1 *= o1;
-        p2 *= o2;
-      }
-    }
-    tout[(int64_t)rhs * g.NG + side * n + along] = (near + far) * NEG_INV_2PI / (g.h * g.h) * g.h;
+  for (int i = lane; i < (L + 1) * p; i += 32) {  // (ancestor run, coefficient) pairs over the lanes
+    const int l = i / p, k = i % p, nl = n >> l;
+    const int64_t id = ((int64_t)side << l) + along / nl;
+    const cpx<R> c = Lb[((int64_t)rhs * g.nbcell + blevel_offset(l) + id) * p + k];
+    const int q = (side * k) & 3;  // e^k = i^q
+    const R v = q == 0 ? c.re : (q == 1 ? -c.im : (q == 2 ? -c.re : c.im));
+    acc = fma(wt[((int64_t)(2 * n - 2 * nl) + along % nl) * p + k], (double)v, acc);
   }
+  acc = warp_sum(acc);
+  if (lane == 0) tout[(int64_t)rhs * g.NG + side * n + along] = acc * NEG_INV_2PI / (g.h * g.h) * g.h;
 }
 
-// The same integrals formed once at set-up (FP64, stored FP32) for the single-precision
-// forms: K[(first[slot] m + idx) m^2 + t] = h int_{element idx} ln|x_t - y| ds, so each apply
-// is a product with q instead of ~5e6 log/atan2 evaluations at 1024^2.
-__global__ void __launch_bounds__(256) k_bnd_near_mat(Geo g, int64_t nbnear, const int32_t *__restrict__ leaf,
+// Near-boundary operators formed once in FP64 and stored as T, between the boundary elements of
+// a volume leaf's near boundary runs and the leaf's nodes: K[(first[slot] m + idx) m^2 + t] =
+// h int_{element idx} ln|x_t - y| ds (KIND 0), the log kernel at the element's midpoint (1: the
+// point sources of the transpose pass), or the double layer -atan2(l d, d^2 + s1 s2) (2: the
+// signed angle the element subtends at the node, as in k_dl_near).
+template <typename T, int KIND>
+__global__ void __launch_bounds__(256) k_bnd_near_mat(Geo g, const int32_t *__restrict__ leaf,
                                                       const int32_t *__restrict__ first,
-                                                      const int32_t *__restrict__ src, float *__restrict__ K) {
+                                                      const int32_t *__restrict__ src, T *__restrict__ K) {
   const int slot = blockIdx.x;
   const int n = g.n, m = g.m, L = g.L, mm = m * m;
   const int ngrp = blockDim.x / mm;
@@ -1310,47 +1242,83 @@ __global__ void __launch_bounds__(256) k_bnd_near_mat(Geo g, int64_t nbnear, con
     const int64_t kk = bl & ((int64_t(1) << L) - 1);
     int u, d;
     side_coords(side, n + 1, x, y, u, d);
-    const int64_t num = (kk * m + e) * (int64_t)(n + 1) - (int64_t)u * n;
-    K[((int64_t)f0 * m + idx) * mm + t] = (float)(g.h * seg_log_int<double>((double)num / n, ell, (double)d));
+    double v;
+    if (KIND == 1) {  // midpoint minus node along the side: ((2(k m + e) + 1)(n + 1) - 2 u n) / (2n)
+      const double ds = (double)((2 * (kk * m + e) + 1) * (int64_t)(n + 1) - 2 * (int64_t)u * n) / (2.0 * n);
+      v = 0.5 * log(ds * ds + (double)d * (double)d);
+    } else {
+      const int64_t num = (kk * m + e) * (int64_t)(n + 1) - (int64_t)u * n;
+      const double s1 = (double)num / n, dd = (double)d;
+      if (KIND == 0) v = g.h * seg_log_int<double>(s1, ell, dd);
+      else v = -atan2(ell * dd, dd * dd + s1 * (s1 + ell));
+    }
+    K[((int64_t)f0 * m + idx) * mm + t] = (T)v;
   }
 }
 
-// Apply of the precomputed integrals: block per (slot, rhs), 16 groups of 16 threads; a
-// thread takes 4 consecutive nodes (float4) of every 16th element; partials meet in shared
-// memory.  Requires m = 8 (64 nodes per leaf).
-__global__ void __launch_bounds__(256) k_bnd_near_k(Geo g, int64_t nbnear, int nrhs, const int32_t *__restrict__ first,
-                                                    const int32_t *__restrict__ src, const float *__restrict__ K,
-                                                    const double *__restrict__ q, float *__restrict__ phib) {
-  __shared__ float4 red[16][16];
-  const int slot = blockIdx.x, rhs = blockIdx.y;
-  const int n = g.n, m = g.m, L = g.L;
-  const int t4 = threadIdx.x & 15, grp = threadIdx.x >> 4;
-  const double *qr = q + (int64_t)rhs * g.NG;
+// Apply of a near-boundary operator K (k_bnd_near_mat): phib[slot][t] = sum_idx K[idx][t] scale
+// dens[idx] over the elements of the leaf's near boundary runs; with TWO, K2, dens2 and scale2
+// add a second operator (the boundary data's double layer).  Block of 256 per (slot, rhs); a
+// thread takes 16 bytes of the leaf's nodes (V of them) of every (256 V / m^2)-th element; the
+// element densities are converted once into shared memory, so that the sweep over K is
+// independent loads; partials meet in shared memory.  Bound by the table's bytes (FP32, 20 MB at
+// 1024^2) or FP64 multiply-adds (5e6: 8.7 us), where evaluating the FP64 form's integrals in each
+// pass took 1216 us and the transpose's logs 462 us.
+template <typename TK, typename R, bool TWO>
+__global__ void __launch_bounds__(256) k_bnd_tab(Geo g, int64_t nbnear, const int32_t *__restrict__ first,
+                                                 const int32_t *__restrict__ src, const TK *__restrict__ K,
+                                                 const double *__restrict__ dens, TK scale,
+                                                 const TK *__restrict__ K2, const double *__restrict__ dens2, TK scale2,
+                                                 R *__restrict__ phib) {
+  constexpr int V = 16 / sizeof(TK);
+  __shared__ __align__(16) TK red[256 * V];
+  __shared__ TK sden[256];
+  const int slot = blockIdx.x, rhs = blockIdx.y, tid = threadIdx.x;
+  const int n = g.n, m = g.m, L = g.L, mm = m * m;
+  const int ln = mm / V, ngrp = 256 / ln, tv = tid % ln, grp = tid / ln;
   const int f0 = first[slot], cnt = (first[slot + 1] - f0) * m;
-  const float4 *K4 = reinterpret_cast<const float4 *>(K) + (int64_t)f0 * m * 16;
-  float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+  TK sum = 0;
+#pragma unroll
+  for (int op = 0; op < (TWO ? 2 : 1); ++op) {  // two sums: the single layer's is the larger by far
+    TK acc[V];
+#pragma unroll
+    for (int c = 0; c < V; ++c) acc[c] = 0;
+    const double *dr = (op ? dens2 : dens) + (int64_t)rhs * g.NG;
+    const TK *Kr = (op ? K2 : K) + (int64_t)f0 * m * mm + tv * V, sc = op ? scale2 : scale;
+    for (int c0 = 0; c0 < cnt; c0 += 256) {
+      const int nc = min(256, cnt - c0);
+      if (tid < nc) {
+        const int idx = c0 + tid, bl = src[f0 + idx / m];
+        const int64_t kk = bl & ((int64_t(1) << L) - 1);
+        sden[tid] = sc * from_f64<TK>(dr[(int64_t)(bl >> L) * n + kk * m + idx % m]);
+      }
+      __syncthreads();
 #pragma unroll 4
-  for (int idx = grp; idx < cnt; idx += 16) {
-    const int bl = src[f0 + idx / m], e = idx % m;
-    const int64_t kk = bl & ((int64_t(1) << L) - 1);
-    const float qe = (float)qr[(bl >> L) * n + kk * m + e];
-    const float4 kv = K4[(int64_t)idx * 16 + t4];
-    acc.x = fmaf(kv.x, qe, acc.x);
-    acc.y = fmaf(kv.y, qe, acc.y);
-    acc.z = fmaf(kv.z, qe, acc.z);
-    acc.w = fmaf(kv.w, qe, acc.w);
-  }
-  red[grp][t4] = acc;
-  __syncthreads();
-  if (threadIdx.x < 64) {
-    const int tt = threadIdx.x >> 2, c = threadIdx.x & 3;
-    float sacc = 0.f;
-    for (int q2 = 0; q2 < 16; ++q2) {
-      const float4 v = red[q2][tt];
-      sacc += c == 0 ? v.x : (c == 1 ? v.y : (c == 2 ? v.z : v.w));
+      for (int i = grp; i < nc; i += ngrp) {
+        TK kv[V];
+        if constexpr (V == 4) {
+          const float4 v = *reinterpret_cast<const float4 *>(Kr + (int64_t)(c0 + i) * mm);
+          kv[0] = v.x, kv[1] = v.y, kv[2] = v.z, kv[3] = v.w;
+        } else {
+          const double2 v = *reinterpret_cast<const double2 *>(Kr + (int64_t)(c0 + i) * mm);
+          kv[0] = v.x, kv[1] = v.y;
+        }
+#pragma unroll
+        for (int c = 0; c < V; ++c) acc[c] = fma(kv[c], sden[i], acc[c]);
+      }
+      __syncthreads();
     }
-    phib[((int64_t)rhs * nbnear + slot) * 64 + threadIdx.x] = sacc;
+#pragma unroll
+    for (int c = 0; c < V; ++c) red[tid * V + c] = acc[c];  // [group][node]
+    __syncthreads();
+    if (tid < mm) {
+      TK part = 0;
+      for (int q = 0; q < ngrp; ++q) part += red[q * mm + tid];
+      sum += part;
+    }
+    if (TWO) __syncthreads();
   }
+  if (tid < mm) phib[((int64_t)rhs * nbnear + slot) * mm + tid] = (R)sum;
 }
 
 // ------------------------------------------------------------------ near field (P2P)
@@ -1823,32 +1791,28 @@ int run_bnd_near(fmmpc_handle &H, int nrhs, cudaStream_t s) {
   const Geo &g = H.g;
   const Lists &Ls = H.lists;
   const dim3 grid((unsigned)Ls.nbnear, nrhs);
-  if (H.trans_pass) {  // point sources c' at the collocation points (transpose pass)
-    k_pt_near<R><<<grid, 256, 0, s>>>(g, Ls.nbnear, nrhs, Ls.pbv_leaf, Ls.pbv_first, Ls.pbv_src, H.fb.q,
-                                      (R *)H.fb.phib);
-    FMMPC_LAUNCH_CHECK();
-    return 1;
+  const int32_t *first = Ls.pbv_first, *src = Ls.pbv_src;
+  R *phib = (R *)H.fb.phib;
+  const R *knear = (const R *)H.fb.knear, *kdl = (const R *)H.fb.kdl;
+  int launches = 1;
+  if (H.trans_pass) {  // point sources h^2 c' at the collocation points (transpose pass)
+    k_bnd_tab<double, R, false><<<grid, 256, 0, s>>>(g, Ls.nbnear, first, src, H.fb.kpt, H.fb.q, g.h * g.h, nullptr,
+                                                     nullptr, 0.0, phib);
+  } else if (H.bem_form == 1) {  // double-layer correction: D mu only (mu in fb.q)
+    k_bnd_tab<R, R, false><<<grid, 256, 0, s>>>(g, Ls.nbnear, first, src, kdl, H.fb.q, R(1), nullptr, nullptr, R(0),
+                                                phib);
+  } else if (H.bc_g && kdl) {  // single layer, and the boundary data: - D g of Eq. e:uinter
+    k_bnd_tab<R, R, true><<<grid, 256, 0, s>>>(g, Ls.nbnear, first, src, knear, H.fb.q, R(1), kdl, H.bc_g, R(-1), phib);
+  } else {
+    k_bnd_tab<R, R, false><<<grid, 256, 0, s>>>(g, Ls.nbnear, first, src, knear, H.fb.q, R(1), nullptr, nullptr, R(0),
+                                                phib);
+    if (H.bc_g) {  // no table of the double layer (init_bnd_dl)
+      k_dl_near<R><<<grid, 256, 0, s>>>(g, Ls.nbnear, Ls.pbv_leaf, first, src, H.bc_g, R(-1), phib);
+      ++launches;
+    }
   }
-  if (H.bem_form == 1) {  // double-layer correction: D mu only (mu in fb.q)
-    k_dl_near<R><<<grid, 256, 0, s>>>(g, Ls.nbnear, nrhs, Ls.pbv_leaf, Ls.pbv_first, Ls.pbv_src, H.fb.q, R(1), 0,
-                                      (R *)H.fb.phib);
-    FMMPC_LAUNCH_CHECK();
-    return 1;
-  }
-  if (std::is_same<R, float>::value && H.fb.knear && g.m == 8)
-    k_bnd_near_k<<<grid, 256, 0, s>>>(g, Ls.nbnear, nrhs, Ls.pbv_first, Ls.pbv_src, H.fb.knear, H.fb.q,
-                                      (float *)H.fb.phib);
-  else
-    k_bnd_near<R><<<grid, 256, 0, s>>>(g, Ls.nbnear, nrhs, Ls.pbv_leaf, Ls.pbv_first, Ls.pbv_src, H.fb.q,
-                                       (R *)H.fb.phib);
   FMMPC_LAUNCH_CHECK();
-  if (H.bc_g) {  // boundary data: - D g of Eq. e:uinter
-    k_dl_near<R><<<grid, 256, 0, s>>>(g, Ls.nbnear, nrhs, Ls.pbv_leaf, Ls.pbv_first, Ls.pbv_src, H.bc_g, R(-1), 1,
-                                      (R *)H.fb.phib);
-    FMMPC_LAUNCH_CHECK();
-    return 2;
-  }
-  return 1;
+  return launches;
 }
 
 template <typename R, int P>
@@ -1911,6 +1875,7 @@ void apply_impl(fmmpc_handle &H, int part, const double *r, double *out, int nrh
   const bool trans = part == PART_TRANS;       // P^{-T}: element integrals, S^{-T}, point sources
   const bool dl = H.bem_form == 1;             // double-layer correction (mu from -1/2 I + K)
   const bool bc = part == PART_BC && H.bc_g;   // boundary data g (Eqs. e:ubound / e:uinter)
+  const bool bc_tab = bc && H.Kbc;
   // The tensor-core near field and volume M2L do not depend on the boundary chain
   // (collocation values, BEM density, boundary tree, near-boundary correction): for the
   // full apply without stage timing they run on a second stream, forked after the weights
@@ -1929,7 +1894,7 @@ void apply_impl(fmmpc_handle &H, int part, const double *r, double *out, int nrh
     if (split_colloc) {
       FMMPC_CUDA(cudaStreamWaitEvent(H.sstream2, H.sev[0], 0));
       k_colloc<R><<<(unsigned)((int64_t)g.n * nrhs), 128, 0, H.sstream2>>>(
-          g, nrhs, wpad, Lb, Ls.pvb_first, Ls.pvb_src, H.fb.vcol, H.fb.kcol, nullptr, nullptr, 1, (R *)H.fb.vnear);
+          g, nrhs, wpad, Lb, Ls.pvb_first, Ls.pvb_src, H.fb.vcol, (const R *)H.fb.kcol, nullptr, nullptr, 1, (R *)H.fb.vnear);
       FMMPC_LAUNCH_CHECK();
       ++launches;
       FMMPC_CUDA(cudaEventRecord(H.sev[6], H.sstream2));
@@ -1951,18 +1916,23 @@ void apply_impl(fmmpc_handle &H, int part, const double *r, double *out, int nrh
     // vcol after this kernel)
     const bool vt_f2 = H.Sinv_hi && H.fb.vt_hi && !bc && !trans;
     if (trans)  // t = S_OG^T zb: element integrals of the volume potential, into vcol
-      k_colloc_T<R><<<dim3((unsigned)g.nbleaf, nrhs), 256, 0, s>>>(g, nrhs, wpad, Lb, Ls.pvb_first, Ls.pvb_src,
-                                                                   H.fb.vcol);
+      k_colloc_T<R><<<(unsigned)((int64_t)g.n * nrhs), 128, 0, s>>>(g, wpad, Lb, Ls.pvb_first, Ls.pvb_src, H.fb.kcolT,
+                                                                    H.fb.wfarT, H.fb.vcol);
     else {
       if (split_colloc) FMMPC_CUDA(cudaStreamWaitEvent(s, H.sev[6], 0));
       k_colloc<R><<<(unsigned)((int64_t)g.n * nrhs), 128, 0, s>>>(g, nrhs, wpad, Lb, Ls.pvb_first, Ls.pvb_src,
-                                                                 H.fb.vcol, H.fb.kcol, vt_f2 ? H.fb.vt_hi : nullptr,
+                                                                 H.fb.vcol, (const R *)H.fb.kcol, vt_f2 ? H.fb.vt_hi : nullptr,
                                                                  vt_f2 ? H.fb.vt_lo : nullptr, split_colloc ? 2 : 0,
                                                                  (R *)H.fb.vnear);
     }
     FMMPC_LAUNCH_CHECK();
     launches += 2;
-    if (bc) {  // vcol -= (1/2 I + K) g: Eq. e:ubound's data term
+    if (bc_tab) {  // -(1/2 I + K) g, added to vcol where its side DFT is taken
+      k_bem_vt<<<nblk((int64_t)nrhs * g.n), 256, 0, s>>>(g.n, nrhs, H.bc_g, nullptr, H.bc_vt);
+      k_bem_apply<<<g.n / BEM64_ROWS, 64 * BEM64_ROWS, 0, s>>>(g.n, nrhs, H.Kbc, H.bc_vt, H.bc_kg);
+      FMMPC_LAUNCH_CHECK();
+      launches += 2;
+    } else if (bc) {  // vcol -= (1/2 I + K) g: Eq. e:ubound's data term
       k_dl_colloc<<<dim3((unsigned)g.NG, nrhs), 256, 0, s>>>(g.n, nrhs, H.bc_g, H.fb.vcol);
       FMMPC_LAUNCH_CHECK();
       ++launches;
@@ -1982,8 +1952,8 @@ void apply_impl(fmmpc_handle &H, int part, const double *r, double *out, int nrh
       else k_bem_apply_f2<1><<<nb, 64 * BEM_ROWS, 0, s>>>(g.n, nrhs, Th, Tl, H.fb.vt_hi, H.fb.vt_lo, H.fb.q);
       ++launches;
     } else {
-      k_bem_vt<<<nblk((int64_t)nrhs * g.n), 256, 0, s>>>(g.n, nrhs, H.fb.vcol, H.fb.vt);
-      k_bem_apply<<<g.n, 256, 0, s>>>(g.n, nrhs, dl ? H.Kdl_inv : (trans ? H.SinvT : H.Sinv), H.fb.vt, H.fb.q);
+      k_bem_vt<<<nblk((int64_t)nrhs * g.n), 256, 0, s>>>(g.n, nrhs, H.fb.vcol, bc_tab ? H.bc_kg : nullptr, H.fb.vt);
+      k_bem_apply<<<g.n / BEM64_ROWS, 64 * BEM64_ROWS, 0, s>>>(g.n, nrhs, dl ? H.Kdl_inv : (trans ? H.SinvT : H.Sinv), H.fb.vt, H.fb.q);
       launches += 2;
     }
     FMMPC_LAUNCH_CHECK();
@@ -2232,7 +2202,71 @@ void dispatch_apply(fmmpc_handle &H, int part, const double *r, double *out, int
   }
 }
 
+// Near-boundary operators formed once (the geometry is fixed): element integrals at the nodes of
+// volume leaves next to the boundary, and the log kernel at the collocation points.
+template <typename R>
+void form_near(fmmpc_handle &H) {
+  const int64_t nent = H.lists.n_p2p_vb * (int64_t)H.g.m * H.g.m * H.g.m;
+  if (nent <= 0 || H.lists.nbnear <= 0) return;
+  H.fb.knear = H.pool.get<R>(nent);
+  H.fb.kcol = H.pool.get<R>(nent);
+  k_bnd_near_mat<R, 0><<<(unsigned)H.lists.nbnear, 256, 0, H.stream>>>(H.g, H.lists.pbv_leaf, H.lists.pbv_first,
+                                                                          H.lists.pbv_src, (R *)H.fb.knear);
+  k_colloc_mat<R, false><<<nblk((int64_t)H.g.NG * 32, 128), 128, 0, H.stream>>>(H.g, H.lists.pvb_first,
+                                                                               H.lists.pvb_src, (R *)H.fb.kcol);
+  FMMPC_LAUNCH_CHECK();
+  FMMPC_CUDA(cudaStreamSynchronize(H.stream));
+}
+
 }  // namespace
+
+// The near double layer's operator, on first use (false: not formed, see init_bem_bc).
+bool init_bnd_dl(fmmpc_handle &H) {
+  const int64_t nent = H.lists.n_p2p_vb * (int64_t)H.g.m * H.g.m * H.g.m;
+  if (H.fb.kdl || nent <= 0 || H.lists.nbnear <= 0) return true;
+  cudaStreamCaptureStatus cap{};
+  if (cudaStreamIsCapturing(H.stream, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
+    cudaGetLastError();
+    return false;
+  }
+  const bool f64 = H.prec == FMMPC_PREC_FP64;
+  void *K = nullptr;
+  try {
+    K = H.pool.alloc((f64 ? sizeof(double) : sizeof(float)) * (size_t)nent);
+  } catch (const Error &) {
+    return false;
+  }
+  if (f64)
+    k_bnd_near_mat<double, 2><<<(unsigned)H.lists.nbnear, 256, 0, H.stream>>>(
+        H.g, H.lists.pbv_leaf, H.lists.pbv_first, H.lists.pbv_src, (double *)K);
+  else
+    k_bnd_near_mat<float, 2><<<(unsigned)H.lists.nbnear, 256, 0, H.stream>>>(
+        H.g, H.lists.pbv_leaf, H.lists.pbv_first, H.lists.pbv_src, (float *)K);
+  FMMPC_LAUNCH_CHECK();
+  H.fb.kdl = K;
+  return true;
+}
+
+// The transpose pass's near operators (FP64 in every form) and far weights, on first use.
+void init_fmm_transpose(fmmpc_handle &H) {
+  if (H.fb.wfarT) return;
+  const Geo &g = H.g;
+  const int64_t nent = H.lists.n_p2p_vb * (int64_t)g.m * g.m * g.m;
+  if (nent > 0 && H.lists.nbnear > 0) {
+    if (!H.fb.kcolT) H.fb.kcolT = H.pool.get<double>(nent);
+    if (!H.fb.kpt) H.fb.kpt = H.pool.get<double>(nent);
+    k_colloc_mat<double, true><<<nblk((int64_t)g.NG * 32, 128), 128, 0, H.stream>>>(g, H.lists.pvb_first,
+                                                                                   H.lists.pvb_src, H.fb.kcolT);
+    k_bnd_near_mat<double, 1><<<(unsigned)H.lists.nbnear, 256, 0, H.stream>>>(g, H.lists.pbv_leaf, H.lists.pbv_first,
+                                                                                H.lists.pbv_src, H.fb.kpt);
+  }
+  const int64_t runs = 2 * g.n - (g.n >> g.L);  // elements over one side's runs of every level
+  double *w = H.pool.get<double>((size_t)runs * g.p);
+  k_colloc_T_far<<<nblk(runs), 256, 0, H.stream>>>(g, w);
+  FMMPC_LAUNCH_CHECK();
+  FMMPC_CUDA(cudaStreamSynchronize(H.stream));
+  H.fb.wfarT = w;
+}
 
 void init_fmm(fmmpc_handle &H) {
   const int side = 1 << H.g.L;
@@ -2258,20 +2292,9 @@ void init_fmm(fmmpc_handle &H) {
   } else {
     set_p2p_smem_limit<float>();
     alloc_fmm<float>(H);
-    // near-boundary operators formed once (the geometry is fixed): element integrals at the
-    // nodes of volume leaves next to the boundary, and the log kernel at collocation points
-    const int64_t nent = H.lists.n_p2p_vb * (int64_t)H.g.m * H.g.m * H.g.m;
-    if (nent > 0 && H.lists.nbnear > 0) {
-      H.fb.knear = H.pool.get<float>(nent);
-      H.fb.kcol = H.pool.get<float>(nent);
-      k_bnd_near_mat<<<(unsigned)H.lists.nbnear, 256, 0, H.stream>>>(H.g, H.lists.nbnear, H.lists.pbv_leaf,
-                                                                    H.lists.pbv_first, H.lists.pbv_src, H.fb.knear);
-      k_colloc_mat<<<nblk((int64_t)H.g.NG * 32, 128), 128, 0, H.stream>>>(H.g, H.lists.pvb_first, H.lists.pvb_src,
-                                                                         H.fb.kcol);
-      FMMPC_LAUNCH_CHECK();
-      FMMPC_CUDA(cudaStreamSynchronize(H.stream));
-    }
   }
+  if (H.prec == FMMPC_PREC_FP64) form_near<double>(H);
+  else form_near<float>(H);
   // Stream priorities (copied into the kernel nodes of captured graphs, which are
   // instantiated to use them): the apply's critical chain (weights, upward pass, boundary
   // chain, downward pass) runs on the graph stream at the highest priority; the near-

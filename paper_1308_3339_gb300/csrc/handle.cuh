@@ -34,8 +34,12 @@ struct FmmBufs {
   double *q = nullptr;       // [nrhs][NG] BEM density
   double *vt = nullptr;      // [nrhs][NG] side-DFT of vcol for the block-circulant apply
   float *vt_hi = nullptr, *vt_lo = nullptr;  // the same as two FP32 words (single-precision forms)
-  float *knear = nullptr;    // near-boundary element integrals (single-precision forms)
-  float *kcol = nullptr;     // collocation-point near-field log kernel (single-precision forms)
+  void *knear = nullptr;     // near-boundary element integrals (R)
+  void *kcol = nullptr;      // collocation-point near-field log kernel (R)
+  double *kcolT = nullptr;   // element integrals in kcol's layout, made on the first transpose pass
+  double *kpt = nullptr;     // point log kernel in knear's layout, made on the first transpose pass
+  void *kdl = nullptr;       // near double layer (R), knear's layout, made on first use
+  double *wfarT = nullptr;   // integrals of z^k over the elements of every boundary run, likewise
   void *vnear = nullptr;     // [nrhs][NG] near part of V r at the collocation points (R)
   void *Lvb = nullptr;       // [nrhs][n_vbv_cells][p] boundary-source part of L of those cells
   int *up_count = nullptr;   // [nrhs][up_ncount] upward-pass arrival counts (zero between launches)
@@ -128,6 +132,8 @@ struct fmmpc_handle {
   double *Kdl_inv = nullptr;  // the same for -1/2 I + K (double-layer correction), made on first use
   double *SinvT = nullptr;    // the same for S^T (the transpose pass), made on first use
   float *Kdl_hi = nullptr, *Kdl_lo = nullptr;  // and as two FP32 words (single-precision forms)
+  double *Kbc = nullptr;      // 1/2 I + K in the same form (apply_bc), made on first use
+  double *bc_vt = nullptr, *bc_kg = nullptr;  // [nrhs][NG] side DFT of the boundary data, -(1/2 I + K) g
   int bem_form = 0;         // 0: single-layer correction (Eq. e:ubound), 1: second-kind double layer
   const double *bc_g = nullptr;  // boundary data of the running fmmpc_apply_bc call (else NULL)
   bool trans_pass = false;       // the running apply is the transpose pass
@@ -177,9 +183,12 @@ cudaGraphExec_t solve_graph(std::vector<fmmpc_handle *> &hs, int method, int m, 
 int solve_batched_graphed(std::vector<fmmpc_handle *> &hs, const double *const *f, const double *const *gb,
                           double *const *u, const fmmpc_solve_opts &o, fmmpc_solve_info *infos);
 void init_fmm(fmmpc_handle &H);
+void init_fmm_transpose(fmmpc_handle &H);
 void init_bem(fmmpc_handle &H, DevPool &tmp);
 void init_bem_dl(fmmpc_handle &H);
 void init_bem_transpose(fmmpc_handle &H);
+bool init_bem_bc(fmmpc_handle &H);
+bool init_bnd_dl(fmmpc_handle &H);
 void spmv5(fmmpc_handle &H, const double *x, double *y, int nrhs);
 int solve(fmmpc_handle &H, const double *f, const double *g, double *u, int nrhs,
           const fmmpc_solve_opts &o, fmmpc_solve_info &info);

@@ -41,3 +41,29 @@ def test_q1_mass_solve_windows(n, leaf_max, nrhs):
         check_close(f"q1 windows n={n} rhs={r}", u[r].cpu().numpy().ravel(), uo, 1e-8, 1e-8)
     assert info["iters"] <= max(counts) + 1, (info["iters"], counts)
     P.close()
+
+
+@pytest.mark.parametrize("n,leaf_max,prec,nrhs", [(32, 16, "fp64", 2), (64, 256, "fp32", 3), (128, 64, "mixed_tf32", 1),
+                                                  (128, 16, "fp32", 1)])
+def test_first_apply_bc_under_capture_sums_directly(n, leaf_max, prec, nrhs):
+    # a first apply_bc inside a stream capture cannot form its tables and sums the boundary data
+    # directly; later calls take the tables.  Same operator either way: FP64 to its rounding,
+    # single precision to FP32 sums of ~100 terms (1e-5).
+    from paper_1308_3339_gb300 import FmmPreconditioner
+    f = dev(np.stack([S.gaussian_mixture(n, 60 + r) for r in range(nrhs)]))
+    g = dev(np.stack([S.random_field(n, 70 + r)[: 4 * n] for r in range(nrhs)]))
+    st = torch.cuda.Stream()
+    with torch.cuda.stream(st):
+        P = FmmPreconditioner(n, p=10, leaf_max=leaf_max, precision=prec, n_rhs=nrhs, stream=st)
+        u = torch.empty_like(f)
+        st.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=st):
+            P.apply_bc(f, g, out=u)
+        graph.replay()
+        st.synchronize()
+        ut = P.apply_bc(f, g)
+        st.synchronize()
+    tol = 1e-12 if prec == "fp64" else 1e-5
+    check_close(f"apply_bc direct vs tables {prec} n={n}", ut.cpu().numpy(), u.cpu().numpy(), tol, tol)
+    P.close()
