@@ -94,7 +94,9 @@ void setup(fmmpc_handle &H, const fmmpc_grid &g, const fmmpc_params &p) {
     G.npad = n + 2 * G.pad;
     init_fmm(H);
     init_tc_p2p(H);
+    init_p2p_oz(H);
     init_tc_m2l(H, tmp);
+    init_m2l_oz(H, tmp);
     init_bem(H, tmp);
     FMMPC_CUDA(cudaStreamSynchronize(H.stream));
   } catch (...) {
@@ -383,10 +385,16 @@ int fmmpc_query(const fmmpc_handle *h, int32_t what, int64_t *value) {
         return FMMPC_ERR_CUDA;
       if (h->tcm.err && cudaMemcpy(&e2, h->tcm.err, sizeof(int), cudaMemcpyDeviceToHost) != cudaSuccess)
         return FMMPC_ERR_CUDA;
-      *value = e | (e2 << 8);
+      int e3 = 0;
+      if (h->ozp.err && cudaMemcpy(&e3, h->ozp.err, sizeof(int), cudaMemcpyDeviceToHost) != cudaSuccess)
+        return FMMPC_ERR_CUDA;
+      int e4 = 0;
+      if (h->ozm.err && cudaMemcpy(&e4, h->ozm.err, sizeof(int), cudaMemcpyDeviceToHost) != cudaSuccess)
+        return FMMPC_ERR_CUDA;
+      *value = e | e3 | ((e2 | e4) << 8);
       break;
     }
-    case 13: *value = (h->tcp.enabled && h->p2p_engine == 0) ? 1 : 0; break;
+    case 13: *value = ((h->tcp.enabled || h->ozp.enabled) && h->p2p_engine == 0) ? 1 : 0; break;
     case 14: *value = h->tcm.enabled ? (h->tcm.kind == 0 ? 1 : 2) : 0; break;
     default: return FMMPC_ERR_INVALID;
   }

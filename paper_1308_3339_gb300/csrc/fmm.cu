@@ -17,9 +17,9 @@
 // weight image with a table of ln|d| over the stencil of leaf offsets that the dual tree
 // traversal produced.
 //
-// Without stage timing the full apply forks the tensor-core near field, the volume M2L and
-// the near-boundary correction onto streams of their own; they overlap the boundary chain
-// (collocation values, BEM density, boundary tree) and join before the downward pass.
+// Without stage timing the applies fork the near field, the volume M2L and the near-boundary
+// correction onto streams of their own; they overlap the boundary chain (collocation values, BEM
+// density, boundary tree) and join before the downward pass.
 #include <algorithm>
 #include <cmath>
 #include <complex>
@@ -806,14 +806,15 @@ __global__ void k_colloc(Geo g, int nrhs, const R *__restrict__ wpad, const cpx<
     acc = vnear[(int64_t)rhs * g.NG + ge];
   } else {
     constexpr int V = 16 / sizeof(R);
-    const int e0 = pfirst[bl], c_near = pfirst[bl + 1] - e0, lgv = 2 * (31 - __clz(m)) - (V == 4 ? 2 : 1);
+    const int e0 = pfirst[bl], c_near = pfirst[bl + 1] - e0;
+    const int lgm = 31 - __clz(m), lgv = 2 * lgm - (V == 4 ? 2 : 1);  // m is a power of two
     const R *kr = Kc + ((int64_t)e0 * m + (int64_t)(along % m) * c_near) * (m * m);
 #pragma unroll 4
     for (int it = lane; it < c_near << lgv; it += 32) {
       const int el = it >> lgv, t = (it & ((1 << lgv) - 1)) * V;
       int a, b;
       morton_decode((uint32_t)psrc[e0 + el], a, b);
-      const R *wr = W + (int64_t)(b * m + t / m + g.pad) * g.npad + a * m + t % m + g.pad;
+      const R *wr = W + (int64_t)(b * m + (t >> lgm) + g.pad) * g.npad + a * m + (t & (m - 1)) + g.pad;
       if constexpr (V == 4) {
         const float4 wv = *reinterpret_cast<const float4 *>(wr), kv = reinterpret_cast<const float4 *>(kr)[it];
         acc += wv.x * kv.x + wv.y * kv.y + wv.z * kv.z + wv.w * kv.w;
@@ -1183,7 +1184,7 @@ __global__ void __launch_bounds__(128) k_colloc_T(Geo g, const R *__restrict__ w
   const int64_t bl = ((int64_t)side << L) + along / m;
   const R *W = wpad + (int64_t)rhs * g.npad * g.npad;
   double acc = 0.0;
-  const int e0 = pfirst[bl], c_near = pfirst[bl + 1] - e0, lgv = 2 * (31 - __clz(m)) - 1;
+  const int e0 = pfirst[bl], c_near = pfirst[bl + 1] - e0, lgm = 31 - __clz(m), lgv = 2 * lgm - 1;
   const double2 *kr =
       reinterpret_cast<const double2 *>(Kt + ((int64_t)e0 * m + (int64_t)(along % m) * c_near) * (m * m));
 #pragma unroll 4
@@ -1191,7 +1192,7 @@ __global__ void __launch_bounds__(128) k_colloc_T(Geo g, const R *__restrict__ w
     const int el = it >> lgv, t = (it & ((1 << lgv) - 1)) * 2;
     int a, b;
     morton_decode((uint32_t)psrc[e0 + el], a, b);
-    const R *wr = W + (int64_t)(b * m + t / m + g.pad) * g.npad + a * m + t % m + g.pad;
+    const R *wr = W + (int64_t)(b * m + (t >> lgm) + g.pad) * g.npad + a * m + (t & (m - 1)) + g.pad;
     const double2 kv = kr[it];
     double w0, w1;
     if constexpr (sizeof(R) == 4) {
@@ -1275,7 +1276,8 @@ __global__ void __launch_bounds__(256) k_bnd_tab(Geo g, int64_t nbnear, const in
   __shared__ TK sden[256];
   const int slot = blockIdx.x, rhs = blockIdx.y, tid = threadIdx.x;
   const int n = g.n, m = g.m, L = g.L, mm = m * m;
-  const int ln = mm / V, ngrp = 256 / ln, tv = tid % ln, grp = tid / ln;
+  const int lgm = 31 - __clz(m), lgl = 2 * lgm - (V == 4 ? 2 : 1);  // m is a power of two
+  const int ngrp = 256 >> lgl, tv = tid & ((1 << lgl) - 1), grp = tid >> lgl;
   const int f0 = first[slot], cnt = (first[slot + 1] - f0) * m;
   TK sum = 0;
 #pragma unroll
@@ -1288,9 +1290,9 @@ __global__ void __launch_bounds__(256) k_bnd_tab(Geo g, int64_t nbnear, const in
     for (int c0 = 0; c0 < cnt; c0 += 256) {
       const int nc = min(256, cnt - c0);
       if (tid < nc) {
-        const int idx = c0 + tid, bl = src[f0 + idx / m];
+        const int idx = c0 + tid, bl = src[f0 + (idx >> lgm)];
         const int64_t kk = bl & ((int64_t(1) << L) - 1);
-        sden[tid] = sc * from_f64<TK>(dr[(int64_t)(bl >> L) * n + kk * m + idx % m]);
+        sden[tid] = sc * from_f64<TK>(dr[(int64_t)(bl >> L) * n + kk * m + (idx & (m - 1))]);
       }
       __syncthreads();
 #pragma unroll 4
@@ -1424,13 +1426,12 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 4 : 2) k_p2p(P2PArgs<R> 
   for (int t = 0; t < M; ++t) o[t] = ((double)sum[t] - (double)comp[t]) * NEG_INV_2PI;
 }
 
-// -(1/2pi) (a + b) + u, u = v (float)(-1/2pi): a + b exactly as a two-word sum (Knuth's
-// TwoSum), times -1/(2pi) held as two floats (the product's error word from an FMA, as in
-// Dekker's product), u added with TwoSum, and the two words converted to FP64 and added.
-__device__ __forceinline__ double near_far_sum(float a, float b, float v) {
+// -(1/2pi) (s + s_lo) + u, u = v (float)(-1/2pi): the two-word sum s + s_lo times -1/(2pi) held
+// as two floats (the product's error word from an FMA, as in Dekker's product), u added with
+// Knuth's TwoSum, and the two words converted to FP64 and added.
+__device__ __forceinline__ double near_far_sum(float s, float s_lo, float v) {
   constexpr float c_hi = (float)NEG_INV_2PI;
   constexpr float c_lo = (float)(NEG_INV_2PI - (double)c_hi);
-  const float s = a + b, bb = s - a, s_lo = (a - (s - bb)) + (b - bb);
   const float p = __fmul_rn(s, c_hi);  // rounded products, never fused into the sums below
   const float p_lo = fmaf(s, c_hi, -p) + fmaf(s, c_lo, s_lo * c_hi);
   const float u = __fmul_rn(v, c_hi);
@@ -1452,8 +1453,7 @@ __global__ void __launch_bounds__(256) k_downward_tree(Geo g, int nrhs, int do_b
                                                        const cpx<R> *__restrict__ Lv, const int32_t *__restrict__ vslot,
                                                        const cpx<R> *__restrict__ Lsep, int64_t nsep,
                                                        const R *__restrict__ phib, const int32_t *__restrict__ bslot,
-                                                       double *__restrict__ out, const float *__restrict__ near1,
-                                                       const float *__restrict__ near2) {
+                                                       double *out, const R *nearp, int np, int64_t nstride) {
   __shared__ cpx<R> sS[4 * P * P], sanc[24][P], s1[4][P], s2[16][P];
   const int tid = threadIdx.x, nthr = blockDim.x, rhs = blockIdx.y;
   const uint32_t blk = blockIdx.x;
@@ -1549,15 +1549,37 @@ __global__ void __launch_bounds__(256) k_downward_tree(Geo g, int nrhs, int do_b
     for (int e = 0; e < NPT; ++e) acc[e] = acc[e] * mk<R>((tx0 + e - R(0.5) * (M - 1)) / M, zy) + Lk;
   }
   double *o = out + off;
-  if (near1) {
-    // tensor-core near field: the two raw halves often cancel, so they are added exactly
-    // and scaled by -1/(2 pi) in two-word FP32 arithmetic, the far term added, and the
-    // two-word result converted to FP64 with one FP64 addition (FP64 is scarce here)
+  if (nearp) {  // tensor-core near field: raw parts (of one part, in out itself)
+    if constexpr (std::is_same<R, double>::value) {
+      double sn[NPT];
 #pragma unroll
-    for (int e = 0; e < NPT; ++e) {
-      float v = (float)acc[e].re;
-      if (pb) v += (float)pb[e];
-      o[e] = near_far_sum(near1[off + e], near2[off + e], v);
+      for (int e = 0; e < NPT; ++e) sn[e] = nearp[off + e];
+      for (int q = 1; q < np; ++q) {
+#pragma unroll
+        for (int e = 0; e < NPT; ++e) sn[e] += nearp[q * nstride + off + e];
+      }
+#pragma unroll
+      for (int e = 0; e < NPT; ++e) o[e] = (sn[e] + acc[e].re + (pb ? pb[e] : 0.0)) * NEG_INV_2PI;
+    } else {
+      // the parts often cancel, so they are added as a two-word FP32 sum (TwoSum) and scaled by
+      // -1/(2 pi) in two-word arithmetic, the far term added, and the two-word result converted
+      // to FP64 with one FP64 addition (FP64 is scarce here)
+      float sn[NPT], sl[NPT];
+#pragma unroll
+      for (int e = 0; e < NPT; ++e) {
+        sn[e] = nearp[off + e];
+        sl[e] = 0.0f;
+      }
+      for (int q = 1; q < np; ++q) {
+#pragma unroll
+        for (int e = 0; e < NPT; ++e) two_sum_acc(sn[e], sl[e], nearp[q * nstride + off + e]);
+      }
+#pragma unroll
+      for (int e = 0; e < NPT; ++e) {
+        float v = (float)acc[e].re;
+        if (pb) v += (float)pb[e];
+        o[e] = near_far_sum(sn[e], sl[e], v);
+      }
     }
   } else {
 #pragma unroll
@@ -1574,8 +1596,7 @@ __global__ void __launch_bounds__(256) k_downward_tree(Geo g, int nrhs, int do_b
 template <typename R, int M>
 __global__ void k_far_final(int n, int L, int p, int64_t ncell, int64_t nbnear, int nrhs, int do_bnd,
                             const cpx<R> *__restrict__ Lv, const R *__restrict__ phib,
-                            const int32_t *__restrict__ bslot, double *__restrict__ out,
-                            const float *__restrict__ near1, const float *__restrict__ near2) {
+                            const int32_t *__restrict__ bslot, double *__restrict__ out) {
   const int64_t nleaf = int64_t(1) << (2 * L);
   const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= nleaf * M * nrhs) return;
@@ -1601,22 +1622,11 @@ __global__ void k_far_final(int n, int L, int p, int64_t ncell, int64_t nbnear, 
   }
   const int64_t off = (int64_t)rhs * n * n + (int64_t)(gy * M + ty) * n + gx * M;
   double *o = out + off;
-  if (near1) {
-    // tensor-core near field: the two raw halves and the far term meet in FP64 (they often
-    // cancel) -- one add and one fused multiply-add per node
 #pragma unroll
-    for (int q = 0; q < M; ++q) {
-      float v = (float)acc[q].re;
-      if (pb) v += (float)pb[q];
-      o[q] = fma((double)near1[off + q] + (double)near2[off + q], NEG_INV_2PI, (double)(v * (float)NEG_INV_2PI));
-    }
-  } else {
-#pragma unroll
-    for (int q = 0; q < M; ++q) {
-      double v = (double)acc[q].re;
-      if (pb) v += (double)pb[q];
-      o[q] += v * NEG_INV_2PI;
-    }
+  for (int q = 0; q < M; ++q) {
+    double v = (double)acc[q].re;
+    if (pb) v += (double)pb[q];
+    o[q] += v * NEG_INV_2PI;
   }
 }
 
@@ -1691,16 +1701,15 @@ void run_p2p(fmmpc_handle &H, const void *table, double *out, int nrhs, cudaStre
 }
 
 template <typename R>
-void run_far_final(fmmpc_handle &H, double *out, int nrhs, int do_bnd, cudaStream_t s,
-                   const float *near1 = nullptr, const float *near2 = nullptr) {
+void run_far_final(fmmpc_handle &H, double *out, int nrhs, int do_bnd, cudaStream_t s) {
   const Geo &g = H.g;
   const int64_t tasks = g.nleaf * g.m * nrhs;
   const cpx<R> *Lv = (const cpx<R> *)H.fb.Lv;
   const R *pb = (const R *)H.fb.phib;
   switch (g.m) {
-    case 4: k_far_final<R, 4><<<nblk(tasks, 128), 128, 0, s>>>(g.n, g.L, g.p, g.ncell, H.lists.nbnear, nrhs, do_bnd, Lv, pb, H.lists.leaf_bslot, out, near1, near2); break;
-    case 8: k_far_final<R, 8><<<nblk(tasks, 128), 128, 0, s>>>(g.n, g.L, g.p, g.ncell, H.lists.nbnear, nrhs, do_bnd, Lv, pb, H.lists.leaf_bslot, out, near1, near2); break;
-    default: k_far_final<R, 16><<<nblk(tasks, 128), 128, 0, s>>>(g.n, g.L, g.p, g.ncell, H.lists.nbnear, nrhs, do_bnd, Lv, pb, H.lists.leaf_bslot, out, near1, near2); break;
+    case 4: k_far_final<R, 4><<<nblk(tasks, 128), 128, 0, s>>>(g.n, g.L, g.p, g.ncell, H.lists.nbnear, nrhs, do_bnd, Lv, pb, H.lists.leaf_bslot, out); break;
+    case 8: k_far_final<R, 8><<<nblk(tasks, 128), 128, 0, s>>>(g.n, g.L, g.p, g.ncell, H.lists.nbnear, nrhs, do_bnd, Lv, pb, H.lists.leaf_bslot, out); break;
+    default: k_far_final<R, 16><<<nblk(tasks, 128), 128, 0, s>>>(g.n, g.L, g.p, g.ncell, H.lists.nbnear, nrhs, do_bnd, Lv, pb, H.lists.leaf_bslot, out); break;
   }
   FMMPC_LAUNCH_CHECK();
 }
@@ -1765,8 +1774,13 @@ int run_l2l(fmmpc_handle &H, int nrhs, cudaStream_t s) {
 // includes the boundary weight.
 template <typename R, int P>
 void run_downward(fmmpc_handle &H, double *out, int nrhs, int do_bnd, int with_bnd_w, cudaStream_t s,
-                  const float *near1 = nullptr, const float *near2 = nullptr, bool sep = false) {
+                  bool tc_near = false, bool sep = false) {
   const Geo &g = H.g;
+  constexpr bool f64 = std::is_same<R, double>::value;
+  const R *nearp = nullptr;
+  if (tc_near) nearp = (const R *)(f64 ? (const void *)(H.ozp.nparts > 1 ? H.ozp.near : out) : (const void *)H.tcp.near);
+  const int np = f64 ? H.ozp.nparts : H.tcp.nparts;
+  const int64_t nstride = f64 ? H.ozp.part_stride : H.tcp.part_stride;
   const int32_t *vslot = sep ? H.lists.vbv_slot : nullptr;
   const cpx<R> *Lsep = (const cpx<R> *)H.fb.Lvb;
   const int64_t nsep = H.lists.n_vbv_cells;
@@ -1776,9 +1790,9 @@ void run_downward(fmmpc_handle &H, double *out, int nrhs, int do_bnd, int with_b
   const cpx<R> *vl2l = mats_of<R>(H).vl2l;
   const dim3 grid((unsigned)(int64_t(1) << (2 * (g.L - 2))), nrhs);
   switch (g.m) {
-    case 4: k_downward_tree<R, P, 4><<<grid, 256, 0, s>>>(g, nrhs, do_bnd, H.lists.nbnear, Mv, Mb, with_bnd_w, vl2l, Lv, vslot, Lsep, nsep, pb, H.lists.leaf_bslot, out, near1, near2); break;
-    case 8: k_downward_tree<R, P, 8><<<grid, 256, 0, s>>>(g, nrhs, do_bnd, H.lists.nbnear, Mv, Mb, with_bnd_w, vl2l, Lv, vslot, Lsep, nsep, pb, H.lists.leaf_bslot, out, near1, near2); break;
-    case 16: k_downward_tree<R, P, 16><<<grid, 256, 0, s>>>(g, nrhs, do_bnd, H.lists.nbnear, Mv, Mb, with_bnd_w, vl2l, Lv, vslot, Lsep, nsep, pb, H.lists.leaf_bslot, out, near1, near2); break;
+    case 4: k_downward_tree<R, P, 4><<<grid, 256, 0, s>>>(g, nrhs, do_bnd, H.lists.nbnear, Mv, Mb, with_bnd_w, vl2l, Lv, vslot, Lsep, nsep, pb, H.lists.leaf_bslot, out, nearp, np, nstride); break;
+    case 8: k_downward_tree<R, P, 8><<<grid, 256, 0, s>>>(g, nrhs, do_bnd, H.lists.nbnear, Mv, Mb, with_bnd_w, vl2l, Lv, vslot, Lsep, nsep, pb, H.lists.leaf_bslot, out, nearp, np, nstride); break;
+    case 16: k_downward_tree<R, P, 16><<<grid, 256, 0, s>>>(g, nrhs, do_bnd, H.lists.nbnear, Mv, Mb, with_bnd_w, vl2l, Lv, vslot, Lsep, nsep, pb, H.lists.leaf_bslot, out, nearp, np, nstride); break;
     default: throw Error(FMMPC_ERR_UNSUPPORTED, "leaf side must be 4, 8 or 16");
   }
   FMMPC_LAUNCH_CHECK();
@@ -1851,9 +1865,10 @@ void apply_impl(fmmpc_handle &H, int part, const double *r, double *out, int nrh
   if (H.timing)
     for (int k = 0; k < fmmpc_handle::NSTAGE; ++k) H.stage_hit[k] = false;
   mark(0);
-  const bool tc = std::is_same<R, float>::value && H.tcp.enabled && H.p2p_engine == 0;
-  if (tc) {
-    launches += prep_p2p_tc(H, r, nrhs, s, (float *)wpad);  // strips and weight image in one pass
+  constexpr bool f64 = std::is_same<R, double>::value;
+  const bool tc = (f64 ? H.ozp.enabled : H.tcp.enabled) && H.p2p_engine == 0;  // near field on the tensor cores
+  if (tc) {  // its operands and the weight image in one pass
+    launches += f64 ? prep_p2p_oz(H, r, nrhs, s, (double *)wpad) : prep_p2p_tc(H, r, nrhs, s, (float *)wpad);
   } else {
     k_weights<R><<<nblk(N * nrhs), 256, 0, s>>>(g.n, g.npad, g.pad, g.h * g.h, N * nrhs, r, wpad);
     FMMPC_LAUNCH_CHECK();
@@ -1862,8 +1877,8 @@ void apply_impl(fmmpc_handle &H, int part, const double *r, double *out, int nrh
   if (part == PART_NEAR) {
     mark(9);
     if (tc) {
-      launches += run_p2p_tc(H, true, out, nrhs, s);
-      launches += add_near2(H, out, nrhs, s);
+      launches += f64 ? run_p2p_oz(H, true, out, nrhs, s) : run_p2p_tc(H, true, nrhs, s);
+      launches += f64 ? add_near_oz(H, out, nrhs, s) : add_near(H, out, nrhs, s);
     }
     else { run_p2p<R>(H, H.fb.table_lnh, out, nrhs, s); ++launches; }
     mark_end();
@@ -1876,37 +1891,78 @@ void apply_impl(fmmpc_handle &H, int part, const double *r, double *out, int nrh
   const bool dl = H.bem_form == 1;             // double-layer correction (mu from -1/2 I + K)
   const bool bc = part == PART_BC && H.bc_g;   // boundary data g (Eqs. e:ubound / e:uinter)
   const bool bc_tab = bc && H.Kbc;
-  // The tensor-core near field and volume M2L do not depend on the boundary chain
-  // (collocation values, BEM density, boundary tree, near-boundary correction): for the
-  // full apply without stage timing they run on a second stream, forked after the weights
-  // and after the upward pass and joined before the boundary-to-volume M2L.
-  const bool side = tc && part == PART_FULL && H.timing == 0 && H.sstream;
-  const bool m2l_side = side && std::is_same<R, float>::value && H.tcm.enabled;
+  auto boundary_data = [&](cudaStream_t st) {  // -(1/2 I + K) g, added to vcol where its side DFT is taken
+    k_bem_vt<<<nblk((int64_t)nrhs * g.n), 256, 0, st>>>(g.n, nrhs, H.bc_g, nullptr, H.bc_vt);
+    k_bem_apply<<<g.n / BEM64_ROWS, 64 * BEM64_ROWS, 0, st>>>(g.n, nrhs, H.Kbc, H.bc_vt, H.bc_kg);
+    FMMPC_LAUNCH_CHECK();
+    launches += 2;
+  };
+  // The near field and the volume M2L do not depend on the boundary chain (collocation values,
+  // BEM density, boundary tree, near-boundary correction): without stage timing they run on
+  // streams of their own, forked after the weights and after the upward pass and joined before
+  // the downward pass, in every form and for the plain, boundary-data and transpose applies.
+  // (One stream for them all kept the chain's latency-bound kernels in line behind the long
+  // ones: 128^2 FP32 83 -> 56 us.)
+  const bool side = with_bnd && part != PART_VCOL && part != PART_Q && g.L >= 2 && H.timing == 0;
   cudaStream_t ss = H.sstream;
   // the near part of the collocation values needs only the weights: with the side streams
   // it runs on the third one beside the volume upward pass, and the collocation kernel on
   // the main stream adds the far part
-  const bool split_colloc = side && with_bnd && part != PART_TRANS && H.fb.vnear && H.fb.kcol;
+  const bool split_colloc = side && !trans && H.fb.kcol;
+  // boundary sources of the volume locals kept apart, for the downward pass to add, so that they
+  // need not wait for the volume M2L
+  const bool vbv_sep = with_bnd && g.L >= 2 && Ls.n_vbv_cells > 0;
+  auto near_field = [&](cudaStream_t st) {
+    if (tc) launches += f64 ? run_p2p_oz(H, false, out, nrhs, st) : run_p2p_tc(H, false, nrhs, st);
+    else {
+      run_p2p<R>(H, H.fb.table, out, nrhs, st);  // writes the near field into out
+      ++launches;
+    }
+  };
+  auto volume_m2l = [&](cudaStream_t st) {
+    if (std::is_same<R, float>::value && H.tcm.enabled) {
+      launches += run_m2l_tc(H, Mv, Lv, nrhs, st);
+    } else if (f64 && H.ozm.enabled) {
+      launches += run_m2l_oz(H, Mv, Lv, nrhs, st);
+    } else {
+      k_m2l_vol<R, P><<<nblk(g.ncell * nrhs * 32), 256, 0, st>>>(gd, g.ncell, g.nbcell, nrhs, 1,
+                                                                with_bnd && !vbv_sep ? 1 : 0, 0, Ls.m2l_first,
+                                                                Ls.m2l_src, Ls.vbv_first, Ls.vbv_src, Mv, Mb, Lv);
+      FMMPC_LAUNCH_CHECK();
+      ++launches;
+    }
+  };
   if (side) {
     FMMPC_CUDA(cudaEventRecord(H.sev[0], s));
-    FMMPC_CUDA(cudaStreamWaitEvent(ss, H.sev[0], 0));
-    launches += run_p2p_tc(H, false, out, nrhs, ss);
+    if (!tc) {
+      FMMPC_CUDA(cudaStreamWaitEvent(ss, H.sev[0], 0));
+      near_field(ss);
+    }
+    if (split_colloc || bc_tab) FMMPC_CUDA(cudaStreamWaitEvent(H.sstream2, H.sev[0], 0));
     if (split_colloc) {
-      FMMPC_CUDA(cudaStreamWaitEvent(H.sstream2, H.sev[0], 0));
       k_colloc<R><<<(unsigned)((int64_t)g.n * nrhs), 128, 0, H.sstream2>>>(
           g, nrhs, wpad, Lb, Ls.pvb_first, Ls.pvb_src, H.fb.vcol, (const R *)H.fb.kcol, nullptr, nullptr, 1, (R *)H.fb.vnear);
       FMMPC_LAUNCH_CHECK();
       ++launches;
-      FMMPC_CUDA(cudaEventRecord(H.sev[6], H.sstream2));
     }
+    if (bc_tab) boundary_data(H.sstream2);
+    if (split_colloc || bc_tab) FMMPC_CUDA(cudaEventRecord(H.sev[6], H.sstream2));
   }
   mark(1);
   launches += run_upward<R, P>(H, nrhs, s);
-  if (m2l_side) {  // its own stream, so that it need not wait for the near field
+  if (side) {  // its own stream, so that it need not wait for the near field
     FMMPC_CUDA(cudaEventRecord(H.sev[1], s));
     FMMPC_CUDA(cudaStreamWaitEvent(H.sstream3, H.sev[1], 0));
-    launches += run_m2l_tc(H, Mv, Lv, nrhs, H.sstream3);
+    volume_m2l(H.sstream3);
     FMMPC_CUDA(cudaEventRecord(H.sev[5], H.sstream3));
+    if (tc) {
+      // the tensor-core near field fills the SMs' shared memory: started with the upward pass, which
+      // the whole chain waits for, it doubles that pass's time (16 -> 31 us at 1024^2), so it starts
+      // after it (1024^2 apply 131 -> 123 us); the CUDA-core one, of small grids, is longer than its
+      // slack and starts at once (128^2: 54 -> 50 us)
+      FMMPC_CUDA(cudaStreamWaitEvent(ss, H.sev[1], 0));
+      near_field(ss);
+    }
   }
   if (with_bnd) {
     mark(2);
@@ -1919,7 +1975,7 @@ void apply_impl(fmmpc_handle &H, int part, const double *r, double *out, int nrh
       k_colloc_T<R><<<(unsigned)((int64_t)g.n * nrhs), 128, 0, s>>>(g, wpad, Lb, Ls.pvb_first, Ls.pvb_src, H.fb.kcolT,
                                                                     H.fb.wfarT, H.fb.vcol);
     else {
-      if (split_colloc) FMMPC_CUDA(cudaStreamWaitEvent(s, H.sev[6], 0));
+      if (split_colloc) FMMPC_CUDA(cudaStreamWaitEvent(s, H.sev[6], 0));  // and the boundary data's
       k_colloc<R><<<(unsigned)((int64_t)g.n * nrhs), 128, 0, s>>>(g, nrhs, wpad, Lb, Ls.pvb_first, Ls.pvb_src,
                                                                  H.fb.vcol, (const R *)H.fb.kcol, vt_f2 ? H.fb.vt_hi : nullptr,
                                                                  vt_f2 ? H.fb.vt_lo : nullptr, split_colloc ? 2 : 0,
@@ -1927,11 +1983,9 @@ void apply_impl(fmmpc_handle &H, int part, const double *r, double *out, int nrh
     }
     FMMPC_LAUNCH_CHECK();
     launches += 2;
-    if (bc_tab) {  // -(1/2 I + K) g, added to vcol where its side DFT is taken
-      k_bem_vt<<<nblk((int64_t)nrhs * g.n), 256, 0, s>>>(g.n, nrhs, H.bc_g, nullptr, H.bc_vt);
-      k_bem_apply<<<g.n / BEM64_ROWS, 64 * BEM64_ROWS, 0, s>>>(g.n, nrhs, H.Kbc, H.bc_vt, H.bc_kg);
-      FMMPC_LAUNCH_CHECK();
-      launches += 2;
+    if (bc_tab) {
+      if (!side) boundary_data(s);
+      else if (!split_colloc) FMMPC_CUDA(cudaStreamWaitEvent(s, H.sev[6], 0));
     } else if (bc) {  // vcol -= (1/2 I + K) g: Eq. e:ubound's data term
       k_dl_colloc<<<dim3((unsigned)g.NG, nrhs), 256, 0, s>>>(g.n, nrhs, H.bc_g, H.fb.vcol);
       FMMPC_LAUNCH_CHECK();
@@ -1993,9 +2047,6 @@ void apply_impl(fmmpc_handle &H, int part, const double *r, double *out, int nrh
     FMMPC_LAUNCH_CHECK();
     ++launches;
   }
-  // with the tensor-core M2L (L >= 2) the boundary-source part of the volume locals is kept
-  // apart for the downward pass to add, so it can run while the volume M2L still runs
-  const bool vbv_sep = std::is_same<R, float>::value && H.tcm.enabled && with_bnd && Ls.n_vbv_cells > 0;
   auto run_vbv_sep = [&]() {
     k_m2l_vbv<R, P><<<nblk(Ls.n_vbv_cells * nrhs * 8), 256, 0, s>>>(gd, g.ncell, g.nbcell, nrhs, Ls.vbv_first,
                                                                      Ls.vbv_src, Mb, Lv, Ls.vbv_cells,
@@ -2007,21 +2058,12 @@ void apply_impl(fmmpc_handle &H, int part, const double *r, double *out, int nrh
     if (vbv_sep) run_vbv_sep();
     FMMPC_CUDA(cudaEventRecord(H.sev[2], ss));
     FMMPC_CUDA(cudaStreamWaitEvent(s, H.sev[2], 0));
-    if (m2l_side) FMMPC_CUDA(cudaStreamWaitEvent(s, H.sev[5], 0));
+    FMMPC_CUDA(cudaStreamWaitEvent(s, H.sev[5], 0));
   }
   mark(5);
-  if (std::is_same<R, float>::value && H.tcm.enabled) {
-    // volume-to-volume M2L on the tensor cores (mixed forms); boundary sources added after
-    if (!m2l_side) launches += run_m2l_tc(H, Mv, Lv, nrhs, s);
-    mark(6);
-    if (vbv_sep && !side) run_vbv_sep();
-  } else {
-    k_m2l_vol<R, P><<<nblk(g.ncell * nrhs * 32), 256, 0, s>>>(gd, g.ncell, g.nbcell, nrhs, 1, with_bnd ? 1 : 0, 0,
-                                                             Ls.m2l_first, Ls.m2l_src, Ls.vbv_first, Ls.vbv_src,
-                                                             Mv, Mb, Lv);
-    ++launches;
-    mark(6);  // closes the M2L stage (its boundary sources are inside this kernel)
-  }
+  if (!side) volume_m2l(s);
+  mark(6);
+  if (vbv_sep && !side) run_vbv_sep();
   if (g.L < 2) {  // else the downward kernel adds the root constant
     k_root_const<R><<<1, 32, 0, s>>>(P, g.ncell, g.nbcell, nrhs, g.lnh, with_bnd ? 2 : 1, Mv, Mb, Lv, Lb);
     FMMPC_LAUNCH_CHECK();
@@ -2035,19 +2077,11 @@ void apply_impl(fmmpc_handle &H, int part, const double *r, double *out, int nrh
   }
   mark(9);
   const int do_bnd = (with_bnd && Ls.nbnear > 0) ? 1 : 0;
-  const float *n1 = nullptr, *n2 = nullptr;
-  if (tc) {
-    if (!side) launches += run_p2p_tc(H, false, out, nrhs, s);
-    n1 = H.tcp.near1;
-    n2 = H.tcp.near2;
-  } else {
-    run_p2p<R>(H, H.fb.table, out, nrhs, s);  // writes the near field into out
-    ++launches;
-  }
+  if (!side) near_field(s);
   if (side && Ls.nbnear > 0) FMMPC_CUDA(cudaStreamWaitEvent(s, H.sev[4], 0));
   mark(10);
-  if (g.L >= 2) run_downward<R, P>(H, out, nrhs, do_bnd, with_bnd ? 1 : 0, s, n1, n2, vbv_sep);
-  else run_far_final<R>(H, out, nrhs, do_bnd, s, n1, n2);
+  if (g.L >= 2) run_downward<R, P>(H, out, nrhs, do_bnd, with_bnd ? 1 : 0, s, tc, vbv_sep);
+  else run_far_final<R>(H, out, nrhs, do_bnd, s);
   ++launches;
   mark_end();
   H.launches = launches;

@@ -2,6 +2,7 @@
 // workspace.  Shared by api.cu, fmm.cu and krylov.cu.
 #pragma once
 
+#include <array>
 #include <string>
 
 #include "common.cuh"
@@ -56,8 +57,24 @@ struct TcP2P {
   int row_oy[33] = {}, row_q0[33] = {}, row_q1[33] = {}, row_ox0[33] = {};
   uint16_t *ahi = nullptr, *alo = nullptr;        // FP16 weight strips (scaled), hi and lo words
   uint16_t *bmat = nullptr, *bmat_lnh = nullptr;  // FP16 kernel tables, hi and lo words
-  float *near1 = nullptr, *near2 = nullptr;  // the two halves of the near-field sum, FP32 images
+  float *near = nullptr;                     // [part][nrhs][n][n] the two parts of the near-field sum, FP32
+  int nparts = 2;
+  int64_t part_stride = 0;
   float *lsc = nullptr;                      // [nrhs][NLY][NLX] 2^-e of each leaf's FP16 weights
+  int *err = nullptr;
+};
+
+// the FP64 form's tensor-core lattice P2P (p2p_f64.cu)
+struct OzP2P {
+  bool enabled = false;
+  int P = 0, ntiles = 0, nparts = 1, nbs = 0, sh = 0, nsr = 0, smem = 0, nrows = 0;
+  int row_oy[33] = {}, row_ox0[33] = {}, row_cnt[33] = {};
+  int part_r[8] = {}, part_q[8] = {}, part_n[8] = {}, part_o[8] = {}, eb[2] = {};
+  int64_t rows = 0, part_stride = 0;
+  uint16_t *img = nullptr;              // [nrhs][digit][rows][64] digit rows of the leaves
+  int2 *lexp = nullptr;                 // [nrhs][rows] exponent of each leaf's weights and their L1 norm / 2^E
+  unsigned char *bmat[2] = {};          // table digits without and with ln h
+  double *near = nullptr;               // [part][nrhs][n][n] parts of the sums (several parts only)
   int *err = nullptr;
 };
 
@@ -77,6 +94,26 @@ struct TcM2L {
   int2 *tiles = nullptr;
   int4 *groups = nullptr;
   int *dxs = nullptr, *err = nullptr;
+};
+
+// the FP64 form's tensor-core M2L (m2l_f64.cu)
+struct OzM2L {
+  bool enabled = false;
+  int width = 32, ntiles = 0, nparts = 1, part_s[2][5] = {}, lev_P[24] = {}, rb[34] = {};
+  int64_t rows = 0, lev_row0[24] = {}, part_stride = 0;
+  unsigned char *img = nullptr, *bmat = nullptr;
+  int2 *lexp = nullptr, *tiles = nullptr;
+  int4 *shifts = nullptr;
+  double *Lp = nullptr;  // [part][nrhs][ncell][p] complex parts of L~
+  int *err = nullptr;
+};
+
+// shifts (source parity, dy, dx) of the lattice M2L by (source parity, dy) group, with the offset
+// that each parity class translates over it (index (oy + 7) 15 + ox + 7, -1: none)
+struct M2lShifts {
+  std::vector<int4> groups;  // (source parity, dy, first shift, count)
+  std::vector<int> dxs;
+  std::vector<std::array<int, 4>> shift_ofs;
 };
 
 struct GraphEntry {
@@ -128,7 +165,7 @@ struct fmmpc_handle {
   fmmpc::TreeOut tree{};
   fmmpc::Lists lists{};
   fmmpc::FmmBufs fb{};
-  double *Sinv = nullptr;   // [n][4n] first block row of the FP64 inverse of the single-layer matrix
+  double *Sinv = nullptr;   // [n/2][4n] FP64 inverse of the single-layer matrix, folded form (bem.cu)
   double *Kdl_inv = nullptr;  // the same for -1/2 I + K (double-layer correction), made on first use
   double *SinvT = nullptr;    // the same for S^T (the transpose pass), made on first use
   float *Kdl_hi = nullptr, *Kdl_lo = nullptr;  // and as two FP32 words (single-precision forms)
@@ -141,7 +178,9 @@ struct fmmpc_handle {
   double *stage_in = nullptr, *stage_out = nullptr, *stage_g = nullptr;  // device staging for *_host calls
   fmmpc::KrylovWs kw{};
   fmmpc::TcP2P tcp{};
+  fmmpc::OzP2P ozp{};
   fmmpc::TcM2L tcm{};
+  fmmpc::OzM2L ozm{};
   int p2p_engine = 0;       // 0: tensor cores where eligible, 1: CUDA cores
   // operator of the Krylov solves (fmmpc_set_operator): 0 five-point, 1 five-point with the
   // coefficient acoef [(n+2)^2], 2 Q1 stiffness (q1tab: Thomas coefficients of the mass solve)
@@ -195,11 +234,19 @@ int solve(fmmpc_handle &H, const double *f, const double *g, double *u, int nrhs
 bool tc_p2p_eligible(const fmmpc_handle &H);
 void init_tc_p2p(fmmpc_handle &H);
 int prep_p2p_tc(fmmpc_handle &H, const double *r, int nrhs, cudaStream_t s, float *wimg);
+bool oz_p2p_eligible(const fmmpc_handle &H);
+void init_p2p_oz(fmmpc_handle &H);
+int prep_p2p_oz(fmmpc_handle &H, const double *r, int nrhs, cudaStream_t s, double *wimg);
+int run_p2p_oz(fmmpc_handle &H, bool with_lnh, double *out, int nrhs, cudaStream_t s);
+int add_near_oz(fmmpc_handle &H, double *out, int nrhs, cudaStream_t s);
+bool m2l_shift_sets(fmmpc_handle &H, DevPool &tmp, M2lShifts &out);
+void init_m2l_oz(fmmpc_handle &H, DevPool &tmp);
+int run_m2l_oz(fmmpc_handle &H, const void *Mv, void *Lv, int nrhs, cudaStream_t s);
 bool tc_m2l_eligible(const fmmpc_handle &H);
 void init_tc_m2l(fmmpc_handle &H, DevPool &tmp);
 int run_m2l_tc(fmmpc_handle &H, const void *Mv, void *Lv, int nrhs, cudaStream_t s);
-int run_p2p_tc(fmmpc_handle &H, bool with_lnh, double *out, int nrhs, cudaStream_t s);
-int add_near2(fmmpc_handle &H, double *out, int nrhs, cudaStream_t s);
+int run_p2p_tc(fmmpc_handle &H, bool with_lnh, int nrhs, cudaStream_t s);
+int add_near(fmmpc_handle &H, double *out, int nrhs, cudaStream_t s);
 // message for fmmpc_last_error(NULL), kept in a fixed thread-local buffer; returns code
 int set_global_error(int code, const char *msg);
 int solve_batched(std::vector<fmmpc_handle *> &hs, const double *const *f, const double *const *gb,

@@ -486,6 +486,51 @@ float tf32_round_host_m2l(double v) {
 
 }  // namespace
 
+// The shifts of the volume M2L as a lattice convolution: the offset sets of the four parity classes,
+// taken from the M2L lists themselves; false if a list is not exactly its class's offsets.
+bool m2l_shift_sets(fmmpc_handle &H, DevPool &tmp, M2lShifts &out) {
+  const int L = H.g.L;
+  // offset sets by class, from the lists themselves, then checked against every list
+  int *dtab = tmp.get<int>(4 * 225), *derr = tmp.get<int>(1);
+  FMMPC_CUDA(cudaMemsetAsync(dtab, 0, sizeof(int) * 4 * 225, H.stream));
+  FMMPC_CUDA(cudaMemsetAsync(derr, 0, sizeof(int), H.stream));
+  const int64_t nt = level_offset(L + 1) - level_offset(2);
+  k_m2l_offsets<<<nblk(nt), 256, 0, H.stream>>>(L, H.lists.m2l_first, H.lists.m2l_src, dtab, derr);
+  k_m2l_verify<<<nblk(nt), 256, 0, H.stream>>>(L, H.lists.m2l_first, dtab, derr);
+  FMMPC_LAUNCH_CHECK();
+  std::vector<int> tab(4 * 225);
+  int herr = 0;
+  FMMPC_CUDA(cudaMemcpyAsync(tab.data(), dtab, sizeof(int) * 4 * 225, cudaMemcpyDeviceToHost, H.stream));
+  FMMPC_CUDA(cudaMemcpyAsync(&herr, derr, sizeof(int), cudaMemcpyDeviceToHost, H.stream));
+  FMMPC_CUDA(cudaStreamSynchronize(H.stream));
+  if (herr) return false;
+  // shifts (source parity, dy, dx) with the offset each class translates over it, grouped
+  // by (source parity, dy) and sorted by dx: target (i, j) of class c = (cx, cy) takes
+  // source cell 2 (i, j) + (cx, cy) - o, which sits in source parity sub-image
+  // ((cx - ox) & 1, (cy - oy) & 1) at (i + dx, j + dy), dx = floor((cx - ox) / 2)
+  std::map<std::pair<int, int>, std::map<int, std::array<int, 4>>> bykey;  // (sp, dy) -> dx -> offset per class
+  for (int c = 0; c < 4; ++c) {
+    const int cx = c & 1, cy = c >> 1;
+    for (int oy = -7; oy <= 7; ++oy)
+      for (int ox = -7; ox <= 7; ++ox) {
+        if (!tab[c * 225 + (oy + 7) * 15 + ox + 7]) continue;
+        const int spx = (cx - ox) & 1, spy = (cy - oy) & 1;
+        const int dx = (cx - ox - spx) / 2, dy = (cy - oy - spy) / 2;
+        auto &row = bykey[{spx + 2 * spy, dy}];
+        if (!row.count(dx)) row[dx] = {-1, -1, -1, -1};
+        row[dx][c] = (oy + 7) * 15 + ox + 7;
+      }
+  }
+  for (auto &kv : bykey) {
+    out.groups.push_back(make_int4(kv.first.first, kv.first.second, (int)out.dxs.size(), (int)kv.second.size()));
+    for (auto &e : kv.second) {
+      out.dxs.push_back(e.first);
+      out.shift_ofs.push_back(e.second);
+    }
+  }
+  return true;
+}
+
 bool tc_m2l_eligible(const fmmpc_handle &H) {
   // W <= 32 outputs per class hold 2p + 2; K (32 TF32 or BF16 inputs per 128-byte row) holds 2p
   return (H.prec == FMMPC_PREC_MIXED_BF16 || H.prec == FMMPC_PREC_MIXED_TF32) && H.g.L >= 2 && 2 * H.g.p + 2 <= 32;
@@ -507,47 +552,12 @@ void init_tc_m2l(fmmpc_handle &H, DevPool &tmp) {
   const int kcap = T.kind == 0 ? 32 : 48;
   T.sbase = 2 * p;
   T.nsplit = std::max(0, std::min(p, (kcap - T.sbase) / 4));
-  // offset sets by class, from the lists themselves, then checked against every list
-  int *dtab = tmp.get<int>(4 * 225), *derr = tmp.get<int>(1);
-  FMMPC_CUDA(cudaMemsetAsync(dtab, 0, sizeof(int) * 4 * 225, H.stream));
-  FMMPC_CUDA(cudaMemsetAsync(derr, 0, sizeof(int), H.stream));
-  const int64_t nt = level_offset(L + 1) - level_offset(2);
-  k_m2l_offsets<<<nblk(nt), 256, 0, H.stream>>>(L, H.lists.m2l_first, H.lists.m2l_src, dtab, derr);
-  k_m2l_verify<<<nblk(nt), 256, 0, H.stream>>>(L, H.lists.m2l_first, dtab, derr);
-  FMMPC_LAUNCH_CHECK();
-  std::vector<int> tab(4 * 225);
-  int herr = 0;
-  FMMPC_CUDA(cudaMemcpyAsync(tab.data(), dtab, sizeof(int) * 4 * 225, cudaMemcpyDeviceToHost, H.stream));
-  FMMPC_CUDA(cudaMemcpyAsync(&herr, derr, sizeof(int), cudaMemcpyDeviceToHost, H.stream));
-  FMMPC_CUDA(cudaStreamSynchronize(H.stream));
-  if (herr) throw Error(FMMPC_ERR_INVALID, "tensor-core M2L: the M2L lists are not translation invariant");
-  // shifts (source parity, dy, dx) with the offset each class translates over it, grouped
-  // by (source parity, dy) and sorted by dx: target (i, j) of class c = (cx, cy) takes
-  // source cell 2 (i, j) + (cx, cy) - o, which sits in source parity sub-image
-  // ((cx - ox) & 1, (cy - oy) & 1) at (i + dx, j + dy), dx = floor((cx - ox) / 2)
-  std::map<std::pair<int, int>, std::map<int, std::array<int, 4>>> bykey;  // (sp, dy) -> dx -> offset per class
-  for (int c = 0; c < 4; ++c) {
-    const int cx = c & 1, cy = c >> 1;
-    for (int oy = -7; oy <= 7; ++oy)
-      for (int ox = -7; ox <= 7; ++ox) {
-        if (!tab[c * 225 + (oy + 7) * 15 + ox + 7]) continue;
-        const int spx = (cx - ox) & 1, spy = (cy - oy) & 1;
-        const int dx = (cx - ox - spx) / 2, dy = (cy - oy - spy) / 2;
-        auto &row = bykey[{spx + 2 * spy, dy}];
-        if (!row.count(dx)) row[dx] = {-1, -1, -1, -1};
-        row[dx][c] = (oy + 7) * 15 + ox + 7;
-      }
-  }
-  std::vector<int4> groups;
-  std::vector<int> dxs;
-  std::vector<std::array<int, 4>> shift_ofs;
-  for (auto &kv : bykey) {
-    groups.push_back(make_int4(kv.first.first, kv.first.second, (int)dxs.size(), (int)kv.second.size()));
-    for (auto &e : kv.second) {
-      dxs.push_back(e.first);
-      shift_ofs.push_back(e.second);
-    }
-  }
+  M2lShifts sets;
+  if (!m2l_shift_sets(H, tmp, sets))
+    throw Error(FMMPC_ERR_INVALID, "tensor-core M2L: the M2L lists are not translation invariant");
+  const std::vector<int4> &groups = sets.groups;
+  const std::vector<int> &dxs = sets.dxs;
+  const std::vector<std::array<int, 4>> &shift_ofs = sets.shift_ofs;
   const int nshift = (int)dxs.size(), ngrp = (int)groups.size();
   // the 144-row window holds the 128 targets shifted by dx in [-4, 4]
   for (int dx : dxs)

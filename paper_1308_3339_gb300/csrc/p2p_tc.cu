@@ -426,8 +426,9 @@ void init_tc_p2p(fmmpc_handle &H) {
     }
     H.tcp.usplit = best;
   }
-  H.tcp.near1 = H.pool.get<float>((size_t)H.nrhs_max * g.n * g.n);
-  H.tcp.near2 = H.pool.get<float>((size_t)H.nrhs_max * g.n * g.n);
+  H.tcp.part_stride = (int64_t)H.nrhs_max * g.n * g.n;
+  H.tcp.nparts = 2;
+  H.tcp.near = H.pool.get<float>((size_t)2 * H.tcp.part_stride);
   H.tcp.lsc = H.pool.get<float>((size_t)H.nrhs_max * NL * NL);
   FMMPC_CUDA(cudaMemsetAsync(H.tcp.lsc, 0, sizeof(float) * H.nrhs_max * NL * NL, H.stream));  // padding leaves
   H.tcp.err = H.pool.get<int>(1);
@@ -449,16 +450,15 @@ int prep_p2p_tc(fmmpc_handle &H, const double *r, int nrhs, cudaStream_t s, floa
   return 1;
 }
 
-// out[...] = -near / (2 pi) on the tensor cores, from the strips prep_p2p_tc wrote.
-int run_p2p_tc(fmmpc_handle &H, bool with_lnh, double *out, int nrhs, cudaStream_t s) {
+// The two parts of the near field (raw sums) into tcp.near, from the strips prep_p2p_tc wrote.
+int run_p2p_tc(fmmpc_handle &H, bool with_lnh, int nrhs, cudaStream_t s) {
   const Geo &g = H.g;
   TcArgs a{};
   a.ahi = H.tcp.ahi;
   a.alo = H.tcp.alo;
   a.bmat = with_lnh ? H.tcp.bmat_lnh : H.tcp.bmat;
   a.lsc = H.tcp.lsc;
-  a.out1 = H.tcp.near1;
-  (void)out;
+  a.out1 = H.tcp.near;
   a.err = H.tcp.err;
   a.n = g.n;
   a.R = g.R;
@@ -468,7 +468,7 @@ int run_p2p_tc(fmmpc_handle &H, bool with_lnh, double *out, int nrhs, cudaStream
   a.nrows = H.tcp.nrows;
   a.nofs = H.tcp.nofs;
   a.usplit = H.tcp.usplit;
-  a.out2 = H.tcp.near2;
+  a.out2 = H.tcp.near + H.tcp.part_stride;
   a.npass = H.tcp.npass;
   for (int i = 0; i < a.nrows; ++i) {
     a.row_oy[i] = H.tcp.row_oy[i];
@@ -483,9 +483,9 @@ int run_p2p_tc(fmmpc_handle &H, bool with_lnh, double *out, int nrhs, cudaStream
 }
 
 // out = the two parts of the near field (PART_NEAR, where no L2P pass follows).
-int add_near2(fmmpc_handle &H, double *out, int nrhs, cudaStream_t s) {
+int add_near(fmmpc_handle &H, double *out, int nrhs, cudaStream_t s) {
   const int64_t total = (int64_t)H.g.n * H.g.n * nrhs;
-  k_near_combine<<<nblk(total), 256, 0, s>>>(total, H.tcp.near1, H.tcp.near2, out);
+  k_near_combine<<<nblk(total), 256, 0, s>>>(total, H.tcp.near, H.tcp.near + H.tcp.part_stride, out);
   FMMPC_LAUNCH_CHECK();
   return 1;
 }

@@ -1,5 +1,6 @@
 """Kernels and dispatch rules at the sizes where they can go wrong, each against the oracle or
-the general path: window edges of the Q1 mass solve."""
+the general path: window edges of the Q1 mass solve, tables formed on first use, and
+the FP64 form's tensor-core kernels."""
 import numpy as np
 import pytest
 
@@ -66,4 +67,69 @@ def test_first_apply_bc_under_capture_sums_directly(n, leaf_max, prec, nrhs):
         st.synchronize()
     tol = 1e-12 if prec == "fp64" else 1e-5
     check_close(f"apply_bc direct vs tables {prec} n={n}", ut.cpu().numpy(), u.cpu().numpy(), tol, tol)
+    P.close()
+
+
+@pytest.mark.parametrize("n,theta,nrhs", [(64, 0.4, 1), (64, 0.3, 2), (128, 0.5, 1), (256, 0.4, 3), (1024, 0.4, 1)])
+def test_fp64_tensor_core_near_field_matches_cuda_cores(n, theta, nrhs):
+    # 8-leaf rows (one partly filled tile) up to a part per CTA; the digit sums are exact, so the
+    # two differ by the CUDA-core kernel's FP64 rounding, ~1e-15 of sums of 37 x 64 terms (gates: ten
+    # times that, and again for the largest node)
+    from paper_1308_3339_gb300 import FmmPreconditioner
+    r = dev(np.stack([S.random_field(n, 80 + k) for k in range(nrhs)]))
+    P = FmmPreconditioner(n, p=8, theta=theta, precision="fp64", n_rhs=nrhs)
+    assert P.query("tc_p2p") == 1
+    a = P.apply_part("near", r).cpu().numpy()
+    za = P.apply(r).cpu().numpy()
+    assert P.query("device_errors") == 0
+    P.set_p2p_engine("simt")
+    b = P.apply_part("near", r).cpu().numpy()
+    zb = P.apply(r).cpu().numpy()
+    check_close(f"fp64 near n={n} theta={theta}", a, b, 1e-14, 1e-13)
+    check_close(f"fp64 apply n={n} theta={theta}", za, zb, 1e-13, 1e-12)
+    P.close()
+
+
+def test_fp64_tensor_core_near_field_scales_and_special_values():
+    # 20 decades between the halves: the small half alone; zero; and a NaN and an Inf reach exactly
+    # the target leaves whose stencil holds them, as on the CUDA cores
+    from paper_1308_3339_gb300 import FmmPreconditioner
+    n = 128
+    f = S.random_field(n, 3).reshape(n, n)
+    f[:, n // 2:] *= 1e-20
+    f[0, 0] = 5e-324
+    P = FmmPreconditioner(n, p=8, precision="fp64")
+    near = {}
+    for engine in ("tc", "simt"):
+        P.set_p2p_engine(engine)
+        near[engine] = P.apply_part("near", dev(f)).cpu().numpy().reshape(n, n)
+        assert not P.apply_part("near", dev(0 * f)).cpu().numpy().any()
+    small = slice(n // 2 + 32, n)
+    check_close("fp64 near, small half", near["tc"][:, small], near["simt"][:, small], 1e-14, 1e-13)
+    for bad in (np.nan, np.inf):
+        g = S.random_field(n, 4).reshape(n, n)
+        g[37, 70] = bad
+        out = {}
+        for engine in ("tc", "simt"):
+            P.set_p2p_engine(engine)
+            out[engine] = P.apply_part("near", dev(g)).cpu().numpy()
+        assert np.array_equal(np.isfinite(out["tc"]), np.isfinite(out["simt"]))
+    P.close()
+
+
+@pytest.mark.parametrize("p,leaf_max", [(4, 64), (12, 64), (12, 16)])
+def test_fp64_tensor_core_m2l_matches_oracle(p, leaf_max):
+    # both widths of the translation matrices, four and six levels, two right-hand sides, and 12
+    # decades between the quadrants' weights: V r within the FP64 form's bar (1e-12), and in the
+    # small quadrant's far corner relative to its own values
+    from paper_1308_3339_gb300 import FmmPreconditioner
+    n = 256
+    f = np.stack([S.random_field(n, 90), S.gaussian_mixture(n, 91)])
+    f[0].reshape(n, n)[n // 2:, n // 2:] *= 1e-12
+    P = FmmPreconditioner(n, p=p, leaf_max=leaf_max, precision="fp64", n_rhs=2)
+    vr = P.apply_part("vr", dev(f)).cpu().numpy().reshape(2, -1)
+    assert P.query("device_errors") == 0
+    R = O.Problem(n, p=p, leaf_max=leaf_max)
+    for k in range(2):
+        check_close(f"fp64 vr p={p} leaf={leaf_max} rhs={k}", vr[k], R.apply(f[k], "fmm", stages=True)["vr"], 1e-12, 1e-12)
     P.close()
