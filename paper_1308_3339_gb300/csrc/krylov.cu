@@ -9,6 +9,7 @@
 #include <algorithm>
 #include <chrono>
 #include <cmath>
+#include <type_traits>
 
 #include "handle.cuh"
 
@@ -22,14 +23,33 @@ constexpr int MAXJ = 64;         // largest Krylov basis handled by the fused ke
 
 inline unsigned nblk(int64_t n, int t = 256) { return (unsigned)((n + t - 1) / t); }
 
-// Blocks of a reduction grid: four per SM (enough loads in flight for the vector sweeps;
-// every further warp adds its own FP64 cross-lane sums, and FP64 issue is the scarce
-// resource of these kernels on this GPU).
-int red_blocks() {
+// Blocks of a reduction grid over N elements: four per SM (enough loads in flight for the vector
+// sweeps; every further warp adds its own FP64 cross-lane sums, and FP64 issue is the scarce
+// resource of these kernels on this GPU), and no more than the elements fill two at a time: on a
+// 64^2 grid 608 blocks for 2048 pairs left the last block 608 partials to add.
+int red_blocks(int64_t N) {
   int dev = 0, nsm = 0;
   FMMPC_CUDA(cudaGetDevice(&dev));
   FMMPC_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
-  return std::min(std::max(4 * nsm, 1), RED_BLOCKS);
+  const int64_t fill = (N / 2 + RED_THREADS - 1) / RED_THREADS;
+  return (int)std::max<int64_t>(1, std::min<int64_t>({4 * (int64_t)nsm, fill, RED_BLOCKS}));
+}
+
+// f(integral_constant<int, k>) for a block-uniform k in [1, 8]: the FP64 loops over a group of
+// vectors are compiled for each count.  (As one loop of eight predicated steps, the multiply-adds of
+// absent vectors still took the FP64 pipe: the norm of one 1024^2 vector 19.8 us.)
+template <typename F>
+__device__ __forceinline__ void with_count8(int k, F &&f) {
+  switch (k) {
+    case 1: f(std::integral_constant<int, 1>{}); break;
+    case 2: f(std::integral_constant<int, 2>{}); break;
+    case 3: f(std::integral_constant<int, 3>{}); break;
+    case 4: f(std::integral_constant<int, 4>{}); break;
+    case 5: f(std::integral_constant<int, 5>{}); break;
+    case 6: f(std::integral_constant<int, 6>{}); break;
+    case 7: f(std::integral_constant<int, 7>{}); break;
+    default: f(std::integral_constant<int, 8>{}); break;
+  }
 }
 
 // The operator A of the solves (fmmpc_set_operator), zero Dirichlet values outside the
@@ -82,9 +102,35 @@ __device__ __forceinline__ double op_at(const OpDev &o, const double *__restrict
   return o.s * fma(4.0, x[t], -((xw + xe) + (xs + xn)));
 }
 
+// A x at elements 2k and 2k + 1 of one right-hand side (n is even: the same grid row), c = x there.
+// For the five-point stencil five loads a pair, three of them 16 bytes wide.
+__device__ __forceinline__ double2 op_pair(const OpDev &o, const double *__restrict__ x, int64_t base, int64_t k,
+                                           double2 &c) {
+  const int64_t t = base + 2 * k;
+  c = *reinterpret_cast<const double2 *>(x + t);
+  if (o.op != 0) return make_double2(op_at(o, x, t), op_at(o, x, t + 1));
+  const int n = o.n, i = (int)((2 * k) & (n - 1));
+  const int64_t N = (int64_t)n * n;
+  const double2 zero = make_double2(0.0, 0.0);
+  const double xw = i > 0 ? x[t - 1] : 0.0, xe = i < n - 2 ? x[t + 2] : 0.0;
+  const double2 xs = 2 * k >= n ? *reinterpret_cast<const double2 *>(x + t - n) : zero;
+  const double2 xn = 2 * k < N - n ? *reinterpret_cast<const double2 *>(x + t + n) : zero;
+  return make_double2(o.s * fma(4.0, c.x, -((xw + c.y) + (xs.x + xn.x))),
+                      o.s * fma(4.0, c.y, -((c.x + xe) + (xs.y + xn.y))));
+}
+
+// PAIR: two elements a thread (x and y 16-byte aligned), else one.
+template <bool PAIR>
 __global__ void k_spmv5(OpDev o, int64_t total, const double *__restrict__ x, double *__restrict__ y) {
-  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t < total) y[t] = op_at(o, x, t);
+  const int64_t t = (PAIR ? 2 : 1) * ((int64_t)blockIdx.x * blockDim.x + threadIdx.x);
+  if (t >= total) return;
+  if (PAIR) {
+    const int64_t N = (int64_t)o.n * o.n, k = t & (N - 1);
+    double2 c;
+    *reinterpret_cast<double2 *>(y + t) = op_pair(o, x, t - k, k >> 1, c);
+  } else {
+    y[t] = op_at(o, x, t);
+  }
 }
 
 // Right-hand side of A u = b: op 0, b = f + g / h^2 at the stencil neighbours outside the
@@ -197,25 +243,43 @@ __global__ void __launch_bounds__(MS_THREADS) k_mass_sweep(int n, int64_t lines,
   }
 }
 
-// acc[q] += <V_{i0+q}, w> (q < 8, i0 + q < nv; with self, index nv is <w, w>) over this
-// thread's share of the N elements of one right-hand side, two elements per load (N is even
-// and every vector starts 16-byte aligned).  Vr and wr point at that right-hand side.
+// acc[q] += <V_{i0+q}, w>, q < NQ (with self, the last of them is <w, w>), over this thread's share
+// of the N elements of one right-hand side, two elements per load (N is even and every vector
+// starts 16-byte aligned).  Vr and wr point at that right-hand side.
+template <int NQ>
 __device__ __forceinline__ void mdot_chunk(int64_t N, const double *__restrict__ Vr, int64_t vs,
-                                           const double *__restrict__ wr, int i0, int nv, bool with_self,
-                                           double (&acc)[8]) {
+                                           const double *__restrict__ wr, int i0, bool self, double (&acc)[8]) {
   const int64_t N2 = N >> 1;
   const double2 *w2 = reinterpret_cast<const double2 *>(wr);
   for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < N2; k += (int64_t)gridDim.x * blockDim.x) {
     const double2 wk = w2[k];
+    double2 v[NQ];
 #pragma unroll
-    for (int q = 0; q < 8; ++q) {
-      if (i0 + q < nv) {
-        const double2 v = reinterpret_cast<const double2 *>(Vr + (int64_t)(i0 + q) * vs)[k];
-        acc[q] = fma(v.x, wk.x, fma(v.y, wk.y, acc[q]));
-      } else if (with_self && i0 + q == nv) {
-        acc[q] = fma(wk.x, wk.x, fma(wk.y, wk.y, acc[q]));
-      }
+    for (int q = 0; q < NQ; ++q)
+      v[q] = (q == NQ - 1 && self) ? wk : reinterpret_cast<const double2 *>(Vr + (int64_t)(i0 + q) * vs)[k];
+#pragma unroll
+    for (int q = 0; q < NQ; ++q) acc[q] = fma(v[q].x, wk.x, fma(v[q].y, wk.y, acc[q]));
+  }
+}
+
+// v -= sum_{i < nv} c[i] V_i at element pair k, four loads at a time
+__device__ __forceinline__ void update_pair(const double *__restrict__ Vr, int64_t vs, int64_t k,
+                                            const double *__restrict__ c, int nv, double2 &v) {
+  int i = 0;
+  for (; i + 4 <= nv; i += 4) {
+    double2 b[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) b[q] = reinterpret_cast<const double2 *>(Vr + (int64_t)(i + q) * vs)[k];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      v.x = fma(-c[i + q], b[q].x, v.x);
+      v.y = fma(-c[i + q], b[q].y, v.y);
     }
+  }
+  for (; i < nv; ++i) {
+    const double2 b = reinterpret_cast<const double2 *>(Vr + (int64_t)i * vs)[k];
+    v.x = fma(-c[i], b.x, v.x);
+    v.y = fma(-c[i], b.y, v.y);
   }
 }
 
@@ -228,11 +292,7 @@ __device__ __forceinline__ double update_chunk(int64_t N, const double *__restri
   double sq = 0.0;
   for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < N2; k += (int64_t)gridDim.x * blockDim.x) {
     double2 v = w2[k];
-    for (int i = 0; i < nv; ++i) {
-      const double2 b = reinterpret_cast<const double2 *>(Vr + (int64_t)i * vs)[k];
-      v.x = fma(-c[i], b.x, v.x);
-      v.y = fma(-c[i], b.y, v.y);
-    }
+    update_pair(Vr, vs, k, c, nv, v);
     w2[k] = v;
     sq = fma(v.x, v.x, fma(v.y, v.y, sq));
   }
@@ -315,8 +375,10 @@ __global__ void __launch_bounds__(RED_THREADS) k_mdot_partial(int64_t N, int nv,
     double acc[8];
 #pragma unroll
     for (int q = 0; q < 8; ++q) acc[q] = 0.0;
-    mdot_chunk(N, V + (int64_t)rhs * N, vs, wr, i0, nv, with_self != 0, acc);
     const int nq = min(8, nt - i0);
+    with_count8(nq, [&](auto q) {
+      mdot_chunk<q()>(N, V + (int64_t)rhs * N, vs, wr, i0, with_self != 0 && i0 + nq == nt, acc);
+    });
     block_sum8(acc, nq, red);
     if (threadIdx.x < nq) part[((int64_t)rhs * MAXJ + i0 + threadIdx.x) * gridDim.x + blockIdx.x] = red[threadIdx.x];
     __syncthreads();
@@ -500,7 +562,7 @@ void ensure_ws(fmmpc_handle &H, int64_t nvec, bool flexible) {
 // with_self: out[rhs][nv] = <w, w> as well (not accumulated into acc)
 void mdot(Ctx &c, int nv, const double *V, int64_t vs, const double *w, double *out, double *acc,
           bool with_self = false) {
-  const int nb = red_blocks();
+  const int nb = red_blocks(c.N);
   k_mdot_partial<<<dim3(nb, c.nrhs), RED_THREADS, 0, c.s>>>(c.N, nv, V, vs, w, c.H.kw.part, with_self ? 1 : 0);
   const int nt = nv + (with_self ? 1 : 0);
   k_mdot_final<<<dim3(c.nrhs, (nt + 7) / 8), 256, 0, c.s>>>(nt, nb, c.H.kw.part, out, acc, nv);
@@ -509,7 +571,7 @@ void mdot(Ctx &c, int nv, const double *V, int64_t vs, const double *w, double *
 
 // w -= V coef (nv vectors), then out[rhs][0] = ||w||^2
 void update_sq(Ctx &c, int nv, const double *V, int64_t vs, const double *coef, double *w, double *out) {
-  const int nb = red_blocks();
+  const int nb = red_blocks(c.N);
   k_mupdate_sq<<<dim3(nb, c.nrhs), RED_THREADS, 0, c.s>>>(c.N, nv, V, vs, coef, w, c.H.kw.part);
   k_mdot_final<<<dim3(c.nrhs, 1), 256, 0, c.s>>>(1, nb, c.H.kw.part, out, nullptr, 0);
   FMMPC_LAUNCH_CHECK();
@@ -750,7 +812,10 @@ int pcg(Ctx &c, int maxit, double rtol, const double *b, double *x, fmmpc_solve_
 
 void spmv5(fmmpc_handle &H, const double *x, double *y, int nrhs) {
   const int64_t total = (int64_t)H.g.n * H.g.n * nrhs;
-  k_spmv5<<<nblk(total), 256, 0, H.stream>>>(op_of(H), total, x, y);
+  if (((uintptr_t)x | (uintptr_t)y) & 15)  // a caller's vectors need only be FP64-aligned
+    k_spmv5<false><<<nblk(total), 256, 0, H.stream>>>(op_of(H), total, x, y);
+  else
+    k_spmv5<true><<<nblk(total / 2), 256, 0, H.stream>>>(op_of(H), total, x, y);
   FMMPC_LAUNCH_CHECK();
 }
 
@@ -1089,30 +1154,29 @@ __global__ void __launch_bounds__(RED_THREADS) k_gapdots(const int *__restrict__
   const int rhs = blockIdx.y, j = ctl[KC_J], nv = j + 1;
   const int64_t N2 = N >> 1, base = (int64_t)rhs * N;
   double2 *w2 = reinterpret_cast<double2 *>(w + base);
-  const double2 *x2 = reinterpret_cast<const double2 *>(x + base);
   double2 *z2 = Zb ? reinterpret_cast<double2 *>(Zb + (int64_t)j * vs + base) : nullptr;
   for (int i0 = 0; i0 < nv; i0 += 8) {
     double acc[8];
 #pragma unroll
     for (int q = 0; q < 8; ++q) acc[q] = 0.0;
-    for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < N2; k += (int64_t)gridDim.x * blockDim.x) {
-      double2 wk;
-      if (i0 == 0) {
-        wk.x = op_at(o, x, base + 2 * k);
-        wk.y = op_at(o, x, base + 2 * k + 1);
-        w2[k] = wk;
-        if (z2) z2[k] = x2[k];
-      } else {
-        wk = w2[k];
-      }
-#pragma unroll
-      for (int q = 0; q < 8; ++q)
-        if (i0 + q < nv) {
-          const double2 v = reinterpret_cast<const double2 *>(V + (int64_t)(i0 + q) * vs + base)[k];
-          acc[q] = fma(v.x, wk.x, fma(v.y, wk.y, acc[q]));
-        }
-    }
     const int nq = min(8, nv - i0);
+    with_count8(nq, [&](auto nqc) {
+      constexpr int NQ = nqc();
+      for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < N2; k += (int64_t)gridDim.x * blockDim.x) {
+        double2 v[NQ], wk, c;
+#pragma unroll
+        for (int q = 0; q < NQ; ++q) v[q] = reinterpret_cast<const double2 *>(V + (int64_t)(i0 + q) * vs + base)[k];
+        if (i0 == 0) {
+          wk = op_pair(o, x, base, k, c);
+          w2[k] = wk;
+          if (z2) z2[k] = c;
+        } else {
+          wk = w2[k];
+        }
+#pragma unroll
+        for (int q = 0; q < NQ; ++q) acc[q] = fma(v[q].x, wk.x, fma(v[q].y, wk.y, acc[q]));
+      }
+    });
     block_sum8(acc, nq, red);
     if (threadIdx.x < nq) part[((int64_t)rhs * MAXJ + i0 + threadIdx.x) * gridDim.x + blockIdx.x] = red[threadIdx.x];
     __syncthreads();
@@ -1125,7 +1189,7 @@ __global__ void __launch_bounds__(RED_THREADS) k_gapdots(const int *__restrict__
 
 // The middle of CGS2 in one pass: w -= sum_{i <= j} c[rhs][i] V_i (c the first pass's
 // coefficients, in the order of update_chunk), then d[rhs][i] = <V_i, w> (hsum += d): one
-// sweep over the basis from memory, the second pass's reads served by L1 and L2.
+// sweep over the basis, a group of eight vectors held in registers for both.
 __global__ void __launch_bounds__(RED_THREADS) k_gupdots(const int *__restrict__ ctl, int64_t N, const double *__restrict__ V,
                                                          int64_t vs, const double *__restrict__ c, double *__restrict__ w,
                                                          double *__restrict__ part, int *__restrict__ cnt,
@@ -1139,25 +1203,26 @@ __global__ void __launch_bounds__(RED_THREADS) k_gupdots(const int *__restrict__
     double acc[8];
 #pragma unroll
     for (int q = 0; q < 8; ++q) acc[q] = 0.0;
-    for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < N2; k += (int64_t)gridDim.x * blockDim.x) {
-      double2 wk = w2[k];
-      if (i0 == 0) {
-        for (int i = 0; i < nv; ++i) {
-          const double2 b = reinterpret_cast<const double2 *>(V + (int64_t)i * vs + base)[k];
-          wk.x = fma(-cr[i], b.x, wk.x);
-          wk.y = fma(-cr[i], b.y, wk.y);
-        }
-        w2[k] = wk;
-      }
-      // the second pass rereads V_i, which the update just brought into L1
-#pragma unroll
-      for (int q = 0; q < 8; ++q)
-        if (i0 + q < nv) {
-          const double2 v = reinterpret_cast<const double2 *>(V + (int64_t)(i0 + q) * vs + base)[k];
-          acc[q] = fma(v.x, wk.x, fma(v.y, wk.y, acc[q]));
-        }
-    }
     const int nq = min(8, nv - i0);
+    with_count8(nq, [&](auto nqc) {
+      constexpr int NQ = nqc();
+      for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < N2; k += (int64_t)gridDim.x * blockDim.x) {
+        double2 v[NQ], wk = w2[k];
+#pragma unroll
+        for (int q = 0; q < NQ; ++q) v[q] = reinterpret_cast<const double2 *>(V + (int64_t)(i0 + q) * vs + base)[k];
+        if (i0 == 0) {  // the update: this group's vectors from registers, then the others
+#pragma unroll
+          for (int q = 0; q < NQ; ++q) {
+            wk.x = fma(-cr[q], v[q].x, wk.x);
+            wk.y = fma(-cr[q], v[q].y, wk.y);
+          }
+          if (nv > NQ) update_pair(V + (int64_t)NQ * vs + base, vs, k, cr + NQ, nv - NQ, wk);
+          w2[k] = wk;
+        }
+#pragma unroll
+        for (int q = 0; q < NQ; ++q) acc[q] = fma(v[q].x, wk.x, fma(v[q].y, wk.y, acc[q]));
+      }
+    });
     block_sum8(acc, nq, red);
     if (threadIdx.x < nq) part[((int64_t)rhs * MAXJ + i0 + threadIdx.x) * gridDim.x + blockIdx.x] = red[threadIdx.x];
     __syncthreads();
@@ -1229,44 +1294,60 @@ __global__ void k_grestart(int *__restrict__ ctl, GmState st, int nrhs, const do
 // |w| (wsq), the previous rotations, a new rotation, the residual estimate |g_{j+1}| / |b|,
 // the scale of V_{j+1}; the cycle ends when every right-hand side is within rtol (or has
 // a zero |w|), at j + 1 = m, at maxit, or on a NaN; then y from the triangular system.
-// Sets the condition of the end-of-cycle IF node.  Run by all threads of one block (one
-// thread per right-hand side, nrhs <= blockDim.x).
+// Sets the condition of the end-of-cycle IF node.  Run by all threads of one block.
 __device__ __forceinline__ void gtail_run(int *__restrict__ ctl, GmState st, int nrhs, int m,
                                           const double *__restrict__ hsum, const double *__restrict__ wsq,
                                           double *__restrict__ y, cudaGraphConditionalHandle if_end) {
   __shared__ int s_ok, s_nan, s_cyc;
-  const int r = threadIdx.x;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
   const int j = ctl[KC_J], it = ctl[KC_IT] + 1;
-  if (r == 0) { s_ok = 1; s_nan = 0; }
+  if (threadIdx.x == 0) { s_ok = 1; s_nan = 0; }
   __syncthreads();
-  if (r < nrhs) {
+  // a warp per right-hand side: lane i holds entries i and i + 32 of the column and the rotations,
+  // loaded at once; the serial recurrence runs on shuffles instead of memory round trips
+  for (int r = wid; r < nrhs; r += nw) {
     double *Hr = st.Hm + (int64_t)r * (MAXJ + 1) * MAXJ;
     double *cs = st.cs + r * MAXJ, *sn = st.sn + r * MAXJ, *g = st.g + r * (MAXJ + 1);
-    for (int i = 0; i <= j; ++i) Hr[i * MAXJ + j] = hsum[r * MAXJ + i];
-    const double hn = sqrt(fmax(0.0, wsq[r * MAXJ]));
-    Hr[(j + 1) * MAXJ + j] = hn;
-    for (int i = 0; i < j; ++i) {
-      const double a = Hr[i * MAXJ + j], b = Hr[(i + 1) * MAXJ + j];
-      Hr[i * MAXJ + j] = cs[i] * a + sn[i] * b;
-      Hr[(i + 1) * MAXJ + j] = -sn[i] * a + cs[i] * b;
+    double hv[2], cv[2], sv[2], rot[2] = {0.0, 0.0};
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      const int i = lane + 32 * q;
+      hv[q] = i <= j ? __ldcg(hsum + r * MAXJ + i) : 0.0;
+      cv[q] = i < j ? cs[i] : 0.0;
+      sv[q] = i < j ? sn[i] : 0.0;
     }
-    const double a = Hr[j * MAXJ + j], b = Hr[(j + 1) * MAXJ + j], rr = hypot(a, b);
-    if (rr == 0.0) { cs[j] = 1.0; sn[j] = 0.0; }
-    else { cs[j] = a / rr; sn[j] = b / rr; }
-    Hr[j * MAXJ + j] = rr;
-    Hr[(j + 1) * MAXJ + j] = 0.0;
-    g[j + 1] = -sn[j] * g[j];
-    g[j] = cs[j] * g[j];
-    const double est = fabs(g[j + 1]) / st.bn[r];
-    if (!isfinite(est)) atomicOr(&s_nan, 1);
-    const int done = st.done[r];
-    if (!done) st.iters[r] = it;
-    const bool ok = done || est <= st.rtol[0] || hn == 0.0;
-    if (!ok) atomicAnd(&s_ok, 0);
-    st.sc[r] = (hn > 0.0 && !done) ? 1.0 / hn : 0.0;
+    const double hn = sqrt(fmax(0.0, __ldcg(wsq + r * MAXJ)));
+    auto pick = [&](const double(&v)[2], int i) { return __shfl_sync(0xffffffffu, i < 32 ? v[0] : v[1], i & 31); };
+    double a = pick(hv, 0);
+    for (int i = 0; i < j; ++i) {
+      const double b = pick(hv, i + 1), c = pick(cv, i), sn_i = pick(sv, i);
+      const double hi = c * a + sn_i * b;
+      a = -sn_i * a + c * b;
+      if (lane == (i & 31)) rot[i >> 5] = hi;
+    }
+    const double rr = hypot(a, hn), cj = rr == 0.0 ? 1.0 : a / rr, sj = rr == 0.0 ? 0.0 : hn / rr;
+#pragma unroll
+    for (int q = 0; q < 2; ++q)
+      if (lane + 32 * q < j) Hr[(lane + 32 * q) * MAXJ + j] = rot[q];
+    if (lane == 0) {
+      Hr[j * MAXJ + j] = rr;
+      Hr[(j + 1) * MAXJ + j] = 0.0;
+      cs[j] = cj;
+      sn[j] = sj;
+      const double gj = g[j];
+      g[j + 1] = -sj * gj;
+      g[j] = cj * gj;
+      const double est = fabs(sj * gj) / st.bn[r];
+      if (!isfinite(est)) atomicOr(&s_nan, 1);
+      const int done = st.done[r];
+      if (!done) st.iters[r] = it;
+      const bool ok = done || est <= st.rtol[0] || hn == 0.0;
+      if (!ok) atomicAnd(&s_ok, 0);
+      st.sc[r] = (hn > 0.0 && !done) ? 1.0 / hn : 0.0;
+    }
   }
   __syncthreads();
-  if (r == 0) {
+  if (threadIdx.x == 0) {
     const int cyc = (s_ok || s_nan || j + 1 >= m || it >= ctl[KC_MAXIT]) ? 1 : 0;
     s_cyc = cyc;
     ctl[KC_IT] = it;
@@ -1277,18 +1358,30 @@ __device__ __forceinline__ void gtail_run(int *__restrict__ ctl, GmState st, int
     cudaGraphSetConditional(if_end, (unsigned)cyc);
   }
   __syncthreads();
-  if (s_cyc && r < nrhs) {  // back substitution (zeros for a finished right-hand side)
+  if (!s_cyc) return;
+  // back substitution by columns (zeros for a finished right-hand side)
+  for (int r = wid; r < nrhs; r += nw) {
     const double *Hr = st.Hm + (int64_t)r * (MAXJ + 1) * MAXJ;
     const double *g = st.g + r * (MAXJ + 1);
-    double *yr = y + r * MAXJ;
-    const int jn = j + 1;
-    for (int i = 0; i < MAXJ; ++i) yr[i] = 0.0;
-    if (!st.done[r])
-      for (int i = jn - 1; i >= 0; --i) {
-        double acc = g[i];
-        for (int k = i + 1; k < jn; ++k) acc -= Hr[i * MAXJ + k] * yr[k];
-        yr[i] = (Hr[i * MAXJ + i] != 0.0) ? acc / Hr[i * MAXJ + i] : 0.0;
+    const bool live = !st.done[r];
+    double gv[2], yv[2] = {0.0, 0.0};
+#pragma unroll
+    for (int q = 0; q < 2; ++q) gv[q] = lane + 32 * q <= j && live ? g[lane + 32 * q] : 0.0;
+    for (int i = j; i >= 0; --i) {
+      double col[2];
+#pragma unroll
+      for (int q = 0; q < 2; ++q) col[q] = lane + 32 * q <= i ? Hr[(lane + 32 * q) * MAXJ + i] : 0.0;
+      const double d = __shfl_sync(0xffffffffu, i < 32 ? col[0] : col[1], i & 31);
+      const double gi = __shfl_sync(0xffffffffu, i < 32 ? gv[0] : gv[1], i & 31);
+      const double yi = d != 0.0 ? gi / d : 0.0;
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        if (lane + 32 * q == i) yv[q] = yi;
+        gv[q] -= col[q] * yi;
       }
+    }
+#pragma unroll
+    for (int q = 0; q < 2; ++q) y[r * MAXJ + lane + 32 * q] = yv[q];
   }
 }
 
@@ -1392,17 +1485,40 @@ __device__ __forceinline__ bool block_partial_last(double v, double *__restrict_
   return true;
 }
 
+// r = b - A x with |r|^2 in dots[rhs][0]: one pass for the residual checks of the graph solves
+// (operator, subtraction and norm were three launches, 36 us at 1024^2).
+__global__ void __launch_bounds__(RED_THREADS) k_gresid(OpDev o, int64_t N, const double *__restrict__ b,
+                                                      const double *__restrict__ x, double *__restrict__ r,
+                                                      double *__restrict__ part, int *cnt, double *__restrict__ dots) {
+  const int rhs = blockIdx.y;
+  const int64_t base = (int64_t)rhs * N;
+  const double2 *b2 = reinterpret_cast<const double2 *>(b + base);
+  double2 *r2 = reinterpret_cast<double2 *>(r + base);
+  double acc = 0.0;
+  for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < N >> 1; k += (int64_t)gridDim.x * blockDim.x) {
+    double2 c;
+    const double2 bk = b2[k], a = op_pair(o, x, base, k, c);
+    const double2 v = make_double2(bk.x - a.x, bk.y - a.y);
+    r2[k] = v;
+    acc = fma(v.x, v.x, fma(v.y, v.y, acc));
+  }
+  double tot;
+  if (block_partial_last(acc, part, rhs, cnt, tot) && threadIdx.x == 0) dots[rhs * MAXJ] = tot;
+}
+
 // q = A p and <p, q>; then alpha = <r, z> / <p, q> (0 for a finished right-hand side)
 __global__ void __launch_bounds__(RED_THREADS) k_cgf_apdot(OpDev o, int64_t N, GmState st, const double *__restrict__ p,
                                                          double *__restrict__ q, double *__restrict__ part, int *cnt,
                                                          double *__restrict__ pq, const double *__restrict__ rz_old) {
   const int rhs = blockIdx.y;
+  const int64_t base = (int64_t)rhs * N;
+  double2 *q2 = reinterpret_cast<double2 *>(q + base);
   double acc = 0.0;
-  for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < N; k += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t t = (int64_t)rhs * N + k;
-    const double v = op_at(o, p, t);
-    q[t] = v;
-    acc = fma(p[t], v, acc);
+  for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < N >> 1; k += (int64_t)gridDim.x * blockDim.x) {
+    double2 c;
+    const double2 v = op_pair(o, p, base, k, c);
+    q2[k] = v;
+    acc = fma(c.x, v.x, fma(c.y, v.y, acc));
   }
   double tot;
   if (block_partial_last(acc, part, rhs, cnt, tot) && threadIdx.x == 0) {
@@ -1422,13 +1538,21 @@ __global__ void __launch_bounds__(RED_THREADS) k_cgf_xr(int *__restrict__ ctl, i
   __shared__ int s_fin, s_all, s_nan;
   const int rhs = blockIdx.y;
   const double al = st.sc[rhs];
+  const int64_t base2 = (int64_t)rhs * (N >> 1);
+  const double2 *p2 = reinterpret_cast<const double2 *>(p) + base2, *q2 = reinterpret_cast<const double2 *>(q) + base2;
+  double2 *x2 = reinterpret_cast<double2 *>(x) + base2, *r2 = reinterpret_cast<double2 *>(r) + base2;
   double acc = 0.0;
-  for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < N; k += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t t = (int64_t)rhs * N + k;
-    x[t] = fma(al, p[t], x[t]);
-    const double rv = fma(-al, q[t], r[t]);
-    r[t] = rv;
-    acc = fma(rv, rv, acc);
+#pragma unroll 2
+  for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < N >> 1; k += (int64_t)gridDim.x * blockDim.x) {
+    const double2 pk = p2[k], qk = q2[k];
+    double2 xk = x2[k], rk = r2[k];
+    xk.x = fma(al, pk.x, xk.x);
+    xk.y = fma(al, pk.y, xk.y);
+    rk.x = fma(-al, qk.x, rk.x);
+    rk.y = fma(-al, qk.y, rk.y);
+    x2[k] = xk;
+    r2[k] = rk;
+    acc = fma(rk.x, rk.x, fma(rk.y, rk.y, acc));
   }
   double tot;
   if (!block_partial_last(acc, part, rhs, cnt, tot)) return;
@@ -1468,10 +1592,13 @@ __global__ void __launch_bounds__(RED_THREADS) k_cgf_rz(int64_t N, GmState st, c
                                                       const double *__restrict__ z, double *__restrict__ part, int *cnt,
                                                       double *__restrict__ rz_old) {
   const int rhs = blockIdx.y;
+  const double2 *r2 = reinterpret_cast<const double2 *>(r + (int64_t)rhs * N);
+  const double2 *z2 = reinterpret_cast<const double2 *>(z + (int64_t)rhs * N);
   double acc = 0.0;
-  for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < N; k += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t t = (int64_t)rhs * N + k;
-    acc = fma(r[t], z[t], acc);
+#pragma unroll 4
+  for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < N >> 1; k += (int64_t)gridDim.x * blockDim.x) {
+    const double2 rk = r2[k], zk = z2[k];
+    acc = fma(rk.x, zk.x, fma(rk.y, zk.y, acc));
   }
   double tot;
   if (block_partial_last(acc, part, rhs, cnt, tot) && threadIdx.x == 0) {
@@ -1534,7 +1661,7 @@ GmState gm_state(KrylovWs &K) {
 
 // norms |v[rhs]|^2 into dots[rhs][0] (captured)
 void gnorm2(Ctx &c, const double *v) {
-  const int nb = red_blocks();
+  const int nb = red_blocks(c.N);
   k_mdot_partial<<<dim3(nb, c.nrhs), RED_THREADS, 0, c.H.stream>>>(c.N, 1, v, 0, v, c.H.kw.part, 0);
   k_mdot_final<<<dim3(c.nrhs, 1), 256, 0, c.H.stream>>>(1, nb, c.H.kw.part, c.H.kw.dots, nullptr, 0);
   FMMPC_LAUNCH_CHECK();
@@ -1563,9 +1690,9 @@ void build_chain(fmmpc_handle &H, cudaGraph_t G, int method, int m, int nrhs, bo
   auto precond = [&](const double *in, double *out, double *scratch) {
     precond_op(H, in, out, scratch, nrhs, true);
   };
-  auto residual_c = [&](const double *b, const double *x, double *r) {
-    k_spmv5<<<nblk(NR), 256, 0, H.stream>>>(od, NR, x, r);
-    k_resid<<<nblk(NR), 256, 0, H.stream>>>(NR, b, r);
+  const dim3 rgrid((unsigned)red_blocks(N), nrhs);
+  auto residual_norm = [&]() {  // r = b - A x and |r|^2 into dots[rhs][0]
+    k_gresid<<<rgrid, RED_THREADS, 0, H.stream>>>(od, N, K.b, K.x, K.r, K.part, K.g_cnt, K.dots);
     FMMPC_LAUNCH_CHECK();
   };
   // ---- set-up
@@ -1575,8 +1702,7 @@ void build_chain(fmmpc_handle &H, cudaGraph_t G, int method, int m, int nrhs, bo
     k_fold_rhs<<<nblk(NR), 256, 0, H.stream>>>(od, NR, K.fin, has_g ? K.gin : nullptr, K.b);
     gnorm2(c, K.b);
     k_ginit<<<1, 64, 0, H.stream>>>(ctl, st, nrhs, K.dots);
-    residual_c(K.b, K.x, K.r);
-    gnorm2(c, K.r);
+    residual_norm();
     if (method == FMMPC_CG) {
       // the loop body starts with z = P^{-1} r; p = 0 and <r, z>_old = 0 make its first
       // beta 0, so that p = z
@@ -1604,7 +1730,6 @@ void build_chain(fmmpc_handle &H, cudaGraph_t G, int method, int m, int nrhs, bo
     // one iteration, rotated so that the convergence test ends it and sets the loop's own
     // condition (no IF node): z = P^{-1} r, beta, p = z + beta p, q = A p with alpha, then
     // x, r and the test
-    const dim3 rgrid((unsigned)red_blocks(), nrhs);
     f_step = capture_into(H, cs, body, none, [&] {
       c.s = H.stream;
       precond(K.r, z, K.zin);
@@ -1622,7 +1747,6 @@ void build_chain(fmmpc_handle &H, cudaGraph_t G, int method, int m, int nrhs, bo
       // w = A z_j with the first CGS pass, the first update with the second pass, the second
       // update with |w|^2: three sweeps over the basis, each reduction finished in its grid's
       // last block (a grid of a few blocks per SM keeps enough loads in flight)
-      const dim3 rgrid((unsigned)red_blocks(), nrhs);
       double *d2 = K.dots + (size_t)2 * nrhs * MAXJ;
       k_gapdots<<<rgrid, RED_THREADS, 0, H.stream>>>(ctl, od, N, K.zin, K.w, flexible ? K.Z : nullptr, K.V, vs,
                                                      K.part, K.g_cnt, K.dots, hsum);
@@ -1643,8 +1767,7 @@ void build_chain(fmmpc_handle &H, cudaGraph_t G, int method, int m, int nrhs, bo
         precond(K.t, K.w, K.t);
         k_add<<<nblk(NR), 256, 0, H.stream>>>(NR, K.w, K.x);
       }
-      residual_c(K.b, K.x, K.r);
-      gnorm2(c, K.r);
+      residual_norm();
       k_grestart<<<1, 64, 0, H.stream>>>(ctl, st, nrhs, K.dots);
       k_gscale_col<<<nblk(NR), 256, 0, H.stream>>>(ctl, N, nrhs, K.g_sc, K.r, K.V, vs, K.t);
       FMMPC_LAUNCH_CHECK();
@@ -1657,8 +1780,7 @@ void build_chain(fmmpc_handle &H, cudaGraph_t G, int method, int m, int nrhs, bo
   // ---- final: the true residual
   capture_into(H, cs, G, {n_loop}, [&] {
     c.s = H.stream;
-    residual_c(K.b, K.x, K.r);
-    gnorm2(c, K.r);
+    residual_norm();
     k_gfinal<<<1, 64, 0, H.stream>>>(st, nrhs, K.dots);
     FMMPC_LAUNCH_CHECK();
   });

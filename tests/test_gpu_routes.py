@@ -1,6 +1,6 @@
 """Kernels and dispatch rules at the sizes where they can go wrong, each against the oracle or
-the general path: window edges of the Q1 mass solve, tables formed on first use, and
-the FP64 form's tensor-core kernels."""
+the general path: window edges of the Q1 mass solve, tables formed on first use, the FP64 form's
+tensor-core kernels, and alignment."""
 import numpy as np
 import pytest
 
@@ -132,4 +132,21 @@ def test_fp64_tensor_core_m2l_matches_oracle(p, leaf_max):
     R = O.Problem(n, p=p, leaf_max=leaf_max)
     for k in range(2):
         check_close(f"fp64 vr p={p} leaf={leaf_max} rhs={k}", vr[k], R.apply(f[k], "fmm", stages=True)["vr"], 1e-12, 1e-12)
+    P.close()
+
+
+def test_spmv_takes_vectors_aligned_for_fp64_only():
+    # the pair loads need 16-byte alignment: vectors one double into an allocation take the scalar path
+    from paper_1308_3339_gb300 import FmmPreconditioner
+    n = 64
+    P = FmmPreconditioner(n, p=8, precision="fp64")
+    x = dev(S.random_field(n, 1))
+    big, out = torch.zeros(n * n + 1, dtype=torch.float64, device="cuda"), torch.zeros(n * n + 1, dtype=torch.float64, device="cuda")
+    big[1:] = x
+    assert torch.equal(P.spmv(big[1:], out=out[1:]), P.spmv(x))
+    z = P.apply(x)
+    assert torch.equal(P.apply(big[1:], out=out[1:]), z)
+    u, _ = P.solve(x, use_graphs=0)
+    v, _ = P.solve(big[1:], u0=big[1:] * 0, use_graphs=0)
+    assert float((u - v).norm() / u.norm()) < 1e-8
     P.close()
