@@ -1,11 +1,21 @@
 // Boundary-element set-up (Sec. 4.3): constant elements, no nodes at the corners, 4n
 // equal elements on the square, collocation at their midpoints.  The single-layer
 // matrix S_mk = int_{Gamma_k} G(y_m, y) dGamma (left side of Eq. e:ubound) is assembled in
-// FP64 from the closed-form element integral (Sec. 4.2).  The square's 90-degree rotation
-// symmetry makes S block circulant over the four sides, so a 4-point DFT over the side
-// index splits it into three n x n blocks (one complex); each is inverted once (LU with
-// partial pivoting by cuSOLVER, then the triangular solves against the identity), and the
-// apply works in that basis.  The inversion is set-up, not the apply's path.
+// FP64 from the closed-form element integral (Sec. 4.2).  The square's symmetries split it:
+//
+//  Rotation.  S is block circulant over the four sides, so a 4-point DFT over the side index gives
+//  C^0 = S0+S1+S2+S3, C^2 = S0-S1+S2-S3 and A + iB, A = S0 - S2, B = S1 - S3 (n x n).
+//  Reflection.  Reversing the elements of every side (J) maps side 1 to side 3: J C^0 J = C^0,
+//  J C^2 J = C^2, J A J = A, J B J = -B.  On the sums and differences of mirrored elements,
+//  v_e[k] = v[k] + v[n-1-k] and v_o[k] = v[k] - v[n-1-k], k < h = n / 2, each matrix X acts through
+//  h x h blocks X_e = X[m][k] + X[m][n-1-k], X_o = X[m][k] - X[m][n-1-k]: (X v)_e = X_e v_e and
+//  (X v)_o = X_o v_o for C^0, C^2 and A; (B v)_e = B_o v_o and (B v)_o = B_e v_e.
+//
+// So a matrix of this kind is stored as h rows of [C0e | C0o | C2e | C2o | Ae | Ao | Bo | Be], 4n values
+// each (the folded form): half the entries and multiply-adds of the side-DFT form alone.  The
+// inverse of S has the form again; its blocks are inverted once (LU with partial pivoting by
+// cuSOLVER, then the triangular solves against the identity): four h x h, and A + iB, which in
+// the basis diag(1, i) is the real [[Ae, -Bo], [Be, Ao]].  The inversion is set-up, not the apply's path.
 #include <cusolverDn.h>
 
 #include <algorithm>
@@ -90,67 +100,71 @@ __global__ void k_bem_Kdl(int n, double diag, double *__restrict__ A) {
   A[t] = v;
 }
 
-// From the first block row of S (n x 4n): S^0 and S^2 (n x n, real) and
-// S^1 = (S0 - S2) + i (S1 - S3) (n x n, complex, interleaved re / im).
-__global__ void k_bem_blocks(int n, const double *__restrict__ S, double *__restrict__ B0, double *__restrict__ B2,
-                             double *__restrict__ C1) {
+// The folded form of a first block row A = [S0 | S1 | S2 | S3] (n x 4n), row m < h: T[m] (4n values).
+__global__ void k_bem_fold(int n, const double *__restrict__ A, double *__restrict__ T) {
+  const int h = n >> 1;
   const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= (int64_t)n * n) return;
-  const int64_t m = t / n;
-  const int k = (int)(t % n);
-  const double *row = S + m * 4 * n;
-  const double s0 = row[k], s1 = row[n + k], s2 = row[2 * n + k], s3 = row[3 * n + k];
-  B0[m * n + k] = (s0 + s2) + (s1 + s3);
-  B2[m * n + k] = (s0 + s2) - (s1 + s3);
-  C1[2 * (m * n + k)] = s0 - s2;
-  C1[2 * (m * n + k) + 1] = s1 - s3;
+  if (t >= (int64_t)h * h) return;
+  const int64_t m = t / h;
+  const int k = (int)(t % h);
+  const double *r = A + m * 4 * n;
+  double x[2][4];  // C^0, C^2, A, B at columns k and n - 1 - k
+#pragma unroll
+  for (int j = 0; j < 2; ++j) {
+    const int c = j ? n - 1 - k : k;
+    const double s0 = r[c], s1 = r[n + c], s2 = r[2 * n + c], s3 = r[3 * n + c];
+    x[j][0] = (s0 + s2) + (s1 + s3);
+    x[j][1] = (s0 + s2) - (s1 + s3);
+    x[j][2] = s0 - s2;
+    x[j][3] = s1 - s3;
+  }
+  double *o = T + m * 4 * n + k;
+#pragma unroll
+  for (int q = 0; q < 3; ++q) {
+    o[(2 * q) * h] = x[0][q] + x[1][q];
+    o[(2 * q + 1) * h] = x[0][q] - x[1][q];
+  }
+  o[6 * h] = x[0][3] - x[1][3];  // Bo
+  o[7 * h] = x[0][3] + x[1][3];  // Be
 }
 
-// T[m] = [inv(S^0) | inv(S^2) | A | B][m] with A + i B = inv(S^1).
-__global__ void k_bem_pack(int n, const double *__restrict__ B0, const double *__restrict__ B2,
-                           const double *__restrict__ C1, double *__restrict__ T) {
+// The blocks to invert, from the folded form: X[4] (h x h each) and M = [[Ae, -Bo], [Be, Ao]] (n x n);
+// and back (the inverse's Bo is minus the upper right block).
+template <bool PACK>
+__global__ void k_bem_blocks(int n, double *__restrict__ T, double *__restrict__ X, double *__restrict__ M) {
+  const int h = n >> 1;
   const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= (int64_t)n * n) return;
-  const int64_t m = t / n;
-  const int k = (int)(t % n);
-  double *o = T + m * 4 * n;
-  o[k] = B0[m * n + k];
-  o[n + k] = B2[m * n + k];
-  o[2 * n + k] = C1[2 * (m * n + k)];
-  o[3 * n + k] = C1[2 * (m * n + k) + 1];
-}
-
-// In place, row m of a first block row [S0 | S1 | S2 | S3] to its side-DFT form
-// [S0+S1+S2+S3 | S0-S1+S2-S3 | S0-S2 | S1-S3] (the blocks that k_bem_apply multiplies by).
-__global__ void k_bem_dft(int n, double *__restrict__ A) {
-  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= (int64_t)n * n) return;
-  double *o = A + (t / n) * 4 * n + t % n;
-  const double s0 = o[0], s1 = o[n], s2 = o[2 * n], s3 = o[3 * n];
-  o[0] = (s0 + s2) + (s1 + s3);
-  o[n] = (s0 + s2) - (s1 + s3);
-  o[2 * n] = s0 - s2;
-  o[3 * n] = s1 - s3;
-}
-
-__global__ void k_identity(int N, double *__restrict__ B, int cplx) {
-  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= (int64_t)N * N) return;
-  const double v = (t / N == t % N) ? 1.0 : 0.0;
-  if (cplx) {
-    B[2 * t] = v;
-    B[2 * t + 1] = 0.0;
+  if (t >= (int64_t)h * h) return;
+  const int64_t m = t / h;
+  const int k = (int)(t % h);
+  double *o = T + m * 4 * n + k, *ae = M + m * n + k, *bo = ae + h, *be = M + (m + h) * n + k, *ao = be + h;
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    if (PACK) o[q * h] = X[q * (int64_t)h * h + t];
+    else X[q * (int64_t)h * h + t] = o[q * h];
+  }
+  if (PACK) {
+    o[4 * h] = *ae;
+    o[5 * h] = *ao;
+    o[6 * h] = -*bo;
+    o[7 * h] = *be;
   } else {
-    B[t] = v;
+    *ae = o[4 * h];
+    *ao = o[5 * h];
+    *bo = -o[6 * h];
+    *be = o[7 * h];
   }
 }
 
-// |A_kk| of the N x N (real or interleaved complex) matrix A
-__global__ void k_diag_abs(int N, const double *__restrict__ A, double *__restrict__ d, int cplx) {
+__global__ void k_identity(int N, double *__restrict__ B) {
+  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (t < (int64_t)N * N) B[t] = (t / N == t % N) ? 1.0 : 0.0;
+}
+
+// |A_kk| of the N x N matrix A
+__global__ void k_diag_abs(int N, const double *__restrict__ A, double *__restrict__ d) {
   const int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= N) return;
-  const int64_t i = (int64_t)k * N + k;
-  d[k] = cplx ? hypot(A[2 * i], A[2 * i + 1]) : fabs(A[i]);
+  if (k < N) d[k] = fabs(A[(int64_t)k * N + k]);
 }
 
 #define FMMPC_CUSOLVER(call)                                                                   \
@@ -175,35 +189,26 @@ cusolverDnHandle_t solver_handle() {
   return h;
 }
 
-// In-place inverse of the N x N matrix A (row-major, device; real, or complex with re / im
-// interleaved), by LU with partial pivoting and the two triangular solves against the
-// identity.  Row-major A is the column-major A^T, and inv(A^T) read row-major is inv(A), so
-// the factorisation runs on the buffer as it is.  Returns the smallest |U_kk| (0 for a
-// singular matrix).  Calls are serialised on the handle's stream.
-double lu_invert(double *A, int N, bool cplx, cudaStream_t s, DevPool &tmp) {
+// In-place inverse of the N x N matrix A (row-major, device), by LU with partial pivoting and the
+// two triangular solves against the identity.  Row-major A is the column-major A^T, and
+// inv(A^T) read row-major is inv(A), so the factorisation runs on the buffer as it is.  Returns
+// the smallest |U_kk| (0 for a singular matrix).  Calls are serialised on the handle's stream.
+double lu_invert(double *A, int N, cudaStream_t s, DevPool &tmp) {
   static std::mutex mu;
   std::lock_guard<std::mutex> lock(mu);  // the per-device solver handle is shared
   cusolverDnHandle_t h = solver_handle();
   FMMPC_CUSOLVER(cusolverDnSetStream(h, s));
-  const size_t w = cplx ? 2 : 1;
   int lwork = 0;
-  cuDoubleComplex *Az = reinterpret_cast<cuDoubleComplex *>(A);
-  if (cplx) FMMPC_CUSOLVER(cusolverDnZgetrf_bufferSize(h, N, N, Az, N, &lwork));
-  else FMMPC_CUSOLVER(cusolverDnDgetrf_bufferSize(h, N, N, A, N, &lwork));
-  double *work = tmp.get<double>(w * (size_t)std::max(lwork, 1));
+  FMMPC_CUSOLVER(cusolverDnDgetrf_bufferSize(h, N, N, A, N, &lwork));
+  double *work = tmp.get<double>((size_t)std::max(lwork, 1));
   int *ipiv = tmp.get<int>(N), *info = tmp.get<int>(2);
-  double *dabs = tmp.get<double>(N), *B = tmp.get<double>(w * (size_t)N * N);
-  if (cplx) FMMPC_CUSOLVER(cusolverDnZgetrf(h, N, N, Az, N, reinterpret_cast<cuDoubleComplex *>(work), ipiv, info));
-  else FMMPC_CUSOLVER(cusolverDnDgetrf(h, N, N, A, N, work, ipiv, info));
-  k_diag_abs<<<nblk(N), 256, 0, s>>>(N, A, dabs, cplx ? 1 : 0);
-  k_identity<<<nblk((int64_t)N * N), 256, 0, s>>>(N, B, cplx ? 1 : 0);
+  double *dabs = tmp.get<double>(N), *B = tmp.get<double>((size_t)N * N);
+  FMMPC_CUSOLVER(cusolverDnDgetrf(h, N, N, A, N, work, ipiv, info));
+  k_diag_abs<<<nblk(N), 256, 0, s>>>(N, A, dabs);
+  k_identity<<<nblk((int64_t)N * N), 256, 0, s>>>(N, B);
   FMMPC_LAUNCH_CHECK();
-  if (cplx)
-    FMMPC_CUSOLVER(cusolverDnZgetrs(h, CUBLAS_OP_N, N, N, Az, N, ipiv, reinterpret_cast<cuDoubleComplex *>(B), N,
-                                    info + 1));
-  else
-    FMMPC_CUSOLVER(cusolverDnDgetrs(h, CUBLAS_OP_N, N, N, A, N, ipiv, B, N, info + 1));
-  FMMPC_CUDA(cudaMemcpyAsync(A, B, sizeof(double) * w * N * N, cudaMemcpyDeviceToDevice, s));
+  FMMPC_CUSOLVER(cusolverDnDgetrs(h, CUBLAS_OP_N, N, N, A, N, ipiv, B, N, info + 1));
+  FMMPC_CUDA(cudaMemcpyAsync(A, B, sizeof(double) * N * N, cudaMemcpyDeviceToDevice, s));
   std::vector<double> ha(N);
   int hinfo[2] = {0, 0};
   FMMPC_CUDA(cudaMemcpyAsync(ha.data(), dabs, sizeof(double) * N, cudaMemcpyDeviceToHost, s));
@@ -215,6 +220,21 @@ double lu_invert(double *A, int N, bool cplx, cudaStream_t s, DevPool &tmp) {
   double amin = ha[0];
   for (int k = 0; k < N; ++k) amin = std::min(amin, ha[k]);
   return amin;
+}
+
+// T: the folded form of a matrix of the square's symmetry, replaced by its inverse's.  False if a
+// block is singular.
+bool invert_folded(int n, double *T, cudaStream_t s, DevPool &tmp) {
+  const int h = n >> 1;
+  double *X = tmp.get<double>((size_t)4 * h * h), *M = tmp.get<double>((size_t)n * n);
+  k_bem_blocks<false><<<nblk((int64_t)h * h), 256, 0, s>>>(n, T, X, M);
+  FMMPC_LAUNCH_CHECK();
+  for (int q = 0; q < 4; ++q)
+    if (!(lu_invert(X + (size_t)q * h * h, h, s, tmp) > 0.0)) return false;
+  if (!(lu_invert(M, n, s, tmp) > 0.0)) return false;
+  k_bem_blocks<true><<<nblk((int64_t)h * h), 256, 0, s>>>(n, T, X, M);
+  FMMPC_LAUNCH_CHECK();
+  return true;
 }
 
 }  // namespace
@@ -232,87 +252,73 @@ __global__ void k_split_f2(int64_t total, const double *__restrict__ x, float *_
 }  // namespace
 
 void init_bem(fmmpc_handle &H, DevPool &tmp) {
-  // S is block circulant in the four sides (the 90-degree rotation of the square maps
-  // element (s, k) to (s+1, k)), so a 4-point DFT over the side index block-diagonalises
-  // it: with S_d = S[(0, .), (d, .)], S^0 = S0+S1+S2+S3, S^2 = S0-S1+S2-S3 (real) and
-  // S^1 = (S0 - S2) + i (S1 - S3).  The apply needs exactly the inverses of these blocks,
-  // [inv(S^0) | inv(S^2) | Re inv(S^1) | Im inv(S^1)] per row, so only the first block row
-  // of S is assembled and three n x n systems are inverted (two real, one complex).
   const Geo &g = H.g;
   const int n = g.n, N = g.NG;
+  const size_t nt = (size_t)(n / 2) * N;  // the folded form
   cudaStream_t s = H.stream;
   double *S = tmp.get<double>((size_t)n * N);  // first block row, n x 4n
   k_bem_S<<<nblk((int64_t)n * N), 256, 0, s>>>(n, g.h, g.lnh, S);
+  H.Sinv = H.pool.get<double>(nt);
+  k_bem_fold<<<nblk((int64_t)(n / 2) * (n / 2)), 256, 0, s>>>(n, S, H.Sinv);
   FMMPC_LAUNCH_CHECK();
-  double *B0 = tmp.get<double>((size_t)n * n), *B2 = tmp.get<double>((size_t)n * n);
-  double *C1 = tmp.get<double>((size_t)2 * n * n);
-  k_bem_blocks<<<nblk((int64_t)n * n), 256, 0, s>>>(n, S, B0, B2, C1);
-  FMMPC_LAUNCH_CHECK();
-  const double a0 = lu_invert(B0, n, false, s, tmp), a2 = lu_invert(B2, n, false, s, tmp), a1 = lu_invert(C1, n, true, s, tmp);
-  if (!(a0 > 0.0) || !(a2 > 0.0) || !(a1 > 0.0))
+  if (!invert_folded(n, H.Sinv, s, tmp))
     throw Error(FMMPC_ERR_INVALID, "single-layer BEM matrix is singular for this domain");
-  H.Sinv = H.pool.get<double>((size_t)n * N);
-  k_bem_pack<<<nblk((int64_t)n * n), 256, 0, s>>>(n, B0, B2, C1, H.Sinv);
-  FMMPC_LAUNCH_CHECK();
   if (H.prec != FMMPC_PREC_FP64) {  // the single-precision forms apply it in two-word FP32
-    H.Sinv_hi = H.pool.get<float>((size_t)n * N);
-    H.Sinv_lo = H.pool.get<float>((size_t)n * N);
-    k_split_f2<<<nblk((int64_t)n * N), 256, 0, s>>>((int64_t)n * N, H.Sinv, H.Sinv_hi, H.Sinv_lo);
+    H.Sinv_hi = H.pool.get<float>(nt);
+    H.Sinv_lo = H.pool.get<float>(nt);
+    k_split_f2<<<nblk((int64_t)nt), 256, 0, s>>>((int64_t)nt, H.Sinv, H.Sinv_hi, H.Sinv_lo);
     FMMPC_LAUNCH_CHECK();
   }
   FMMPC_CUDA(cudaStreamSynchronize(s));
 }
 
-// T' for S^T from T for S (first block rows in the side-DFT form [C0 | C2 | A | B]): S^T is
-// block circulant with the blocks transposed and the side index reversed, so its DFT blocks
-// are C0^T, C2^T and (A + iB)^H = A^T - i B^T: T'[m][blk n + k] = +-T[k][blk n + m].
+// The folded form T' of S^T from T of S: the side index is reversed, so C^0, C^2 and A transpose and
+// B becomes -B^T, whose folded blocks are Bo' = -Be^T, Be' = -Bo^T.
 __global__ void k_bem_transpose(int n, const double *__restrict__ T, double *__restrict__ Tt) {
+  const int h = n >> 1;
   const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= (int64_t)n * 4 * n) return;
+  if (t >= (int64_t)h * 4 * n) return;
   const int64_t mrow = t / (4 * n);
-  const int c = (int)(t % (4 * n)), blk = c / n, k = c % n;
-  const double v = T[(int64_t)k * 4 * n + blk * n + mrow];
-  Tt[t] = (blk == 3) ? -v : v;
+  const int c = (int)(t % (4 * n)), blk = c / h, k = c % h;
+  const int from = blk == 6 ? 7 : (blk == 7 ? 6 : blk);
+  const double v = T[(int64_t)k * 4 * n + (int64_t)from * h + mrow];
+  Tt[t] = blk >= 6 ? -v : v;
 }
 
 // S^{-T} for the transpose pass, formed on first use.
 void init_bem_transpose(fmmpc_handle &H) {
   if (H.SinvT) return;
   const int n = H.g.n;
-  double *Tt = H.pool.get<double>((size_t)n * 4 * n);
-  k_bem_transpose<<<nblk((int64_t)n * 4 * n), 256, 0, H.stream>>>(n, H.Sinv, Tt);
+  const size_t nt = (size_t)(n / 2) * 4 * n;
+  double *Tt = H.pool.get<double>(nt);
+  k_bem_transpose<<<nblk((int64_t)nt), 256, 0, H.stream>>>(n, H.Sinv, Tt);
   FMMPC_LAUNCH_CHECK();
   FMMPC_CUDA(cudaStreamSynchronize(H.stream));
   H.SinvT = Tt;
 }
 
-// The inverse of -1/2 I + K in the side-DFT form of the single-layer inverse (the same
-// 90-degree rotation symmetry), for the double-layer correction; formed on first use.
+// The inverse of -1/2 I + K in the folded form (the same symmetries), for the double-layer
+// correction; formed on first use.
 void init_bem_dl(fmmpc_handle &H) {
   if (H.Kdl_inv) return;
   const Geo &g = H.g;
   const int n = g.n, N = g.NG;
+  const size_t nt = (size_t)(n / 2) * N;
   cudaStream_t s = H.stream;
   DevPool tmp;
   try {
     double *A = tmp.get<double>((size_t)n * N);
     k_bem_Kdl<<<nblk((int64_t)n * N), 256, 0, s>>>(n, -0.5, A);
+    double *T = H.pool.get<double>(nt);
+    k_bem_fold<<<nblk((int64_t)(n / 2) * (n / 2)), 256, 0, s>>>(n, A, T);
     FMMPC_LAUNCH_CHECK();
-    double *B0 = tmp.get<double>((size_t)n * n), *B2 = tmp.get<double>((size_t)n * n);
-    double *C1 = tmp.get<double>((size_t)2 * n * n);
-    k_bem_blocks<<<nblk((int64_t)n * n), 256, 0, s>>>(n, A, B0, B2, C1);
-    FMMPC_LAUNCH_CHECK();
-    const double a0 = lu_invert(B0, n, false, s, tmp), a2 = lu_invert(B2, n, false, s, tmp), a1 = lu_invert(C1, n, true, s, tmp);
-    if (!(a0 > 0.0) || !(a2 > 0.0) || !(a1 > 0.0))
+    if (!invert_folded(n, T, s, tmp))
       throw Error(FMMPC_ERR_INVALID, "double-layer BEM matrix is singular for this domain");
-    double *T = H.pool.get<double>((size_t)n * N);
-    k_bem_pack<<<nblk((int64_t)n * n), 256, 0, s>>>(n, B0, B2, C1, T);
-    FMMPC_LAUNCH_CHECK();
     float *th = nullptr, *tl = nullptr;
     if (H.prec != FMMPC_PREC_FP64) {
-      th = H.pool.get<float>((size_t)n * N);
-      tl = H.pool.get<float>((size_t)n * N);
-      k_split_f2<<<nblk((int64_t)n * N), 256, 0, s>>>((int64_t)n * N, T, th, tl);
+      th = H.pool.get<float>(nt);
+      tl = H.pool.get<float>(nt);
+      k_split_f2<<<nblk((int64_t)nt), 256, 0, s>>>((int64_t)nt, T, th, tl);
       FMMPC_LAUNCH_CHECK();
     }
     FMMPC_CUDA(cudaStreamSynchronize(s));
@@ -325,9 +331,9 @@ void init_bem_dl(fmmpc_handle &H) {
   }
 }
 
-// 1/2 I + K in the side-DFT form, the boundary data term of Eq. e:ubound, for apply_bc; formed
+// 1/2 I + K in the folded form, the boundary data term of Eq. e:ubound, for apply_bc; formed
 // on its first call.  Summing the 16 n^2 atan2 of K g directly took 1160 us at n = 1024; the
-// 6 n^2 multiply-adds of the block-circulant form take 15 us.  Not formed (false) while the
+// 3 n^2 multiply-adds of the folded form take 9 us.  Not formed (false) while the
 // handle's stream is being captured, or without memory for it: the caller sums directly.
 bool init_bem_bc(fmmpc_handle &H) {
   if (H.Kbc) return true;
@@ -338,18 +344,21 @@ bool init_bem_bc(fmmpc_handle &H) {
   }
   const int n = H.g.n;
   const size_t nv = (size_t)H.g.NG * H.nrhs_max;
-  double *A = nullptr;
+  double *A = nullptr, *T = nullptr;
+  DevPool tmp;
   try {
     if (!H.bc_vt) H.bc_vt = H.pool.get<double>(nv);
     if (!H.bc_kg) H.bc_kg = H.pool.get<double>(nv);
-    A = H.pool.get<double>((size_t)n * H.g.NG);
+    A = tmp.get<double>((size_t)n * H.g.NG);
+    T = H.pool.get<double>((size_t)(n / 2) * H.g.NG);
   } catch (const Error &) {
     return false;
   }
   k_bem_Kdl<<<nblk((int64_t)n * H.g.NG), 256, 0, H.stream>>>(n, 0.5, A);
-  k_bem_dft<<<nblk((int64_t)n * n), 256, 0, H.stream>>>(n, A);
+  k_bem_fold<<<nblk((int64_t)(n / 2) * (n / 2)), 256, 0, H.stream>>>(n, A, T);
   FMMPC_LAUNCH_CHECK();
-  H.Kbc = A;
+  FMMPC_CUDA(cudaStreamSynchronize(H.stream));  // A goes out of scope
+  H.Kbc = T;
   return true;
 }
 

@@ -184,7 +184,7 @@ __device__ __forceinline__ void m2m_levels_smem(const cpx<R> *sT, cpx<R> (*buf)[
 // reset by that block) computes the k levels above it.  Any block that does a step
 // computes the same sums, so the result does not depend on which block it is.
 template <typename R, int P, int MS>
-__global__ void __launch_bounds__(256, (sizeof(R) == 4 && P <= 10 && MS <= 8) ? 6 : 1) k_upward_tree(Geo g, const R *__restrict__ wpad, const cpx<R> *__restrict__ vm2m,
+__global__ void __launch_bounds__(256, (sizeof(R) == 4 && P <= 10 && MS <= 8) ? 7 : 1) k_upward_tree(Geo g, const R *__restrict__ wpad, const cpx<R> *__restrict__ vm2m,
                                                      cpx<R> *__restrict__ Mv, int *__restrict__ counter, int64_t ncount) {
   // three-level steps need 64 cells in shared memory; two-level steps where that would not fit
   constexpr int NBUF = sizeof(cpx<R>) * P * (4 * P + 128) <= 45000 ? 64 : 16, MAXSTEP = NBUF == 64 ? 3 : 2;
@@ -372,6 +372,42 @@ __device__ __forceinline__ void m2l_accum(cpx<R> (&H)[P], const cpx<R> *__restri
   }
 }
 
+// The same for half of the outputs, n = s + i, s = half P / 2, i < P / 2, by one lane: two lanes share
+// a source, which shortens the chain of the latency-bound boundary passes by a third (and their
+// registers, so that all their warps are resident at once).  K_m = I_{s+m}.
+template <typename R, int P>
+__device__ __forceinline__ void m2l_accum_half(cpx<R> (&H)[P / 2], const cpx<R> *__restrict__ Ms, cpx<R> z, R lnrho,
+                                               int half) {
+  constexpr int PH = P / 2;
+  cpx<R> m[P];
+#pragma unroll
+  for (int k = 0; k < P; ++k) m[k] = Ms[k];
+  const cpx<R> inv = cinv(z);
+  cpx<R> c = inv;  // I_PH
+#pragma unroll
+  for (int j = 2; j <= PH; ++j) c = R(j - 1) * (c * inv);
+  const R s = half ? R(PH) : R(0);
+  cpx<R> K[PH + P - 1];
+  K[0] = half ? c : mk<R>(0, 0);
+  K[1] = half ? R(PH) * (c * inv) : inv;
+#pragma unroll
+  for (int j = 2; j < PH + P - 1; ++j) K[j] = (s + R(j - 1)) * (K[j - 1] * inv);
+#pragma unroll
+  for (int i = 0; i < PH; ++i) cmac(H[i], mk<R>(-m[0].re, -m[0].im), K[i]);
+#pragma unroll
+  for (int k = 1; k < P; ++k) {
+    const cpx<R> a = R(inv_fact_d(k - 1)) * m[k];
+#pragma unroll
+    for (int i = 0; i < PH; ++i) cmac(H[i], a, K[i + k]);
+  }
+  if (half == 0) {
+    const R lz = R(0.5) * dev_log<R>(z.re * z.re + z.im * z.im) + lnrho;
+    const R az = atan2(z.im, z.re);
+    H[0].re += m[0].re * lz - m[0].im * az;
+    H[0].im += m[0].re * az + m[0].im * lz;
+  }
+}
+
 // warp-reduce H, scale by (-1)^n/n!, then store (add = 0) or accumulate (add = 1)
 // Offset between a volume and a boundary cell centre in cell units, d * scale with
 // scale = 1 / (rho 2^(L+1)) and d an integer in those fine units.  When the scale is a power
@@ -473,13 +509,13 @@ __global__ void k_m2l_vol(GeoDev gd, int64_t ncell, int64_t nbcell, int nrhs, in
 
 // Boundary sources added to volume locals, for the cells that have them (cells[0, ntgt)):
 // eight lanes per (cell, rhs), four cells per warp, a segmented shuffle reduction, and
-// L += (-1)^n/n! H_n (deterministic: no atomics).  The lists average ~8 sources per cell.
-// With Lsep the result is written there instead ([rhs][index in cells][P]), for the
-// downward pass to add, so that this pass need not wait for the volume M2L.
+// (-1)^n/n! H_n (deterministic: no atomics).  The lists average ~8 sources per cell.  The result goes
+// to Lsep ([rhs][index in cells][P]), for the downward pass to add, so that this pass need not
+// wait for the volume M2L.
 template <typename R, int P>
 __global__ void k_m2l_vbv(GeoDev gd, int64_t ncell, int64_t nbcell, int nrhs, const int32_t *__restrict__ bfirst,
-                          const int32_t *__restrict__ bsrc, const cpx<R> *__restrict__ Mb, cpx<R> *__restrict__ Lv,
-                          const int32_t *__restrict__ cells, int64_t ntgt, cpx<R> *__restrict__ Lsep = nullptr) {
+                          const int32_t *__restrict__ bsrc, const cpx<R> *__restrict__ Mb,
+                          const int32_t *__restrict__ cells, int64_t ntgt, cpx<R> *__restrict__ Lsep) {
   const int64_t grp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 3;
   const int sub = threadIdx.x & 7;
   const bool active = grp < ntgt * nrhs;
@@ -510,7 +546,7 @@ __global__ void k_m2l_vbv(GeoDev gd, int64_t ncell, int64_t nbcell, int nrhs, co
     }
   }
   R f = 1;
-  cpx<R> *out = Lsep ? Lsep + ((int64_t)rhs * ntgt + gg % ntgt) * P : Lv + (int64_t)rhs * ncell * P + gidx * P;
+  cpx<R> *out = Lsep + ((int64_t)rhs * ntgt + gg % ntgt) * P;
 #pragma unroll
   for (int n = 0; n < P; ++n) {
     if (n > 0) f = -f / R(n);
@@ -520,7 +556,128 @@ __global__ void k_m2l_vbv(GeoDev gd, int64_t ncell, int64_t nbcell, int nrhs, co
       re += __shfl_xor_sync(0xffffffffu, re, o);
       im += __shfl_xor_sync(0xffffffffu, im, o);
     }
-    if (active && sub == 0) out[n] = Lsep ? mk(f * re, f * im) : out[n] + mk(f * re, f * im);
+    if (active && sub == 0) out[n] = mk(f * re, f * im);
+  }
+}
+
+// k_m2l_vbv in FP32 with two lanes per source: 16 lanes per (cell, rhs), two cells per warp, into Lsep.
+template <int P>
+__global__ void __launch_bounds__(256) k_m2l_vbv_half(GeoDev gd, int64_t nbcell, int nrhs,
+                                                     const int32_t *__restrict__ bfirst,
+                                                     const int32_t *__restrict__ bsrc,
+                                                     const cpx<float> *__restrict__ Mb,
+                                                     const int32_t *__restrict__ cells, int64_t ntgt,
+                                                     cpx<float> *__restrict__ Lsep) {
+  constexpr int PH = P / 2;
+  const int64_t grp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 4;
+  const int sub = (threadIdx.x & 15) >> 1, half = threadIdx.x & 1;
+  const bool active = grp < ntgt * nrhs;
+  const int64_t gg = active ? grp : 0;
+  const int rhs = (int)(gg / ntgt);
+  const int64_t gidx = cells[gg % ntgt];
+  int l = 0;
+  while (level_offset(l + 1) <= gidx) ++l;
+  const uint32_t c = (uint32_t)(gidx - level_offset(l));
+  const int rho = gd.n >> l;
+  const float lnrho = logf((float)rho);
+  cpx<float> H[PH];
+#pragma unroll
+  for (int i = 0; i < PH; ++i) H[i] = mk<float>(0, 0);
+  if (active) {
+    int64_t X, Y, sw;
+    vol_geom(gd, l, c, X, Y, sw);
+    X <<= gd.L;
+    Y <<= gd.L;
+    const OffsetScale scale = offset_scale(rho, gd.L);
+    const cpx<float> *MB = Mb + (int64_t)rhs * nbcell * P + blevel_offset(l) * P;
+    const int e1 = bfirst[gidx + 1];
+    for (int e = bfirst[gidx] + sub; e < e1; e += 8) {
+      const uint32_t b = (uint32_t)bsrc[e];
+      int64_t BX, BY, bs;
+      bnd_geom(gd, l, b, BX, BY, bs);
+      m2l_accum_half<float, P>(H, MB + (int64_t)b * P,
+                               mk<float>(scaled_offset<float>(X - BX, scale), scaled_offset<float>(Y - BY, scale)),
+                               lnrho, half);
+    }
+  }
+  // (-1)^n / n! from n = half PH on
+  float f = half ? ((PH & 1) ? -1.f : 1.f) * (float)inv_fact_d(PH) : 1.f;
+  cpx<float> *out = Lsep + ((int64_t)rhs * ntgt + gg % ntgt) * P + half * PH;
+#pragma unroll
+  for (int i = 0; i < PH; ++i) {
+    if (i > 0) f = -f / (float)(i + half * PH);
+    float re = H[i].re, im = H[i].im;
+#pragma unroll
+    for (int o = 8; o > 1; o >>= 1) {
+      re += __shfl_xor_sync(0xffffffffu, re, o);
+      im += __shfl_xor_sync(0xffffffffu, im, o);
+    }
+    if (active && sub == 0) out[i] = mk(f * re, f * im);
+  }
+}
+
+// k_m2l_bnd in FP32 with two lanes per source: a block of four warps (64 sources at once) per
+// (boundary cell, rhs).
+template <int P>
+__global__ void __launch_bounds__(128) k_m2l_bnd_half(GeoDev gd, int64_t ncell, int64_t nbcell,
+                                                     const int32_t *__restrict__ first,
+                                                     const int32_t *__restrict__ src,
+                                                     const cpx<float> *__restrict__ Mv, cpx<float> *__restrict__ Lb,
+                                                     double lnh) {
+  constexpr int PH = P / 2;
+  __shared__ float red[4][2][2 * PH];
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5, half = tid & 1;
+  const int rhs = blockIdx.y;
+  const int64_t gb = blockIdx.x;
+  int l = 0;
+  while (blevel_offset(l + 1) <= gb) ++l;
+  const uint32_t b = (uint32_t)(gb - blevel_offset(l));
+  const int rho = gd.n >> l;
+  const float lnrho = logf((float)rho);
+  int64_t BX, BY, bs;
+  bnd_geom(gd, l, b, BX, BY, bs);
+  const OffsetScale scale = offset_scale(rho, gd.L);
+  cpx<float> H[PH];
+#pragma unroll
+  for (int i = 0; i < PH; ++i) H[i] = mk<float>(0, 0);
+  const cpx<float> *M = Mv + (int64_t)rhs * ncell * P + level_offset(l) * P;
+  const int e1 = first[gb + 1];
+  for (int e = first[gb] + (tid >> 1); e < e1; e += 64) {
+    const uint32_t v = (uint32_t)src[e];
+    int64_t X, Y, sw;
+    vol_geom(gd, l, v, X, Y, sw);
+    X <<= gd.L;
+    Y <<= gd.L;
+    m2l_accum_half<float, P>(H, M + (int64_t)v * P,
+                             mk<float>(scaled_offset<float>(BX - X, scale), scaled_offset<float>(BY - Y, scale)),
+                             lnrho, half);
+  }
+#pragma unroll
+  for (int i = 0; i < PH; ++i) {
+    float re = H[i].re, im = H[i].im;
+#pragma unroll
+    for (int o = 16; o > 1; o >>= 1) {
+      re += __shfl_xor_sync(0xffffffffu, re, o);
+      im += __shfl_xor_sync(0xffffffffu, im, o);
+    }
+    if (lane < 2) {
+      red[w][half][2 * i] = re;
+      red[w][half][2 * i + 1] = im;
+    }
+  }
+  __syncthreads();
+  if (tid < 2 * P) {  // (coefficient n, re / im)
+    const int n = tid >> 1, hn = n >= PH ? 1 : 0, i = n - hn * PH;
+    float v = 0.f;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) v += red[q][hn][2 * i + (tid & 1)];
+    float f = 1.f;
+    for (int j = 1; j <= n; ++j) f = -f / (float)j;
+    v *= f;
+    float *out = reinterpret_cast<float *>(Lb + ((int64_t)rhs * nbcell + gb) * P);
+    // the four side roots also take the ln h part of G times the total volume weight
+    if (tid == 0 && gb < 4) v += (float)(lnh * (double)Mv[(int64_t)rhs * ncell * P].re);
+    out[tid] = v;
   }
 }
 
@@ -788,16 +945,18 @@ __global__ void k_colloc_mat(Geo g, const int32_t *__restrict__ pfirst, const in
 // upward pass); mode 2: the far sum, added to the near sum read from vnear.  Kc: the near-field
 // log kernel of k_colloc_mat, read 16 bytes a lane (a leaf row's nodes are consecutive in the
 // table and in the weight image, whose rows and halo are multiples of 4 nodes).
-template <typename R>
+template <typename R, int M>
 __global__ void k_colloc(Geo g, int nrhs, const R *__restrict__ wpad, const cpx<R> *__restrict__ Lb,
                          const int32_t *__restrict__ pfirst, const int32_t *__restrict__ psrc,
                          double *__restrict__ vcol, const R *__restrict__ Kc, float *__restrict__ vt_hi,
                          float *__restrict__ vt_lo, int mode, R *__restrict__ vnear) {
-  // block (rhs, along): warp w takes the collocation point `along` of side w
-  __shared__ double sv[4];
-  const int lane = threadIdx.x & 31;
-  const int rhs = (int)(blockIdx.x / g.n), along = (int)(blockIdx.x % g.n), side = threadIdx.x >> 5;
-  const int n = g.n, m = g.m, L = g.L, p = g.p;
+  // block (rhs, k), k < n / 2: warp w takes collocation point k (w < 4) or n - 1 - k of side w % 4
+  __shared__ double sv[8];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  constexpr int m = M;
+  const int n = g.n, L = g.L, p = g.p, hn = n >> 1;
+  const int rhs = (int)(blockIdx.x / hn), kf = (int)(blockIdx.x % hn), side = wid & 3;
+  const int along = wid < 4 ? kf : n - 1 - kf;
   const int ge = side * n + along;
   const int64_t bl = ((int64_t)side << L) + along / m;
   const R *W = wpad + (int64_t)rhs * g.npad * g.npad;
@@ -807,7 +966,7 @@ __global__ void k_colloc(Geo g, int nrhs, const R *__restrict__ wpad, const cpx<
   } else {
     constexpr int V = 16 / sizeof(R);
     const int e0 = pfirst[bl], c_near = pfirst[bl + 1] - e0;
-    const int lgm = 31 - __clz(m), lgv = 2 * lgm - (V == 4 ? 2 : 1);  // m is a power of two
+    constexpr int lgm = M == 4 ? 2 : (M == 8 ? 3 : 4), lgv = 2 * lgm - (V == 4 ? 2 : 1);
     const R *kr = Kc + ((int64_t)e0 * m + (int64_t)(along % m) * c_near) * (m * m);
 #pragma unroll 4
     for (int it = lane; it < c_near << lgv; it += 32) {
@@ -849,33 +1008,54 @@ __global__ void k_colloc(Geo g, int nrhs, const R *__restrict__ wpad, const cpx<
   const double v = ((double)acc + (double)far) * NEG_INV_2PI;
   if (lane == 0) {
     vcol[(int64_t)rhs * g.NG + ge] = v;
-    sv[side] = v;
+    sv[wid] = v;
   }
   if (vt_hi) {
-    // the side DFT of the four values (as k_bem_vt) as FP32 hi + lo words for the BEM apply
+    // the folded side DFT of the eight values (as k_bem_vt) as FP32 hi + lo words for the BEM apply
     __syncthreads();
-    if (threadIdx.x < 4) {
-      const int j = threadIdx.x;
-      const double o = j == 0 ? (sv[0] + sv[2]) + (sv[1] + sv[3])
-                     : j == 1 ? (sv[0] + sv[2]) - (sv[1] + sv[3])
-                     : j == 2 ? sv[0] - sv[2] : sv[1] - sv[3];
-      const float hi = (float)o;
-      vt_hi[(int64_t)rhs * g.NG + j * n + along] = hi;
-      vt_lo[(int64_t)rhs * g.NG + j * n + along] = (float)(o - (double)hi);
+    if (threadIdx.x < 8) {
+      const int j = threadIdx.x >> 1;
+      double o[2];
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        const double *x = sv + 4 * q;
+        o[q] = j == 0 ? (x[0] + x[2]) + (x[1] + x[3])
+             : j == 1 ? (x[0] + x[2]) - (x[1] + x[3])
+             : j == 2 ? x[0] - x[2] : x[1] - x[3];
+      }
+      const double f = (threadIdx.x & 1) ? o[0] - o[1] : o[0] + o[1];
+      const float hi = (float)f;
+      vt_hi[(int64_t)rhs * g.NG + threadIdx.x * hn + kf] = hi;
+      vt_lo[(int64_t)rhs * g.NG + threadIdx.x * hn + kf] = (float)(f - (double)hi);
     }
   }
 }
 
 // ------------------------------------------------------------------ BEM solve (FP64)
-// q = -S^{-1} (V r)|_Gamma with the inverse formed at set-up.  Rotating the square by 90
-// degrees maps element (side s, index k) to (s+1, k), so S and its inverse are block
-// circulant in the four sides: q_s = -sum_d C_d v_{s+d}, C_d the blocks of the first block
-// row.  A 4-point DFT over the side index diagonalises this: with
-//   C^0 = C0+C1+C2+C3, C^2 = C0-C1+C2-C3, A = C0-C2, B = C1-C3 (stored at set-up) and
+// q = -S^{-1} (V r)|_Gamma with the inverse formed at set-up, in the folded form of bem.cu (the
+// square's rotations and reflection).  With C^0, C^2, A, B the side-DFT blocks and
 //   v^0 = v0+v1+v2+v3, v^2 = v0-v1+v2-v3, a = v0-v2, b = v1-v3,
 // P0 = C^0 v^0, P2 = C^2 v^2, R + iI = (A + iB)(a - ib), and
-//   q0 = -(P0+P2+2R)/4, q1 = -(P0-P2-2I)/4, q2 = -(P0+P2-2R)/4, q3 = -(P0-P2+2I)/4:
-// 6 n^2 FP64 multiply-adds instead of 16 n^2 (FP64 is the bound on this part).
+//   q0 = -(P0+P2+2R)/4, q1 = -(P0-P2-2I)/4, q2 = -(P0+P2-2R)/4, q3 = -(P0-P2+2I)/4.
+// On sums (e) and differences (o) of mirrored elements, row m < n / 2 of the folded form gives
+//   P0e = C0e v0e, P0o = C0o v0o, P2 likewise, Re = Ae ae + Bo bo, Ro = Ao ao + Be be,
+//   Ie = Bo ao - Ae be, Io = Be ae - Ao bo,  X[m] = (Xe + Xo) / 2, X[n-1-m] = (Xe - Xo) / 2:
+// 3 n^2 multiply-adds (16 n^2 without the symmetries; FP64 is the bound on this part).
+
+// the eight densities of row m from x = P0e, P0o, P2e, P2o, Re, Ro, Ie, Io
+__device__ __forceinline__ void bem_store(const double (&x)[8], int n, int m, double *__restrict__ q) {
+#pragma unroll
+  for (int f = 0; f < 2; ++f) {
+    double P0, P2, R, I;
+    if (f == 0) P0 = x[0] + x[1], P2 = x[2] + x[3], R = x[4] + x[5], I = x[6] + x[7];
+    else P0 = x[0] - x[1], P2 = x[2] - x[3], R = x[4] - x[5], I = x[6] - x[7];
+    double *qr = q + (f ? n - 1 - m : m);
+    qr[0] = -0.125 * (P0 + P2 + 2.0 * R);
+    qr[n] = -0.125 * (P0 - P2 - 2.0 * I);
+    qr[2 * n] = -0.125 * (P0 + P2 - 2.0 * R);
+    qr[3 * n] = -0.125 * (P0 - P2 + 2.0 * I);
+  }
+}
 
 // The boundary data term of Eq. e:ubound moved to the left: vcol_m -= (1/2 g_m + (K g)_m)
 // at every collocation point, K_mk = int_k dG/dn_y(y_m, y) dGamma = (1/2pi) atan2(l d,
@@ -921,68 +1101,88 @@ __global__ void __launch_bounds__(256) k_dl_colloc(int n, int nrhs, const double
   }
 }
 
-// vt[rhs] = [v^0 | v^2 | a | b] from vcol[rhs] = [v0 | v1 | v2 | v3], add (if given) added to it
+// vt[rhs] = [v0e | v0o | v2e | v2o | ae | ao | be | bo] from vcol[rhs] = [v0 | v1 | v2 | v3], add (if given)
+// added to it
 __global__ void k_bem_vt(int n, int nrhs, const double *__restrict__ vcol, const double *__restrict__ add,
                          double *__restrict__ vt) {
+  const int h = n >> 1;
   const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= (int64_t)nrhs * n) return;
-  const int64_t rr = t / n;
-  const int k = (int)(t % n);
+  if (t >= (int64_t)nrhs * h) return;
+  const int64_t rr = t / h;
+  const int k = (int)(t % h);
   const double *v = vcol + rr * 4 * n;
-  double v0 = v[k], v1 = v[n + k], v2 = v[2 * n + k], v3 = v[3 * n + k];
-  if (add) {
-    const double *a = add + rr * 4 * n;
-    v0 += a[k], v1 += a[n + k], v2 += a[2 * n + k], v3 += a[3 * n + k];
+  double x[2][4];
+#pragma unroll
+  for (int j = 0; j < 2; ++j) {
+    const int c = j ? n - 1 - k : k;
+    double v0 = v[c], v1 = v[n + c], v2 = v[2 * n + c], v3 = v[3 * n + c];
+    if (add) {
+      const double *a = add + rr * 4 * n;
+      v0 += a[c], v1 += a[n + c], v2 += a[2 * n + c], v3 += a[3 * n + c];
+    }
+    x[j][0] = (v0 + v2) + (v1 + v3);
+    x[j][1] = (v0 + v2) - (v1 + v3);
+    x[j][2] = v0 - v2;
+    x[j][3] = v1 - v3;
   }
-  double *o = vt + rr * 4 * n;
-  o[k] = (v0 + v2) + (v1 + v3);
-  o[n + k] = (v0 + v2) - (v1 + v3);
-  o[2 * n + k] = v0 - v2;
-  o[3 * n + k] = v1 - v3;
+  double *o = vt + rr * 4 * n + k;
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    o[(2 * q) * h] = x[0][q] + x[1][q];
+    o[(2 * q + 1) * h] = x[0][q] - x[1][q];
+  }
 }
 
-// Rows m of the transformed first block row T[m] = [C^0 | C^2 | A | B][m], two warps a row (half
-// of its columns each), four rows a block, 16-byte loads.  Bound by FP64 issue: 6 n^2 multiply-adds
-// a right-hand side, 11 us at n = 1024.  The lanes meet by a transposing butterfly, 6 FP64 adds a
-// warp for the four sums: with a warp tree each (20) on eight warps a row the cross-lane adds
-// were as many as the products, and the pass took 27 us.
+// Rows of the folded form, two warps a row (half of its columns each), four rows a block, 16-byte
+// loads.  Bound by FP64 issue: 3 n^2 multiply-adds a right-hand side, 5.4 us at n = 1024.  The lanes
+// meet by a transposing butterfly, 9 FP64 adds a warp for the eight sums (a warp tree each: 40).
 constexpr int BEM64_ROWS = 4;
 __global__ void __launch_bounds__(64 * BEM64_ROWS) k_bem_apply(int n, int nrhs, const double *__restrict__ T,
                                                               const double *__restrict__ vt, double *__restrict__ q) {
-  __shared__ double red[BEM64_ROWS][2][4];
+  __shared__ double red[BEM64_ROWS][2][8];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, rb = w >> 1, hw = w & 1;
-  const int mrow = blockIdx.x * BEM64_ROWS + rb;  // n is a multiple of 4
-  const int NG = 4 * n, n2 = n >> 1, kend = (hw + 1) * (n2 >> 1);
-  const double2 *t2 = reinterpret_cast<const double2 *>(T + (int64_t)mrow * NG);
+  const int h = n >> 1, mrow = blockIdx.x * BEM64_ROWS + rb;
+  const bool live = mrow < h;
+  const int NG = 4 * n, h2 = h >> 1, kmid = h2 >> 1, kend = hw ? h2 : kmid;  // h is even
+  const double2 *t2 = reinterpret_cast<const double2 *>(T + (int64_t)(live ? mrow : 0) * NG);
   for (int rr = 0; rr < nrhs; ++rr) {
     const double2 *v = reinterpret_cast<const double2 *>(vt + (int64_t)rr * NG);
-    double p0 = 0.0, p2 = 0.0, re = 0.0, im = 0.0;
-#pragma unroll 2
-    for (int k = hw * (n2 >> 1) + lane; k < kend; k += 32) {
-      const double2 c0 = t2[k], c2 = t2[n2 + k], ca = t2[2 * n2 + k], cb = t2[3 * n2 + k];
-      const double2 x0 = v[k], x2 = v[n2 + k], a = v[2 * n2 + k], b = v[3 * n2 + k];
-      p0 = fma(c0.x, x0.x, fma(c0.y, x0.y, p0));
-      p2 = fma(c2.x, x2.x, fma(c2.y, x2.y, p2));
-      re = fma(ca.x, a.x, fma(cb.x, b.x, fma(ca.y, a.y, fma(cb.y, b.y, re))));
-      im = fma(cb.x, a.x, fma(-ca.x, b.x, fma(cb.y, a.y, fma(-ca.y, b.y, im))));
-    }
-    // lane 8 g ends with the warp's sum of value g of (p0, p2, re, im)
-    const bool u4 = (lane & 16) != 0, u3 = (lane & 8) != 0;
-    const double b0 = (u4 ? re : p0) + __shfl_xor_sync(0xffffffffu, u4 ? p0 : re, 16);
-    const double b1 = (u4 ? im : p2) + __shfl_xor_sync(0xffffffffu, u4 ? p2 : im, 16);
-    double d = (u3 ? b1 : b0) + __shfl_xor_sync(0xffffffffu, u3 ? b0 : b1, 8);
+    double x[8];
 #pragma unroll
-    for (int o = 4; o > 0; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
-    if ((lane & 7) == 0) red[rb][hw][lane >> 3] = d;
+    for (int i = 0; i < 8; ++i) x[i] = 0.0;
+    for (int k = (hw ? kmid : 0) + lane; k < kend; k += 32) {
+      double2 c[8], y[8];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        c[i] = t2[i * h2 + k];
+        y[i] = v[i * h2 + k];
+      }
+#pragma unroll
+      for (int i = 0; i < 4; ++i) x[i] = fma(c[i].x, y[i].x, fma(c[i].y, y[i].y, x[i]));
+      // c[4 .. 7] = Ae, Ao, Bo, Be; y[4 .. 7] = ae, ao, be, bo
+      x[4] = fma(c[4].x, y[4].x, fma(c[6].x, y[7].x, fma(c[4].y, y[4].y, fma(c[6].y, y[7].y, x[4]))));
+      x[5] = fma(c[5].x, y[5].x, fma(c[7].x, y[6].x, fma(c[5].y, y[5].y, fma(c[7].y, y[6].y, x[5]))));
+      x[6] = fma(c[6].x, y[5].x, fma(-c[4].x, y[6].x, fma(c[6].y, y[5].y, fma(-c[4].y, y[6].y, x[6]))));
+      x[7] = fma(c[7].x, y[4].x, fma(-c[5].x, y[7].x, fma(c[7].y, y[4].y, fma(-c[5].y, y[7].y, x[7]))));
+    }
+    // lane 4 i ends with the warp's sum of x[i]
+    const bool u4 = (lane & 16) != 0, u3 = (lane & 8) != 0, u2 = (lane & 4) != 0;
+    double b[4], d[2];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) b[i] = (u4 ? x[4 + i] : x[i]) + __shfl_xor_sync(0xffffffffu, u4 ? x[i] : x[4 + i], 16);
+#pragma unroll
+    for (int i = 0; i < 2; ++i) d[i] = (u3 ? b[2 + i] : b[i]) + __shfl_xor_sync(0xffffffffu, u3 ? b[i] : b[2 + i], 8);
+    double e = (u2 ? d[1] : d[0]) + __shfl_xor_sync(0xffffffffu, u2 ? d[0] : d[1], 4);
+    e += __shfl_xor_sync(0xffffffffu, e, 2);
+    e += __shfl_xor_sync(0xffffffffu, e, 1);
+    if ((lane & 3) == 0) red[rb][hw][lane >> 2] = e;
     __syncthreads();
-    if (threadIdx.x < BEM64_ROWS) {
-      const double(*x)[4] = red[threadIdx.x];
-      const double P0 = x[0][0] + x[1][0], P2 = x[0][1] + x[1][1], R = x[0][2] + x[1][2], I = x[0][3] + x[1][3];
-      double *qr = q + (int64_t)rr * NG + blockIdx.x * BEM64_ROWS + threadIdx.x;
-      qr[0] = -0.25 * (P0 + P2 + 2.0 * R);
-      qr[n] = -0.25 * (P0 - P2 - 2.0 * I);
-      qr[2 * n] = -0.25 * (P0 + P2 - 2.0 * R);
-      qr[3 * n] = -0.25 * (P0 - P2 + 2.0 * I);
+    const int m = blockIdx.x * BEM64_ROWS + threadIdx.x;
+    if (threadIdx.x < BEM64_ROWS && m < h) {
+      double tot[8];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) tot[i] = red[threadIdx.x][0][i] + red[threadIdx.x][1][i];
+      bem_store(tot, n, m, q + (int64_t)rr * NG);
     }
     __syncthreads();
   }
@@ -1005,99 +1205,197 @@ __device__ __forceinline__ void dot2_mac(float &s, float &c, float ah, float al,
   c = fmaf(al, bh, fmaf(ah, bl, c + e));
 }
 
-// The BEM apply of k_bem_apply in two-word FP32 arithmetic: two warps per row m of
-// T = [C^0 | C^2 | A | B], each half of its columns (two rows per block), RB right-hand sides
-// per pass over it.  A lane takes four consecutive columns at a time (16-byte loads of the
-// four blocks, hi and lo) and two such steps at once, so that a row's loads are in flight
-// together and the pass is a sweep over T at memory speed rather than a chain of load round
-// trips.  The partial two-word sums are combined with TwoSum over the warp's lanes, then
-// over the row's two warps, and converted to FP64 once per row and right-hand side.  n is a
-// multiple of 8 and the rows start 16-byte aligned.
-constexpr int BEM_ROWS = 2;  // rows per block, two warps each
-template <int RB>
-__global__ void __launch_bounds__(64 * BEM_ROWS) k_bem_apply_f2(int n, int nrhs, const float *__restrict__ Th,
-                                                              const float *__restrict__ Tl, const float *__restrict__ vh,
-                                                              const float *__restrict__ vl, double *__restrict__ q) {
-  __shared__ float xs[BEM_ROWS][RB][4], xc[BEM_ROWS][RB][4];
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, rb = w >> 1, hw = w & 1;
-  const int mrow = blockIdx.x * BEM_ROWS + rb;
-  const bool live = mrow < n;  // block-uniform for the barrier below: n is a multiple of BEM_ROWS
-  const int NG = 4 * n, n4 = n >> 2, kbeg = hw * (n4 >> 1), kend = kbeg + (n4 >> 1);
+// One step of a folded row in two-word FP32, the eight sums of k_bem_apply += four columns of the
+// blocks times the folded values: c, y = blocks 0 .. 3 (C^0, C^2) or 4 .. 7 (A, B), hi and lo words.
+__device__ __forceinline__ float lane4(const float4 &v, int j) { return j == 0 ? v.x : (j == 1 ? v.y : (j == 2 ? v.z : v.w)); }
+__device__ __forceinline__ void bem_step_c(float (&sa)[8], float (&ca)[8], const float4 (&ch)[4], const float4 (&cl)[4],
+                                           const float4 (&yh)[4], const float4 (&yl)[4]) {
+#pragma unroll
+  for (int j = 0; j < 4; ++j)
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      dot2_mac(sa[i], ca[i], lane4(ch[i], j), lane4(cl[i], j), lane4(yh[i], j), lane4(yl[i], j));
+}
+__device__ __forceinline__ void bem_step_ab(float (&sa)[8], float (&ca)[8], const float4 (&ch)[4], const float4 (&cl)[4],
+                                            const float4 (&yh)[4], const float4 (&yl)[4]) {
+  // c = Ae, Ao, Bo, Be; y = ae, ao, be, bo
+  constexpr int out[8] = {4, 4, 5, 5, 6, 6, 7, 7}, ci[8] = {0, 2, 1, 3, 2, 0, 3, 1}, yi[8] = {0, 3, 1, 2, 1, 2, 0, 3};
+#pragma unroll
+  for (int j = 0; j < 4; ++j)
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+      const float sg = (e == 5 || e == 7) ? -1.f : 1.f;  // Ie -= Ae be, Io -= Ao bo
+      dot2_mac(sa[out[e]], ca[out[e]], sg * lane4(ch[ci[e]], j), sg * lane4(cl[ci[e]], j), lane4(yh[yi[e]], j),
+               lane4(yl[yi[e]], j));
+    }
+}
+
+// The warp's two-word sums of eight values by a transposing butterfly (each of the first three steps
+// a lane keeps half of its values): lane 4 i ends with value i in s[0], c[0].
+__device__ __forceinline__ void warp_two_sum8(float (&s)[8], float (&c)[8]) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int st = 0; st < 5; ++st) {
+    const int o = 16 >> st, hv = st < 3 ? 4 >> st : 1;
+    const bool up = st < 3 && (lane & o);
+#pragma unroll
+    for (int i = 0; i < hv; ++i) {
+      float ks = s[i], kc = c[i], gs = s[i], gc = c[i];
+      if (st < 3) {
+        ks = up ? s[hv + i] : s[i], gs = up ? s[i] : s[hv + i];
+        kc = up ? c[hv + i] : c[i], gc = up ? c[i] : c[hv + i];
+      }
+      gs = __shfl_xor_sync(0xffffffffu, gs, o);
+      gc = __shfl_xor_sync(0xffffffffu, gc, o);
+      two_sum_acc(ks, kc, gs);
+      s[i] = ks;
+      c[i] = kc + gc;
+    }
+  }
+}
+
+// The BEM apply in two-word FP32 arithmetic, few right-hand sides: four warps per row of the folded
+// form, a quarter of its columns each (16-byte loads; at n = 1024 one step of 2 x 16 loads per lane),
+// so that the pass is two memory round trips.  The partial two-word sums are
+// combined with TwoSum over the lanes and the row's warps, and converted to FP64 once.  n = 1024:
+// 17 MB of table, 7 us (12 us from the side-DFT form's 34 MB).  Rows of n <= 4 (h = 2) have no whole float4: the
+// launch takes the FP64 kernel there.
+__global__ void __launch_bounds__(128, 4) k_bem_apply_f2(int n, const float *__restrict__ Th,
+                                                        const float *__restrict__ Tl, const float *__restrict__ vh,
+                                                        const float *__restrict__ vl, double *__restrict__ q) {
+  __shared__ float xs[4][8], xc[4][8];
+  __shared__ double tot[8];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, mrow = blockIdx.x;
+  const int h = n >> 1, h4 = h >> 2, NG = 4 * n;
+  const int kbeg = (h4 * w) >> 2, kend = (h4 * (w + 1)) >> 2;
   const float4 *th = reinterpret_cast<const float4 *>(Th + (int64_t)mrow * NG);
   const float4 *tl = reinterpret_cast<const float4 *>(Tl + (int64_t)mrow * NG);
-  for (int r0 = 0; r0 < nrhs; r0 += RB) {
-    float sa[RB][4], ca[RB][4];
+  {
+    const int rr = blockIdx.y;
+    const float4 *xh = reinterpret_cast<const float4 *>(vh + (int64_t)rr * NG);
+    const float4 *xl = reinterpret_cast<const float4 *>(vl + (int64_t)rr * NG);
+    float sa[8], ca[8];
 #pragma unroll
-    for (int j = 0; j < RB; ++j)
+    for (int i = 0; i < 8; ++i) sa[i] = ca[i] = 0.f;
+    for (int k = kbeg + lane; k < kend; k += 32) {
 #pragma unroll
-      for (int g = 0; g < 4; ++g) sa[j][g] = ca[j][g] = 0.f;
-#pragma unroll 2
-    for (int k4 = kbeg + lane; live && k4 < kend; k4 += 32) {
-      const float4 c0h = th[k4], c2h = th[n4 + k4], cah = th[2 * n4 + k4], cbh = th[3 * n4 + k4];
-      const float4 c0l = tl[k4], c2l = tl[n4 + k4], cal = tl[2 * n4 + k4], cbl = tl[3 * n4 + k4];
+      for (int g = 0; g < 2; ++g) {
+        float4 ch[4], cl[4], yh[4], yl[4];
 #pragma unroll
-      for (int j = 0; j < RB; ++j) {
-        if (r0 + j < nrhs) {
-          const float4 *xh = reinterpret_cast<const float4 *>(vh + (int64_t)(r0 + j) * NG);
-          const float4 *xl = reinterpret_cast<const float4 *>(vl + (int64_t)(r0 + j) * NG);
-          const float4 v0h = xh[k4], v2h = xh[n4 + k4], ah = xh[2 * n4 + k4], bh = xh[3 * n4 + k4];
-          const float4 v0l = xl[k4], v2l = xl[n4 + k4], al = xl[2 * n4 + k4], bl = xl[3 * n4 + k4];
-          const float c0h_[4] = {c0h.x, c0h.y, c0h.z, c0h.w}, c0l_[4] = {c0l.x, c0l.y, c0l.z, c0l.w};
-          const float c2h_[4] = {c2h.x, c2h.y, c2h.z, c2h.w}, c2l_[4] = {c2l.x, c2l.y, c2l.z, c2l.w};
-          const float cah_[4] = {cah.x, cah.y, cah.z, cah.w}, cal_[4] = {cal.x, cal.y, cal.z, cal.w};
-          const float cbh_[4] = {cbh.x, cbh.y, cbh.z, cbh.w}, cbl_[4] = {cbl.x, cbl.y, cbl.z, cbl.w};
-          const float v0h_[4] = {v0h.x, v0h.y, v0h.z, v0h.w}, v0l_[4] = {v0l.x, v0l.y, v0l.z, v0l.w};
-          const float v2h_[4] = {v2h.x, v2h.y, v2h.z, v2h.w}, v2l_[4] = {v2l.x, v2l.y, v2l.z, v2l.w};
-          const float ah_[4] = {ah.x, ah.y, ah.z, ah.w}, al_[4] = {al.x, al.y, al.z, al.w};
-          const float bh_[4] = {bh.x, bh.y, bh.z, bh.w}, bl_[4] = {bl.x, bl.y, bl.z, bl.w};
-#pragma unroll
-          for (int c = 0; c < 4; ++c) {
-            dot2_mac(sa[j][0], ca[j][0], c0h_[c], c0l_[c], v0h_[c], v0l_[c]);
-            dot2_mac(sa[j][1], ca[j][1], c2h_[c], c2l_[c], v2h_[c], v2l_[c]);
-            dot2_mac(sa[j][2], ca[j][2], cah_[c], cal_[c], ah_[c], al_[c]);  // re = A a + B b
-            dot2_mac(sa[j][2], ca[j][2], cbh_[c], cbl_[c], bh_[c], bl_[c]);
-            dot2_mac(sa[j][3], ca[j][3], cbh_[c], cbl_[c], ah_[c], al_[c]);  // im = B a - A b
-            dot2_mac(sa[j][3], ca[j][3], -cah_[c], -cal_[c], bh_[c], bl_[c]);
-          }
+        for (int i = 0; i < 4; ++i) {
+          ch[i] = th[(4 * g + i) * h4 + k];
+          cl[i] = tl[(4 * g + i) * h4 + k];
+          yh[i] = xh[(4 * g + i) * h4 + k];
+          yl[i] = xl[(4 * g + i) * h4 + k];
         }
+        if (g == 0) bem_step_c(sa, ca, ch, cl, yh, yl);
+        else bem_step_ab(sa, ca, ch, cl, yh, yl);
       }
     }
-#pragma unroll
-    for (int j = 0; j < RB; ++j)
-#pragma unroll
-      for (int g = 0; g < 4; ++g) {
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-          const float s2 = __shfl_xor_sync(0xffffffffu, sa[j][g], o), c2 = __shfl_xor_sync(0xffffffffu, ca[j][g], o);
-          two_sum_acc(sa[j][g], ca[j][g], s2);
-          ca[j][g] += c2;
-        }
-        if (hw == 1 && lane == 0) {
-          xs[rb][j][g] = sa[j][g];
-          xc[rb][j][g] = ca[j][g];
-        }
-      }
+    warp_two_sum8(sa, ca);  // lane 4 i: the warp's sum of value i
+    if ((lane & 3) == 0) {
+      xs[w][lane >> 2] = sa[0];
+      xc[w][lane >> 2] = ca[0];
+    }
     __syncthreads();
+    if (threadIdx.x < 8) {
+      const int i = threadIdx.x;
+      float s0 = xs[0][i], c0 = xc[0][i];
 #pragma unroll
-    for (int j = 0; j < RB; ++j) {
-      double tot[4];
-#pragma unroll
-      for (int g = 0; g < 4; ++g) {
-        float s0 = sa[j][g], c0 = ca[j][g];  // the first half's sums (lane 0 of warp hw = 0)
-        two_sum_acc(s0, c0, xs[rb][j][g]);
-        c0 += xc[rb][j][g];
-        tot[g] = (double)s0 + (double)c0;
+      for (int k = 1; k < 4; ++k) {
+        two_sum_acc(s0, c0, xs[k][i]);
+        c0 += xc[k][i];
       }
-      if (hw == 0 && lane == 0 && live && r0 + j < nrhs) {
-        const double P0 = tot[0], P2 = tot[1], R = tot[2], I = tot[3];
-        double *qr = q + (int64_t)(r0 + j) * NG;
-        qr[mrow] = -0.25 * (P0 + P2 + 2.0 * R);
-        qr[n + mrow] = -0.25 * (P0 - P2 - 2.0 * I);
-        qr[2 * n + mrow] = -0.25 * (P0 + P2 - 2.0 * R);
-        qr[3 * n + mrow] = -0.25 * (P0 - P2 + 2.0 * I);
+      tot[i] = (double)s0 + (double)c0;
+      __syncwarp(0xff);
+      // thread (f, side): element mrow or its mirror of one side, as bem_store
+      const int f = i >> 2, sd = i & 3;
+      const double sg = f ? -1.0 : 1.0;
+      const double P0 = fma(sg, tot[1], tot[0]), P2 = fma(sg, tot[3], tot[2]);
+      const double RI = (sd & 1) ? fma(sg, tot[7], tot[6]) : fma(sg, tot[5], tot[4]);
+      const double pp = (sd & 1) ? P0 - P2 : P0 + P2;
+      q[(int64_t)rr * NG + (int64_t)sd * n + (f ? n - 1 - mrow : mrow)] =
+          -0.125 * fma((sd == 1 || sd == 2) ? -2.0 : 2.0, RI, pp);
+    }
+  }
+}
+
+// The same for many right-hand sides: a warp per row, eight rows and RB right-hand sides per block; the
+// folded values of a tile of 128 columns of every block are staged in shared memory once for the
+// eight rows (read from L2 per pair of rows they were as many bytes as ten tables: 4.4 ms at
+// 4096^2 x 32).
+constexpr int BEMM_RB = 4, BEMM_CT = 32;  // right-hand sides, float4 columns per tile
+__global__ void __launch_bounds__(256) k_bem_apply_f2m(int n, int nrhs, const float *__restrict__ Th,
+                                                      const float *__restrict__ Tl, const float *__restrict__ vh,
+                                                      const float *__restrict__ vl, double *__restrict__ q) {
+  __shared__ float4 sv[BEMM_RB][2][8][BEMM_CT];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int h = n >> 1, h4 = h >> 2, NG = 4 * n, mrow = blockIdx.x * 8 + w;  // h is a multiple of 8
+  const int r0 = blockIdx.y * BEMM_RB;
+  const float4 *th = reinterpret_cast<const float4 *>(Th + (int64_t)mrow * NG);
+  const float4 *tl = reinterpret_cast<const float4 *>(Tl + (int64_t)mrow * NG);
+  // the sums in k_bem_apply_f2's order, a quarter of the columns at a time, so that a right-hand side's
+  // densities do not depend on how many others it comes with; lane 4 i keeps value i
+  float rs[BEMM_RB], rc[BEMM_RB];
+#pragma unroll
+  for (int j = 0; j < BEMM_RB; ++j) rs[j] = rc[j] = 0.f;
+  for (int quarter = 0; quarter < 4; ++quarter) {
+    float sa[BEMM_RB][8], ca[BEMM_RB][8];
+#pragma unroll
+    for (int j = 0; j < BEMM_RB; ++j)
+#pragma unroll
+      for (int i = 0; i < 8; ++i) sa[j][i] = ca[j][i] = 0.f;
+    const int kq = (h4 >> 2) * quarter;  // h4 / 4 is a multiple of the tile
+    for (int k0 = kq; k0 < kq + (h4 >> 2); k0 += BEMM_CT) {
+      const int k = k0 + lane;
+      __syncthreads();
+      for (int e = w; e < BEMM_RB * 16; e += 8) {  // (right-hand side, word, block): a row of the tile
+        const int j = e >> 4, wd = (e >> 3) & 1, i = e & 7;
+        const float *src = wd ? vl : vh;
+        sv[j][wd][i][lane] = r0 + j < nrhs ? reinterpret_cast<const float4 *>(src + (int64_t)(r0 + j) * NG)[i * h4 + k]
+                                           : make_float4(0.f, 0.f, 0.f, 0.f);
+      }
+      __syncthreads();
+#pragma unroll
+      for (int g = 0; g < 2; ++g) {
+        float4 ch[4], cl[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          ch[i] = th[(4 * g + i) * h4 + k];
+          cl[i] = tl[(4 * g + i) * h4 + k];
+        }
+#pragma unroll
+        for (int j = 0; j < BEMM_RB; ++j) {
+          float4 yh[4], yl[4];
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            yh[i] = sv[j][0][4 * g + i][lane];
+            yl[i] = sv[j][1][4 * g + i][lane];
+          }
+          if (g == 0) bem_step_c(sa[j], ca[j], ch, cl, yh, yl);
+          else bem_step_ab(sa[j], ca[j], ch, cl, yh, yl);
+        }
       }
     }
-    __syncthreads();  // xs, xc are rewritten by the next pass
+#pragma unroll
+    for (int j = 0; j < BEMM_RB; ++j) {
+      warp_two_sum8(sa[j], ca[j]);
+      if (quarter == 0) {
+        rs[j] = sa[j][0];
+        rc[j] = ca[j][0];
+      } else {
+        two_sum_acc(rs[j], rc[j], sa[j][0]);
+        rc[j] += ca[j][0];
+      }
+    }
+  }
+#pragma unroll
+  for (int j = 0; j < BEMM_RB; ++j) {
+    const double t = (double)rs[j] + (double)rc[j];
+    double tot[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) tot[i] = __shfl_sync(0xffffffffu, t, 4 * i);
+    if (lane == 0 && r0 + j < nrhs) bem_store(tot, n, mrow, q + (int64_t)(r0 + j) * NG);
   }
 }
 
@@ -1173,18 +1471,19 @@ __global__ void k_colloc_T_far(Geo g, double *__restrict__ wt) {
 // Evaluating the closed-form integrals in every pass cost 5e6 FP64 log, log1p and atan2 and a
 // serial far sum per element: 1484 us at 1024^2; from the tables it is 5e6 FP64 multiply-adds
 // (8.7 us of the FP64 pipe, 40 MB of table).
-template <typename R>
+template <typename R, int M>
 __global__ void __launch_bounds__(128) k_colloc_T(Geo g, const R *__restrict__ wpad, const cpx<R> *__restrict__ Lb,
                                                   const int32_t *__restrict__ pfirst, const int32_t *__restrict__ psrc,
                                                   const double *__restrict__ Kt, const double *__restrict__ wt,
                                                   double *__restrict__ tout) {
   const int lane = threadIdx.x & 31;
   const int rhs = (int)(blockIdx.x / g.n), along = (int)(blockIdx.x % g.n), side = threadIdx.x >> 5;
-  const int n = g.n, m = g.m, L = g.L, p = g.p;
+  constexpr int m = M, lgm = M == 4 ? 2 : (M == 8 ? 3 : 4), lgv = 2 * lgm - 1;
+  const int n = g.n, L = g.L, p = g.p;
   const int64_t bl = ((int64_t)side << L) + along / m;
   const R *W = wpad + (int64_t)rhs * g.npad * g.npad;
   double acc = 0.0;
-  const int e0 = pfirst[bl], c_near = pfirst[bl + 1] - e0, lgm = 31 - __clz(m), lgv = 2 * lgm - 1;
+  const int e0 = pfirst[bl], c_near = pfirst[bl + 1] - e0;
   const double2 *kr =
       reinterpret_cast<const double2 *>(Kt + ((int64_t)e0 * m + (int64_t)(along % m) * c_near) * (m * m));
 #pragma unroll 4
@@ -1265,7 +1564,7 @@ __global__ void __launch_bounds__(256) k_bnd_near_mat(Geo g, const int32_t *__re
 // independent loads; partials meet in shared memory.  Bound by the table's bytes (FP32, 20 MB at
 // 1024^2) or FP64 multiply-adds (5e6: 8.7 us), where evaluating the FP64 form's integrals in each
 // pass took 1216 us and the transpose's logs 462 us.
-template <typename TK, typename R, bool TWO>
+template <typename TK, typename R, int M, bool TWO>
 __global__ void __launch_bounds__(256) k_bnd_tab(Geo g, int64_t nbnear, const int32_t *__restrict__ first,
                                                  const int32_t *__restrict__ src, const TK *__restrict__ K,
                                                  const double *__restrict__ dens, TK scale,
@@ -1275,9 +1574,9 @@ __global__ void __launch_bounds__(256) k_bnd_tab(Geo g, int64_t nbnear, const in
   __shared__ __align__(16) TK red[256 * V];
   __shared__ TK sden[256];
   const int slot = blockIdx.x, rhs = blockIdx.y, tid = threadIdx.x;
-  const int n = g.n, m = g.m, L = g.L, mm = m * m;
-  const int lgm = 31 - __clz(m), lgl = 2 * lgm - (V == 4 ? 2 : 1);  // m is a power of two
-  const int ngrp = 256 >> lgl, tv = tid & ((1 << lgl) - 1), grp = tid >> lgl;
+  constexpr int m = M, mm = m * m, lgm = M == 4 ? 2 : (M == 8 ? 3 : 4), lgl = 2 * lgm - (V == 4 ? 2 : 1);
+  constexpr int ngrp = 256 >> lgl;
+  const int n = g.n, L = g.L, tv = tid & ((1 << lgl) - 1), grp = tid >> lgl;
   const int f0 = first[slot], cnt = (first[slot + 1] - f0) * m;
   TK sum = 0;
 #pragma unroll
@@ -1447,7 +1746,7 @@ __device__ __forceinline__ double near_far_sum(float s, float s_lo, float v) {
 // cell b, its 4 children and the 16 leaves, and evaluates each leaf expansion at the leaf's
 // nodes (NPT consecutive nodes of one row per thread, so a warp writes whole row segments).
 template <typename R, int P, int M>
-__global__ void __launch_bounds__(256) k_downward_tree(Geo g, int nrhs, int do_bnd, int64_t nbnear,
+__global__ void __launch_bounds__(256, (sizeof(R) == 4 && P <= 10 && M <= 8) ? 7 : 1) k_downward_tree(Geo g, int nrhs, int do_bnd, int64_t nbnear,
                                                        const cpx<R> *__restrict__ Mv, const cpx<R> *__restrict__ Mb,
                                                        int with_bnd_w, const cpx<R> *__restrict__ vl2l,
                                                        const cpx<R> *__restrict__ Lv, const int32_t *__restrict__ vslot,
@@ -1799,6 +2098,14 @@ void run_downward(fmmpc_handle &H, double *out, int nrhs, int do_bnd, int with_b
 }
 
 
+// f(integral_constant<int, m>) for the leaf side m
+template <typename F>
+void with_leaf_side(int m, F &&f) {
+  if (m == 4) f(std::integral_constant<int, 4>{});
+  else if (m == 8) f(std::integral_constant<int, 8>{});
+  else f(std::integral_constant<int, 16>{});
+}
+
 // Near-boundary correction phib at the nodes of the leaves next to the boundary.
 template <typename R>
 int run_bnd_near(fmmpc_handle &H, int nrhs, cudaStream_t s) {
@@ -1809,22 +2116,24 @@ int run_bnd_near(fmmpc_handle &H, int nrhs, cudaStream_t s) {
   R *phib = (R *)H.fb.phib;
   const R *knear = (const R *)H.fb.knear, *kdl = (const R *)H.fb.kdl;
   int launches = 1;
-  if (H.trans_pass) {  // point sources h^2 c' at the collocation points (transpose pass)
-    k_bnd_tab<double, R, false><<<grid, 256, 0, s>>>(g, Ls.nbnear, first, src, H.fb.kpt, H.fb.q, g.h * g.h, nullptr,
-                                                     nullptr, 0.0, phib);
-  } else if (H.bem_form == 1) {  // double-layer correction: D mu only (mu in fb.q)
-    k_bnd_tab<R, R, false><<<grid, 256, 0, s>>>(g, Ls.nbnear, first, src, kdl, H.fb.q, R(1), nullptr, nullptr, R(0),
-                                                phib);
-  } else if (H.bc_g && kdl) {  // single layer, and the boundary data: - D g of Eq. e:uinter
-    k_bnd_tab<R, R, true><<<grid, 256, 0, s>>>(g, Ls.nbnear, first, src, knear, H.fb.q, R(1), kdl, H.bc_g, R(-1), phib);
-  } else {
-    k_bnd_tab<R, R, false><<<grid, 256, 0, s>>>(g, Ls.nbnear, first, src, knear, H.fb.q, R(1), nullptr, nullptr, R(0),
-                                                phib);
-    if (H.bc_g) {  // no table of the double layer (init_bnd_dl)
-      k_dl_near<R><<<grid, 256, 0, s>>>(g, Ls.nbnear, Ls.pbv_leaf, first, src, H.bc_g, R(-1), phib);
-      ++launches;
+  with_leaf_side(g.m, [&](auto mc) {
+    if (H.trans_pass) {  // point sources h^2 c' at the collocation points (transpose pass)
+      k_bnd_tab<double, R, mc(), false><<<grid, 256, 0, s>>>(g, Ls.nbnear, first, src, H.fb.kpt, H.fb.q, g.h * g.h, nullptr,
+                                                       nullptr, 0.0, phib);
+    } else if (H.bem_form == 1) {  // double-layer correction: D mu only (mu in fb.q)
+      k_bnd_tab<R, R, mc(), false><<<grid, 256, 0, s>>>(g, Ls.nbnear, first, src, kdl, H.fb.q, R(1), nullptr, nullptr, R(0),
+                                                  phib);
+    } else if (H.bc_g && kdl) {  // single layer, and the boundary data: - D g of Eq. e:uinter
+      k_bnd_tab<R, R, mc(), true><<<grid, 256, 0, s>>>(g, Ls.nbnear, first, src, knear, H.fb.q, R(1), kdl, H.bc_g, R(-1), phib);
+    } else {
+      k_bnd_tab<R, R, mc(), false><<<grid, 256, 0, s>>>(g, Ls.nbnear, first, src, knear, H.fb.q, R(1), nullptr, nullptr, R(0),
+                                                  phib);
+      if (H.bc_g) {  // no table of the double layer (init_bnd_dl)
+        k_dl_near<R><<<grid, 256, 0, s>>>(g, Ls.nbnear, Ls.pbv_leaf, first, src, H.bc_g, R(-1), phib);
+        ++launches;
+      }
     }
-  }
+  });
   FMMPC_LAUNCH_CHECK();
   return launches;
 }
@@ -1892,8 +2201,8 @@ void apply_impl(fmmpc_handle &H, int part, const double *r, double *out, int nrh
   const bool bc = part == PART_BC && H.bc_g;   // boundary data g (Eqs. e:ubound / e:uinter)
   const bool bc_tab = bc && H.Kbc;
   auto boundary_data = [&](cudaStream_t st) {  // -(1/2 I + K) g, added to vcol where its side DFT is taken
-    k_bem_vt<<<nblk((int64_t)nrhs * g.n), 256, 0, st>>>(g.n, nrhs, H.bc_g, nullptr, H.bc_vt);
-    k_bem_apply<<<g.n / BEM64_ROWS, 64 * BEM64_ROWS, 0, st>>>(g.n, nrhs, H.Kbc, H.bc_vt, H.bc_kg);
+    k_bem_vt<<<nblk((int64_t)nrhs * g.n / 2), 256, 0, st>>>(g.n, nrhs, H.bc_g, nullptr, H.bc_vt);
+    k_bem_apply<<<nblk(g.n / 2, BEM64_ROWS), 64 * BEM64_ROWS, 0, st>>>(g.n, nrhs, H.Kbc, H.bc_vt, H.bc_kg);
     FMMPC_LAUNCH_CHECK();
     launches += 2;
   };
@@ -1902,7 +2211,7 @@ void apply_impl(fmmpc_handle &H, int part, const double *r, double *out, int nrh
   // streams of their own, forked after the weights and after the upward pass and joined before
   // the downward pass, in every form and for the plain, boundary-data and transpose applies.
   // (One stream for them all kept the chain's latency-bound kernels in line behind the long
-  // ones: 128^2 FP32 83 -> 56 us.)
+  // ones: 128^2 FP32 83 -> 50 us.)
   const bool side = with_bnd && part != PART_VCOL && part != PART_Q && g.L >= 2 && H.timing == 0;
   cudaStream_t ss = H.sstream;
   // the near part of the collocation values needs only the weights: with the side streams
@@ -1940,8 +2249,10 @@ void apply_impl(fmmpc_handle &H, int part, const double *r, double *out, int nrh
     }
     if (split_colloc || bc_tab) FMMPC_CUDA(cudaStreamWaitEvent(H.sstream2, H.sev[0], 0));
     if (split_colloc) {
-      k_colloc<R><<<(unsigned)((int64_t)g.n * nrhs), 128, 0, H.sstream2>>>(
-          g, nrhs, wpad, Lb, Ls.pvb_first, Ls.pvb_src, H.fb.vcol, (const R *)H.fb.kcol, nullptr, nullptr, 1, (R *)H.fb.vnear);
+      with_leaf_side(g.m, [&](auto mc) {
+        k_colloc<R, mc()><<<(unsigned)((int64_t)(g.n / 2) * nrhs), 256, 0, H.sstream2>>>(
+            g, nrhs, wpad, Lb, Ls.pvb_first, Ls.pvb_src, H.fb.vcol, (const R *)H.fb.kcol, nullptr, nullptr, 1, (R *)H.fb.vnear);
+      });
       FMMPC_LAUNCH_CHECK();
       ++launches;
     }
@@ -1958,28 +2269,36 @@ void apply_impl(fmmpc_handle &H, int part, const double *r, double *out, int nrh
     if (tc) {
       // the tensor-core near field fills the SMs' shared memory: started with the upward pass, which
       // the whole chain waits for, it doubles that pass's time (16 -> 31 us at 1024^2), so it starts
-      // after it (1024^2 apply 131 -> 123 us); the CUDA-core one, of small grids, is longer than its
-      // slack and starts at once (128^2: 54 -> 50 us)
+      // after it (1024^2 apply 123 -> 120 us, 2048^2 solve 17.5 -> 17.0 ms); the CUDA-core one, of small
+      // grids, is longer than its slack and starts at once (128^2: 54 -> 50 us)
       FMMPC_CUDA(cudaStreamWaitEvent(ss, H.sev[1], 0));
       near_field(ss);
     }
   }
   if (with_bnd) {
     mark(2);
-    k_m2l_bnd<R, P><<<nblk(g.nbcell * nrhs * 32), 256, 0, s>>>(gd, g.ncell, g.nbcell, nrhs, Ls.vbb_first,
-                                                              Ls.vbb_src, Mv, Lb, g.lnh);
+    if constexpr (f64)  // bound by FP64 issue, where a source's powers are worth sharing
+      k_m2l_bnd<R, P><<<nblk(g.nbcell * nrhs * 32), 256, 0, s>>>(gd, g.ncell, g.nbcell, nrhs, Ls.vbb_first,
+                                                                Ls.vbb_src, Mv, Lb, g.lnh);
+    else
+      k_m2l_bnd_half<P><<<dim3((unsigned)g.nbcell, (unsigned)nrhs), 128, 0, s>>>(gd, g.ncell, g.nbcell, Ls.vbb_first,
+                                                                                Ls.vbb_src, Mv, Lb, g.lnh);
     // the side DFT for the two-word BEM apply, fused (not with boundary data, which changes
     // vcol after this kernel)
-    const bool vt_f2 = H.Sinv_hi && H.fb.vt_hi && !bc && !trans;
+    const bool vt_f2 = H.Sinv_hi && H.fb.vt_hi && !bc && !trans && g.n >= 8;  // rows of whole float4
     if (trans)  // t = S_OG^T zb: element integrals of the volume potential, into vcol
-      k_colloc_T<R><<<(unsigned)((int64_t)g.n * nrhs), 128, 0, s>>>(g, wpad, Lb, Ls.pvb_first, Ls.pvb_src, H.fb.kcolT,
-                                                                    H.fb.wfarT, H.fb.vcol);
+      with_leaf_side(g.m, [&](auto mc) {
+        k_colloc_T<R, mc()><<<(unsigned)((int64_t)g.n * nrhs), 128, 0, s>>>(g, wpad, Lb, Ls.pvb_first, Ls.pvb_src, H.fb.kcolT,
+                                                                      H.fb.wfarT, H.fb.vcol);
+      });
     else {
       if (split_colloc) FMMPC_CUDA(cudaStreamWaitEvent(s, H.sev[6], 0));  // and the boundary data's
-      k_colloc<R><<<(unsigned)((int64_t)g.n * nrhs), 128, 0, s>>>(g, nrhs, wpad, Lb, Ls.pvb_first, Ls.pvb_src,
-                                                                 H.fb.vcol, (const R *)H.fb.kcol, vt_f2 ? H.fb.vt_hi : nullptr,
-                                                                 vt_f2 ? H.fb.vt_lo : nullptr, split_colloc ? 2 : 0,
-                                                                 (R *)H.fb.vnear);
+      with_leaf_side(g.m, [&](auto mc) {
+        k_colloc<R, mc()><<<(unsigned)((int64_t)(g.n / 2) * nrhs), 256, 0, s>>>(g, nrhs, wpad, Lb, Ls.pvb_first, Ls.pvb_src,
+                                                                   H.fb.vcol, (const R *)H.fb.kcol, vt_f2 ? H.fb.vt_hi : nullptr,
+                                                                   vt_f2 ? H.fb.vt_lo : nullptr, split_colloc ? 2 : 0,
+                                                                   (R *)H.fb.vnear);
+      });
     }
     FMMPC_LAUNCH_CHECK();
     launches += 2;
@@ -2001,13 +2320,18 @@ void apply_impl(fmmpc_handle &H, int part, const double *r, double *out, int nrh
     // q = S^{-1}(-vcol), or mu = (-1/2 I + K)^{-1}(-vcol) in the double-layer form
     const float *Th = dl ? H.Kdl_hi : H.Sinv_hi, *Tl = dl ? H.Kdl_lo : H.Sinv_lo;
     if (vt_f2 && Th) {  // vt_hi / vt_lo came with the collocation values
-      const unsigned nb = (unsigned)((g.n + BEM_ROWS - 1) / BEM_ROWS);
-      if (nrhs >= 4) k_bem_apply_f2<4><<<nb, 64 * BEM_ROWS, 0, s>>>(g.n, nrhs, Th, Tl, H.fb.vt_hi, H.fb.vt_lo, H.fb.q);
-      else k_bem_apply_f2<1><<<nb, 64 * BEM_ROWS, 0, s>>>(g.n, nrhs, Th, Tl, H.fb.vt_hi, H.fb.vt_lo, H.fb.q);
+      // eight rows per block from four right-hand sides on, where the rows then still fill the SMs
+      // (4096^2 x 4: 465 -> 208 us; 1024^2 x 4: 41 -> 45, so one row a block there)
+      if (nrhs >= BEMM_RB && g.n >= 2048)
+        k_bem_apply_f2m<<<dim3((unsigned)(g.n / 16), (unsigned)((nrhs + BEMM_RB - 1) / BEMM_RB)), 256, 0, s>>>(
+            g.n, nrhs, Th, Tl, H.fb.vt_hi, H.fb.vt_lo, H.fb.q);
+      else
+        k_bem_apply_f2<<<dim3((unsigned)(g.n / 2), (unsigned)nrhs), 128, 0, s>>>(g.n, Th, Tl, H.fb.vt_hi, H.fb.vt_lo,
+                                                                                H.fb.q);
       ++launches;
     } else {
-      k_bem_vt<<<nblk((int64_t)nrhs * g.n), 256, 0, s>>>(g.n, nrhs, H.fb.vcol, bc_tab ? H.bc_kg : nullptr, H.fb.vt);
-      k_bem_apply<<<g.n / BEM64_ROWS, 64 * BEM64_ROWS, 0, s>>>(g.n, nrhs, dl ? H.Kdl_inv : (trans ? H.SinvT : H.Sinv), H.fb.vt, H.fb.q);
+      k_bem_vt<<<nblk((int64_t)nrhs * g.n / 2), 256, 0, s>>>(g.n, nrhs, H.fb.vcol, bc_tab ? H.bc_kg : nullptr, H.fb.vt);
+      k_bem_apply<<<nblk(g.n / 2, BEM64_ROWS), 64 * BEM64_ROWS, 0, s>>>(g.n, nrhs, dl ? H.Kdl_inv : (trans ? H.SinvT : H.Sinv), H.fb.vt, H.fb.q);
       launches += 2;
     }
     FMMPC_LAUNCH_CHECK();
@@ -2048,9 +2372,14 @@ void apply_impl(fmmpc_handle &H, int part, const double *r, double *out, int nrh
     ++launches;
   }
   auto run_vbv_sep = [&]() {
-    k_m2l_vbv<R, P><<<nblk(Ls.n_vbv_cells * nrhs * 8), 256, 0, s>>>(gd, g.ncell, g.nbcell, nrhs, Ls.vbv_first,
-                                                                     Ls.vbv_src, Mb, Lv, Ls.vbv_cells,
-                                                                     Ls.n_vbv_cells, (cpx<R> *)H.fb.Lvb);
+    if constexpr (f64)
+      k_m2l_vbv<R, P><<<nblk(Ls.n_vbv_cells * nrhs * 8), 256, 0, s>>>(gd, g.ncell, g.nbcell, nrhs, Ls.vbv_first,
+                                                                       Ls.vbv_src, Mb, Ls.vbv_cells, Ls.n_vbv_cells,
+                                                                       (cpx<R> *)H.fb.Lvb);
+    else
+      k_m2l_vbv_half<P><<<nblk(Ls.n_vbv_cells * nrhs * 16), 256, 0, s>>>(gd, g.nbcell, nrhs, Ls.vbv_first, Ls.vbv_src, Mb,
+                                                                        Ls.vbv_cells, Ls.n_vbv_cells,
+                                                                        (cpx<R> *)H.fb.Lvb);
     FMMPC_LAUNCH_CHECK();
     ++launches;
   };

@@ -1,6 +1,6 @@
 """Kernels and dispatch rules at the sizes where they can go wrong, each against the oracle or
 the general path: window edges of the Q1 mass solve, tables formed on first use, the FP64 form's
-tensor-core kernels, and alignment."""
+tensor-core kernels, the smallest folded boundary blocks, and alignment."""
 import numpy as np
 import pytest
 
@@ -132,6 +132,29 @@ def test_fp64_tensor_core_m2l_matches_oracle(p, leaf_max):
     R = O.Problem(n, p=p, leaf_max=leaf_max)
     for k in range(2):
         check_close(f"fp64 vr p={p} leaf={leaf_max} rhs={k}", vr[k], R.apply(f[k], "fmm", stages=True)["vr"], 1e-12, 1e-12)
+    P.close()
+
+
+@pytest.mark.parametrize("n,prec,nrhs", [(8, "fp32", 1), (16, "fp32", 3), (32, "fp64", 2), (64, "mixed_tf32", 5)])
+def test_folded_boundary_solve_matches_oracle(n, prec, nrhs):
+    # the smallest folded blocks (two rows; one 16-byte column), several right-hand sides: q, its
+    # transpose pass and the boundary-data solve against the oracle, at the bars of the stage,
+    # transpose and boundary tests
+    from paper_1308_3339_gb300 import FmmPreconditioner
+    leaf_max = 16
+    f = np.stack([S.random_field(n, 30 + k) for k in range(nrhs)])
+    g = np.stack([S.random_field(n, 50 + k)[:4 * n] for k in range(nrhs)]) if n >= 4 else None
+    P = FmmPreconditioner(n, p=10, leaf_max=leaf_max, precision=prec, n_rhs=nrhs)
+    R = O.Problem(n, p=10, leaf_max=leaf_max)
+    q = P.apply_part("q", dev(f)).cpu().numpy()
+    rb = P.apply_transpose(dev(f)).cpu().numpy()
+    u = P.apply_bc(dev(f), dev(g)).cpu().numpy()
+    tol = {"fp64": 1e-12, "fp32": 1e-5, "mixed_tf32": 3e-5}[prec]
+    gate = {"fp64": 1e-7, "fp32": 1e-5, "mixed_tf32": 3e-5}[prec]
+    for k in range(nrhs):
+        check_close(f"q {prec} n={n}", q[k], R.apply(f[k], "fmm", stages=True)["q"], 10 * tol, 10 * tol)
+        check_close(f"transpose {prec} n={n}", rb[k].ravel(), R.apply_transpose(f[k], "fmm"), gate, gate)
+        check_close(f"apply_bc {prec} n={n}", u[k].ravel(), R.apply_bc(f[k], g[k], "fmm"), 10 * gate, 10 * gate)
     P.close()
 
 
