@@ -35,6 +35,40 @@ int red_blocks(int64_t N) {
   return (int)std::max<int64_t>(1, std::min<int64_t>({4 * (int64_t)nsm, fill, RED_BLOCKS}));
 }
 
+// The same for the kernels of the graph solves, as (blocks, threads): two blocks per SM at most, and small
+// blocks where a grid has few pairs.  The sweeps are bound by FP64 issue (2 a clock and SM: 7.2 us per
+// operation and point at 2048^2), so every SM has to take part, and each block ends with a
+// reduction of FP64 adds and an arrival, which 608 blocks of 256 threads paid twice over
+// (second sweep over three vectors of 1024^2: 23.5 -> 18.7 us).
+dim3 sweep_grid(int64_t N, int nrhs, int &threads) {
+  int dev = 0, nsm = 0;
+  FMMPC_CUDA(cudaGetDevice(&dev));
+  FMMPC_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
+  for (threads = 64; threads < RED_THREADS && N / 2 > 2 * (int64_t)nsm * threads; threads *= 2) {}
+  const int64_t fill = (N / 2 + threads - 1) / threads;
+  return dim3((unsigned)std::max<int64_t>(1, std::min<int64_t>({2 * (int64_t)nsm, fill, RED_BLOCKS})), (unsigned)nrhs);
+}
+
+// f(k, count) over the grid's strided element pairs, U at a time (their loads go out together), then
+// the remainder one by one
+template <int U, typename F>
+__device__ __forceinline__ void pair_sweep(int64_t N2, F &&f) {
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if constexpr (U > 1) {
+    for (; k + (U - 1) * stride < N2; k += U * stride) {
+      int64_t kk[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) kk[u] = k + u * stride;
+      f(kk, std::integral_constant<int, U>{});
+    }
+  }
+  for (; k < N2; k += stride) {
+    int64_t kk[1] = {k};
+    f(kk, std::integral_constant<int, 1>{});
+  }
+}
+
 // f(integral_constant<int, k>) for a block-uniform k in [1, 8]: the FP64 loops over a group of
 // vectors are compiled for each count.  (As one loop of eight predicated steps, the multiply-adds of
 // absent vectors still took the FP64 pipe: the norm of one 1024^2 vector 19.8 us.)
@@ -516,6 +550,8 @@ struct Ctx {
   cudaStream_t s;
 };
 
+constexpr int GM_CTL = 16;  // control words of a graph solve
+
 void ensure_ws(fmmpc_handle &H, int64_t nvec, bool flexible) {
   KrylovWs &k = H.kw;
   const int64_t N = (int64_t)H.g.n * H.g.n * H.nrhs_max;
@@ -537,19 +573,20 @@ void ensure_ws(fmmpc_handle &H, int64_t nvec, bool flexible) {
   k.zin = H.kpool.get<double>(N);
   k.gin = H.kpool.get<double>((size_t)4 * H.g.n * H.nrhs_max);
   const int nr = H.nrhs_max;
-  k.g_ctl = H.kpool.get<int>(16);
+  // rtol, control words, relative residuals and iteration counts side by side: one copy in, one out
+  k.g_rtol = H.kpool.get<double>((size_t)1 + GM_CTL / 2 + nr + (nr + 1) / 2);
+  k.g_ctl = reinterpret_cast<int *>(k.g_rtol + 1);
+  k.g_rel = k.g_rtol + 1 + GM_CTL / 2;
+  k.g_iters = reinterpret_cast<int *>(k.g_rel + nr);
   k.g_done = H.kpool.get<int>(nr);
-  k.g_iters = H.kpool.get<int>(nr);
   k.g_H = H.kpool.get<double>((size_t)nr * (MAXJ + 1) * MAXJ);
   k.g_cs = H.kpool.get<double>((size_t)nr * MAXJ);
   k.g_sn = H.kpool.get<double>((size_t)nr * MAXJ);
   k.g_g = H.kpool.get<double>((size_t)nr * (MAXJ + 1));
   k.g_bn = H.kpool.get<double>(nr);
-  k.g_rel = H.kpool.get<double>(nr);
   k.g_sc = H.kpool.get<double>(nr);
-  k.g_rtol = H.kpool.get<double>(1);
   k.g_cnt = H.kpool.get<int>(nr + 1);  // per right-hand side, then one over all of them
-  FMMPC_CUDA(cudaMemsetAsync(k.g_ctl, 0, sizeof(int) * 16, H.stream));
+  FMMPC_CUDA(cudaMemsetAsync(k.g_ctl, 0, sizeof(int) * GM_CTL, H.stream));
   FMMPC_CUDA(cudaMemsetAsync(k.g_cnt, 0, sizeof(int) * (nr + 1), H.stream));
   k.dots = H.kpool.get<double>((size_t)H.nrhs_max * MAXJ * 4);
   k.part = H.kpool.get<double>((size_t)H.nrhs_max * MAXJ * RED_BLOCKS);
@@ -1104,14 +1141,18 @@ __global__ void k_gmaxpy(const int *__restrict__ ctl, int64_t N, int nrhs, const
   x[t] = v;
 }
 
-// V_{ctl[KC_J]}[rhs] = sc[rhs] w[rhs], and the same into t2 (the next preconditioner input)
+// V_{ctl[KC_J]}[rhs] = sc[rhs] w[rhs], and the same into t2 (the next preconditioner input); START: the
+// first vector of a cycle, which opens the loop over the cycle's steps
+template <bool START>
 __global__ void k_gscale_col(const int *__restrict__ ctl, int64_t N, int nrhs, const double *__restrict__ sc,
-                             const double *__restrict__ w, double *__restrict__ V, int64_t vs, double *__restrict__ t2) {
+                             const double *__restrict__ w, double *__restrict__ V, int64_t vs, double *__restrict__ t2,
+                             cudaGraphConditionalHandle steps) {
   const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (START && t == 0) cudaGraphSetConditional(steps, 1u);
   if (t >= N * nrhs) return;
   const double v = sc[t >> (__ffsll(N) - 1)] * w[t];
-  V[(int64_t)ctl[KC_J] * vs + t] = v;
-  if (t2) t2[t] = v;
+  V[(START ? 0 : (int64_t)ctl[KC_J] * vs) + t] = v;
+  t2[t] = v;
 }
 
 // Last block of a reduction grid to arrive: returns true in every thread of that block
@@ -1162,20 +1203,29 @@ __global__ void __launch_bounds__(RED_THREADS) k_gapdots(const int *__restrict__
     const int nq = min(8, nv - i0);
     with_count8(nq, [&](auto nqc) {
       constexpr int NQ = nqc();
-      for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < N2; k += (int64_t)gridDim.x * blockDim.x) {
-        double2 v[NQ], wk, c;
+      pair_sweep<(NQ <= 4 ? 2 : 1)>(N2, [&](const auto &kk, auto uc) {
+        constexpr int U = uc();
+        double2 v[U][NQ], wk[U], c;
 #pragma unroll
-        for (int q = 0; q < NQ; ++q) v[q] = reinterpret_cast<const double2 *>(V + (int64_t)(i0 + q) * vs + base)[k];
-        if (i0 == 0) {
-          wk = op_pair(o, x, base, k, c);
-          w2[k] = wk;
-          if (z2) z2[k] = c;
-        } else {
-          wk = w2[k];
+        for (int u = 0; u < U; ++u) {
+#pragma unroll
+          for (int q = 0; q < NQ; ++q) v[u][q] = reinterpret_cast<const double2 *>(V + (int64_t)(i0 + q) * vs + base)[kk[u]];
         }
 #pragma unroll
-        for (int q = 0; q < NQ; ++q) acc[q] = fma(v[q].x, wk.x, fma(v[q].y, wk.y, acc[q]));
-      }
+        for (int u = 0; u < U; ++u) {
+          if (i0 == 0) {
+            wk[u] = op_pair(o, x, base, kk[u], c);
+            w2[kk[u]] = wk[u];
+            if (z2) z2[kk[u]] = c;
+          } else {
+            wk[u] = w2[kk[u]];
+          }
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+#pragma unroll
+          for (int q = 0; q < NQ; ++q) acc[q] = fma(v[u][q].x, wk[u].x, fma(v[u][q].y, wk[u].y, acc[q]));
+      });
     });
     block_sum8(acc, nq, red);
     if (threadIdx.x < nq) part[((int64_t)rhs * MAXJ + i0 + threadIdx.x) * gridDim.x + blockIdx.x] = red[threadIdx.x];
@@ -1206,22 +1256,30 @@ __global__ void __launch_bounds__(RED_THREADS) k_gupdots(const int *__restrict__
     const int nq = min(8, nv - i0);
     with_count8(nq, [&](auto nqc) {
       constexpr int NQ = nqc();
-      for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < N2; k += (int64_t)gridDim.x * blockDim.x) {
-        double2 v[NQ], wk = w2[k];
+      pair_sweep<(NQ <= 4 ? 2 : 1)>(N2, [&](const auto &kk, auto uc) {
+        constexpr int U = uc();
+        double2 v[U][NQ], wk[U];
 #pragma unroll
-        for (int q = 0; q < NQ; ++q) v[q] = reinterpret_cast<const double2 *>(V + (int64_t)(i0 + q) * vs + base)[k];
-        if (i0 == 0) {  // the update: this group's vectors from registers, then the others
+        for (int u = 0; u < U; ++u) {
+          wk[u] = w2[kk[u]];
 #pragma unroll
-          for (int q = 0; q < NQ; ++q) {
-            wk.x = fma(-cr[q], v[q].x, wk.x);
-            wk.y = fma(-cr[q], v[q].y, wk.y);
-          }
-          if (nv > NQ) update_pair(V + (int64_t)NQ * vs + base, vs, k, cr + NQ, nv - NQ, wk);
-          w2[k] = wk;
+          for (int q = 0; q < NQ; ++q) v[u][q] = reinterpret_cast<const double2 *>(V + (int64_t)(i0 + q) * vs + base)[kk[u]];
         }
 #pragma unroll
-        for (int q = 0; q < NQ; ++q) acc[q] = fma(v[q].x, wk.x, fma(v[q].y, wk.y, acc[q]));
-      }
+        for (int u = 0; u < U; ++u) {
+          if (i0 == 0) {  // the update: this group's vectors from registers, then the others
+#pragma unroll
+            for (int q = 0; q < NQ; ++q) {
+              wk[u].x = fma(-cr[q], v[u][q].x, wk[u].x);
+              wk[u].y = fma(-cr[q], v[u][q].y, wk[u].y);
+            }
+            if (nv > NQ) update_pair(V + (int64_t)NQ * vs + base, vs, kk[u], cr + NQ, nv - NQ, wk[u]);
+            w2[kk[u]] = wk[u];
+          }
+#pragma unroll
+          for (int q = 0; q < NQ; ++q) acc[q] = fma(v[u][q].x, wk[u].x, fma(v[u][q].y, wk[u].y, acc[q]));
+        }
+      });
     });
     block_sum8(acc, nq, red);
     if (threadIdx.x < nq) part[((int64_t)rhs * MAXJ + i0 + threadIdx.x) * gridDim.x + blockIdx.x] = red[threadIdx.x];
@@ -1245,48 +1303,59 @@ struct GmState {
   int *done, *iters;  // [nrhs]
 };
 
-__global__ void k_ginit(int *__restrict__ ctl, GmState st, int nrhs, const double *__restrict__ dots) {
-  const int r = threadIdx.x;
-  if (r < nrhs) {
-    const double b = sqrt(fmax(0.0, dots[r * MAXJ]));
-    st.bn[r] = b > 0.0 ? b : 1.0;
-    st.iters[r] = 0;
-    st.done[r] = 0;
-  }
-  if (r == 0) {
-    ctl[KC_J] = 0;
-    ctl[KC_IT] = 0;
-    ctl[KC_CYC] = 0;
-    ctl[KC_DONE] = 0;
-    ctl[KC_NAN] = 0;
-    ctl[KC_JCNT] = 0;
-  }
-}
-
-// Start of a cycle from the true residual r (|r|^2 in dots[rhs][0]): per right-hand side
-// done = |r| / |b| <= rtol, g = (|r|, 0, ...), scale 1/|r| of V_0 (0 when done); j = 0.
-__global__ void k_grestart(int *__restrict__ ctl, GmState st, int nrhs, const double *__restrict__ dots) {
+// Start of a cycle from the true residual r (|r|^2 in dots[rhs][0]): per right-hand side the
+// relative residual, done = |r| / |b| <= rtol, g = (|r|, 0, ...), scale 1/|r| of V_0 (0 when done);
+// j = 0; and the solve's loop goes on while some right-hand side is above rtol, no NaN was met
+// and fewer than maxit preconditioner applications ran.  Run by all threads of one block.
+__device__ __forceinline__ void gm_restart(int *__restrict__ ctl, GmState st, int nrhs, const double *__restrict__ dots,
+                                           cudaGraphConditionalHandle loop) {
   __shared__ int s_all, s_nan;
-  const int r = threadIdx.x;
-  if (r == 0) { s_all = 1; s_nan = 0; }
+  if (threadIdx.x == 0) { s_all = 1; s_nan = 0; }
   __syncthreads();
-  if (r < nrhs) {
-    const double beta = sqrt(fmax(0.0, dots[r * MAXJ]));
-    const double rtol = st.rtol[0];
-    if (!isfinite(beta) || !isfinite(dots[r * MAXJ])) atomicOr(&s_nan, 1);
-    const int d = (beta / st.bn[r] <= rtol) ? 1 : 0;
+  const double rtol = st.rtol[0];
+  for (int r = threadIdx.x; r < nrhs; r += blockDim.x) {
+    const double sq = __ldcg(dots + r * MAXJ), beta = sqrt(fmax(0.0, sq)), rel = beta / __ldcg(st.bn + r);
+    if (!isfinite(beta) || !isfinite(sq)) atomicOr(&s_nan, 1);
+    const int d = (rel <= rtol) ? 1 : 0;
+    st.rel[r] = rel;
     st.done[r] = d;
-    double *g = st.g + r * (MAXJ + 1);
-    for (int i = 0; i <= MAXJ; ++i) g[i] = 0.0;
-    g[0] = d ? 0.0 : beta;
     st.sc[r] = (d || beta == 0.0) ? 0.0 : 1.0 / beta;
+    st.g[r * (MAXJ + 1)] = d ? 0.0 : beta;  // the steps write g[j + 1] before they read it
     if (!d) atomicAnd(&s_all, 0);
   }
   __syncthreads();
-  if (r == 0) {
+  if (threadIdx.x == 0) {
+    const int nan = ctl[KC_NAN] | s_nan;
     ctl[KC_J] = 0;
     ctl[KC_DONE] = s_all;
-    ctl[KC_NAN] |= s_nan;
+    ctl[KC_NAN] = nan;
+    const int cont = (!s_all && !nan && ctl[KC_IT] < ctl[KC_MAXIT]) ? 1 : 0;
+    ctl[KC_CONT] = cont;
+    cudaGraphSetConditional(loop, (unsigned)cont);
+  }
+}
+
+// Start of CG from the true residual: done flags and the loop's condition.
+__device__ __forceinline__ void cg_start(int *__restrict__ ctl, GmState st, int nrhs, const double *__restrict__ dots,
+                                         cudaGraphConditionalHandle loop) {
+  __shared__ int s_all, s_nan;
+  if (threadIdx.x == 0) { s_all = 1; s_nan = 0; }
+  __syncthreads();
+  for (int r = threadIdx.x; r < nrhs; r += blockDim.x) {
+    const double sq = __ldcg(dots + r * MAXJ);
+    if (!isfinite(sq)) atomicOr(&s_nan, 1);  // fmax(0, NaN) would hide it
+    const int d = sqrt(fmax(0.0, sq)) / __ldcg(st.bn + r) <= st.rtol[0];
+    st.done[r] = d;
+    if (!d) atomicAnd(&s_all, 0);
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    const int nan = ctl[KC_NAN] | s_nan;
+    ctl[KC_DONE] = s_all;
+    ctl[KC_NAN] = nan;
+    const int cont = (!s_all && !nan && ctl[KC_IT] < ctl[KC_MAXIT]) ? 1 : 0;
+    ctl[KC_CONT] = cont;
+    cudaGraphSetConditional(loop, (unsigned)cont);
   }
 }
 
@@ -1294,13 +1363,13 @@ __global__ void k_grestart(int *__restrict__ ctl, GmState st, int nrhs, const do
 // |w| (wsq), the previous rotations, a new rotation, the residual estimate |g_{j+1}| / |b|,
 // the scale of V_{j+1}; the cycle ends when every right-hand side is within rtol (or has
 // a zero |w|), at j + 1 = m, at maxit, or on a NaN; then y from the triangular system.
-// Sets the condition of the end-of-cycle IF node.  Run by all threads of one block.
+// Sets the condition of the loop over the cycle's steps.  Run by all threads of one block.
 __device__ __forceinline__ void gtail_run(int *__restrict__ ctl, GmState st, int nrhs, int m,
                                           const double *__restrict__ hsum, const double *__restrict__ wsq,
-                                          double *__restrict__ y, cudaGraphConditionalHandle if_end) {
+                                          double *__restrict__ y, cudaGraphConditionalHandle steps) {
   __shared__ int s_ok, s_nan, s_cyc;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  const int j = ctl[KC_J], it = ctl[KC_IT] + 1;
+  const int j = ctl[KC_J], it = ctl[KC_IT] + 1, maxit = ctl[KC_MAXIT];
   if (threadIdx.x == 0) { s_ok = 1; s_nan = 0; }
   __syncthreads();
   // a warp per right-hand side: lane i holds entries i and i + 32 of the column and the rotations,
@@ -1308,6 +1377,8 @@ __device__ __forceinline__ void gtail_run(int *__restrict__ ctl, GmState st, int
   for (int r = wid; r < nrhs; r += nw) {
     double *Hr = st.Hm + (int64_t)r * (MAXJ + 1) * MAXJ;
     double *cs = st.cs + r * MAXJ, *sn = st.sn + r * MAXJ, *g = st.g + r * (MAXJ + 1);
+    const double gj = g[j], bn = st.bn[r], rtol = st.rtol[0];  // every load of the step goes out at once
+    const int done = st.done[r];
     double hv[2], cv[2], sv[2], rot[2] = {0.0, 0.0};
 #pragma unroll
     for (int q = 0; q < 2; ++q) {
@@ -1325,7 +1396,12 @@ __device__ __forceinline__ void gtail_run(int *__restrict__ ctl, GmState st, int
       a = -sn_i * a + c * b;
       if (lane == (i & 31)) rot[i >> 5] = hi;
     }
-    const double rr = hypot(a, hn), cj = rr == 0.0 ? 1.0 : a / rr, sj = rr == 0.0 ? 0.0 : hn / rr;
+    // the rotation; the three divisions (a / rr, hn / rr, 1 / hn) go out together, one per lane
+    const double big = fmax(fabs(a), hn);
+    const double rr = big > 1e-140 && big < 1e140 ? sqrt(fma(a, a, hn * hn)) : hypot(a, hn);
+    const double quo = (lane == 0 ? a : (lane == 1 ? hn : 1.0)) / (lane == 2 ? hn : rr);
+    const double qa = __shfl_sync(0xffffffffu, quo, 0), qh = __shfl_sync(0xffffffffu, quo, 1);
+    const double cj = rr == 0.0 ? 1.0 : qa, sj = rr == 0.0 ? 0.0 : qh, inv_hn = __shfl_sync(0xffffffffu, quo, 2);
 #pragma unroll
     for (int q = 0; q < 2; ++q)
       if (lane + 32 * q < j) Hr[(lane + 32 * q) * MAXJ + j] = rot[q];
@@ -1334,28 +1410,26 @@ __device__ __forceinline__ void gtail_run(int *__restrict__ ctl, GmState st, int
       Hr[(j + 1) * MAXJ + j] = 0.0;
       cs[j] = cj;
       sn[j] = sj;
-      const double gj = g[j];
       g[j + 1] = -sj * gj;
       g[j] = cj * gj;
-      const double est = fabs(sj * gj) / st.bn[r];
+      const double est = fabs(sj * gj) / bn;
       if (!isfinite(est)) atomicOr(&s_nan, 1);
-      const int done = st.done[r];
       if (!done) st.iters[r] = it;
-      const bool ok = done || est <= st.rtol[0] || hn == 0.0;
+      const bool ok = done || est <= rtol || hn == 0.0;
       if (!ok) atomicAnd(&s_ok, 0);
-      st.sc[r] = (hn > 0.0 && !done) ? 1.0 / hn : 0.0;
+      st.sc[r] = (hn > 0.0 && !done) ? inv_hn : 0.0;
     }
   }
   __syncthreads();
   if (threadIdx.x == 0) {
-    const int cyc = (s_ok || s_nan || j + 1 >= m || it >= ctl[KC_MAXIT]) ? 1 : 0;
+    const int cyc = (s_ok || s_nan || j + 1 >= m || it >= maxit) ? 1 : 0;
     s_cyc = cyc;
     ctl[KC_IT] = it;
     ctl[KC_CYC] = cyc;
     ctl[KC_JCNT] = j + 1;
     ctl[KC_J] = j + 1;
     ctl[KC_NAN] |= s_nan;
-    cudaGraphSetConditional(if_end, (unsigned)cyc);
+    cudaGraphSetConditional(steps, (unsigned)!cyc);
   }
   __syncthreads();
   if (!s_cyc) return;
@@ -1393,20 +1467,46 @@ __global__ void __launch_bounds__(RED_THREADS) k_gupdate_tail(int *__restrict__ 
                                                               double *__restrict__ w, double *__restrict__ part,
                                                               int *__restrict__ cnt, double *__restrict__ wsq, GmState st,
                                                               int nrhs, int m, const double *__restrict__ hsum,
-                                                              double *__restrict__ y, cudaGraphConditionalHandle if_end) {
+                                                              double *__restrict__ y, cudaGraphConditionalHandle steps) {
   __shared__ double red[RED_THREADS / 32];
   __shared__ int s_fin;
   const int rhs = blockIdx.y;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int nv = ctl[KC_J] + 1;
-  double sq = update_chunk(N, V + (int64_t)rhs * N, vs, c + rhs * MAXJ, nv, w + (int64_t)rhs * N);
+  const double *Vr = V + (int64_t)rhs * N, *cr = c + rhs * MAXJ;
+  double2 *w2 = reinterpret_cast<double2 *>(w + (int64_t)rhs * N);
+  double sq = 0.0;
+  with_count8(min(8, nv), [&](auto nqc) {
+    constexpr int NQ = nqc();
+    pair_sweep<(NQ <= 4 ? 2 : 1)>(N >> 1, [&](const auto &kk, auto uc) {
+      constexpr int U = uc();
+      double2 v[U][NQ], wk[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        wk[u] = w2[kk[u]];
+#pragma unroll
+        for (int q = 0; q < NQ; ++q) v[u][q] = reinterpret_cast<const double2 *>(Vr + (int64_t)q * vs)[kk[u]];
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+#pragma unroll
+        for (int q = 0; q < NQ; ++q) {
+          wk[u].x = fma(-cr[q], v[u][q].x, wk[u].x);
+          wk[u].y = fma(-cr[q], v[u][q].y, wk[u].y);
+        }
+        if (nv > NQ) update_pair(Vr + (int64_t)NQ * vs, vs, kk[u], cr + NQ, nv - NQ, wk[u]);
+        w2[kk[u]] = wk[u];
+        sq = fma(wk[u].x, wk[u].x, fma(wk[u].y, wk[u].y, sq));
+      }
+    });
+  });
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
   if (lane == 0) red[wid] = sq;
   __syncthreads();
   if (threadIdx.x == 0) {
     double t = 0.0;
-    for (int q = 0; q < RED_THREADS / 32; ++q) t += red[q];
+    for (int q = 0; q < (int)(blockDim.x >> 5); ++q) t += red[q];
     part[(int64_t)rhs * MAXJ * gridDim.x + blockIdx.x] = t;
   }
   if (!last_block(cnt + rhs)) return;
@@ -1414,51 +1514,20 @@ __global__ void __launch_bounds__(RED_THREADS) k_gupdate_tail(int *__restrict__ 
   __syncthreads();
   if (threadIdx.x == 0) {
     cnt[rhs] = 0;
-    __threadfence();
-    s_fin = atomicAdd(cnt + nrhs, 1) == nrhs - 1;
-    if (s_fin) cnt[nrhs] = 0;
+    s_fin = 1;
+    if (nrhs > 1) {
+      __threadfence();
+      s_fin = atomicAdd(cnt + nrhs, 1) == nrhs - 1;
+      if (s_fin) cnt[nrhs] = 0;
+    }
   }
   __syncthreads();
   if (!s_fin) return;
   __threadfence();
-  gtail_run(ctl, st, nrhs, m, hsum, wsq, y, if_end);
+  gtail_run(ctl, st, nrhs, m, hsum, wsq, y, steps);
 }
 
-// Condition of the loop: continue while some right-hand side is above rtol, no NaN was met
-// and fewer than maxit preconditioner applications ran.
-__global__ void k_gcond(int *__restrict__ ctl, cudaGraphConditionalHandle loop) {
-  const int cont = (!ctl[KC_DONE] && !ctl[KC_NAN] && ctl[KC_IT] < ctl[KC_MAXIT]) ? 1 : 0;
-  ctl[KC_CONT] = cont;
-  cudaGraphSetConditional(loop, (unsigned)cont);
-}
-
-// Final report: true relative residual per right-hand side.
-__global__ void k_gfinal(GmState st, int nrhs, const double *__restrict__ dots) {
-  const int r = threadIdx.x;
-  if (r < nrhs) st.rel[r] = sqrt(fmax(0.0, dots[r * MAXJ])) / st.bn[r];
-}
-
-// ---- CG (Sec. 3.1) with per-right-hand-side masks: the iteration's kernels are the fused
-// k_cgf_* below
-__global__ void k_cg_init(int *__restrict__ ctl, GmState st, int nrhs, const double *__restrict__ dots) {
-  const int r = threadIdx.x;
-  __shared__ int s_all, s_nan;
-  if (r == 0) { s_all = 1; s_nan = 0; }
-  __syncthreads();
-  if (r < nrhs) {
-    const double rn = sqrt(fmax(0.0, dots[r * MAXJ]));
-    if (!isfinite(dots[r * MAXJ])) atomicOr(&s_nan, 1);  // fmax(0, NaN) would hide it
-    const int d = rn / st.bn[r] <= st.rtol[0];
-    st.done[r] = d;
-    if (!d) atomicAnd(&s_all, 0);
-  }
-  __syncthreads();
-  if (r == 0) {
-    ctl[KC_DONE] = s_all;
-    ctl[KC_NAN] |= s_nan;
-  }
-}
-
+// ---- CG (Sec. 3.1) with per-right-hand-side masks
 // ---- fused CG steps: each vector pass carries its inner product, finished in the grid's last
 // block per right-hand side (a fixed order of block partials), which also takes the scalar
 // step that follows, so one CG iteration is four vector kernels and the preconditioner.
@@ -1485,16 +1554,44 @@ __device__ __forceinline__ bool block_partial_last(double v, double *__restrict_
   return true;
 }
 
+// |b| of every right-hand side (1 where b = 0), counts and control words cleared: norm, its
+// reduction and the initial state in one launch.
+__global__ void __launch_bounds__(RED_THREADS) k_gbnorm(int *__restrict__ ctl, int64_t N, GmState st,
+                                                      const double *__restrict__ b, double *__restrict__ part, int *cnt) {
+  const int rhs = blockIdx.y;
+  const double2 *b2 = reinterpret_cast<const double2 *>(b + (int64_t)rhs * N);
+  double acc = 0.0;
+#pragma unroll 4
+  for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < N >> 1; k += (int64_t)gridDim.x * blockDim.x) {
+    const double2 v = b2[k];
+    acc = fma(v.x, v.x, fma(v.y, v.y, acc));
+  }
+  double tot;
+  if (!block_partial_last(acc, part, rhs, cnt, tot) || threadIdx.x != 0) return;
+  const double nb = sqrt(fmax(0.0, tot));
+  st.bn[rhs] = nb > 0.0 ? nb : 1.0;
+  st.iters[rhs] = 0;
+  st.done[rhs] = 0;
+  if (rhs == 0) {
+    ctl[KC_J] = ctl[KC_IT] = ctl[KC_CYC] = ctl[KC_DONE] = ctl[KC_NAN] = ctl[KC_JCNT] = 0;
+  }
+}
+
 // r = b - A x with |r|^2 in dots[rhs][0]: one pass for the residual checks of the graph solves
-// (operator, subtraction and norm were three launches, 36 us at 1024^2).
-__global__ void __launch_bounds__(RED_THREADS) k_gresid(OpDev o, int64_t N, const double *__restrict__ b,
-                                                      const double *__restrict__ x, double *__restrict__ r,
-                                                      double *__restrict__ part, int *cnt, double *__restrict__ dots) {
+// (operator, subtraction and norm were three launches, 36 us at 1024^2); the last right-hand side to
+// finish then takes the scalar step that follows: a cycle's start, CG's start, or the final report.
+enum class AfterResid { CYCLE, CG_START, REPORT };
+template <AfterResid WHAT>
+__global__ void __launch_bounds__(RED_THREADS) k_gresid(int *__restrict__ ctl, OpDev o, int64_t N, int nrhs, GmState st,
+                                                      const double *__restrict__ b, const double *__restrict__ x,
+                                                      double *__restrict__ r, double *__restrict__ part, int *cnt,
+                                                      double *__restrict__ dots, cudaGraphConditionalHandle loop) {
   const int rhs = blockIdx.y;
   const int64_t base = (int64_t)rhs * N;
   const double2 *b2 = reinterpret_cast<const double2 *>(b + base);
   double2 *r2 = reinterpret_cast<double2 *>(r + base);
   double acc = 0.0;
+#pragma unroll 2
   for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < N >> 1; k += (int64_t)gridDim.x * blockDim.x) {
     double2 c;
     const double2 bk = b2[k], a = op_pair(o, x, base, k, c);
@@ -1503,7 +1600,23 @@ __global__ void __launch_bounds__(RED_THREADS) k_gresid(OpDev o, int64_t N, cons
     acc = fma(v.x, v.x, fma(v.y, v.y, acc));
   }
   double tot;
-  if (block_partial_last(acc, part, rhs, cnt, tot) && threadIdx.x == 0) dots[rhs * MAXJ] = tot;
+  if (!block_partial_last(acc, part, rhs, cnt, tot)) return;
+  if constexpr (WHAT == AfterResid::REPORT) {
+    if (threadIdx.x == 0) st.rel[rhs] = sqrt(fmax(0.0, tot)) / st.bn[rhs];
+  } else {
+    __shared__ int s_fin;
+    if (threadIdx.x == 0) {
+      dots[rhs * MAXJ] = tot;
+      __threadfence();
+      s_fin = atomicAdd(cnt + nrhs, 1) == nrhs - 1;
+      if (s_fin) cnt[nrhs] = 0;
+    }
+    __syncthreads();
+    if (!s_fin) return;
+    __threadfence();
+    if constexpr (WHAT == AfterResid::CYCLE) gm_restart(ctl, st, nrhs, dots, loop);
+    else cg_start(ctl, st, nrhs, dots, loop);
+  }
 }
 
 // q = A p and <p, q>; then alpha = <r, z> / <p, q> (0 for a finished right-hand side)
@@ -1514,6 +1627,7 @@ __global__ void __launch_bounds__(RED_THREADS) k_cgf_apdot(OpDev o, int64_t N, G
   const int64_t base = (int64_t)rhs * N;
   double2 *q2 = reinterpret_cast<double2 *>(q + base);
   double acc = 0.0;
+#pragma unroll 2
   for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < N >> 1; k += (int64_t)gridDim.x * blockDim.x) {
     double2 c;
     const double2 v = op_pair(o, p, base, k, c);
@@ -1659,16 +1773,11 @@ GmState gm_state(KrylovWs &K) {
   return GmState{K.g_H, K.g_cs, K.g_sn, K.g_g, K.g_bn, K.g_rel, K.g_sc, K.g_rtol, K.g_done, K.g_iters};
 }
 
-// norms |v[rhs]|^2 into dots[rhs][0] (captured)
-void gnorm2(Ctx &c, const double *v) {
-  const int nb = red_blocks(c.N);
-  k_mdot_partial<<<dim3(nb, c.nrhs), RED_THREADS, 0, c.H.stream>>>(c.N, 1, v, 0, v, c.H.kw.part, 0);
-  k_mdot_final<<<dim3(c.nrhs, 1), 256, 0, c.H.stream>>>(1, nb, c.H.kw.part, c.H.kw.dots, nullptr, 0);
-  FMMPC_LAUNCH_CHECK();
-}
-
-// Builds one problem's chain [set-up] -> WHILE [step (-> IF cycle end)] -> [final] into
-// graph G.  Solves A u = b for the handle's internal vectors: b is folded from K.fin
+// Builds one problem's chain [set-up] -> WHILE [step] -> [final] (CG), or [set-up] -> WHILE cycle
+// [V_0 -> WHILE [step] -> cycle end] ((F)GMRES: the last cycle's end is the final residual) into
+// graph G.  Every condition is set by the last block of the kernel that decides it: an IF node for the
+// cycle's end and a kernel for the condition in every pass were 2.5 to 10 us of it (64^2 FGMRES, with
+// the copies of solve_graphed, 983 -> 916 us).  Solves A u = b for the handle's internal vectors: b is folded from K.fin
 // (and K.gin), the iterate is K.x.
 void build_chain(fmmpc_handle &H, cudaGraph_t G, int method, int m, int nrhs, bool has_g) {
   KrylovWs &K = H.kw;
@@ -1690,39 +1799,34 @@ void build_chain(fmmpc_handle &H, cudaGraph_t G, int method, int m, int nrhs, bo
   auto precond = [&](const double *in, double *out, double *scratch) {
     precond_op(H, in, out, scratch, nrhs, true);
   };
-  const dim3 rgrid((unsigned)red_blocks(N), nrhs);
-  auto residual_norm = [&]() {  // r = b - A x and |r|^2 into dots[rhs][0]
-    k_gresid<<<rgrid, RED_THREADS, 0, H.stream>>>(od, N, K.b, K.x, K.r, K.part, K.g_cnt, K.dots);
+  int rth = 0;
+  const dim3 rgrid = sweep_grid(N, nrhs, rth);
+  auto residual = [&](auto what) {  // r = b - A x and |r|^2, with what follows from it
+    k_gresid<what()><<<rgrid, rth, 0, H.stream>>>(ctl, od, N, nrhs, st, K.b, K.x, K.r, K.part, K.g_cnt, K.dots,
+                                                          hloop);
     FMMPC_LAUNCH_CHECK();
   };
+  using Cycle = std::integral_constant<AfterResid, AfterResid::CYCLE>;
   // ---- set-up
   const std::vector<cudaGraphNode_t> none;
   auto f_init = capture_into(H, cs, G, none, [&] {
     c.s = H.stream;
     k_fold_rhs<<<nblk(NR), 256, 0, H.stream>>>(od, NR, K.fin, has_g ? K.gin : nullptr, K.b);
-    gnorm2(c, K.b);
-    k_ginit<<<1, 64, 0, H.stream>>>(ctl, st, nrhs, K.dots);
-    residual_norm();
+    k_gbnorm<<<rgrid, rth, 0, H.stream>>>(ctl, N, st, K.b, K.part, K.g_cnt);
+    FMMPC_LAUNCH_CHECK();
     if (method == FMMPC_CG) {
       // the loop body starts with z = P^{-1} r; p = 0 and <r, z>_old = 0 make its first
       // beta 0, so that p = z
-      k_cg_init<<<1, 64, 0, H.stream>>>(ctl, st, nrhs, K.dots);
+      residual(std::integral_constant<AfterResid, AfterResid::CG_START>{});
       FMMPC_CUDA(cudaMemsetAsync(K.V, 0, sizeof(double) * NR, H.stream));
       FMMPC_CUDA(cudaMemsetAsync(K.dots + (size_t)nrhs * MAXJ, 0, sizeof(double) * nrhs * MAXJ, H.stream));
     } else {
-      k_grestart<<<1, 64, 0, H.stream>>>(ctl, st, nrhs, K.dots);
-      k_gscale_col<<<nblk(NR), 256, 0, H.stream>>>(ctl, N, nrhs, K.g_sc, K.r, K.V, vs, K.t);
+      residual(Cycle{});
     }
-    k_gcond<<<1, 1, 0, H.stream>>>(ctl, hloop);
-    FMMPC_LAUNCH_CHECK();
   });
   cudaGraph_t body = nullptr;
   cudaGraphNode_t n_loop = add_conditional(G, f_init, hloop, cudaGraphCondTypeWhile, &body);
-  cudaGraphConditionalHandle hif{};
-  if (method != FMMPC_CG) FMMPC_CUDA(cudaGraphConditionalHandleCreate(&hif, body, 0, 0));
   double *hsum = K.dots + (size_t)nrhs * MAXJ, *wsq = K.scal + (size_t)nrhs * MAXJ;
-  std::vector<cudaGraphNode_t> f_step;
-  cudaGraph_t ifb = nullptr;
   if (method == FMMPC_CG) {
     // p in V_0, q in t, z in w; <r, z> of the last iteration in the second dots block
     double *p = K.V, *q = K.t, *z = K.w, *rz_old = K.dots + (size_t)nrhs * MAXJ;
@@ -1730,34 +1834,46 @@ void build_chain(fmmpc_handle &H, cudaGraph_t G, int method, int m, int nrhs, bo
     // one iteration, rotated so that the convergence test ends it and sets the loop's own
     // condition (no IF node): z = P^{-1} r, beta, p = z + beta p, q = A p with alpha, then
     // x, r and the test
-    f_step = capture_into(H, cs, body, none, [&] {
+    capture_into(H, cs, body, none, [&] {
       c.s = H.stream;
       precond(K.r, z, K.zin);
-      k_cgf_rz<<<rgrid, RED_THREADS, 0, H.stream>>>(N, st, K.r, z, K.part, K.g_cnt, rz_old);
+      k_cgf_rz<<<rgrid, rth, 0, H.stream>>>(N, st, K.r, z, K.part, K.g_cnt, rz_old);
       k_cg_p<<<nblk(NR), 256, 0, H.stream>>>(N, nrhs, K.g_sc, z, p);
-      k_cgf_apdot<<<rgrid, RED_THREADS, 0, H.stream>>>(od, N, st, p, q, K.part, K.g_cnt, pq, rz_old);
-      k_cgf_xr<<<rgrid, RED_THREADS, 0, H.stream>>>(ctl, N, nrhs, st, p, q, K.x, K.r, K.part, K.g_cnt, K.dots,
+      k_cgf_apdot<<<rgrid, rth, 0, H.stream>>>(od, N, st, p, q, K.part, K.g_cnt, pq, rz_old);
+      k_cgf_xr<<<rgrid, rth, 0, H.stream>>>(ctl, N, nrhs, st, p, q, K.x, K.r, K.part, K.g_cnt, K.dots,
                                                      hloop);
       FMMPC_LAUNCH_CHECK();
     });
+    // the recurrence's residual drifts from the true one
+    capture_into(H, cs, G, {n_loop}, [&] {
+      c.s = H.stream;
+      residual(std::integral_constant<AfterResid, AfterResid::REPORT>{});
+    });
   } else {
-    f_step = capture_into(H, cs, body, none, [&] {
+    cudaGraphConditionalHandle hsteps;
+    FMMPC_CUDA(cudaGraphConditionalHandleCreate(&hsteps, body, 0, 0));
+    auto f_begin = capture_into(H, cs, body, none, [&] {
+      k_gscale_col<true><<<nblk(NR), 256, 0, H.stream>>>(ctl, N, nrhs, K.g_sc, K.r, K.V, vs, K.t, hsteps);
+      FMMPC_LAUNCH_CHECK();
+    });
+    cudaGraph_t step = nullptr;
+    cudaGraphNode_t n_steps = add_conditional(body, f_begin, hsteps, cudaGraphCondTypeWhile, &step);
+    capture_into(H, cs, step, none, [&] {
       c.s = H.stream;
       precond(K.t, K.zin, K.t);  // K.t holds v_j (written with V_j by the previous step)
       // w = A z_j with the first CGS pass, the first update with the second pass, the second
       // update with |w|^2: three sweeps over the basis, each reduction finished in its grid's
       // last block (a grid of a few blocks per SM keeps enough loads in flight)
       double *d2 = K.dots + (size_t)2 * nrhs * MAXJ;
-      k_gapdots<<<rgrid, RED_THREADS, 0, H.stream>>>(ctl, od, N, K.zin, K.w, flexible ? K.Z : nullptr, K.V, vs,
+      k_gapdots<<<rgrid, rth, 0, H.stream>>>(ctl, od, N, K.zin, K.w, flexible ? K.Z : nullptr, K.V, vs,
                                                      K.part, K.g_cnt, K.dots, hsum);
-      k_gupdots<<<rgrid, RED_THREADS, 0, H.stream>>>(ctl, N, K.V, vs, K.dots, K.w, K.part, K.g_cnt, d2, hsum);
-      k_gupdate_tail<<<rgrid, RED_THREADS, 0, H.stream>>>(ctl, N, K.V, vs, d2, K.w, K.part, K.g_cnt, wsq, st, nrhs, m,
-                                                            hsum, K.scal, hif);
-      k_gscale_col<<<nblk(NR), 256, 0, H.stream>>>(ctl, N, nrhs, K.g_sc, K.w, K.V, vs, K.t);
+      k_gupdots<<<rgrid, rth, 0, H.stream>>>(ctl, N, K.V, vs, K.dots, K.w, K.part, K.g_cnt, d2, hsum);
+      k_gupdate_tail<<<rgrid, rth, 0, H.stream>>>(ctl, N, K.V, vs, d2, K.w, K.part, K.g_cnt, wsq, st, nrhs, m,
+                                                            hsum, K.scal, hsteps);
+      k_gscale_col<false><<<nblk(NR), 256, 0, H.stream>>>(ctl, N, nrhs, K.g_sc, K.w, K.V, vs, K.t, hsteps);
       FMMPC_LAUNCH_CHECK();
     });
-    cudaGraphNode_t n_if = add_conditional(body, f_step, hif, cudaGraphCondTypeIf, &ifb);
-    capture_into(H, cs, ifb, none, [&] {
+    capture_into(H, cs, body, {n_steps}, [&] {
       c.s = H.stream;
       if (flexible) {
         k_gmaxpy<<<nblk(NR), 256, 0, H.stream>>>(ctl, N, nrhs, K.Z, vs, K.scal, K.x);
@@ -1767,23 +1883,9 @@ void build_chain(fmmpc_handle &H, cudaGraph_t G, int method, int m, int nrhs, bo
         precond(K.t, K.w, K.t);
         k_add<<<nblk(NR), 256, 0, H.stream>>>(NR, K.w, K.x);
       }
-      residual_norm();
-      k_grestart<<<1, 64, 0, H.stream>>>(ctl, st, nrhs, K.dots);
-      k_gscale_col<<<nblk(NR), 256, 0, H.stream>>>(ctl, N, nrhs, K.g_sc, K.r, K.V, vs, K.t);
-      FMMPC_LAUNCH_CHECK();
-    });
-    capture_into(H, cs, body, {n_if}, [&] {
-      k_gcond<<<1, 1, 0, H.stream>>>(ctl, hloop);
-      FMMPC_LAUNCH_CHECK();
+      residual(Cycle{});
     });
   }
-  // ---- final: the true residual
-  capture_into(H, cs, G, {n_loop}, [&] {
-    c.s = H.stream;
-    residual_norm();
-    k_gfinal<<<1, 64, 0, H.stream>>>(st, nrhs, K.dots);
-    FMMPC_LAUNCH_CHECK();
-  });
 }
 
 }  // namespace
@@ -1824,6 +1926,27 @@ cudaGraphExec_t solve_graph(std::vector<fmmpc_handle *> &hs, int method, int m, 
   return e.exec;
 }
 
+// The limits of a solve into the handle's control words, and its report (control words, relative
+// residuals, iteration counts) back into pinned memory: one copy each (every small copy is ~6 us of
+// a solve's start or end).
+void send_solve_limits(KrylovWs &K, const fmmpc_solve_opts &o, cudaStream_t s) {
+  int *hc = reinterpret_cast<int *>(K.hbuf + 1);
+  K.hbuf[0] = o.rtol;
+  for (int i = 0; i < GM_CTL; ++i) hc[i] = 0;
+  hc[KC_MAXIT] = o.maxit;
+  FMMPC_CUDA(cudaMemcpyAsync(K.g_rtol, K.hbuf, sizeof(double) * (1 + GM_CTL / 2), cudaMemcpyHostToDevice, s));
+}
+
+void fetch_solve_report(fmmpc_handle &H, cudaStream_t s, const int *&ctl, const double *&rel, const int *&iters) {
+  KrylovWs &K = H.kw;
+  const int nr = H.nrhs_max;
+  double *out = K.hbuf + 16;
+  FMMPC_CUDA(cudaMemcpyAsync(out, K.g_ctl, sizeof(double) * (GM_CTL / 2 + nr) + sizeof(int) * nr, cudaMemcpyDeviceToHost, s));
+  ctl = reinterpret_cast<const int *>(out);
+  rel = out + GM_CTL / 2;
+  iters = reinterpret_cast<const int *>(rel + nr);
+}
+
 // Solve through the graph: inputs copied into the handle's vectors, one launch, the report
 // read back once.
 int solve_graphed(fmmpc_handle &H, const double *f, const double *g, double *u, int nrhs, const fmmpc_solve_opts &o,
@@ -1837,19 +1960,12 @@ int solve_graphed(fmmpc_handle &H, const double *f, const double *g, double *u, 
   FMMPC_CUDA(cudaMemcpyAsync(K.fin, f, sizeof(double) * NR, cudaMemcpyDeviceToDevice, s));
   if (g) FMMPC_CUDA(cudaMemcpyAsync(K.gin, g, sizeof(double) * 4 * H.g.n * nrhs, cudaMemcpyDeviceToDevice, s));
   FMMPC_CUDA(cudaMemcpyAsync(K.x, u, sizeof(double) * NR, cudaMemcpyDeviceToDevice, s));
-  int *hc = reinterpret_cast<int *>(K.hbuf);
-  double *hp = K.hbuf + 8;
-  hc[0] = o.maxit;
-  hp[0] = o.rtol;
-  FMMPC_CUDA(cudaMemcpyAsync(K.g_ctl + KC_MAXIT, hc, sizeof(int), cudaMemcpyHostToDevice, s));
-  FMMPC_CUDA(cudaMemcpyAsync(K.g_rtol, hp, sizeof(double), cudaMemcpyHostToDevice, s));
+  send_solve_limits(K, o, s);
   FMMPC_CUDA(cudaGraphLaunch(ex, s));
   FMMPC_CUDA(cudaMemcpyAsync(u, K.x, sizeof(double) * NR, cudaMemcpyDeviceToDevice, s));
-  double *hrel = K.hbuf + 16;
-  int *hit = reinterpret_cast<int *>(K.hbuf + 16 + MAXJ), *hctl = hit + MAXJ;
-  FMMPC_CUDA(cudaMemcpyAsync(hrel, K.g_rel, sizeof(double) * nrhs, cudaMemcpyDeviceToHost, s));
-  FMMPC_CUDA(cudaMemcpyAsync(hit, K.g_iters, sizeof(int) * nrhs, cudaMemcpyDeviceToHost, s));
-  FMMPC_CUDA(cudaMemcpyAsync(hctl, K.g_ctl, sizeof(int) * KC_COUNT, cudaMemcpyDeviceToHost, s));
+  const double *hrel;
+  const int *hit, *hctl;
+  fetch_solve_report(H, s, hctl, hrel, hit);
   FMMPC_CUDA(cudaStreamSynchronize(s));
   double worst = 0.0;
   int status = FMMPC_OK;
@@ -1888,32 +2004,25 @@ int solve_batched_graphed(std::vector<fmmpc_handle *> &hs, const double *const *
       else FMMPC_CUDA(cudaMemsetAsync(K.gin, 0, sizeof(double) * 4 * H.g.n, s0));
     }
     FMMPC_CUDA(cudaMemcpyAsync(K.x, u[p], sizeof(double) * N, cudaMemcpyDeviceToDevice, s0));
-    int *hc = reinterpret_cast<int *>(K.hbuf);
-    double *hp = K.hbuf + 8;
-    hc[0] = o.maxit;
-    hp[0] = o.rtol;
-    FMMPC_CUDA(cudaMemcpyAsync(K.g_ctl + KC_MAXIT, hc, sizeof(int), cudaMemcpyHostToDevice, s0));
-    FMMPC_CUDA(cudaMemcpyAsync(K.g_rtol, hp, sizeof(double), cudaMemcpyHostToDevice, s0));
+    send_solve_limits(K, o, s0);
   }
   FMMPC_CUDA(cudaGraphLaunch(ex, s0));
+  std::vector<const double *> hrel(np);
+  std::vector<const int *> hit(np), hctl(np);
   for (int p = 0; p < np; ++p) {
     fmmpc_handle &H = *hs[p];
     KrylovWs &K = H.kw;
     const int64_t N = (int64_t)H.g.n * H.g.n;
     FMMPC_CUDA(cudaMemcpyAsync(u[p], K.x, sizeof(double) * N, cudaMemcpyDeviceToDevice, s0));
-    FMMPC_CUDA(cudaMemcpyAsync(K.hbuf + 16, K.g_rel, sizeof(double), cudaMemcpyDeviceToHost, s0));
-    FMMPC_CUDA(cudaMemcpyAsync(K.hbuf + 17, K.g_iters, sizeof(int), cudaMemcpyDeviceToHost, s0));
-    FMMPC_CUDA(cudaMemcpyAsync(K.hbuf + 18, K.g_ctl, sizeof(int) * KC_COUNT, cudaMemcpyDeviceToHost, s0));
+    fetch_solve_report(H, s0, hctl[p], hrel[p], hit[p]);
   }
   FMMPC_CUDA(cudaStreamSynchronize(s0));
   int worst = FMMPC_OK;
   for (int p = 0; p < np; ++p) {
-    KrylovWs &K = hs[p]->kw;
-    const double rel = K.hbuf[16];
-    const int iters = *reinterpret_cast<int *>(K.hbuf + 17);
-    const int *hctl = reinterpret_cast<int *>(K.hbuf + 18);
+    const double rel = hrel[p][0];
+    const int iters = hit[p][0];
     int status = FMMPC_OK;
-    if (!std::isfinite(rel) || hctl[KC_NAN]) status = FMMPC_ERR_NAN;
+    if (!std::isfinite(rel) || hctl[p][KC_NAN]) status = FMMPC_ERR_NAN;
     else if (rel > o.rtol) status = FMMPC_ERR_NOT_CONVERGED;
     if (infos) {
       infos[p].iters = iters;

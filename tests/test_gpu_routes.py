@@ -1,6 +1,7 @@
 """Kernels and dispatch rules at the sizes where they can go wrong, each against the oracle or
 the general path: window edges of the Q1 mass solve, tables formed on first use, the FP64 form's
-tensor-core kernels, the smallest folded boundary blocks, and alignment."""
+tensor-core kernels, the smallest folded boundary blocks, alignment, and the block sizes of the graph
+solves' sweeps."""
 import numpy as np
 import pytest
 
@@ -172,4 +173,24 @@ def test_spmv_takes_vectors_aligned_for_fp64_only():
     u, _ = P.solve(x, use_graphs=0)
     v, _ = P.solve(big[1:], u0=big[1:] * 0, use_graphs=0)
     assert float((u - v).norm() / u.norm()) < 1e-8
+    P.close()
+
+
+@pytest.mark.parametrize("n,method,restart,nrhs", [(16, "fgmres", 3, 2), (32, "cg", 30, 1), (256, "gmres", 5, 1),
+                                                   (512, "fgmres", 9, 1)])
+def test_graph_solve_sweeps_at_every_block_size(n, method, restart, nrhs):
+    # blocks of 64, 128 and 256 threads, full and ragged grids, cycles that end early and late, more
+    # than eight vectors, one and several right-hand sides: the same solution as the host-driven loop
+    # within the solves' tolerance, and the reported residual is the true one
+    from paper_1308_3339_gb300 import FmmPreconditioner
+    f = dev(np.stack([S.random_field(n, 70 + k) for k in range(nrhs)]))
+    P = FmmPreconditioner(n, p=6, leaf_max=16 if n < 64 else 64, precision="fp32", n_rhs=nrhs)
+    u0, i0 = P.solve(f, method=method, restart=restart, rtol=1e-9, use_graphs=0)
+    u2, i2 = P.solve(f, method=method, restart=restart, rtol=1e-9, use_graphs=2)
+    assert i0["status"] == 0 and i2["status"] == 0 and i2["rel_res"] <= 1e-9
+    assert abs(i0["iters"] - i2["iters"]) <= 1
+    check_close(f"graph vs host {method} n={n}", u2.cpu().numpy(), u0.cpu().numpy(), 1e-7, 1e-7)
+    r = f - P.spmv(u2)
+    true = (r.reshape(nrhs, -1).norm(dim=1) / f.reshape(nrhs, -1).norm(dim=1)).max().item()
+    assert abs(true - i2["rel_res"]) <= 1e-6 * true + 1e-13
     P.close()
