@@ -124,27 +124,62 @@ __device__ __forceinline__ cpx<R> m2m_row(const cpx<R> *__restrict__ T, const cp
   return acc;
 }
 
-// Sums acc[k] (P <= 16 complex values) over the 16 lanes of a half-warp, transposed: lane c
-// of the half ends with the total of acc[c].  The 2P real values, padded to 32, go through a
-// butterfly in which each lane keeps half of its values at each of the four steps and adds
-// the partner's copy of that half: 30 shuffles where separate trees take 8P.
-template <typename R, int P>
-__device__ __forceinline__ cpx<R> seg16_sum_coeffs(const cpx<R> (&acc)[P], int c) {
+// One step of the butterfly below: of the values v[0 .. N), numbers lo .. hi of the whole, the lanes with
+// bit o of c keep the upper part, the others the lower one.
+template <typename R, int N, int NV>
+__device__ __forceinline__ void seg16_half(R (&v)[NV], int c, int o, int &lo, int &hi) {
+  constexpr int H = (N + 1) / 2;
+  const bool up = (c & o) != 0;
+#pragma unroll
+  for (int i = 0; i < H; ++i) {
+    const R top = H + i < N ? v[(H + i) % NV] : R(0);
+    const R keep = up ? top : v[i], give = up ? v[i] : top;
+    v[i] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+  }
+  if (up) lo += H;
+  else hi = min(hi, lo + H);
+}
+
+// Sums the 2P real parts of acc[k] (P <= 16) over the 16 lanes of a half-warp, transposed: a butterfly
+// in which each lane keeps half of its values (rounded up) at each of the four steps and adds
+// the partner's copy of that half, 20 shuffles and adds at P = 10 where separate trees take 8P.
+// f(i, v): lane c is given the totals v of its one or two real parts i (2k: Re, 2k + 1: Im).
+template <typename R, int P, typename F>
+__device__ __forceinline__ void seg16_sum_coeffs(const cpx<R> (&acc)[P], int c, F &&f) {
   static_assert(P <= 16, "two values per lane after the butterfly");
-  R v[32];
+  R v[2 * P];
 #pragma unroll
-  for (int i = 0; i < 32; ++i) v[i] = i < 2 * P ? ((i & 1) ? acc[i >> 1].im : acc[i >> 1].re) : R(0);
+  for (int i = 0; i < 2 * P; ++i) v[i] = (i & 1) ? acc[i >> 1].im : acc[i >> 1].re;
+  constexpr int N1 = P, N2 = (N1 + 1) / 2, N3 = (N2 + 1) / 2, N4 = (N3 + 1) / 2;
+  int lo = 0, hi = 2 * P;
+  seg16_half<R, 2 * P>(v, c, 8, lo, hi);
+  seg16_half<R, N1>(v, c, 4, lo, hi);
+  seg16_half<R, N2>(v, c, 2, lo, hi);
+  seg16_half<R, N3>(v, c, 1, lo, hi);
 #pragma unroll
-  for (int st = 0; st < 4; ++st) {
-    const int o = 8 >> st, h = 16 >> st;
-    const bool up = (c & o) != 0;
+  for (int i = 0; i < N4; ++i)
+    if (lo + i < hi) f(lo + i, v[i]);
+}
+
+// The four mirror images of a node z = x + i y of a leaf (x, y > 0 in units of the leaf side): z, -z,
+// conj z and -conj z have the powers (a, b), (-1)^k (a, b), (a, -b) and (-1)^k (a, -b), so P2M takes the
+// four weights as four folded sums and L2P gives the four values from four sums over the
+// coefficients: a quarter of the multiply-adds and table reads of node by node.
+// Powers z^k (P2M: -z^k / k, k > 0), k < P, of the M^2 / 4 nodes with x, y > 0 into zt (a row of PZ per node).
+template <typename R, int P, int PZ, int M, bool P2M>
+__device__ __forceinline__ void quad_powers(cpx<R> (*zt)[PZ], int tid, int nthr) {
+  constexpr int H = M / 2;
+  for (int pt = tid; pt < H * H; pt += nthr) {
+    const cpx<R> z = mk<R>((pt % H + R(0.5)) / M, (pt / H + R(0.5)) / M);
+    cpx<R> pw = z;
+    zt[pt][0] = mk<R>(1, 0);
 #pragma unroll
-    for (int i = 0; i < h; ++i) {
-      const R keep = up ? v[h + i] : v[i], give = up ? v[i] : v[h + i];
-      v[i] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+    for (int k = 1; k < P; ++k) {
+      const R s = P2M ? R(-1) / R(k) : R(1);
+      zt[pt][k] = mk<R>(s * pw.re, s * pw.im);
+      pw = pw * z;
     }
   }
-  return mk<R>(v[0], v[1]);
 }
 
 // k M2M levels (item 2) over the 4^k consecutive (Morton) cells of level l held in
@@ -177,8 +212,8 @@ __device__ __forceinline__ void m2m_levels_smem(const cpx<R> *sT, cpx<R> (*buf)[
 
 // The whole upward pass of the volume tree in one launch.  Block (b, rhs) takes the 4x4
 // Morton block b of leaves (MS x MS nodes each): P2M (item 1; Mt_0 = sum w_j,
-// Mt_k = -sum w_j zt_j^k / k; 16 threads per leaf, each summing every 16th node with all
-// its loads issued first, then a shuffle reduction), then M2M (item 2) to the 4 parents and
+// Mt_k = -sum w_j zt_j^k / k; 16 threads per leaf, each with every 16th mirrored quadruple of nodes
+// (or node), all its loads issued first, then a shuffle reduction), then M2M (item 2) to the 4 parents and
 // to cell b of level L - 2.  Above that, M2M proceeds up to three levels at a time: the
 // last of the blocks that complete a Morton group of 4^k cells (an atomic count per group,
 // reset by that block) computes the k levels above it.  Any block that does a step
@@ -188,10 +223,15 @@ __global__ void __launch_bounds__(256, (sizeof(R) == 4 && P <= 10 && MS <= 8) ? 
                                                      cpx<R> *__restrict__ Mv, int *__restrict__ counter, int64_t ncount) {
   // three-level steps need 64 cells in shared memory; two-level steps where that would not fit
   constexpr int NBUF = sizeof(cpx<R>) * P * (4 * P + 128) <= 45000 ? 64 : 16, MAXSTEP = NBUF == 64 ? 3 : 2;
-  // z^k of each node position in a leaf (the same for every leaf), where it fits
-  constexpr bool ZTAB = sizeof(cpx<R>) * MS * MS * P <= 16384;
-  constexpr int ZN = ZTAB ? MS * MS : 1;
-  __shared__ cpx<R> sT[4 * P * P], buf[NBUF][P], part[NBUF][P], zt[ZN][P];
+  // P2M by mirrored quadruples of nodes: 16 or 64 of them per leaf, powers in shared memory where they fit
+  // (an odd row length: no bank conflicts).  Node by node, table reads and multiply-adds bound it: 1024^2
+  // FP32 16.4 -> 13.4 us, FP64 121 -> 84, 4096^2 x 32 3.1 -> 2.1 ms
+  constexpr int PZ = P | 1, NQ = MS * MS / 64;
+  constexpr bool FOLD = MS == 8 || (MS == 16 && sizeof(cpx<R>) * (4 * P * P + 2 * NBUF * P + MS * MS / 4 * PZ) <= 47000);
+  // otherwise z^k of each node position in a leaf (the same for every leaf), where it fits
+  constexpr bool ZTAB = !FOLD && sizeof(cpx<R>) * MS * MS * P <= 16384;
+  constexpr int ZN = FOLD ? MS * MS / 4 : (ZTAB ? MS * MS : 1);
+  __shared__ cpx<R> sT[4 * P * P], buf[NBUF][P], part[NBUF][P], zt[ZN][PZ];
   __shared__ int s_last;
   const int tid = threadIdx.x, nthr = blockDim.x;
   const int rhs = blockIdx.y;
@@ -206,56 +246,85 @@ __global__ void __launch_bounds__(256, (sizeof(R) == 4 && P <= 10 && MS <= 8) ? 
     morton_decode(lc, a, b);
     const R half = R(0.5) * (MS - 1), invm = R(1) / MS;
     const R *W = wpad + (int64_t)rhs * g.npad * g.npad + (int64_t)(b * MS + g.pad) * g.npad + a * MS + g.pad;
-    R w[NP];
-#pragma unroll
-    for (int e = 0; e < NP; ++e) {
-      const int pt = c + 16 * e;
-      w[e] = pt < MS * MS ? W[(int64_t)(pt / MS) * g.npad + pt % MS] : R(0);
-    }
-    if (ZTAB) {  // the same chain of products as below, so the same values
-      for (int pt = tid; pt < ZN; pt += nthr) {
-        const cpx<R> z = mk<R>((pt % MS - half) * invm, (pt / MS - half) * invm);
-        cpx<R> pw = z;
-        for (int k = 1; k < P; ++k) {
-          zt[pt][k] = pw;
-          pw = pw * z;
-        }
-      }
-      __syncthreads();
-    }
     cpx<R> acc[P];
 #pragma unroll
     for (int k = 0; k < P; ++k) acc[k] = mk<R>(0, 0);
+    if constexpr (FOLD) {
+      constexpr int H = MS / 2;
+      R w[NQ][4];  // at z, -z, conj z, -conj z
 #pragma unroll
-    for (int e = 0; e < NP; ++e) {
-      const int pt = c + 16 * e;
-      acc[0].re += w[e];
-      if (ZTAB) {
-        const int ptc = pt < ZN ? pt : 0;  // w[e] is 0 past the leaf
+      for (int e = 0; e < NQ; ++e) {
+        const int q = c + 16 * e, qx = q % H, qy = q / H;
+        const R *Wp = W + (int64_t)(H + qy) * g.npad + H, *Wm = W + (int64_t)(H - 1 - qy) * g.npad + H;
+        w[e][0] = Wp[qx];
+        w[e][1] = Wm[-1 - qx];
+        w[e][2] = Wm[qx];
+        w[e][3] = Wp[-1 - qx];
+      }
+      quad_powers<R, P, PZ, MS, true>(zt, tid, nthr);
+      __syncthreads();
+#pragma unroll
+      for (int e = 0; e < NQ; ++e) {
+        const R s1 = w[e][0] + w[e][1], d1 = w[e][0] - w[e][1], s2 = w[e][2] + w[e][3], d2 = w[e][2] - w[e][3];
+        const R er = s1 + s2, ei = s1 - s2, odr = d1 + d2, odi = d1 - d2;
+        const cpx<R> *z = zt[c + 16 * e];
+        acc[0].re += er;
 #pragma unroll
         for (int k = 1; k < P; ++k) {
-          const cpx<R> zk = zt[ptc][k];
-          acc[k].re = fma(w[e], zk.re, acc[k].re);
-          acc[k].im = fma(w[e], zk.im, acc[k].im);
+          const cpx<R> zk = z[k];
+          acc[k].re = fma((k & 1) ? odr : er, zk.re, acc[k].re);
+          acc[k].im = fma((k & 1) ? odi : ei, zk.im, acc[k].im);
         }
-      } else {
-        const cpx<R> z = mk<R>((pt % MS - half) * invm, (pt / MS - half) * invm);
-        cpx<R> pw = z;
+      }
+    } else {
+      R w[NP];
 #pragma unroll
-        for (int k = 1; k < P; ++k) {
-          acc[k].re = fma(w[e], pw.re, acc[k].re);
-          acc[k].im = fma(w[e], pw.im, acc[k].im);
-          pw = pw * z;
+      for (int e = 0; e < NP; ++e) {
+        const int pt = c + 16 * e;
+        w[e] = pt < MS * MS ? W[(int64_t)(pt / MS) * g.npad + pt % MS] : R(0);
+      }
+      if (ZTAB) {  // the same chain of products as below, so the same values
+        for (int pt = tid; pt < ZN; pt += nthr) {
+          const cpx<R> z = mk<R>((pt % MS - half) * invm, (pt / MS - half) * invm);
+          cpx<R> pw = z;
+          for (int k = 1; k < P; ++k) {
+            zt[pt][k] = pw;
+            pw = pw * z;
+          }
+        }
+        __syncthreads();
+      }
+#pragma unroll
+      for (int e = 0; e < NP; ++e) {
+        const int pt = c + 16 * e;
+        acc[0].re += w[e];
+        if (ZTAB) {
+          const int ptc = pt < ZN ? pt : 0;  // w[e] is 0 past the leaf
+#pragma unroll
+          for (int k = 1; k < P; ++k) {
+            const cpx<R> zk = zt[ptc][k];
+            acc[k].re = fma(w[e], zk.re, acc[k].re);
+            acc[k].im = fma(w[e], zk.im, acc[k].im);
+          }
+        } else {
+          const cpx<R> z = mk<R>((pt % MS - half) * invm, (pt / MS - half) * invm);
+          cpx<R> pw = z;
+#pragma unroll
+          for (int k = 1; k < P; ++k) {
+            acc[k].re = fma(w[e], pw.re, acc[k].re);
+            acc[k].im = fma(w[e], pw.im, acc[k].im);
+            pw = pw * z;
+          }
         }
       }
     }
-    const cpx<R> tot = seg16_sum_coeffs<R, P>(acc, c);  // lane c: coefficient c
-    if (c < P) {
-      const R sk = c == 0 ? R(1) : R(-1) / R(c);
-      const cpx<R> v = mk<R>(sk * tot.re, sk * tot.im);
-      buf[leaf][c] = v;
-      M[(level_offset(g.L) + lc) * P + c] = v;
-    }
+    R *bl = reinterpret_cast<R *>(buf[leaf]), *ml = reinterpret_cast<R *>(M + (level_offset(g.L) + lc) * P);
+    seg16_sum_coeffs<R, P>(acc, c, [&](int i, R tot) {
+      const int k = i >> 1;
+      const R v = FOLD || k == 0 ? tot : R(-1) / R(k) * tot;
+      bl[i] = v;
+      ml[i] = v;
+    });
   }
   __syncthreads();
   m2m_levels_smem<R, P>(sT, buf, part, M, g.L, 16 * blk, 2, tid, nthr);
@@ -1753,7 +1822,12 @@ __global__ void __launch_bounds__(256, (sizeof(R) == 4 && P <= 10 && M <= 8) ? 7
                                                        const cpx<R> *__restrict__ Lsep, int64_t nsep,
                                                        const R *__restrict__ phib, const int32_t *__restrict__ bslot,
                                                        double *out, const R *nearp, int np, int64_t nstride) {
-  __shared__ cpx<R> sS[4 * P * P], sanc[24][P], s1[4][P], s2[16][P];
+  // L2P by mirrored quadruples of nodes, staged so that the stores stay rows (node by node, the FP64 form
+  // spent 160 multiply-adds per thread: 1024^2 162 -> 76 us; 4096^2 x 32 FP32 4.6 -> 4.2 ms)
+  constexpr bool FOLD = M == 8 || (M == 16 && sizeof(R) == 4);
+  constexpr int PZ = P | 1, NQ = M * M / 64, SVW = 4 * M + 4;
+  __shared__ cpx<R> sS[4 * P * P], sanc[24][P], s1[4][P], s2[16][P], zt[FOLD ? M * M / 4 : 1][PZ];
+  __shared__ alignas(16) R sv[FOLD ? 4 * M : 1][SVW];  // the far field at the block's nodes
   const int tid = threadIdx.x, nthr = blockDim.x, rhs = blockIdx.y;
   const uint32_t blk = blockIdx.x;
   const int L = g.L;
@@ -1777,6 +1851,7 @@ __global__ void __launch_bounds__(256, (sizeof(R) == 4 && P <= 10 && M <= 8) ? 7
   }
   for (int i = tid; i < 4 * P; i += nthr) s1[i / P][i % P] = lval(level_offset(L - 1) + 4 * blk + i / P, i % P);
   for (int i = tid; i < 16 * P; i += nthr) s2[i / P][i % P] = lval(level_offset(L) + 16 * blk + i / P, i % P);
+  if constexpr (FOLD) quad_powers<R, P, PZ, M, false>(zt, nthr - 1 - tid, nthr);
   if (tid == 0) {  // the root also takes ln h times the total weight (volume, and boundary if present)
     double W = (double)Mv[(int64_t)rhs * g.ncell * P].re;
     if (with_bnd_w)
@@ -1838,14 +1913,49 @@ __global__ void __launch_bounds__(256, (sizeof(R) == 4 && P <= 10 && M <= 8) ? 7
     const int slot = bslot[16 * (int64_t)blk + lf];
     if (slot >= 0) pb = phib + ((int64_t)rhs * nbnear + slot) * M * M + ty * M + tx0;
   }
-  const R zy = (ty - R(0.5) * (M - 1)) / M;
-  cpx<R> acc[NPT];
+  R far[NPT];
+  if constexpr (FOLD) {
+    constexpr int H = M / 2;
+    const int ql = tid >> 4;  // the leaf whose quadruples this thread evaluates
+    int lx, ly;
+    morton_decode((uint32_t)ql, lx, ly);
 #pragma unroll
-  for (int e = 0; e < NPT; ++e) acc[e] = mk<R>(0, 0);
-  for (int k = P - 1; k >= 0; --k) {
-    const cpx<R> Lk = s2[lf][k];
+    for (int e = 0; e < NQ; ++e) {
+      const int q = (tid & 15) + 16 * e, qx = q % H, qy = q / H;
+      R ae = s2[ql][0].re, ao = R(0), be = R(0), bo = R(0);
 #pragma unroll
-    for (int e = 0; e < NPT; ++e) acc[e] = acc[e] * mk<R>((tx0 + e - R(0.5) * (M - 1)) / M, zy) + Lk;
+      for (int k = 1; k < P; ++k) {
+        const cpx<R> Lk = s2[ql][k], zk = zt[q][k];
+        if (k & 1) {
+          ao = fma(Lk.re, zk.re, ao);
+          bo = fma(Lk.im, zk.im, bo);
+        } else {
+          ae = fma(Lk.re, zk.re, ae);
+          be = fma(Lk.im, zk.im, be);
+        }
+      }
+      const int xp = lx * M + H + qx, xm = lx * M + H - 1 - qx, yp = ly * M + H + qy, ym = ly * M + H - 1 - qy;
+      const R u = ae + ao, v = be + bo, um = ae - ao, vm = be - bo;
+      sv[yp][xp] = u - v;    // z
+      sv[ym][xp] = u + v;    // conj z
+      sv[ym][xm] = um - vm;  // -z
+      sv[yp][xm] = um + vm;  // -conj z
+    }
+    __syncthreads();
+#pragma unroll
+    for (int e = 0; e < NPT; ++e) far[e] = sv[y][x0 + e];
+  } else {
+    const R zy = (ty - R(0.5) * (M - 1)) / M;
+    cpx<R> acc[NPT];
+#pragma unroll
+    for (int e = 0; e < NPT; ++e) acc[e] = mk<R>(0, 0);
+    for (int k = P - 1; k >= 0; --k) {
+      const cpx<R> Lk = s2[lf][k];
+#pragma unroll
+      for (int e = 0; e < NPT; ++e) acc[e] = acc[e] * mk<R>((tx0 + e - R(0.5) * (M - 1)) / M, zy) + Lk;
+    }
+#pragma unroll
+    for (int e = 0; e < NPT; ++e) far[e] = acc[e].re;
   }
   double *o = out + off;
   if (nearp) {  // tensor-core near field: raw parts (of one part, in out itself)
@@ -1858,7 +1968,7 @@ __global__ void __launch_bounds__(256, (sizeof(R) == 4 && P <= 10 && M <= 8) ? 7
         for (int e = 0; e < NPT; ++e) sn[e] += nearp[q * nstride + off + e];
       }
 #pragma unroll
-      for (int e = 0; e < NPT; ++e) o[e] = (sn[e] + acc[e].re + (pb ? pb[e] : 0.0)) * NEG_INV_2PI;
+      for (int e = 0; e < NPT; ++e) o[e] = (sn[e] + far[e] + (pb ? pb[e] : 0.0)) * NEG_INV_2PI;
     } else {
       // the parts often cancel, so they are added as a two-word FP32 sum (TwoSum) and scaled by
       // -1/(2 pi) in two-word arithmetic, the far term added, and the two-word result converted
@@ -1875,7 +1985,7 @@ __global__ void __launch_bounds__(256, (sizeof(R) == 4 && P <= 10 && M <= 8) ? 7
       }
 #pragma unroll
       for (int e = 0; e < NPT; ++e) {
-        float v = (float)acc[e].re;
+        float v = (float)far[e];
         if (pb) v += (float)pb[e];
         o[e] = near_far_sum(sn[e], sl[e], v);
       }
@@ -1883,7 +1993,7 @@ __global__ void __launch_bounds__(256, (sizeof(R) == 4 && P <= 10 && M <= 8) ? 7
   } else {
 #pragma unroll
     for (int e = 0; e < NPT; ++e) {
-      double v = (double)acc[e].re;
+      double v = (double)far[e];
       if (pb) v += (double)pb[e];
       o[e] += v * NEG_INV_2PI;
     }
@@ -2661,9 +2771,12 @@ void init_fmm(fmmpc_handle &H) {
   // Stream priorities (copied into the kernel nodes of captured graphs, which are
   // instantiated to use them): the apply's critical chain (weights, upward pass, boundary
   // chain, downward pass) runs on the graph stream at the highest priority; the near-
-  // boundary correction, which joins later, in between; the near field and the volume M2L,
-  // which have slack, at the lowest, so that their many CTAs do not hold back the chain's
-  // latency-bound kernels.
+  // boundary correction, which joins later, in between; the near field and the volume M2L, which have
+  // slack, at the lowest, so that their many CTAs do not hold back the chain's latency-bound kernels.
+  // The mixed forms' M2L, whose CTAs take an SM each, goes in between too: behind the near field's it
+  // was what the downward pass waited for (at the lowest: 1024^2 apply 116 -> 125 us, 2048^2 solve
+  // 15.9 -> 16.6 ms; FP64 and FP32 forms are 5% faster with it at the lowest).
+  const bool mixed = H.prec == FMMPC_PREC_MIXED_TF32 || H.prec == FMMPC_PREC_MIXED_BF16;
   int prio_low = 0, prio_high = 0;
   FMMPC_CUDA(cudaDeviceGetStreamPriorityRange(&prio_low, &prio_high));
   FMMPC_CUDA(cudaStreamCreateWithPriority(&H.gstream, cudaStreamNonBlocking, prio_high));
@@ -2671,7 +2784,8 @@ void init_fmm(fmmpc_handle &H) {
   FMMPC_CUDA(cudaEventCreateWithFlags(&H.gev_out, cudaEventDisableTiming));
   FMMPC_CUDA(cudaStreamCreateWithPriority(&H.sstream, cudaStreamNonBlocking, prio_low));
   FMMPC_CUDA(cudaStreamCreateWithPriority(&H.sstream2, cudaStreamNonBlocking, (prio_low + prio_high) / 2));
-  FMMPC_CUDA(cudaStreamCreateWithPriority(&H.sstream3, cudaStreamNonBlocking, prio_low));
+  FMMPC_CUDA(cudaStreamCreateWithPriority(&H.sstream3, cudaStreamNonBlocking,
+                                          mixed ? (prio_low + prio_high) / 2 : prio_low));
   for (auto &e : H.sev) FMMPC_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
 }
 

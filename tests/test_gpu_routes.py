@@ -1,7 +1,7 @@
 """Kernels and dispatch rules at the sizes where they can go wrong, each against the oracle or
 the general path: window edges of the Q1 mass solve, tables formed on first use, the FP64 form's
-tensor-core kernels, the smallest folded boundary blocks, alignment, and the block sizes of the graph
-solves' sweeps."""
+tensor-core kernels, the smallest folded boundary blocks, alignment, the block sizes of the graph solves'
+sweeps, and mirrored nodes."""
 import numpy as np
 import pytest
 
@@ -193,4 +193,20 @@ def test_graph_solve_sweeps_at_every_block_size(n, method, restart, nrhs):
     r = f - P.spmv(u2)
     true = (r.reshape(nrhs, -1).norm(dim=1) / f.reshape(nrhs, -1).norm(dim=1)).max().item()
     assert abs(true - i2["rel_res"]) <= 1e-6 * true + 1e-13
+    P.close()
+
+
+@pytest.mark.parametrize("leaf_max,p,prec", [(64, 4, "fp32"), (64, 16, "fp64"), (64, 10, "fp64"), (256, 8, "fp32"),
+                                             (256, 16, "fp32"), (16, 6, "fp32")])
+def test_mirrored_p2m_l2p_matches_oracle(leaf_max, p, prec):
+    # one and four quadruples per thread, powers in shared memory or not, and leaves of 4 x 4, which stay
+    # node by node: V r at the stage tests' bars, for a field without any symmetry
+    from paper_1308_3339_gb300 import FmmPreconditioner
+    n = 64
+    f = S.random_field(n, 95)
+    P = FmmPreconditioner(n, p=p, leaf_max=leaf_max, precision=prec)
+    vr = P.apply_part("vr", dev(f)).cpu().numpy().ravel()
+    R = O.Problem(n, p=p, leaf_max=leaf_max)
+    tol = 1e-12 if prec == "fp64" else 1e-5
+    check_close(f"vr p={p} leaf={leaf_max} {prec}", vr, R.apply(f, "fmm", stages=True)["vr"], tol, tol)
     P.close()
