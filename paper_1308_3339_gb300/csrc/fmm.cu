@@ -127,7 +127,7 @@ __device__ __forceinline__ cpx<R> m2m_row(const cpx<R> *__restrict__ T, const cp
 // One step of the butterfly below: of the values v[0 .. N), numbers lo .. hi of the whole, the lanes with
 // bit o of c keep the upper part, the others the lower one.
 template <typename R, int N, int NV>
-__device__ __forceinline__ void seg16_half(R (&v)[NV], int c, int o, int &lo, int &hi) {
+__device__ __forceinline__ void seg_half(R (&v)[NV], int c, int o, int &lo, int &hi) {
   constexpr int H = (N + 1) / 2;
   const bool up = (c & o) != 0;
 #pragma unroll
@@ -140,24 +140,26 @@ __device__ __forceinline__ void seg16_half(R (&v)[NV], int c, int o, int &lo, in
   else hi = min(hi, lo + H);
 }
 
-// Sums the 2P real parts of acc[k] (P <= 16) over the 16 lanes of a half-warp, transposed: a butterfly
-// in which each lane keeps half of its values (rounded up) at each of the four steps and adds
-// the partner's copy of that half, 20 shuffles and adds at P = 10 where separate trees take 8P.
-// f(i, v): lane c is given the totals v of its one or two real parts i (2k: Re, 2k + 1: Im).
-template <typename R, int P, typename F>
-__device__ __forceinline__ void seg16_sum_coeffs(const cpx<R> (&acc)[P], int c, F &&f) {
-  static_assert(P <= 16, "two values per lane after the butterfly");
+// Sums the 2P real parts of acc[k] over groups of W lanes (16 with P <= 16, or 4), transposed: a
+// butterfly in which each lane keeps half of its values (rounded up) at each step and adds the
+// partner's copy of that half, 20 shuffles and adds at P = 10, W = 16 where separate trees take 8P.
+// f(i, v): lane c of a group is given the totals v of its real parts i (2k: Re, 2k + 1: Im).
+template <typename R, int P, int W, typename F>
+__device__ __forceinline__ void seg_sum_coeffs(const cpx<R> (&acc)[P], int c, F &&f) {
+  static_assert(W == 4 || W == 16, "four or sixteen lanes");
   R v[2 * P];
 #pragma unroll
   for (int i = 0; i < 2 * P; ++i) v[i] = (i & 1) ? acc[i >> 1].im : acc[i >> 1].re;
-  constexpr int N1 = P, N2 = (N1 + 1) / 2, N3 = (N2 + 1) / 2, N4 = (N3 + 1) / 2;
+  constexpr int N1 = P, N2 = (N1 + 1) / 2, N3 = (N2 + 1) / 2, N4 = (N3 + 1) / 2, N = W == 4 ? N2 : N4;
   int lo = 0, hi = 2 * P;
-  seg16_half<R, 2 * P>(v, c, 8, lo, hi);
-  seg16_half<R, N1>(v, c, 4, lo, hi);
-  seg16_half<R, N2>(v, c, 2, lo, hi);
-  seg16_half<R, N3>(v, c, 1, lo, hi);
+  seg_half<R, 2 * P>(v, c, W / 2, lo, hi);
+  seg_half<R, N1>(v, c, W / 4, lo, hi);
+  if constexpr (W == 16) {
+    seg_half<R, N2>(v, c, 2, lo, hi);
+    seg_half<R, N3>(v, c, 1, lo, hi);
+  }
 #pragma unroll
-  for (int i = 0; i < N4; ++i)
+  for (int i = 0; i < N; ++i)
     if (lo + i < hi) f(lo + i, v[i]);
 }
 
@@ -210,23 +212,27 @@ __device__ __forceinline__ void m2m_levels_smem(const cpx<R> *sT, cpx<R> (*buf)[
   }
 }
 
-// The whole upward pass of the volume tree in one launch.  Block (b, rhs) takes the 4x4
-// Morton block b of leaves (MS x MS nodes each): P2M (item 1; Mt_0 = sum w_j,
+// The whole upward pass of the volume tree in one launch.  Block (b, rhs) takes the Morton block b of
+// 4x4 or 8x8 leaves (MS x MS nodes each): P2M (item 1; Mt_0 = sum w_j,
 // Mt_k = -sum w_j zt_j^k / k; 16 threads per leaf, each with every 16th mirrored quadruple of nodes
-// (or node), all its loads issued first, then a shuffle reduction), then M2M (item 2) to the 4 parents and
-// to cell b of level L - 2.  Above that, M2M proceeds up to three levels at a time: the
+// (or node), all its loads issued first, then a shuffle reduction; with 8x8 leaves 4 threads and every
+// 4th quadruple, which halves the instructions), then M2M (item 2) to the parents and on to cell b of
+// level L - 2 (L - 3).  Above that, M2M proceeds up to three levels at a time: the
 // last of the blocks that complete a Morton group of 4^k cells (an atomic count per group,
 // reset by that block) computes the k levels above it.  Any block that does a step
 // computes the same sums, so the result does not depend on which block it is.
-template <typename R, int P, int MS>
-__global__ void __launch_bounds__(256, (sizeof(R) == 4 && P <= 10 && MS <= 8) ? 7 : 1) k_upward_tree(Geo g, const R *__restrict__ wpad, const cpx<R> *__restrict__ vm2m,
+template <typename R, int P>
+constexpr int up_nbuf() { return sizeof(cpx<R>) * P * (4 * P + 128) <= 45000 ? 64 : 16; }
+template <typename R, int P, int MS, bool WIDE>
+__global__ void __launch_bounds__(256, (sizeof(R) == 4 && P <= 10 && MS <= 8) ? (WIDE ? 5 : 7) : 1) k_upward_tree(Geo g, const R *__restrict__ wpad, const cpx<R> *__restrict__ vm2m,
                                                      cpx<R> *__restrict__ Mv, int *__restrict__ counter, int64_t ncount) {
   // three-level steps need 64 cells in shared memory; two-level steps where that would not fit
-  constexpr int NBUF = sizeof(cpx<R>) * P * (4 * P + 128) <= 45000 ? 64 : 16, MAXSTEP = NBUF == 64 ? 3 : 2;
+  constexpr int NBUF = up_nbuf<R, P>(), MAXSTEP = NBUF == 64 ? 3 : 2;
+  static_assert(!WIDE || (MS == 8 && NBUF == 64), "8x8 leaves of 8x8 nodes");
   // P2M by mirrored quadruples of nodes: 16 or 64 of them per leaf, powers in shared memory where they fit
   // (an odd row length: no bank conflicts).  Node by node, table reads and multiply-adds bound it: 1024^2
   // FP32 16.4 -> 13.4 us, FP64 121 -> 84, 4096^2 x 32 3.1 -> 2.1 ms
-  constexpr int PZ = P | 1, NQ = MS * MS / 64;
+  constexpr int PZ = P | 1, TPL = WIDE ? 4 : 16, NLEAF = 256 / TPL, NQ = MS * MS / (4 * TPL);  // threads per leaf
   constexpr bool FOLD = MS == 8 || (MS == 16 && sizeof(cpx<R>) * (4 * P * P + 2 * NBUF * P + MS * MS / 4 * PZ) <= 47000);
   // otherwise z^k of each node position in a leaf (the same for every leaf), where it fits
   constexpr bool ZTAB = !FOLD && sizeof(cpx<R>) * MS * MS * P <= 16384;
@@ -240,8 +246,8 @@ __global__ void __launch_bounds__(256, (sizeof(R) == 4 && P <= 10 && MS <= 8) ? 
   cpx<R> *M = Mv + (int64_t)rhs * g.ncell * P;
   {
     constexpr int NP = (MS * MS + 15) / 16;  // nodes per thread
-    const int leaf = tid >> 4, c = tid & 15;
-    const uint32_t lc = 16 * blk + leaf;
+    const int leaf = tid / TPL, c = tid % TPL;
+    const uint32_t lc = NLEAF * blk + leaf;
     int a, b;
     morton_decode(lc, a, b);
     const R half = R(0.5) * (MS - 1), invm = R(1) / MS;
@@ -254,7 +260,7 @@ __global__ void __launch_bounds__(256, (sizeof(R) == 4 && P <= 10 && MS <= 8) ? 
       R w[NQ][4];  // at z, -z, conj z, -conj z
 #pragma unroll
       for (int e = 0; e < NQ; ++e) {
-        const int q = c + 16 * e, qx = q % H, qy = q / H;
+        const int q = c + TPL * e, qx = q % H, qy = q / H;
         const R *Wp = W + (int64_t)(H + qy) * g.npad + H, *Wm = W + (int64_t)(H - 1 - qy) * g.npad + H;
         w[e][0] = Wp[qx];
         w[e][1] = Wm[-1 - qx];
@@ -267,7 +273,7 @@ __global__ void __launch_bounds__(256, (sizeof(R) == 4 && P <= 10 && MS <= 8) ? 
       for (int e = 0; e < NQ; ++e) {
         const R s1 = w[e][0] + w[e][1], d1 = w[e][0] - w[e][1], s2 = w[e][2] + w[e][3], d2 = w[e][2] - w[e][3];
         const R er = s1 + s2, ei = s1 - s2, odr = d1 + d2, odi = d1 - d2;
-        const cpx<R> *z = zt[c + 16 * e];
+        const cpx<R> *z = zt[c + TPL * e];
         acc[0].re += er;
 #pragma unroll
         for (int k = 1; k < P; ++k) {
@@ -319,7 +325,7 @@ __global__ void __launch_bounds__(256, (sizeof(R) == 4 && P <= 10 && MS <= 8) ? 
       }
     }
     R *bl = reinterpret_cast<R *>(buf[leaf]), *ml = reinterpret_cast<R *>(M + (level_offset(g.L) + lc) * P);
-    seg16_sum_coeffs<R, P>(acc, c, [&](int i, R tot) {
+    seg_sum_coeffs<R, P, TPL>(acc, c, [&](int i, R tot) {
       const int k = i >> 1;
       const R v = FOLD || k == 0 ? tot : R(-1) / R(k) * tot;
       bl[i] = v;
@@ -327,8 +333,9 @@ __global__ void __launch_bounds__(256, (sizeof(R) == 4 && P <= 10 && MS <= 8) ? 
     });
   }
   __syncthreads();
-  m2m_levels_smem<R, P>(sT, buf, part, M, g.L, 16 * blk, 2, tid, nthr);
-  int l = g.L - 2;
+  constexpr int K0 = WIDE ? 3 : 2;  // levels within the block
+  m2m_levels_smem<R, P>(sT, buf, part, M, g.L, NLEAF * blk, K0, tid, nthr);
+  int l = g.L - K0;
   uint32_t cell = blk;
   while (l > 0) {
     const int step = l < MAXSTEP ? l : MAXSTEP, pl = l - step;
@@ -1809,13 +1816,15 @@ __device__ __forceinline__ double near_far_sum(float s, float s_lo, float v) {
 
 // The whole downward pass of the volume tree, L2L (item 4) and L2P (item 5), in one launch,
 // with the final sum z = -(1/2pi) (near field + far field + near-boundary correction).
-// Block (b, rhs) takes the 4x4 Morton block b of leaves (cell b of level L - 2): it first
+// Block (b, rhs) takes NB Morton blocks of 4x4 leaves (cells NB b .. of level L - 2): it first
 // forms the complete local expansion of each of its ancestors from the root down (its own
 // copy: L(cell) = L_M2L(cell) + L2L(L(parent)), at most P terms per output), then those of
-// cell b, its 4 children and the 16 leaves, and evaluates each leaf expansion at the leaf's
-// nodes (NPT consecutive nodes of one row per thread, so a warp writes whole row segments).
-template <typename R, int P, int M>
-__global__ void __launch_bounds__(256, (sizeof(R) == 4 && P <= 10 && M <= 8) ? 7 : 1) k_downward_tree(Geo g, int nrhs, int do_bnd, int64_t nbnear,
+// its cells, their 4 children and 16 leaves, and evaluates each leaf expansion at the leaf's
+// nodes.
+// The ancestors are one warp's serial chain that the others wait for (barrier stalls were 8.8 of 20 warp
+// cycles per issue at 2048^2 x 4); NB = 4 takes it once for four blocks, a level less of it.
+template <typename R, int P, int M, int NB>
+__global__ void __launch_bounds__(256, P <= 10 && M <= 8 ? (sizeof(R) == 8 ? 3 : (NB == 4 ? 6 : 7)) : 1) k_downward_tree(Geo g, int nrhs, int do_bnd, int64_t nbnear,
                                                        const cpx<R> *__restrict__ Mv, const cpx<R> *__restrict__ Mb,
                                                        int with_bnd_w, const cpx<R> *__restrict__ vl2l,
                                                        const cpx<R> *__restrict__ Lv, const int32_t *__restrict__ vslot,
@@ -1826,15 +1835,17 @@ __global__ void __launch_bounds__(256, (sizeof(R) == 4 && P <= 10 && M <= 8) ? 7
   // spent 160 multiply-adds per thread: 1024^2 162 -> 76 us; 4096^2 x 32 FP32 4.6 -> 4.2 ms)
   constexpr bool FOLD = M == 8 || (M == 16 && sizeof(R) == 4);
   constexpr int PZ = P | 1, NQ = M * M / 64, SVW = 4 * M + 4;
-  __shared__ cpx<R> sS[4 * P * P], sanc[24][P], s1[4][P], s2[16][P], zt[FOLD ? M * M / 4 : 1][PZ];
-  __shared__ alignas(16) R sv[FOLD ? 4 * M : 1][SVW];  // the far field at the block's nodes
+  static_assert(NB == 1 || NB == 4, "one block of leaves, or four of one parent");
+  constexpr int LT = NB == 4 ? 3 : 2;  // the chain ends LT levels above the leaves
+  __shared__ cpx<R> sS[4 * P * P], sanc[24][P], s0[NB][P], s1[4 * NB][P], s2[16 * NB][P], zt[FOLD ? M * M / 4 : 1][PZ];
+  __shared__ alignas(16) R sv[FOLD ? 4 * M : 1][SVW];  // the far field at a block of leaves' nodes
   const int tid = threadIdx.x, nthr = blockDim.x, rhs = blockIdx.y;
-  const uint32_t blk = blockIdx.x;
+  const uint32_t blk0 = NB * blockIdx.x;
   const int L = g.L;
   const cpx<R> *Lr = Lv + (int64_t)rhs * g.ncell * P;
 
   // every value the block needs, loaded at once: the translation matrices, the M2L parts of
-  // the ancestors (levels 0 .. L - 2), of the 4 children and of the 16 leaves
+  // the ancestors (levels 0 .. L - 2), of the children and of the leaves
   for (int i = tid; i < 4 * P * P; i += nthr) sS[i] = vl2l[i];
   // L of cell c (global index), coefficient n, with the boundary-source part kept apart
   auto lval = [&](int64_t c, int n) -> cpx<R> {
@@ -1845,12 +1856,14 @@ __global__ void __launch_bounds__(256, (sizeof(R) == 4 && P <= 10 && M <= 8) ? 7
     }
     return v;
   };
-  for (int i = tid; i < (L - 1) * P; i += nthr) {
+  for (int i = tid; i < (L - LT + 1) * P; i += nthr) {
     const int l = i / P, n = i % P;
-    sanc[l][n] = lval(level_offset(l) + (blk >> (2 * (L - 2 - l))), n);
+    sanc[l][n] = lval(level_offset(l) + (blk0 >> (2 * (L - 2 - l))), n);
   }
-  for (int i = tid; i < 4 * P; i += nthr) s1[i / P][i % P] = lval(level_offset(L - 1) + 4 * blk + i / P, i % P);
-  for (int i = tid; i < 16 * P; i += nthr) s2[i / P][i % P] = lval(level_offset(L) + 16 * blk + i / P, i % P);
+  if constexpr (NB > 1)
+    for (int i = tid; i < NB * P; i += nthr) s0[i / P][i % P] = lval(level_offset(L - 2) + blk0 + i / P, i % P);
+  for (int i = tid; i < 4 * NB * P; i += nthr) s1[i / P][i % P] = lval(level_offset(L - 1) + 4 * blk0 + i / P, i % P);
+  for (int i = tid; i < 16 * NB * P; i += nthr) s2[i / P][i % P] = lval(level_offset(L) + 16 * blk0 + i / P, i % P);
   if constexpr (FOLD) quad_powers<R, P, PZ, M, false>(zt, nthr - 1 - tid, nthr);
   if (tid == 0) {  // the root also takes ln h times the total weight (volume, and boundary if present)
     double W = (double)Mv[(int64_t)rhs * g.ncell * P].re;
@@ -1863,8 +1876,8 @@ __global__ void __launch_bounds__(256, (sizeof(R) == 4 && P <= 10 && M <= 8) ? 7
   // by the first warp alone (P <= 32 outputs per step), so the steps meet at warp barriers
   // and the other warps wait at a single block barrier
   if (tid < 32) {
-    for (int l = 1; l <= L - 2; ++l) {
-      const int q = (blk >> (2 * (L - 2 - l))) & 3;
+    for (int l = 1; l <= L - LT; ++l) {
+      const int q = (blk0 >> (2 * (L - 2 - l))) & 3;
       cpx<R> acc = mk<R>(0, 0);
       if (tid < P) {
         const int n = tid;
@@ -1879,123 +1892,125 @@ __global__ void __launch_bounds__(256, (sizeof(R) == 4 && P <= 10 && M <= 8) ? 7
     }
   }
   __syncthreads();
-  const cpx<R> *cur = sanc[L - 2];
-  cpx<R> v1 = mk<R>(0, 0), v2 = mk<R>(0, 0);
-  if (tid < 4 * P) {
-    const int q = tid / P, n = tid % P;
-    v1 = s1[q][n];
+  // a level at a time, in place: a cell's raw value is read by the thread that completes it alone
+  auto descend = [&](const cpx<R>(*par)[P], cpx<R>(*cell)[P], int count) {
+    for (int t = tid; t < count * P; t += nthr) {
+      const int lf = t / P, n = t % P, q = lf & 3;
+      cpx<R> v = cell[lf][n];
 #pragma unroll
-    for (int k = 0; k < P; ++k)
-      if (k >= n) cmac(v1, sS[(q * P + n) * P + k], cur[k]);
-  }
-  __syncthreads();
-  if (tid < 4 * P) s1[tid / P][tid % P] = v1;
-  __syncthreads();
-  if (tid < 16 * P) {
-    const int lf = tid / P, n = tid % P, q = lf & 3;
-    v2 = s2[lf][n];
-#pragma unroll
-    for (int k = 0; k < P; ++k)
-      if (k >= n) cmac(v2, sS[(q * P + n) * P + k], s1[lf >> 2][k]);
-  }
-  __syncthreads();
-  if (tid < 16 * P) s2[tid / P][tid % P] = v2;
-  __syncthreads();
-  constexpr int NPT = M * M / 16;  // nodes per thread: (4M)^2 nodes over 256 threads
-  const int e0 = tid * NPT, y = e0 / (4 * M), x0 = e0 % (4 * M);
-  const int lf = (int)morton_encode((uint32_t)(x0 / M), (uint32_t)(y / M));
-  const int tx0 = x0 % M, ty = y % M;
-  int bx, by;
-  morton_decode(blk, bx, by);
-  const int64_t off = (int64_t)rhs * g.n * g.n + (int64_t)(by * 4 * M + y) * g.n + bx * 4 * M + x0;
-  const R *pb = nullptr;
-  if (do_bnd) {
-    const int slot = bslot[16 * (int64_t)blk + lf];
-    if (slot >= 0) pb = phib + ((int64_t)rhs * nbnear + slot) * M * M + ty * M + tx0;
-  }
-  R far[NPT];
-  if constexpr (FOLD) {
-    constexpr int H = M / 2;
-    const int ql = tid >> 4;  // the leaf whose quadruples this thread evaluates
-    int lx, ly;
-    morton_decode((uint32_t)ql, lx, ly);
-#pragma unroll
-    for (int e = 0; e < NQ; ++e) {
-      const int q = (tid & 15) + 16 * e, qx = q % H, qy = q / H;
-      R ae = s2[ql][0].re, ao = R(0), be = R(0), bo = R(0);
-#pragma unroll
-      for (int k = 1; k < P; ++k) {
-        const cpx<R> Lk = s2[ql][k], zk = zt[q][k];
-        if (k & 1) {
-          ao = fma(Lk.re, zk.re, ao);
-          bo = fma(Lk.im, zk.im, bo);
-        } else {
-          ae = fma(Lk.re, zk.re, ae);
-          be = fma(Lk.im, zk.im, be);
-        }
-      }
-      const int xp = lx * M + H + qx, xm = lx * M + H - 1 - qx, yp = ly * M + H + qy, ym = ly * M + H - 1 - qy;
-      const R u = ae + ao, v = be + bo, um = ae - ao, vm = be - bo;
-      sv[yp][xp] = u - v;    // z
-      sv[ym][xp] = u + v;    // conj z
-      sv[ym][xm] = um - vm;  // -z
-      sv[yp][xm] = um + vm;  // -conj z
+      for (int k = 0; k < P; ++k)
+        if (k >= n) cmac(v, sS[(q * P + n) * P + k], par[lf >> 2][k]);
+      cell[lf][n] = v;
     }
     __syncthreads();
+  };
+  if constexpr (NB > 1) descend(sanc + (L - 3), s0, NB);
+  descend(NB > 1 ? s0 : sanc + (L - 2), s1, 4 * NB);
+  descend(s1, s2, 16 * NB);
+  // nodes per thread: (4M)^2 nodes over 256 threads, every RS-th row, so that a warp's loads and stores are
+  // whole rows (four consecutive nodes per thread took four passes over the same sectors)
+  constexpr int NPT = M * M / 16, RS = 256 / (4 * M);
+  const int y = tid / (4 * M), x = tid % (4 * M);
+#pragma unroll 1
+  for (int sub = 0; sub < NB; ++sub) {
+    int bx, by;
+    morton_decode(blk0 + sub, bx, by);
+    const int64_t off = (int64_t)rhs * g.n * g.n + (int64_t)(by * 4 * M + y) * g.n + bx * 4 * M + x;
+    const int64_t rstep = (int64_t)RS * g.n;
+    // the near field's first two parts, on their way during the L2P where there are registers for them
+    // (the single FP32 block's 7 per SM are one wave at 1024^2)
+    constexpr bool EARLY = NB == 4 || sizeof(R) == 8;
+    R sn[NPT], sm[NPT];
+    auto load_near = [&] {
 #pragma unroll
-    for (int e = 0; e < NPT; ++e) far[e] = sv[y][x0 + e];
-  } else {
-    const R zy = (ty - R(0.5) * (M - 1)) / M;
-    cpx<R> acc[NPT];
-#pragma unroll
-    for (int e = 0; e < NPT; ++e) acc[e] = mk<R>(0, 0);
-    for (int k = P - 1; k >= 0; --k) {
-      const cpx<R> Lk = s2[lf][k];
-#pragma unroll
-      for (int e = 0; e < NPT; ++e) acc[e] = acc[e] * mk<R>((tx0 + e - R(0.5) * (M - 1)) / M, zy) + Lk;
-    }
-#pragma unroll
-    for (int e = 0; e < NPT; ++e) far[e] = acc[e].re;
-  }
-  double *o = out + off;
-  if (nearp) {  // tensor-core near field: raw parts (of one part, in out itself)
-    if constexpr (std::is_same<R, double>::value) {
-      double sn[NPT];
-#pragma unroll
-      for (int e = 0; e < NPT; ++e) sn[e] = nearp[off + e];
-      for (int q = 1; q < np; ++q) {
-#pragma unroll
-        for (int e = 0; e < NPT; ++e) sn[e] += nearp[q * nstride + off + e];
+      for (int e = 0; e < NPT; ++e) {
+        sn[e] = nearp[off + e * rstep];
+        sm[e] = np > 1 ? nearp[nstride + off + e * rstep] : R(0);
       }
+    };
+    if (EARLY && nearp) load_near();
+    R far[NPT];
+    if constexpr (FOLD) {
+      constexpr int H = M / 2;
+      if (NB > 1 && sub > 0) __syncthreads();  // the last block's values are read
+      const int ql = tid >> 4;  // the leaf whose quadruples this thread evaluates
+      int lx, ly;
+      morton_decode((uint32_t)ql, lx, ly);
 #pragma unroll
-      for (int e = 0; e < NPT; ++e) o[e] = (sn[e] + far[e] + (pb ? pb[e] : 0.0)) * NEG_INV_2PI;
+      for (int e = 0; e < NQ; ++e) {
+        const int q = (tid & 15) + 16 * e, qx = q % H, qy = q / H;
+        R ae = s2[16 * sub + ql][0].re, ao = R(0), be = R(0), bo = R(0);
+#pragma unroll
+        for (int k = 1; k < P; ++k) {
+          const cpx<R> Lk = s2[16 * sub + ql][k], zk = zt[q][k];
+          if (k & 1) {
+            ao = fma(Lk.re, zk.re, ao);
+            bo = fma(Lk.im, zk.im, bo);
+          } else {
+            ae = fma(Lk.re, zk.re, ae);
+            be = fma(Lk.im, zk.im, be);
+          }
+        }
+        const int xp = lx * M + H + qx, xm = lx * M + H - 1 - qx, yp = ly * M + H + qy, ym = ly * M + H - 1 - qy;
+        const R u = ae + ao, v = be + bo, um = ae - ao, vm = be - bo;
+        sv[yp][xp] = u - v;    // z
+        sv[ym][xp] = u + v;    // conj z
+        sv[ym][xm] = um - vm;  // -z
+        sv[yp][xm] = um + vm;  // -conj z
+      }
+      __syncthreads();
+#pragma unroll
+      for (int e = 0; e < NPT; ++e) far[e] = sv[y + e * RS][x];
     } else {
-      // the parts often cancel, so they are added as a two-word FP32 sum (TwoSum) and scaled by
-      // -1/(2 pi) in two-word arithmetic, the far term added, and the two-word result converted
-      // to FP64 with one FP64 addition (FP64 is scarce here)
-      float sn[NPT], sl[NPT];
 #pragma unroll
       for (int e = 0; e < NPT; ++e) {
-        sn[e] = nearp[off + e];
-        sl[e] = 0.0f;
-      }
-      for (int q = 1; q < np; ++q) {
-#pragma unroll
-        for (int e = 0; e < NPT; ++e) two_sum_acc(sn[e], sl[e], nearp[q * nstride + off + e]);
-      }
-#pragma unroll
-      for (int e = 0; e < NPT; ++e) {
-        float v = (float)far[e];
-        if (pb) v += (float)pb[e];
-        o[e] = near_far_sum(sn[e], sl[e], v);
+        const int ye = y + e * RS, lf = (int)morton_encode((uint32_t)(x / M), (uint32_t)(ye / M));
+        const cpx<R> z = mk<R>((x % M - R(0.5) * (M - 1)) / M, (ye % M - R(0.5) * (M - 1)) / M);
+        cpx<R> acc = mk<R>(0, 0);
+        for (int k = P - 1; k >= 0; --k) acc = acc * z + s2[16 * sub + lf][k];
+        far[e] = acc.re;
       }
     }
-  } else {
+    if (do_bnd) {  // the near-boundary correction of the leaves that have one
 #pragma unroll
-    for (int e = 0; e < NPT; ++e) {
-      double v = (double)far[e];
-      if (pb) v += (double)pb[e];
-      o[e] += v * NEG_INV_2PI;
+      for (int e = 0; e < NPT; ++e) {
+        const int ye = y + e * RS, lf = (int)morton_encode((uint32_t)(x / M), (uint32_t)(ye / M));
+        const int slot = bslot[16 * (int64_t)(blk0 + sub) + lf];
+        if (slot >= 0) far[e] += phib[((int64_t)rhs * nbnear + slot) * M * M + (ye % M) * M + x % M];
+      }
+    }
+    double *o = out + off;
+    if (nearp) {  // tensor-core near field: raw parts (of one part, in out itself)
+      if (!EARLY) load_near();
+      if constexpr (std::is_same<R, double>::value) {
+#pragma unroll
+        for (int e = 0; e < NPT; ++e) sn[e] += sm[e];
+        for (int q = 2; q < np; ++q) {
+#pragma unroll
+          for (int e = 0; e < NPT; ++e) sn[e] += nearp[q * nstride + off + e * rstep];
+        }
+#pragma unroll
+        for (int e = 0; e < NPT; ++e) o[e * rstep] = (sn[e] + far[e]) * NEG_INV_2PI;
+      } else {
+        // the parts often cancel, so they are added as a two-word FP32 sum (TwoSum) and scaled by
+        // -1/(2 pi) in two-word arithmetic, the far term added, and the two-word result converted
+        // to FP64 with one FP64 addition (FP64 is scarce here)
+        float sl[NPT];
+#pragma unroll
+        for (int e = 0; e < NPT; ++e) {
+          sl[e] = 0.0f;
+          two_sum_acc(sn[e], sl[e], sm[e]);
+        }
+        for (int q = 2; q < np; ++q) {
+#pragma unroll
+          for (int e = 0; e < NPT; ++e) two_sum_acc(sn[e], sl[e], nearp[q * nstride + off + e * rstep]);
+        }
+#pragma unroll
+        for (int e = 0; e < NPT; ++e) o[e * rstep] = near_far_sum(sn[e], sl[e], far[e]);
+      }
+    } else {
+#pragma unroll
+      for (int e = 0; e < NPT; ++e) o[e * rstep] += (double)far[e] * NEG_INV_2PI;
     }
   }
 }
@@ -2138,6 +2153,11 @@ Mats<R> mats_of(fmmpc_handle &H) {
   return mt;
 }
 
+// Blocks of 8x8 leaves from this depth on: at L = 7 (1024^2 with 8x8 nodes per leaf) the pass takes 12.8 us
+// either way and the FP64 form's 68 instead of 84; 2048^2 37 -> 21 us, 4096^2 x 32 2.13 -> 1.18 ms.  The
+// sums depend on it, so it goes by the depth alone, not by the number of right-hand sides.
+constexpr int UP_WIDE_L = 7;
+
 // Upward pass of the volume tree: one launch for L >= 2 (P2M, then every M2M level).
 template <typename R, int P>
 int run_upward(fmmpc_handle &H, int nrhs, cudaStream_t s) {
@@ -2147,10 +2167,17 @@ int run_upward(fmmpc_handle &H, int nrhs, cudaStream_t s) {
   Mats<R> mt = mats_of<R>(H);
   if (g.L >= 2) {
     const dim3 grid((unsigned)(int64_t(1) << (2 * (g.L - 2))), nrhs);
+    if constexpr (up_nbuf<R, P>() == 64) {
+      if (g.m == 8 && g.L >= UP_WIDE_L) {
+        k_upward_tree<R, P, 8, true><<<dim3(grid.x / 4, nrhs), 256, 0, s>>>(g, wpad, mt.vm2m, Mv, H.fb.up_count, H.fb.up_ncount);
+        FMMPC_LAUNCH_CHECK();
+        return 1;
+      }
+    }
     switch (g.m) {
-      case 4: k_upward_tree<R, P, 4><<<grid, 256, 0, s>>>(g, wpad, mt.vm2m, Mv, H.fb.up_count, H.fb.up_ncount); break;
-      case 8: k_upward_tree<R, P, 8><<<grid, 256, 0, s>>>(g, wpad, mt.vm2m, Mv, H.fb.up_count, H.fb.up_ncount); break;
-      case 16: k_upward_tree<R, P, 16><<<grid, 256, 0, s>>>(g, wpad, mt.vm2m, Mv, H.fb.up_count, H.fb.up_ncount); break;
+      case 4: k_upward_tree<R, P, 4, false><<<grid, 256, 0, s>>>(g, wpad, mt.vm2m, Mv, H.fb.up_count, H.fb.up_ncount); break;
+      case 8: k_upward_tree<R, P, 8, false><<<grid, 256, 0, s>>>(g, wpad, mt.vm2m, Mv, H.fb.up_count, H.fb.up_ncount); break;
+      case 16: k_upward_tree<R, P, 16, false><<<grid, 256, 0, s>>>(g, wpad, mt.vm2m, Mv, H.fb.up_count, H.fb.up_ncount); break;
       default: throw Error(FMMPC_ERR_UNSUPPORTED, "leaf side must be 4, 8 or 16");
     }
     FMMPC_LAUNCH_CHECK();
@@ -2179,6 +2206,13 @@ int run_l2l(fmmpc_handle &H, int nrhs, cudaStream_t s) {
   return launches;
 }
 
+// Downward blocks of four 4x4 blocks of leaves from this many 4x4 blocks on: below, the chip would not be
+// filled (FP32 1024^2, 1024 of them: 12.8 us singly, 17.3 in fours; 2048^2, 4096: solve 15.40 ms singly,
+// 15.28 in fours; 4096^2 x 32: 4.2 -> 3.1 ms); FP64, bound by the chain and by issue, gains at 1024
+// already (932 -> 912 us).
+template <typename R>
+constexpr int64_t DOWN_WIDE_BLOCKS = sizeof(R) == 4 ? 4096 : 1024;
+
 // L2L and L2P with the final sum in one launch (L >= 2); with_bnd_w: the root constant
 // includes the boundary weight.
 template <typename R, int P>
@@ -2198,10 +2232,17 @@ void run_downward(fmmpc_handle &H, double *out, int nrhs, int do_bnd, int with_b
   const R *pb = (const R *)H.fb.phib;
   const cpx<R> *vl2l = mats_of<R>(H).vl2l;
   const dim3 grid((unsigned)(int64_t(1) << (2 * (g.L - 2))), nrhs);
+  if constexpr (sizeof(cpx<R>) * P * (4 * P + 24 + 84 + 16) + sizeof(R) * 32 * 36 <= 46000) {
+    if (g.m == 8 && g.L >= 3 && (int64_t)grid.x * nrhs >= DOWN_WIDE_BLOCKS<R>) {
+      k_downward_tree<R, P, 8, 4><<<dim3(grid.x / 4, nrhs), 256, 0, s>>>(g, nrhs, do_bnd, H.lists.nbnear, Mv, Mb, with_bnd_w, vl2l, Lv, vslot, Lsep, nsep, pb, H.lists.leaf_bslot, out, nearp, np, nstride);
+      FMMPC_LAUNCH_CHECK();
+      return;
+    }
+  }
   switch (g.m) {
-    case 4: k_downward_tree<R, P, 4><<<grid, 256, 0, s>>>(g, nrhs, do_bnd, H.lists.nbnear, Mv, Mb, with_bnd_w, vl2l, Lv, vslot, Lsep, nsep, pb, H.lists.leaf_bslot, out, nearp, np, nstride); break;
-    case 8: k_downward_tree<R, P, 8><<<grid, 256, 0, s>>>(g, nrhs, do_bnd, H.lists.nbnear, Mv, Mb, with_bnd_w, vl2l, Lv, vslot, Lsep, nsep, pb, H.lists.leaf_bslot, out, nearp, np, nstride); break;
-    case 16: k_downward_tree<R, P, 16><<<grid, 256, 0, s>>>(g, nrhs, do_bnd, H.lists.nbnear, Mv, Mb, with_bnd_w, vl2l, Lv, vslot, Lsep, nsep, pb, H.lists.leaf_bslot, out, nearp, np, nstride); break;
+    case 4: k_downward_tree<R, P, 4, 1><<<grid, 256, 0, s>>>(g, nrhs, do_bnd, H.lists.nbnear, Mv, Mb, with_bnd_w, vl2l, Lv, vslot, Lsep, nsep, pb, H.lists.leaf_bslot, out, nearp, np, nstride); break;
+    case 8: k_downward_tree<R, P, 8, 1><<<grid, 256, 0, s>>>(g, nrhs, do_bnd, H.lists.nbnear, Mv, Mb, with_bnd_w, vl2l, Lv, vslot, Lsep, nsep, pb, H.lists.leaf_bslot, out, nearp, np, nstride); break;
+    case 16: k_downward_tree<R, P, 16, 1><<<grid, 256, 0, s>>>(g, nrhs, do_bnd, H.lists.nbnear, Mv, Mb, with_bnd_w, vl2l, Lv, vslot, Lsep, nsep, pb, H.lists.leaf_bslot, out, nearp, np, nstride); break;
     default: throw Error(FMMPC_ERR_UNSUPPORTED, "leaf side must be 4, 8 or 16");
   }
   FMMPC_LAUNCH_CHECK();

@@ -116,23 +116,19 @@ __device__ __forceinline__ float m2l_input(const cpx<float> *M, int v, int p, in
   return e < 2 ? m2l_round<KIND>(x - hi) : hi;
 }
 
-// Multipole image rows: thread per (rhs, cell at level >= 2, 16-byte chunk).  Also clears
+// Multipole image rows: thread per (rhs, cell at level >= 2, 16-byte chunk), a grid row per right-hand
+// side (64-bit divisions by the cell count bound it: 2048^2 x 4 41 us).  Also clears
 // the local expansions of levels 0 and 1, which have no M2L sources, and those of every
 // level when the M2L is split into parts that add.
 template <int KIND>
-__global__ void k_m2l_pack(M2lArgs a, int nrhs, int64_t ncell_lo, int64_t ncell_hi, const cpx<float> *__restrict__ Mv) {
+__global__ void k_m2l_pack(M2lArgs a, int64_t ncell_lo, int64_t ncell_hi, const cpx<float> *__restrict__ Mv) {
   const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const int64_t per = (ncell_hi - ncell_lo) * 8;
-  if (t < (int64_t)nrhs * level_offset(2) * a.p) {
-    const int64_t rhs = t / (level_offset(2) * a.p), k = t % (level_offset(2) * a.p);
-    a.Lv[rhs * a.ncell * a.p + k] = mk<float>(0.f, 0.f);
-  }
-  if (t >= (int64_t)nrhs * per) return;
-  const int64_t rhs = t / per, rem = t % per;
-  const int64_t gidx = ncell_lo + rem / 8;
-  const int chunk = (int)(rem % 8);
-  int l = 2;
-  while (level_offset(l + 1) <= gidx) ++l;
+  const int rhs = blockIdx.y;
+  if (t < level_offset(2) * a.p) a.Lv[(int64_t)rhs * a.ncell * a.p + t] = mk<float>(0.f, 0.f);
+  const int64_t gidx = ncell_lo + (t >> 3);
+  if (gidx >= ncell_hi) return;
+  const int chunk = (int)(t & 7);
+  const int l = (63 - __clzll(3 * gidx + 1)) >> 1;  // level_offset(l) = (4^l - 1) / 3
   int x, y;
   morton_decode((uint32_t)(gidx - level_offset(l)), x, y);
   const int P = a.lev_P[l];
@@ -716,10 +712,10 @@ int run_m2l_tc(fmmpc_handle &H, const void *Mv, void *Lv, int nrhs, cudaStream_t
   a.sbase = T.sbase;
   a.nks = T.kind == 0 ? (T.sbase + 4 * T.nsplit + 7) / 8 : (T.sbase + 4 * T.nsplit + 15) / 16;
   const int64_t lo = level_offset(2), hi = level_offset(g.L + 1);
-  const int64_t threads = std::max<int64_t>((int64_t)nrhs * (hi - lo) * 8, (int64_t)nrhs * lo * g.p);
+  const dim3 pgrid(nblk(std::max<int64_t>((hi - lo) * 8, lo * g.p)), (unsigned)nrhs);
   const cpx<float> *M = (const cpx<float> *)Mv;
-  if (T.kind == 0) k_m2l_pack<0><<<nblk(threads), 256, 0, s>>>(a, nrhs, lo, hi, M);
-  else k_m2l_pack<1><<<nblk(threads), 256, 0, s>>>(a, nrhs, lo, hi, M);
+  if (T.kind == 0) k_m2l_pack<0><<<pgrid, 256, 0, s>>>(a, lo, hi, M);
+  else k_m2l_pack<1><<<pgrid, 256, 0, s>>>(a, lo, hi, M);
   FMMPC_LAUNCH_CHECK();
   dim3 grid((unsigned)T.ntiles, (unsigned)T.nparts, (unsigned)nrhs);
   if (T.width == 24) {

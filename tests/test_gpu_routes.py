@@ -210,3 +210,36 @@ def test_mirrored_p2m_l2p_matches_oracle(leaf_max, p, prec):
     tol = 1e-12 if prec == "fp64" else 1e-5
     check_close(f"vr p={p} leaf={leaf_max} {prec}", vr, R.apply(f, "fmm", stages=True)["vr"], tol, tol)
     P.close()
+
+
+@pytest.mark.parametrize("prec,p,n", [("fp64", 10, 512), ("fp64", 16, 256), ("fp32", 10, 1024), ("mixed_tf32", 8, 1024)])
+def test_wide_tree_blocks_match_oracle(prec, p, n):
+    # blocks of 8x8 leaves on the way up and of four 4x4 blocks on the way down, and the depths and types
+    # next to them that keep the small ones; 4 right-hand sides (1024^2: the wide downward blocks)
+    # equal to one alone bit for bit
+    from paper_1308_3339_gb300 import FmmPreconditioner
+    f = np.stack([S.random_field(n, 40 + k) for k in range(4)])
+    P = FmmPreconditioner(n, p=p, precision=prec, n_rhs=4)
+    z4 = P.apply(dev(f))
+    z1 = P.apply(dev(f[2]))
+    assert torch.equal(z4[2].reshape(-1), z1.reshape(-1))
+    if n <= 512:
+        vr = P.apply_part("vr", dev(f)).cpu().numpy().reshape(4, -1)
+        tol = 1e-12 if prec == "fp64" else 1e-5
+        check_close(f"vr {prec} n={n} p={p}", vr[1], O.Problem(n, p=p).apply(f[1], "fmm", stages=True)["vr"], tol, tol)
+    P.close()
+
+
+@pytest.mark.parametrize("prec", ["fp32", "fp64"])
+def test_wide_upward_blocks_keep_the_half_turn(prec):
+    # 1024^2: the potential of weights that a half turn leaves as they are is left so too, while the
+    # Morton order of cells, blocks and mirrored nodes is reversed
+    from paper_1308_3339_gb300 import FmmPreconditioner
+    n = 1024
+    f = S.random_field(n, 7).reshape(n, n)
+    f = f + f[::-1, ::-1]
+    P = FmmPreconditioner(n, p=10, precision=prec)
+    z = P.apply_part("vr", dev(f.ravel().copy())).cpu().numpy().reshape(n, n)
+    tol = 1e-12 if prec == "fp64" else 1e-5
+    check_close(f"half turn {prec}", z, z[::-1, ::-1], tol, tol)
+    P.close()
