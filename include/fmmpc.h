@@ -44,14 +44,16 @@ extern "C" {
 
 /* FMM arithmetic inside the preconditioner.  The Krylov recurrences, inner products,
  * residual checks and the boundary-element solve are FP64 in every mode. */
-#define FMMPC_PREC_FP64 0       /* FMM in FP64 on CUDA cores (plain FP64 form) */
-#define FMMPC_PREC_FP32 1       /* FMM in FP32 on CUDA cores (plain FP32 form) */
+#define FMMPC_PREC_FP64 0       /* FMM in FP64 (plain FP64 form) */
+#define FMMPC_PREC_FP32 1       /* FMM in FP32 (plain FP32 form) */
 #define FMMPC_PREC_MIXED_BF16 2 /* FP32 P2P/expansions, M2L on tensor cores in BF16, FP32 accumulate */
 #define FMMPC_PREC_MIXED_TF32 3 /* FP32 P2P/expansions, M2L on tensor cores in TF32, FP32 accumulate */
 /* In the mixed forms the volume-to-volume M2L (Sec. 5.3 item 3) of every level >= 2 runs as
  * a lattice convolution on the tensor cores: the leading multipoles and their translation
  * columns are split hi + lo, so the apply stays within ~1e-4 of the FP64 FMM (p <= 15;
- * larger p keeps the FP32 CUDA-core M2L).  Boundary-source M2L stays on CUDA cores. */
+ * larger p keeps the FP32 CUDA-core M2L).  Boundary-source M2L stays on CUDA cores.  The FP64
+ * form's near field (8x8 leaves) and volume M2L (p <= 15) are exact products of 9-bit digits on
+ * the tensor cores, summed as integers: closer to the exact sums than FP64 additions. */
 
 #define FMMPC_CG 0
 #define FMMPC_GMRES 1
@@ -154,7 +156,9 @@ int fmmpc_apply_part(fmmpc_handle *h, int32_t part, const double *r_dev, double 
  * the Dirichlet values at the 4n element midpoints (the collocation points: side length
  * / n apart from half an element past each corner), in the order bottom (x increasing),
  * right (y increasing), top (x decreasing), left (y decreasing).  The boundary solve is
- * FP64 in every form.  Uses the single-layer equations whatever fmmpc_set_bem_form set.
+ * FP64 in every form.  Uses the single-layer equations whatever fmmpc_set_bem_form set.  The
+ * first call forms the tables of (1/2 I + K) and of the double layer next to the boundary; a
+ * first call under stream capture, or where they do not fit, sums them directly instead.
  * Asynchronous on the handle's stream.  Errors: _INVALID. */
 int fmmpc_apply_bc(fmmpc_handle *h, const double *f_dev, const double *g_dev, double *u_dev, int32_t n_rhs);
 
@@ -164,8 +168,8 @@ int fmmpc_apply_bc(fmmpc_handle *h, const double *f_dev, const double *g_dev, do
  * P^{-T} = V - V_GO^T S^{-T} S_OG^T, V symmetric.  The FMM-transpose pass runs the apply's
  * volume FMM on zb, takes the element integrals of that potential over the 4n boundary
  * elements (S_OG^T zb: the local expansions integrated in closed form, closed-form log
- * integrals next to the boundary), applies S^{-T} (the side-DFT blocks transposed, FP64;
- * formed on first use), and sums the resulting point sources at the collocation points
+ * integrals next to the boundary, in FP64 tables), applies S^{-T} (the side-DFT blocks transposed,
+ * FP64; all formed on first use), and sums the resulting point sources at the collocation points
  * back into the nodes through the boundary FMM tree (V_GO^T).  Accurate to the FMM
  * truncation against the exact transpose.  zb_dev, rb_dev: [n_rhs][ny][nx] FP64 device,
  * distinct.  Single-layer form only (_UNSUPPORTED after fmmpc_set_bem_form(DOUBLE_LAYER)).
@@ -250,9 +254,9 @@ int fmmpc_set_operator(fmmpc_handle *h, int32_t op, const double *a_dev);
 /* on = 1 (the default): fmmpc_apply records its kernels once per distinct (r, z, n_rhs)
  * into a CUDA graph on an internal stream and replays it (ordered after and before the
  * handle's stream with events); on = 0: launches the kernels one by one.  Either way,
- * with stage timing off, the full apply runs the tensor-core near field, the volume M2L
- * and the near-boundary correction on three further internal streams, forked and joined
- * with events, so they overlap the boundary chain; the result is the same bit for bit as
+ * with stage timing off, the full apply of every form, with boundary data and transposed too,
+ * runs the near field, the volume M2L and the near-boundary correction on three further internal
+ * streams, forked and joined with events, so they overlap the boundary chain; the result is the same bit for bit as
  * with the stages in order on one stream.  fmmpc_solve follows its own opts.use_graphs
  * instead.  Up to 64 graphs are kept per handle. */
 int fmmpc_set_graphs(fmmpc_handle *h, int32_t on);
@@ -264,11 +268,10 @@ int fmmpc_set_graphs(fmmpc_handle *h, int32_t on);
  * rest of the apply runs without event records; 0 turns recording off.
  * fmmpc_get_timing synchronises the stream and writes the durations in milliseconds of
  * the stages of the last apply into ms[0 .. min(cap, count)), *count = 11 stages:
- *  0 weight image, 1 P2M + M2M (Sec. 5.3 items 1-2), 2 collocation pass (M2L to boundary
+ *  0 weight image and strips, 1 P2M + M2M (Sec. 5.3 items 1-2), 2 collocation pass (M2L to boundary
  *  cells, local expansions and near field at the collocation points), 3 BEM solve (FP64,
- *  or two-word FP32 in the single-precision forms), 4 boundary multipoles, 5 M2L (item 3;
- *  with the tensor-core M2L its volume part only), 6 boundary-source M2L with the
- *  tensor-core M2L (kept apart, added by the downward pass), 7 L2L (item 4; only for trees
+ *  or two-word FP32 in the single-precision forms), 4 boundary multipoles, 5 M2L (item 3),
+ *  its volume part, 6 boundary-source M2L (kept apart, added by the downward pass), 7 L2L (item 4; only for trees
  *  of fewer than three levels, else part of stage 10), 8 near-boundary element integrals,
  *  9 P2P near field (item 5, Eq. e:volume_integral), 10 L2L + L2P + the final sum.
  * A stage that did not run reports 0.  Errors: _INVALID if timing is off. */

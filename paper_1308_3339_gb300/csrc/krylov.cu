@@ -1103,11 +1103,11 @@ int solve_batched(std::vector<fmmpc_handle *> &hs, const double *const *f, const
 
 // ====================================================================== graph-resident solves
 // The whole Krylov solve as one CUDA graph: set-up nodes, then a conditional WHILE node whose
-// body is one Arnoldi step (FGMRES/GMRES) or one CG iteration, and final nodes that recompute
-// the true residual.  The Hessenberg column, the Givens rotations, the residual estimate, the
+// body is one CG iteration, and the true residual; or whose body is one cycle of FGMRES/GMRES,
+// a second WHILE node over its Arnoldi steps and the cycle's end.  The Hessenberg column, the Givens rotations, the residual estimate, the
 // convergence decision and (at the end of a cycle) the back substitution run on the device
-// in one small kernel, which also sets the conditions of the loop and of the end-of-cycle
-// IF node, so no step waits for the host: the host launches the graph once and reads the
+// in the last block of the step's last sweep, which also sets the loop's condition, so no step waits
+// for the host: the host launches the graph once and reads the
 // report when it has finished.  Orthogonalisation is classical Gram-Schmidt applied twice
 // (CGS2) at every step.  The loop is bounded: every pass counts one preconditioner
 // application and the loop stops at maxit, on a NaN, or when every right-hand side meets
