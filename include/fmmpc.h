@@ -197,7 +197,8 @@ int fmmpc_spmv(fmmpc_handle *h, const double *x_dev, double *y_dev, int32_t n_rh
  * f_dev [n_rhs][ny][nx]; g_dev [n_rhs][4n] or NULL for g = 0; u_dev holds the initial
  * iterate on entry (zeros for the paper's setting) and the solution on exit.  info may
  * be NULL.  Returns FMMPC_OK when every right-hand side met rtol, FMMPC_ERR_NOT_CONVERGED
- * when one stopped at maxit (u_dev still holds the last iterate), FMMPC_ERR_NAN. */
+ * when one stopped at maxit, or CG where the true residual no longer falls (u_dev still holds
+ * the last iterate), FMMPC_ERR_NAN. */
 int fmmpc_solve(fmmpc_handle *h, const double *f_dev, const double *g_dev, double *u_dev,
                 int32_t n_rhs, const fmmpc_solve_opts *opts, fmmpc_solve_info *info);
 

@@ -333,7 +333,7 @@ int fmmpc_solve(fmmpc_handle *h, const double *f_dev, const double *g_dev, doubl
     fmmpc_solve_info tmp{};
     int st = solve(*h, f_dev, g_dev, u_dev, n_rhs, *opts, tmp);
     if (info) *info = tmp;
-    if (st != FMMPC_OK) h->err = (st == FMMPC_ERR_NOT_CONVERGED) ? "solve: not converged within maxit"
+    if (st != FMMPC_OK) h->err = (st == FMMPC_ERR_NOT_CONVERGED) ? "solve: not converged within maxit or the attainable residual"
                                                                   : "solve: NaN or Inf in a residual";
     return st;
   });

@@ -783,12 +783,9 @@ int pcg(Ctx &c, int maxit, double rtol, const double *b, double *x, fmmpc_solve_
   const int nr = c.nrhs;
   double *r = K.r, *z = K.w, *p = K.V, *q = K.t;
   double *hy = K.hbuf + (size_t)nr * MAXJ * 2;
-  std::vector<double> bn, rn;
+  std::vector<double> bn, rn, rel(nr, INFINITY);
   norms(c, b, bn);
   for (double &v : bn) if (v == 0.0) v = 1.0;
-  residual(c, b, x, r);
-  precond(c, r, z);
-  FMMPC_CUDA(cudaMemcpyAsync(p, z, sizeof(double) * NR, cudaMemcpyDeviceToDevice, c.s));
   auto dotv = [&](const double *a, const double *bb, std::vector<double> &out) {
     mdot(c, 1, a, 0, bb, K.dots, nullptr);
     to_host(c, K.dots, (size_t)nr * MAXJ);
@@ -796,53 +793,63 @@ int pcg(Ctx &c, int maxit, double rtol, const double *b, double *x, fmmpc_solve_
     for (int i = 0; i < nr; ++i) out[i] = K.hbuf[i * MAXJ];
   };
   std::vector<double> rz, pq, rz2;
-  dotv(r, z, rz);
-  norms(c, r, rn);
   std::vector<int> done(nr, 0), its(nr, 0);
   int it = 0;
-  bool all = true;
-  for (int i = 0; i < nr; ++i) { done[i] = rn[i] / bn[i] <= rtol; all = all && done[i]; }
-  while (!all && it < maxit) {
-    spmv5(H, p, q, nr);
-    dotv(p, q, pq);
-    for (int i = 0; i < nr; ++i) hy[i] = (done[i] || pq[i] == 0.0) ? 0.0 : rz[i] / pq[i];
-    FMMPC_CUDA(cudaMemcpyAsync(K.scal, hy, sizeof(double) * nr, cudaMemcpyHostToDevice, c.s));
-    k_cg_xr<<<nblk(NR), 256, 0, c.s>>>(N, nr, K.scal, p, q, x, r);
-    FMMPC_LAUNCH_CHECK();
-    ++it;
+  bool all = false;
+  for (;;) {
+    // the true residual: the recurrence's drifts from it, so a right-hand side that ended above rtol
+    // goes on from here, while that of some unfinished one still falls
+    residual(c, b, x, r);
     norms(c, r, rn);
+    bool falls = false;
     all = true;
     for (int i = 0; i < nr; ++i) {
-      if (!std::isfinite(rn[i])) return FMMPC_ERR_NAN;
-      if (!done[i]) its[i] = it;
-      done[i] = done[i] || rn[i] / bn[i] <= rtol;
+      const double v = rn[i] / bn[i];
+      if (!std::isfinite(v)) return FMMPC_ERR_NAN;
+      done[i] = v <= rtol;
       all = all && done[i];
+      falls = falls || (!done[i] && v < rel[i]);
+      rel[i] = v;
     }
-    if (all) break;
+    if (all || !falls || it >= maxit) break;
     precond(c, r, z);
-    dotv(r, z, rz2);
-    for (int i = 0; i < nr; ++i) {
-      hy[i] = (done[i] || rz[i] == 0.0) ? 0.0 : rz2[i] / rz[i];
-      rz[i] = rz2[i];
+    FMMPC_CUDA(cudaMemcpyAsync(p, z, sizeof(double) * NR, cudaMemcpyDeviceToDevice, c.s));
+    dotv(r, z, rz);
+    for (;;) {
+      spmv5(H, p, q, nr);
+      dotv(p, q, pq);
+      for (int i = 0; i < nr; ++i) hy[i] = (done[i] || pq[i] == 0.0) ? 0.0 : rz[i] / pq[i];
+      FMMPC_CUDA(cudaMemcpyAsync(K.scal, hy, sizeof(double) * nr, cudaMemcpyHostToDevice, c.s));
+      k_cg_xr<<<nblk(NR), 256, 0, c.s>>>(N, nr, K.scal, p, q, x, r);
+      FMMPC_LAUNCH_CHECK();
+      ++it;
+      norms(c, r, rn);
+      all = true;
+      for (int i = 0; i < nr; ++i) {
+        if (!std::isfinite(rn[i])) return FMMPC_ERR_NAN;
+        if (!done[i]) its[i] = it;
+        done[i] = done[i] || rn[i] / bn[i] <= rtol;
+        all = all && done[i];
+      }
+      if (all || it >= maxit) break;
+      precond(c, r, z);
+      dotv(r, z, rz2);
+      for (int i = 0; i < nr; ++i) {
+        hy[i] = (done[i] || rz[i] == 0.0) ? 0.0 : rz2[i] / rz[i];
+        rz[i] = rz2[i];
+      }
+      FMMPC_CUDA(cudaMemcpyAsync(K.scal, hy, sizeof(double) * nr, cudaMemcpyHostToDevice, c.s));
+      k_cg_p<<<nblk(NR), 256, 0, c.s>>>(N, nr, K.scal, z, p);
+      FMMPC_LAUNCH_CHECK();
     }
-    FMMPC_CUDA(cudaMemcpyAsync(K.scal, hy, sizeof(double) * nr, cudaMemcpyHostToDevice, c.s));
-    k_cg_p<<<nblk(NR), 256, 0, c.s>>>(N, nr, K.scal, z, p);
-    FMMPC_LAUNCH_CHECK();
   }
-  residual(c, b, x, r);
-  norms(c, r, rn);
-  double worst = 0.0;
-  int status = FMMPC_OK;
-  for (int i = 0; i < nr; ++i) {
-    const double rel = rn[i] / bn[i];
-    if (!std::isfinite(rel)) status = FMMPC_ERR_NAN;
-    worst = std::max(worst, rel);
-  }
-  if (status == FMMPC_OK && worst > rtol) status = FMMPC_ERR_NOT_CONVERGED;
   info.iters = 0;
-  for (int i = 0; i < nr; ++i) info.iters = std::max(info.iters, its[i]);
-  info.rel_res = worst;
-  return status;
+  info.rel_res = 0.0;
+  for (int i = 0; i < nr; ++i) {
+    info.iters = std::max(info.iters, its[i]);
+    info.rel_res = std::max(info.rel_res, rel[i]);
+  }
+  return all ? FMMPC_OK : FMMPC_ERR_NOT_CONVERGED;
 }
 
 }  // namespace
@@ -1103,8 +1110,8 @@ int solve_batched(std::vector<fmmpc_handle *> &hs, const double *const *f, const
 
 // ====================================================================== graph-resident solves
 // The whole Krylov solve as one CUDA graph: set-up nodes, then a conditional WHILE node whose
-// body is one CG iteration, and the true residual; or whose body is one cycle of FGMRES/GMRES,
-// a second WHILE node over its Arnoldi steps and the cycle's end.  The Hessenberg column, the Givens rotations, the residual estimate, the
+// body is one cycle: a second WHILE node over Arnoldi steps (FGMRES/GMRES) or CG iterations, and the
+// cycle's end with the true residual.  The Hessenberg column, the Givens rotations, the residual estimate, the
 // convergence decision and (at the end of a cycle) the back substitution run on the device
 // in the last block of the step's last sweep, which also sets the loop's condition, so no step waits
 // for the host: the host launches the graph once and reads the
@@ -1335,25 +1342,34 @@ __device__ __forceinline__ void gm_restart(int *__restrict__ ctl, GmState st, in
   }
 }
 
-// Start of CG from the true residual: done flags and the loop's condition.
-__device__ __forceinline__ void cg_start(int *__restrict__ ctl, GmState st, int nrhs, const double *__restrict__ dots,
+// CG's true residual (|r|^2 in dots[rhs][0]), at its start and whenever the recurrence's residual met
+// rtol or maxit: the relative residual of the report, done flags, and the condition of the loop
+// over the runs of iterations.  The recurrence's residual drifts from the true one (2e-11 of |b| at
+// 1024^2), so a right-hand side can end just above rtol; it then goes on from the true residual,
+// while that of some unfinished right-hand side still falls (st.rel holds the last one).
+__device__ __forceinline__ void cg_check(int *__restrict__ ctl, GmState st, int nrhs, const double *__restrict__ dots,
                                          cudaGraphConditionalHandle loop) {
-  __shared__ int s_all, s_nan;
-  if (threadIdx.x == 0) { s_all = 1; s_nan = 0; }
+  __shared__ int s_all, s_nan, s_falls;
+  if (threadIdx.x == 0) { s_all = 1; s_nan = 0; s_falls = 0; }
   __syncthreads();
   for (int r = threadIdx.x; r < nrhs; r += blockDim.x) {
     const double sq = __ldcg(dots + r * MAXJ);
-    if (!isfinite(sq)) atomicOr(&s_nan, 1);  // fmax(0, NaN) would hide it
-    const int d = sqrt(fmax(0.0, sq)) / __ldcg(st.bn + r) <= st.rtol[0];
+    if (!isfinite(sq)) atomicOr(&s_nan, 1);
+    const double rel = sqrt(sq) / __ldcg(st.bn + r);  // a NaN stays one
+    const int d = rel <= st.rtol[0];
+    if (!d) {
+      atomicAnd(&s_all, 0);
+      if (rel < __ldcg(st.rel + r)) atomicOr(&s_falls, 1);
+    }
     st.done[r] = d;
-    if (!d) atomicAnd(&s_all, 0);
+    st.rel[r] = rel;
   }
   __syncthreads();
   if (threadIdx.x == 0) {
     const int nan = ctl[KC_NAN] | s_nan;
     ctl[KC_DONE] = s_all;
     ctl[KC_NAN] = nan;
-    const int cont = (!s_all && !nan && ctl[KC_IT] < ctl[KC_MAXIT]) ? 1 : 0;
+    const int cont = (!s_all && s_falls && !nan && ctl[KC_IT] < ctl[KC_MAXIT]) ? 1 : 0;
     ctl[KC_CONT] = cont;
     cudaGraphSetConditional(loop, (unsigned)cont);
   }
@@ -1572,6 +1588,7 @@ __global__ void __launch_bounds__(RED_THREADS) k_gbnorm(int *__restrict__ ctl, i
   st.bn[rhs] = nb > 0.0 ? nb : 1.0;
   st.iters[rhs] = 0;
   st.done[rhs] = 0;
+  st.rel[rhs] = INFINITY;  // CG's first residual falls from here
   if (rhs == 0) {
     ctl[KC_J] = ctl[KC_IT] = ctl[KC_CYC] = ctl[KC_DONE] = ctl[KC_NAN] = ctl[KC_JCNT] = 0;
   }
@@ -1579,8 +1596,8 @@ __global__ void __launch_bounds__(RED_THREADS) k_gbnorm(int *__restrict__ ctl, i
 
 // r = b - A x with |r|^2 in dots[rhs][0]: one pass for the residual checks of the graph solves
 // (operator, subtraction and norm were three launches, 36 us at 1024^2); the last right-hand side to
-// finish then takes the scalar step that follows: a cycle's start, CG's start, or the final report.
-enum class AfterResid { CYCLE, CG_START, REPORT };
+// finish then takes the scalar step that follows: a cycle's start of (F)GMRES, or CG's check.
+enum class AfterResid { CYCLE, CG };
 template <AfterResid WHAT>
 __global__ void __launch_bounds__(RED_THREADS) k_gresid(int *__restrict__ ctl, OpDev o, int64_t N, int nrhs, GmState st,
                                                       const double *__restrict__ b, const double *__restrict__ x,
@@ -1601,22 +1618,25 @@ __global__ void __launch_bounds__(RED_THREADS) k_gresid(int *__restrict__ ctl, O
   }
   double tot;
   if (!block_partial_last(acc, part, rhs, cnt, tot)) return;
-  if constexpr (WHAT == AfterResid::REPORT) {
-    if (threadIdx.x == 0) st.rel[rhs] = sqrt(fmax(0.0, tot)) / st.bn[rhs];
-  } else {
-    __shared__ int s_fin;
-    if (threadIdx.x == 0) {
-      dots[rhs * MAXJ] = tot;
-      __threadfence();
-      s_fin = atomicAdd(cnt + nrhs, 1) == nrhs - 1;
-      if (s_fin) cnt[nrhs] = 0;
-    }
-    __syncthreads();
-    if (!s_fin) return;
+  __shared__ int s_fin;
+  if (threadIdx.x == 0) {
+    dots[rhs * MAXJ] = tot;
     __threadfence();
-    if constexpr (WHAT == AfterResid::CYCLE) gm_restart(ctl, st, nrhs, dots, loop);
-    else cg_start(ctl, st, nrhs, dots, loop);
+    s_fin = atomicAdd(cnt + nrhs, 1) == nrhs - 1;
+    if (s_fin) cnt[nrhs] = 0;
   }
+  __syncthreads();
+  if (!s_fin) return;
+  __threadfence();
+  if constexpr (WHAT == AfterResid::CYCLE) gm_restart(ctl, st, nrhs, dots, loop);
+  else cg_check(ctl, st, nrhs, dots, loop);
+}
+
+// Start of a run of CG iterations from the true residual: <r, z>_old = 0 makes its first beta 0, so that
+// p = z; opens the loop over the iterations.
+__global__ void k_cg_begin(int nrhs, double *__restrict__ rz_old, cudaGraphConditionalHandle steps) {
+  for (int r = threadIdx.x; r < nrhs; r += blockDim.x) rz_old[r * MAXJ] = 0.0;
+  if (threadIdx.x == 0) cudaGraphSetConditional(steps, 1u);
 }
 
 // q = A p and <p, q>; then alpha = <r, z> / <p, q> (0 for a finished right-hand side)
@@ -1643,12 +1663,12 @@ __global__ void __launch_bounds__(RED_THREADS) k_cgf_apdot(OpDev o, int64_t N, G
 
 // x += alpha p, r -= alpha q and |r|^2; the last right-hand side to finish then does the
 // convergence test of every right-hand side (iteration counts, done flags, NaN) and sets
-// the condition of the solve's WHILE loop: some right-hand side still runs, below maxit
+// the condition of the loop over the iterations: some right-hand side still runs, below maxit
 __global__ void __launch_bounds__(RED_THREADS) k_cgf_xr(int *__restrict__ ctl, int64_t N, int nrhs, GmState st,
                                                       const double *__restrict__ p, const double *__restrict__ q,
                                                       double *__restrict__ x, double *__restrict__ r,
                                                       double *__restrict__ part, int *cnt, double *__restrict__ dots,
-                                                      cudaGraphConditionalHandle loop) {
+                                                      cudaGraphConditionalHandle steps) {
   __shared__ int s_fin, s_all, s_nan;
   const int rhs = blockIdx.y;
   const double al = st.sc[rhs];
@@ -1697,7 +1717,7 @@ __global__ void __launch_bounds__(RED_THREADS) k_cgf_xr(int *__restrict__ ctl, i
     ctl[KC_NAN] |= s_nan;
     const int more = (!s_all && !s_nan && it < ctl[KC_MAXIT]) ? 1 : 0;
     ctl[KC_CONT] = more;
-    cudaGraphSetConditional(loop, (unsigned)more);
+    cudaGraphSetConditional(steps, (unsigned)more);
   }
 }
 
@@ -1773,9 +1793,9 @@ GmState gm_state(KrylovWs &K) {
   return GmState{K.g_H, K.g_cs, K.g_sn, K.g_g, K.g_bn, K.g_rel, K.g_sc, K.g_rtol, K.g_done, K.g_iters};
 }
 
-// Builds one problem's chain [set-up] -> WHILE [step] -> [final] (CG), or [set-up] -> WHILE cycle
-// [V_0 -> WHILE [step] -> cycle end] ((F)GMRES: the last cycle's end is the final residual) into
-// graph G.  Every condition is set by the last block of the kernel that decides it: an IF node for the
+// Builds one problem's chain [set-up] -> WHILE cycle [start -> WHILE [step] -> cycle end] into graph G.  The
+// steps of a cycle are Arnoldi steps, or CG's iterations; its end takes the true residual, the last
+// one the final one.  Every condition is set by the last block of the kernel that decides it: an IF node for the
 // cycle's end and a kernel for the condition in every pass were 2.5 to 10 us of it (64^2 FGMRES, with
 // the copies of solve_graphed, 983 -> 916 us).  Solves A u = b for the handle's internal vectors: b is folded from K.fin
 // (and K.gin), the iterate is K.x.
@@ -1807,6 +1827,7 @@ void build_chain(fmmpc_handle &H, cudaGraph_t G, int method, int m, int nrhs, bo
     FMMPC_LAUNCH_CHECK();
   };
   using Cycle = std::integral_constant<AfterResid, AfterResid::CYCLE>;
+  using Check = std::integral_constant<AfterResid, AfterResid::CG>;
   // ---- set-up
   const std::vector<cudaGraphNode_t> none;
   auto f_init = capture_into(H, cs, G, none, [&] {
@@ -1815,48 +1836,49 @@ void build_chain(fmmpc_handle &H, cudaGraph_t G, int method, int m, int nrhs, bo
     k_gbnorm<<<rgrid, rth, 0, H.stream>>>(ctl, N, st, K.b, K.part, K.g_cnt);
     FMMPC_LAUNCH_CHECK();
     if (method == FMMPC_CG) {
-      // the loop body starts with z = P^{-1} r; p = 0 and <r, z>_old = 0 make its first
-      // beta 0, so that p = z
-      residual(std::integral_constant<AfterResid, AfterResid::CG_START>{});
-      FMMPC_CUDA(cudaMemsetAsync(K.V, 0, sizeof(double) * NR, H.stream));
-      FMMPC_CUDA(cudaMemsetAsync(K.dots + (size_t)nrhs * MAXJ, 0, sizeof(double) * nrhs * MAXJ, H.stream));
+      residual(Check{});
+      FMMPC_CUDA(cudaMemsetAsync(K.V, 0, sizeof(double) * NR, H.stream));  // p, which the first beta = 0 multiplies
     } else {
       residual(Cycle{});
     }
   });
   cudaGraph_t body = nullptr;
-  cudaGraphNode_t n_loop = add_conditional(G, f_init, hloop, cudaGraphCondTypeWhile, &body);
+  add_conditional(G, f_init, hloop, cudaGraphCondTypeWhile, &body);
+  cudaGraphConditionalHandle hsteps;
+  FMMPC_CUDA(cudaGraphConditionalHandleCreate(&hsteps, body, 0, 0));
+  cudaGraph_t step = nullptr;
   double *hsum = K.dots + (size_t)nrhs * MAXJ, *wsq = K.scal + (size_t)nrhs * MAXJ;
   if (method == FMMPC_CG) {
     // p in V_0, q in t, z in w; <r, z> of the last iteration in the second dots block
     double *p = K.V, *q = K.t, *z = K.w, *rz_old = K.dots + (size_t)nrhs * MAXJ;
     double *pq = K.dots + (size_t)2 * nrhs * MAXJ;
+    auto f_begin = capture_into(H, cs, body, none, [&] {
+      k_cg_begin<<<1, 64, 0, H.stream>>>(nrhs, rz_old, hsteps);
+      FMMPC_LAUNCH_CHECK();
+    });
+    cudaGraphNode_t n_steps = add_conditional(body, f_begin, hsteps, cudaGraphCondTypeWhile, &step);
     // one iteration, rotated so that the convergence test ends it and sets the loop's own
     // condition (no IF node): z = P^{-1} r, beta, p = z + beta p, q = A p with alpha, then
     // x, r and the test
-    capture_into(H, cs, body, none, [&] {
+    capture_into(H, cs, step, none, [&] {
       c.s = H.stream;
       precond(K.r, z, K.zin);
       k_cgf_rz<<<rgrid, rth, 0, H.stream>>>(N, st, K.r, z, K.part, K.g_cnt, rz_old);
       k_cg_p<<<nblk(NR), 256, 0, H.stream>>>(N, nrhs, K.g_sc, z, p);
       k_cgf_apdot<<<rgrid, rth, 0, H.stream>>>(od, N, st, p, q, K.part, K.g_cnt, pq, rz_old);
       k_cgf_xr<<<rgrid, rth, 0, H.stream>>>(ctl, N, nrhs, st, p, q, K.x, K.r, K.part, K.g_cnt, K.dots,
-                                                     hloop);
+                                                     hsteps);
       FMMPC_LAUNCH_CHECK();
     });
-    // the recurrence's residual drifts from the true one
-    capture_into(H, cs, G, {n_loop}, [&] {
+    capture_into(H, cs, body, {n_steps}, [&] {
       c.s = H.stream;
-      residual(std::integral_constant<AfterResid, AfterResid::REPORT>{});
+      residual(Check{});
     });
   } else {
-    cudaGraphConditionalHandle hsteps;
-    FMMPC_CUDA(cudaGraphConditionalHandleCreate(&hsteps, body, 0, 0));
     auto f_begin = capture_into(H, cs, body, none, [&] {
       k_gscale_col<true><<<nblk(NR), 256, 0, H.stream>>>(ctl, N, nrhs, K.g_sc, K.r, K.V, vs, K.t, hsteps);
       FMMPC_LAUNCH_CHECK();
     });
-    cudaGraph_t step = nullptr;
     cudaGraphNode_t n_steps = add_conditional(body, f_begin, hsteps, cudaGraphCondTypeWhile, &step);
     capture_into(H, cs, step, none, [&] {
       c.s = H.stream;

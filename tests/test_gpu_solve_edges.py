@@ -1,0 +1,64 @@
+"""Solves at the edge of what they report: CG asked for a residual between the recurrence's and
+the true one."""
+import numpy as np
+import pytest
+
+import synth_inputs as S
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _cuda():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+
+
+def dev(a):
+    return torch.tensor(np.asarray(a), dtype=torch.float64, device="cuda").contiguous()
+
+
+def true_residual(P, f, u):
+    k = f.shape[0]
+    return ((f - P.spmv(u)).reshape(k, -1).norm(dim=1) / f.reshape(k, -1).norm(dim=1)).max().item()
+
+
+@pytest.mark.parametrize("use_graphs", [0, 1, 2])
+@pytest.mark.parametrize("n,prec,nrhs", [(256, "mixed_bf16", 3), (512, "fp32", 1)])
+def test_cg_meets_a_tolerance_just_below_its_true_residual(n, prec, nrhs, use_graphs):
+    # CG stops by its recurrence's residual, which drifts below the true one.  A tolerance just under the
+    # true residual of k iterations lies between the two: the solve has to go on from the true residual
+    # until it is met, not to fail with maxit far away.
+    from paper_1308_3339_gb300 import FmmPreconditioner
+    f = dev(np.stack([S.gaussian_mixture(n, 20 + k) for k in range(nrhs)]))
+    P = FmmPreconditioner(n, p=10, precision=prec, n_rhs=nrhs)
+    asked = 0
+    for k in range(6, 16):
+        _, part = P.solve(f, method="cg", maxit=k, rtol=1e-15, use_graphs=use_graphs, raise_on_fail=False)
+        if not 1e-11 < part["rel_res"] < 1e-8:
+            continue
+        rtol = part["rel_res"] * (1 - 1e-6)
+        u, info = P.solve(f, method="cg", rtol=rtol, use_graphs=use_graphs, raise_on_fail=False)
+        print(f"CG n={n} {prec} after {k}: {part['rel_res']:.6e}; asked just below: {info}", flush=True)
+        assert info["status"] == 0 and info["rel_res"] <= rtol and info["iters"] <= k + 3
+        assert true_residual(P, f, u) <= rtol * (1 + 1e-5)
+        asked += 1
+    assert asked >= 2
+    P.close()
+
+
+@pytest.mark.parametrize("use_graphs", [0, 2])
+def test_cg_stops_where_the_true_residual_no_longer_falls(use_graphs):
+    # below the attainable residual: reported as not converged, long before maxit, with the true residual
+    from paper_1308_3339_gb300 import FmmPreconditioner
+    n = 128
+    f = dev(np.stack([S.gaussian_mixture(n, 30), S.random_field(n, 31)]))
+    P = FmmPreconditioner(n, p=10, precision="fp32", n_rhs=2)
+    u, info = P.solve(f, method="cg", maxit=5000, rtol=1e-30, use_graphs=use_graphs, raise_on_fail=False)
+    assert info["status"] == -4 and info["iters"] < 5000, info
+    # P^-1's FP32 error does not enter the attainable residual, eps |A| |u| / |f| does
+    size = (u.reshape(2, -1).norm(dim=1) / f.reshape(2, -1).norm(dim=1)).max().item()
+    limit = 50 * 2.2e-16 * 8 * (n + 1) ** 2 * size
+    assert info["rel_res"] < limit and abs(true_residual(P, f, u) - info["rel_res"]) < limit, (info, limit)
+    P.close()
