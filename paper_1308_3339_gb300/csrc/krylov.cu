@@ -627,13 +627,14 @@ void residual(Ctx &c, const double *b, const double *x, double *r) {
   FMMPC_LAUNCH_CHECK();
 }
 
-// per-rhs norms of v (length nrhs on host, in out)
+// per-rhs norms of v (length nrhs on host, in out).  Sums of squares are never negative, so here and in
+// every norm below the root is taken as it is: a clamp at zero would turn a NaN into a zero residual.
 void norms(Ctx &c, const double *v, std::vector<double> &out) {
   double *d = c.H.kw.dots;
   mdot(c, 1, v, 0, v, d, nullptr);  // with vs = 0 each rhs dots its own slice with itself
   to_host(c, d, (size_t)c.nrhs * MAXJ);
   out.resize(c.nrhs);
-  for (int r = 0; r < c.nrhs; ++r) out[r] = std::sqrt(std::max(0.0, c.H.kw.hbuf[r * MAXJ]));
+  for (int r = 0; r < c.nrhs; ++r) out[r] = std::sqrt(c.H.kw.hbuf[r * MAXJ]);
 }
 
 int gmres(Ctx &c, bool flexible, int m, int maxit, double rtol, const double *b, double *x,
@@ -703,7 +704,7 @@ int gmres(Ctx &c, bool flexible, int m, int maxit, double rtol, const double *b,
       }
       for (int r = 0; r < nr; ++r) {
         for (int i = 0; i <= j; ++i) hcol[(size_t)r * MAXJ + i] = hb[(size_t)r * MAXJ + i];
-        hn[r] = std::sqrt(std::max(0.0, hb[(size_t)2 * nr * MAXJ + (size_t)r * MAXJ]));
+        hn[r] = std::sqrt(hb[(size_t)2 * nr * MAXJ + (size_t)r * MAXJ]);
       }
       ++it;
       bool conv_all = true;
@@ -965,7 +966,7 @@ int solve_batched(std::vector<fmmpc_handle *> &hs, const double *const *f, const
   }
   sync_all(hs);
   for (int p = 0; p < np; ++p) {
-    st[p].bn = std::sqrt(std::max(0.0, hs[p]->kw.hbuf[0]));
+    st[p].bn = std::sqrt(hs[p]->kw.hbuf[0]);
     if (st[p].bn == 0.0) st[p].bn = 1.0;
   }
   for (;;) {
@@ -984,7 +985,7 @@ int solve_batched(std::vector<fmmpc_handle *> &hs, const double *const *f, const
       s.in_cycle = false;
       if (s.done) continue;
       fmmpc_handle &H = *hs[p];
-      s.beta = std::sqrt(std::max(0.0, H.kw.hbuf[0]));
+      s.beta = std::sqrt(H.kw.hbuf[0]);
       if (!std::isfinite(s.beta)) { s.done = true; s.status = FMMPC_ERR_NAN; continue; }
       if (s.beta / s.bn <= o.rtol) { s.done = true; continue; }
       if (s.iters >= o.maxit) { s.done = true; s.status = FMMPC_ERR_NOT_CONVERGED; continue; }
@@ -1030,7 +1031,7 @@ int solve_batched(std::vector<fmmpc_handle *> &hs, const double *const *f, const
         if (!s.in_cycle) continue;
         fmmpc_handle &H = *hs[p];
         const int j = s.j;
-        const double hn = std::sqrt(std::max(0.0, H.kw.hbuf[0]));
+        const double hn = std::sqrt(H.kw.hbuf[0]);
         double *Hr = s.Hm.data();
         for (int i = 0; i <= j; ++i) Hr[i * m + j] = H.kw.hbuf[MAXJ + i];
         Hr[(j + 1) * m + j] = hn;
@@ -1089,7 +1090,7 @@ int solve_batched(std::vector<fmmpc_handle *> &hs, const double *const *f, const
   const double ms = std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count();
   int worst = FMMPC_OK;
   for (int p = 0; p < np; ++p) {
-    const double rel = std::sqrt(std::max(0.0, hs[p]->kw.hbuf[0])) / st[p].bn;
+    const double rel = std::sqrt(hs[p]->kw.hbuf[0]) / st[p].bn;
     int status = st[p].status;
     if (!std::isfinite(rel)) status = FMMPC_ERR_NAN;
     else if (status == FMMPC_OK && rel > o.rtol) status = FMMPC_ERR_NOT_CONVERGED;
@@ -1321,7 +1322,7 @@ __device__ __forceinline__ void gm_restart(int *__restrict__ ctl, GmState st, in
   __syncthreads();
   const double rtol = st.rtol[0];
   for (int r = threadIdx.x; r < nrhs; r += blockDim.x) {
-    const double sq = __ldcg(dots + r * MAXJ), beta = sqrt(fmax(0.0, sq)), rel = beta / __ldcg(st.bn + r);
+    const double sq = __ldcg(dots + r * MAXJ), beta = sqrt(sq), rel = beta / __ldcg(st.bn + r);
     if (!isfinite(beta) || !isfinite(sq)) atomicOr(&s_nan, 1);
     const int d = (rel <= rtol) ? 1 : 0;
     st.rel[r] = rel;
@@ -1403,7 +1404,7 @@ __device__ __forceinline__ void gtail_run(int *__restrict__ ctl, GmState st, int
       cv[q] = i < j ? cs[i] : 0.0;
       sv[q] = i < j ? sn[i] : 0.0;
     }
-    const double hn = sqrt(fmax(0.0, __ldcg(wsq + r * MAXJ)));
+    const double hn = sqrt(__ldcg(wsq + r * MAXJ));
     auto pick = [&](const double(&v)[2], int i) { return __shfl_sync(0xffffffffu, i < 32 ? v[0] : v[1], i & 31); };
     double a = pick(hv, 0);
     for (int i = 0; i < j; ++i) {
@@ -1584,7 +1585,7 @@ __global__ void __launch_bounds__(RED_THREADS) k_gbnorm(int *__restrict__ ctl, i
   }
   double tot;
   if (!block_partial_last(acc, part, rhs, cnt, tot) || threadIdx.x != 0) return;
-  const double nb = sqrt(fmax(0.0, tot));
+  const double nb = sqrt(tot);
   st.bn[rhs] = nb > 0.0 ? nb : 1.0;
   st.iters[rhs] = 0;
   st.done[rhs] = 0;
@@ -1703,7 +1704,7 @@ __global__ void __launch_bounds__(RED_THREADS) k_cgf_xr(int *__restrict__ ctl, i
   __threadfence();
   const int it = ctl[KC_IT] + 1;
   for (int rr = threadIdx.x; rr < nrhs; rr += blockDim.x) {
-    const double rn = sqrt(fmax(0.0, __ldcg(dots + rr * MAXJ)));
+    const double rn = sqrt(__ldcg(dots + rr * MAXJ));
     if (!isfinite(rn)) atomicOr(&s_nan, 1);
     if (!st.done[rr]) st.iters[rr] = it;
     const int d = st.done[rr] || rn / st.bn[rr] <= st.rtol[0];

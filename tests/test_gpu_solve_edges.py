@@ -1,5 +1,5 @@
 """Solves at the edge of what they report: CG asked for a residual between the recurrence's and
-the true one."""
+the true one, and NaNs, met at the start or made on the way, which are never convergence."""
 import numpy as np
 import pytest
 
@@ -62,3 +62,38 @@ def test_cg_stops_where_the_true_residual_no_longer_falls(use_graphs):
     limit = 50 * 2.2e-16 * 8 * (n + 1) ** 2 * size
     assert info["rel_res"] < limit and abs(true_residual(P, f, u) - info["rel_res"]) < limit, (info, limit)
     P.close()
+
+
+@pytest.mark.parametrize("method,kind", [("cg", "nan in f"), ("gmres", "nan in f"), ("fgmres", "nan in f"),
+                                         ("cg", "overflow on the way")])
+@pytest.mark.parametrize("use_graphs", [0, 1, 2])
+def test_nan_is_not_convergence(method, kind, use_graphs):
+    # a NaN in one right-hand side, or a finite one whose weights h^2 r pass the FP32 range of the
+    # preconditioner (CG's are not normalised), so that P^-1 r is not finite: the solve reports it
+    # whatever drives the loop
+    from paper_1308_3339_gb300 import FmmPreconditioner, FmmpcError
+    n = 64
+    f = np.stack([S.gaussian_mixture(n, 7), S.gaussian_mixture(n, 8)])
+    if kind == "nan in f":
+        f[1, 100] = np.nan
+    else:
+        f[1] *= 1e45
+    P = FmmPreconditioner(n, p=8, precision="fp32", n_rhs=2)
+    with pytest.raises(FmmpcError) as e:
+        P.solve(dev(f), method=method, rtol=1e-8, use_graphs=use_graphs)
+    assert e.value.code == -5, e.value
+    _, info = P.solve(dev(f[:1]), method=method, rtol=1e-8, use_graphs=use_graphs)  # the handle works on
+    assert info["status"] == 0
+    P.close()
+
+
+@pytest.mark.parametrize("use_graphs", [0, 1, 2])
+def test_nan_is_not_convergence_in_a_batch(use_graphs):
+    from paper_1308_3339_gb300 import FmmBatch, FmmpcError
+    B = FmmBatch([64, 32], p=8, precision="fp32")
+    f = [dev(S.gaussian_mixture(64, 1)), dev(S.gaussian_mixture(32, 2))]
+    f[1][100] = float("nan")
+    with pytest.raises(FmmpcError) as e:
+        B.solve(f, use_graphs=use_graphs)
+    assert e.value.code == -5, e.value
+    B.close()
