@@ -2084,18 +2084,6 @@ void launch_p2p(int L, const P2PArgs<R> &a, cudaStream_t s) {
   FMMPC_LAUNCH_CHECK();
 }
 
-// Kernels that need more than 48 KB of dynamic shared memory: raise their limit once, at
-// set-up (the attribute is per function), to the per-block maximum minus static use.
-template <typename K>
-void raise_smem_limit(K kernel) {
-  cudaFuncAttributes fa{};
-  FMMPC_CUDA(cudaFuncGetAttributes(&fa, kernel));
-  int dev = 0, optin = 0;
-  FMMPC_CUDA(cudaGetDevice(&dev));
-  FMMPC_CUDA(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
-  FMMPC_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - (int)fa.sharedSizeBytes));
-}
-
 template <typename R>
 void set_p2p_smem_limit() {
   raise_smem_limit(k_p2p<R, 4>);

@@ -210,6 +210,19 @@ struct fmmpc_handle {
 };
 
 namespace fmmpc {
+// The limit of dynamic shared memory of a kernel, raised at set-up to the per-block maximum minus its
+// static use.  The attribute is one per function, so a handle that set only what its own launches take
+// would lower it under another handle's.
+template <typename K>
+void raise_smem_limit(K kernel) {
+  cudaFuncAttributes fa{};
+  FMMPC_CUDA(cudaFuncGetAttributes(&fa, kernel));
+  int dev = 0, optin = 0;
+  FMMPC_CUDA(cudaGetDevice(&dev));
+  FMMPC_CUDA(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
+  FMMPC_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - (int)fa.sharedSizeBytes));
+}
+
 void apply_fmm(fmmpc_handle &H, int part, const double *r, double *out, int nrhs);
 // the apply's kernels issued on H.stream one by one (no graph of its own; used inside captures)
 void apply_fmm_eager(fmmpc_handle &H, int part, const double *r, double *out, int nrhs);

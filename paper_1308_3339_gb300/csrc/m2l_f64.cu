@@ -536,8 +536,8 @@ void init_m2l_oz(fmmpc_handle &H, DevPool &tmp) {
   FMMPC_CUDA(cudaMemcpyAsync(T.tiles, tiles.data(), sizeof(int2) * tiles.size(), cudaMemcpyHostToDevice, H.stream));
   FMMPC_CUDA(cudaMemcpyAsync(T.shifts, shifts.data(), sizeof(int4) * shifts.size(), cudaMemcpyHostToDevice, H.stream));
   FMMPC_CUDA(cudaMemsetAsync(T.err, 0, sizeof(int), H.stream));
-  if (W == 24) FMMPC_CUDA(cudaFuncSetAttribute(k_m2l_oz<24>, cudaFuncAttributeMaxDynamicSharedMemorySize, OzmShape<24>::SMEM));
-  else FMMPC_CUDA(cudaFuncSetAttribute(k_m2l_oz<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, OzmShape<32>::SMEM));
+  if (W == 24) raise_smem_limit(k_m2l_oz<24>);
+  else raise_smem_limit(k_m2l_oz<32>);
   FMMPC_CUDA(cudaStreamSynchronize(H.stream));
   T.enabled = true;
 }

@@ -673,11 +673,11 @@ void init_tc_m2l(fmmpc_handle &H, DevPool &tmp) {
   FMMPC_CUDA(cudaMemcpyAsync(T.dxs, dxs.data(), sizeof(int) * dxs.size(), cudaMemcpyHostToDevice, H.stream));
   FMMPC_CUDA(cudaMemsetAsync(T.err, 0, sizeof(int), H.stream));
   if (W == 24) {
-    FMMPC_CUDA(cudaFuncSetAttribute(k_m2l_tc<0, 24>, cudaFuncAttributeMaxDynamicSharedMemorySize, T.smem));
-    FMMPC_CUDA(cudaFuncSetAttribute(k_m2l_tc<1, 24>, cudaFuncAttributeMaxDynamicSharedMemorySize, T.smem));
+    raise_smem_limit(k_m2l_tc<0, 24>);
+    raise_smem_limit(k_m2l_tc<1, 24>);
   } else {
-    FMMPC_CUDA(cudaFuncSetAttribute(k_m2l_tc<0, 32>, cudaFuncAttributeMaxDynamicSharedMemorySize, T.smem));
-    FMMPC_CUDA(cudaFuncSetAttribute(k_m2l_tc<1, 32>, cudaFuncAttributeMaxDynamicSharedMemorySize, T.smem));
+    raise_smem_limit(k_m2l_tc<0, 32>);
+    raise_smem_limit(k_m2l_tc<1, 32>);
   }
   FMMPC_CUDA(cudaStreamSynchronize(H.stream));
   T.enabled = true;

@@ -490,7 +490,7 @@ void init_p2p_oz(fmmpc_handle &H) {
   if (T.nparts > 1) T.near = H.pool.get<double>((size_t)T.nparts * T.part_stride);
   T.err = H.pool.get<int>(1);
   FMMPC_CUDA(cudaMemsetAsync(T.err, 0, sizeof(int), H.stream));
-  FMMPC_CUDA(cudaFuncSetAttribute(k_p2p_oz, cudaFuncAttributeMaxDynamicSharedMemorySize, T.smem));
+  raise_smem_limit(k_p2p_oz);
   T.enabled = true;
 }
 

@@ -434,7 +434,7 @@ void init_tc_p2p(fmmpc_handle &H) {
   H.tcp.err = H.pool.get<int>(1);
   FMMPC_CUDA(cudaMemsetAsync(H.tcp.err, 0, sizeof(int), H.stream));
   const int smem = 4 * ((H.tcp.NS * 128 + 1023) & ~1023) + TC_NB * TC_BGRP + 1024;  // + alignment slack
-  FMMPC_CUDA(cudaFuncSetAttribute(k_p2p_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+  raise_smem_limit(k_p2p_tc);
   H.tcp.smem = smem;
 }
 

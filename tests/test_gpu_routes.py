@@ -243,3 +243,21 @@ def test_wide_upward_blocks_keep_the_half_turn(prec):
     tol = 1e-12 if prec == "fp64" else 1e-5
     check_close(f"half turn {prec}", z, z[::-1, ::-1], tol, tol)
     P.close()
+
+
+@pytest.mark.parametrize("prec,n,first,second", [("fp64", 128, 0.4, 0.25), ("fp64", 128, 0.25, 0.4),
+                                                 ("fp32", 1024, 0.25, 0.4), ("fp32", 1024, 0.4, 0.25)])
+def test_tensor_core_near_field_after_a_handle_of_another_theta(prec, n, first, second):
+    # the two stencil radii (3 and 5 leaves) take different amounts of shared memory, whose limit is one per
+    # kernel: making the second handle must leave the first one's launches as they were
+    from paper_1308_3339_gb300 import FmmPreconditioner
+    r = dev(S.random_field(n, 17))
+    P = FmmPreconditioner(n, p=8, theta=first, precision=prec)
+    assert P.query("tc_p2p") == 1
+    before = P.apply_part("near", r).clone()
+    Q = FmmPreconditioner(n, p=8, theta=second, precision=prec)
+    assert Q.query("tc_p2p") == 1
+    Q.apply_part("near", r)
+    assert torch.equal(P.apply_part("near", r), before)
+    Q.close()
+    P.close()
