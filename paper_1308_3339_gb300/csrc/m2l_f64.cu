@@ -393,6 +393,36 @@ __global__ void k_m2l_oz_sum(int64_t per_rhs, int64_t lo, int64_t total, int npa
   L[t] = v;
 }
 
+// The digits of every shift's B block: thread per (shift, row, 16 bytes of a digit's columns).  idx: the
+// matrix of each shift's two classes (-1: none); mats [matrix][2 p + 2 outputs][2 p], scaled columns.
+template <int W>
+__global__ void k_ozm_table(OzmArgs a, int ns, const int2 *__restrict__ idx, const double *__restrict__ mats,
+                            unsigned char *__restrict__ bmat) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= (int64_t)ns * 2 * W * 4) return;
+  const int q = (int)(i / (2 * W * 4)), row = (int)(i >> 2) % (2 * W), vc = (int)i & 3;
+  const int h = row / W, u = row % W, p2 = 2 * a.p, m = h ? idx[q].y : idx[q].x;
+  const bool used = m >= 0 && (u < p2 || u >= W - 2);
+  const double *x = mats + ((int64_t)(used ? m : 0) * (p2 + 2) + (u < p2 ? u : p2 + u - (W - 2))) * p2;
+  uint32_t pk[8][4];
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {
+    const int v = 8 * vc + j;
+    int d[OZ_S];
+    ozm_digits(used && v < p2 ? __double2ll_rn(ldexp(x[v], 62 - a.rb[u])) : 0, d);
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+      const uint32_t hv = __half_as_ushort(__int2half_rn(e < OZ_S ? d[e < OZ_S ? e : 0] : 0));
+      if (j & 1) pk[e][j >> 1] |= hv << 16;
+      else pk[e][j >> 1] = hv;
+    }
+  }
+#pragma unroll
+  for (int e = 0; e < 8; ++e)  // digit e: row set e / 2, columns 32 (e % 2) ..
+    reinterpret_cast<uint4 *>(bmat + ((int64_t)q * 4 + e / 2) * 2 * W * 128 + row * 128)[(vc + 4 * (e & 1)) ^ (row & 7)] =
+        make_uint4(pk[e][0], pk[e][1], pk[e][2], pk[e][3]);
+}
+
 __global__ void k_ozm_fill(int64_t total, int2 *__restrict__ le) {
   const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (t < total) le[t] = make_int2(OZ_NONE, 0);
@@ -454,44 +484,76 @@ void init_m2l_oz(fmmpc_handle &H, DevPool &tmp) {
     for (int q = 0; q < T.nparts; ++q)
       if (T.part_s[cp][q + 1] - T.part_s[cp][q] > OZM_MAXSH) return;
   }
-  // real matrices of every offset, inputs scaled by 2^-c_k
+  // real matrices of every offset, inputs scaled by 2^-c_k.  The powers of an offset in two doubles each
+  // (106 bits), so that an entry is one multiply-add: in long double, which is software on this host,
+  // they were a third of a 64^2 handle's set-up (with the digits, 10 of 27 ms).
   std::vector<double> fact(2 * p + 2, 1.0);
   for (int i = 1; i < (int)fact.size(); ++i) fact[i] = fact[i - 1] * i;
+  struct Two {
+    double hi, lo;
+  };
+  auto two = [](long double x) {
+    const double hi = (double)x;
+    return Two{hi, (double)(x - hi)};
+  };
   typedef std::complex<long double> C;
-  std::vector<C> ipw(2 * p);  // o^-j of the offset at hand
-  C lg;
+  std::vector<Two> pre(2 * p), pim(2 * p);  // o^-j of the offset at hand
+  double lre = 0.0, lim = 0.0;              // log o
   auto set_offset = [&](int oi) {
     const C o((long double)(oi % 15 - 7), (long double)(oi / 15 - 7)), inv = C(1) / o;
-    ipw[0] = C(1);
-    for (int j = 1; j < 2 * p; ++j) ipw[j] = ipw[j - 1] * inv;
-    lg = C(0.5L * std::log(std::norm(o)), std::atan2(o.imag(), o.real()));
+    C pw(1);
+    for (int j = 0; j < 2 * p; ++j, pw = pw * inv) {
+      pre[j] = two(pw.real());
+      pim[j] = two(pw.imag());
+    }
+    lre = (double)(0.5L * std::log(std::norm(o)));
+    lim = (double)std::atan2(o.imag(), o.real());
   };
-  auto entry = [&](int u, int v) -> double {
-    if (u >= W - 2) return u - (W - 2) == v ? 1.0 : 0.0;
-    const int nn = u / 2, k = v / 2;
-    long double f = 1.0L;
-    if (k == 0) f = ((nn % 2) ? 1.0L : -1.0L) / (long double)std::max(nn, 1);
-    else if (nn > 0) f = ((nn % 2) ? -1.0L : 1.0L) * (long double)(fact[nn + k - 1] / (fact[nn] * fact[k - 1]));
-    const C cv = (nn == 0 && k == 0) ? lg : f * ipw[nn + k];
-    return (double)((u & 1) == 0 ? ((v & 1) ? -cv.imag() : cv.real()) : ((v & 1) ? cv.real() : cv.imag()));
+  auto times = [](double f, const Two &x) {
+    const double q = f * x.hi;
+    return q + (std::fma(f, x.hi, -q) + f * x.lo);
   };
-  std::vector<int> outs;
-  for (int u = 0; u < 2 * p; ++u) outs.push_back(u);
-  outs.push_back(W - 2);
-  outs.push_back(W - 1);
-  std::vector<std::vector<double>> mats(225);  // by offset: [W][2p], scaled columns
-  std::vector<double> rmax(W, 0.0);
+  auto over = [](const Two &x, double n) {
+    const double q = x.hi / n;
+    return q + (std::fma(-q, n, x.hi) + x.lo) / n;
+  };
+  // real and imaginary part of output coefficient n from input coefficient k
+  auto coeff = [&](int n, int k, double &re, double &im) {
+    if (n == 0 && k == 0) {
+      re = lre, im = lim;
+    } else if (k == 0) {
+      const double s = (n % 2) ? 1.0 : -1.0;
+      re = s * over(pre[n], n), im = s * over(pim[n], n);
+    } else {
+      const double f = n == 0 ? 1.0 : ((n % 2) ? -1.0 : 1.0) * (fact[n + k - 1] / (fact[n] * fact[k - 1]));
+      re = times(f, pre[n + k]), im = times(f, pim[n + k]);
+    }
+  };
+  const int p2 = 2 * p, nout = p2 + 2;  // outputs: 2p real parts, then the sums M~_0 (rows W - 2, W - 1)
+  std::vector<int> mat_of(225, -1);
+  std::vector<double> mats, rmax(W, 0.0);  // [matrix][nout][2p], scaled columns
   for (int q = 0; q < ns; ++q)
     for (int c = 0; c < 4; ++c) {
       const int oi = S.shift_ofs[q][c];
-      if (oi < 0 || !mats[oi].empty()) continue;
-      mats[oi].assign((size_t)W * 2 * p, 0.0);
+      if (oi < 0 || mat_of[oi] >= 0) continue;
+      mat_of[oi] = (int)(mats.size() / ((size_t)nout * p2));
+      mats.resize(mats.size() + (size_t)nout * p2, 0.0);
+      double *m = mats.data() + (size_t)mat_of[oi] * nout * p2;
       set_offset(oi);
-      for (int u : outs)
-        for (int v = 0; v < 2 * p; ++v) {
-          const double m = std::ldexp(entry(u, v), -ozm_col(v / 2));
-          mats[oi][(size_t)u * 2 * p + v] = m;
-          rmax[u] = std::max(rmax[u], std::fabs(m));
+      for (int n = 0; n < p; ++n)
+        for (int k = 0; k < p; ++k) {
+          double re, im;
+          coeff(n, k, re, im);
+          const double sc = std::ldexp(1.0, -ozm_col(k));
+          m[(2 * n) * p2 + 2 * k] = m[(2 * n + 1) * p2 + 2 * k + 1] = sc * re;
+          m[(2 * n) * p2 + 2 * k + 1] = -(sc * im);
+          m[(2 * n + 1) * p2 + 2 * k] = sc * im;
+        }
+      m[p2 * p2] = m[(p2 + 1) * p2 + 1] = 1.0;
+      for (int u = 0; u < nout; ++u)
+        for (int v = 0; v < p2; ++v) {
+          double &r = rmax[u < p2 ? u : W - 2 + u - p2];
+          r = std::max(r, std::fabs(m[u * p2 + v]));
         }
     }
   for (int u = 0; u < W; ++u) {
@@ -499,40 +561,35 @@ void init_m2l_oz(fmmpc_handle &H, DevPool &tmp) {
     if (rmax[u] > 0.0) std::frexp(rmax[u], &e);  // rmax < 2^e
     T.rb[u] = e;
   }
-  const size_t bbytes = (size_t)4 * 2 * W * 128;
-  std::vector<unsigned char> B(shifts.size() * bbytes, 0);
-  for (size_t q = 0; q < shifts.size(); ++q)
-    for (int h = 0; h < 2; ++h) {
-      const int oi = S.shift_ofs[shq[q]][(q < (size_t)count[0] ? 0 : 2) + h];
-      if (oi < 0) continue;
-      unsigned char *blk = B.data() + q * bbytes;
-      for (int u : outs) {
-        const int row = W * h + u;
-        for (int v = 0; v < 2 * p; ++v) {
-          int d[OZ_S];
-          ozm_digits(std::llrint(std::ldexp(mats[oi][(size_t)u * 2 * p + v], 62 - T.rb[u])), d);
-          for (int i = 0; i < OZ_S; ++i) {
-            const int col = 32 * (i & 1) + v, ch = col / 8;
-            uint16_t *dst = reinterpret_cast<uint16_t *>(blk + (size_t)(i / 2) * 2 * W * 128 + (size_t)row * 128 +
-                                                         ((ch ^ (row & 7)) * 16));
-            dst[col % 8] = __half_as_ushort(__float2half_rn((float)d[i]));
-          }
-        }
-      }
-    }
+  std::vector<int2> idx(shifts.size());
+  for (size_t q = 0; q < shifts.size(); ++q) {
+    const auto &o = S.shift_ofs[shq[q]];
+    const int c = q < (size_t)count[0] ? 0 : 2;
+    idx[q] = make_int2(o[c] < 0 ? -1 : mat_of[o[c]], o[c + 1] < 0 ? -1 : mat_of[o[c + 1]]);
+  }
   const size_t ibytes = (size_t)H.nrhs_max * 4 * rows * 128, nexp = (size_t)H.nrhs_max * rows;
   T.img = H.pool.get<unsigned char>(ibytes);
   FMMPC_CUDA(cudaMemsetAsync(T.img, 0, ibytes, H.stream));
   T.lexp = H.pool.get<int2>(nexp);
   k_ozm_fill<<<nblk(nexp), 256, 0, H.stream>>>((int64_t)nexp, T.lexp);
   FMMPC_LAUNCH_CHECK();
-  T.bmat = H.pool.get<unsigned char>(B.size());
+  T.bmat = H.pool.get<unsigned char>(shifts.size() * 4 * 2 * W * 128);
   T.tiles = H.pool.get<int2>(tiles.size());
   T.shifts = H.pool.get<int4>(shifts.size());
   T.part_stride = (int64_t)H.nrhs_max * g.ncell * p;
   T.Lp = H.pool.get<double>((size_t)2 * T.nparts * T.part_stride);
   T.err = H.pool.get<int>(1);
-  FMMPC_CUDA(cudaMemcpyAsync(T.bmat, B.data(), B.size(), cudaMemcpyHostToDevice, H.stream));
+  double *dmats = tmp.get<double>(mats.size());
+  int2 *didx = tmp.get<int2>(idx.size());
+  FMMPC_CUDA(cudaMemcpyAsync(dmats, mats.data(), sizeof(double) * mats.size(), cudaMemcpyHostToDevice, H.stream));
+  FMMPC_CUDA(cudaMemcpyAsync(didx, idx.data(), sizeof(int2) * idx.size(), cudaMemcpyHostToDevice, H.stream));
+  OzmArgs a{};
+  a.p = p;
+  for (int u = 0; u < W; ++u) a.rb[u] = T.rb[u];
+  const int nsh = (int)shifts.size();
+  if (W == 24) k_ozm_table<24><<<nblk((int64_t)nsh * 2 * W * 4), 256, 0, H.stream>>>(a, nsh, didx, dmats, T.bmat);
+  else k_ozm_table<32><<<nblk((int64_t)nsh * 2 * W * 4), 256, 0, H.stream>>>(a, nsh, didx, dmats, T.bmat);
+  FMMPC_LAUNCH_CHECK();
   FMMPC_CUDA(cudaMemcpyAsync(T.tiles, tiles.data(), sizeof(int2) * tiles.size(), cudaMemcpyHostToDevice, H.stream));
   FMMPC_CUDA(cudaMemcpyAsync(T.shifts, shifts.data(), sizeof(int4) * shifts.size(), cudaMemcpyHostToDevice, H.stream));
   FMMPC_CUDA(cudaMemsetAsync(T.err, 0, sizeof(int), H.stream));

@@ -380,6 +380,36 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_p2p_oz(OzArgs a) {
   }
 }
 
+// The digits of the kernel table's block of every stencil offset (rows of offsets as in OzArgs), from the
+// CUDA-core kernel's table of ln|d|: thread per (offset, target node t, source node row).  On the host
+// the logarithms and digits of 37 x 4096 pairs were half of a 64^2 handle's set-up (11 of 27 ms).
+__global__ void k_oz_table(OzArgs a, int no, int nrows, int eb, const double *__restrict__ table, int Rn, int c0, int stride,
+                           unsigned char *__restrict__ bmat) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= (int64_t)no * 512) return;
+  const int o = (int)(i >> 9), t = (int)(i >> 3) & 63, kc = (int)i & 7;
+  int r = 0, q = o;
+  while (r + 1 < nrows && q >= a.row_cnt[r]) q -= a.row_cnt[r++];
+  const int ox = a.row_ox0[r] + q, oy = a.row_oy[r], dy = (t >> 3) - kc - 8 * oy;
+  const double *row = table + (int64_t)(dy < 0 ? -dy : dy) * stride + c0 + Rn;
+  uint32_t pk[OZ_S][4];
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {
+    int d[OZ_S];
+    oz_digits(__double2ll_rn(ldexp(row[(t & 7) - j - 8 * ox], 62 - eb)), d);
+#pragma unroll
+    for (int s = 0; s < OZ_S; ++s) {
+      const uint32_t hv = __half_as_ushort(__int2half_rn(d[s]));
+      if (j & 1) pk[s][j >> 1] |= hv << 16;
+      else pk[s][j >> 1] = hv;
+    }
+  }
+#pragma unroll
+  for (int s = 0; s < OZ_S; ++s)
+    reinterpret_cast<uint4 *>(bmat + ((int64_t)o * OZ_S + oz_pos(s)) * OZ_BLK + t * 128)[kc ^ (t & 7)] =
+        make_uint4(pk[s][0], pk[s][1], pk[s][2], pk[s][3]);
+}
+
 __global__ void k_oz_fill(int64_t total, int2 *__restrict__ le) {
   const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (t < total) le[t] = make_int2(OZ_NONE, 0);
@@ -395,6 +425,17 @@ __global__ void k_near_combine64(int64_t total, const double *__restrict__ a, in
 }
 
 inline unsigned nblk(int64_t n, int t = 256) { return (unsigned)((n + t - 1) / t); }
+
+// the stencil's rows of offsets
+OzArgs rows_of(const OzP2P &T) {
+  OzArgs a{};
+  for (int r = 0; r < T.nrows; ++r) {
+    a.row_oy[r] = (int16_t)T.row_oy[r];
+    a.row_ox0[r] = (int16_t)T.row_ox0[r];
+    a.row_cnt[r] = (int16_t)T.row_cnt[r];
+  }
+  return a;
+}
 
 }  // namespace
 
@@ -458,7 +499,7 @@ void init_p2p_oz(fmmpc_handle &H) {
   FMMPC_LAUNCH_CHECK();
   const double cself = -0.5 * std::log(2.0) - 1.5 + 0.25 * PI;
   for (int variant = 0; variant < 2; ++variant) {  // without and with ln h
-    auto value = [&](int dx, int dy) {
+    auto value = [&](int dx, int dy) {  // as in the table
       const double v = (dx == 0 && dy == 0) ? cself : 0.5 * std::log((double)dx * dx + (double)dy * dy);
       return variant ? v + g.lnh : v;
     };
@@ -467,22 +508,11 @@ void init_p2p_oz(fmmpc_handle &H) {
     for (auto d : {std::pair<int, int>{0, 0}, {1, 0}, {dm, dm}}) vmax = std::max(vmax, std::fabs(value(d.first, d.second)));
     int eb = 0;
     std::frexp(vmax, &eb);  // vmax < 2^eb
-    std::vector<uint16_t> B((size_t)no * OZ_S * (OZ_BLK / 2));
-    for (int o = 0; o < no; ++o) {
-      const int oy = T.row_oy[ofs[o].first], ox = T.row_ox0[ofs[o].first] + ofs[o].second;
-      for (int t = 0; t < 64; ++t)
-        for (int k = 0; k < 64; ++k) {
-          const double v = value((t % 8) - (k % 8) - 8 * ox, (t / 8) - (k / 8) - 8 * oy);
-          int d[OZ_S];
-          oz_digits(std::llrint(std::ldexp(v, 62 - eb)), d);
-          const size_t e = (size_t)t * 64 + (((k / 8) ^ (t & 7)) * 8) + (k % 8);
-          for (int s = 0; s < OZ_S; ++s)
-            B[((size_t)o * OZ_S + oz_pos(s)) * (OZ_BLK / 2) + e] = __half_as_ushort(__float2half_rn((float)d[s]));
-        }
-    }
-    unsigned char *dB = H.pool.get<unsigned char>(B.size() * 2);
-    FMMPC_CUDA(cudaMemcpyAsync(dB, B.data(), B.size() * 2, cudaMemcpyHostToDevice, H.stream));
-    FMMPC_CUDA(cudaStreamSynchronize(H.stream));
+    unsigned char *dB = H.pool.get<unsigned char>((size_t)no * OZ_S * OZ_BLK);
+    k_oz_table<<<nblk((int64_t)no * 512), 256, 0, H.stream>>>(
+        rows_of(T), no, T.nrows, eb, (const double *)(variant ? H.fb.table_lnh : H.fb.table), H.fb.Rn, H.fb.table_c0,
+        H.fb.table_stride, dB);
+    FMMPC_LAUNCH_CHECK();
     T.bmat[variant] = dB;
     T.eb[variant] = eb;
   }
@@ -508,7 +538,7 @@ int prep_p2p_oz(fmmpc_handle &H, const double *r, int nrhs, cudaStream_t s, doub
 int run_p2p_oz(fmmpc_handle &H, bool with_lnh, double *out, int nrhs, cudaStream_t s) {
   const Geo &g = H.g;
   const OzP2P &T = H.ozp;
-  OzArgs a{};
+  OzArgs a = rows_of(T);
   a.img = T.img;
   a.lexp = T.lexp;
   a.bmat = T.bmat[with_lnh ? 1 : 0];
@@ -526,11 +556,6 @@ int run_p2p_oz(fmmpc_handle &H, bool with_lnh, double *out, int nrhs, cudaStream
   a.sh = T.sh;
   a.nsr = T.nsr;
   a.nparts = T.nparts;
-  for (int r = 0; r < T.nrows; ++r) {
-    a.row_oy[r] = (int16_t)T.row_oy[r];
-    a.row_ox0[r] = (int16_t)T.row_ox0[r];
-    a.row_cnt[r] = (int16_t)T.row_cnt[r];
-  }
   for (int p = 0; p < T.nparts; ++p) {
     a.part_r[p] = (int16_t)T.part_r[p];
     a.part_q[p] = (int16_t)T.part_q[p];

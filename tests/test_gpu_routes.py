@@ -261,3 +261,26 @@ def test_tensor_core_near_field_after_a_handle_of_another_theta(prec, n, first, 
     assert torch.equal(P.apply_part("near", r), before)
     Q.close()
     P.close()
+
+
+def test_fp64_set_up_costs_no_more_than_twice_the_fp32_forms():
+    # the FP64 form's digit tables are formed on the GPU; on the host they were four times the rest of a
+    # small handle's set-up
+    import time
+
+    from paper_1308_3339_gb300 import FmmPreconditioner
+
+    def best(prec):
+        times = []
+        for _ in range(6):
+            torch.cuda.synchronize()
+            t = time.perf_counter()
+            P = FmmPreconditioner(64, p=10, precision=prec)
+            torch.cuda.synchronize()
+            times.append(time.perf_counter() - t)
+            P.close()
+        return min(times)
+
+    fp32, fp64 = best("fp32"), best("fp64")
+    print(f"set-up of 64^2: fp32 {1e3 * fp32:.2f} ms, fp64 {1e3 * fp64:.2f} ms", flush=True)
+    assert fp64 < 2 * fp32
