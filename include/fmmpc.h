@@ -157,9 +157,10 @@ int fmmpc_apply_part(fmmpc_handle *h, int32_t part, const double *r_dev, double 
  * / n apart from half an element past each corner), in the order bottom (x increasing),
  * right (y increasing), top (x decreasing), left (y decreasing).  The boundary solve is
  * FP64 in every form.  Uses the single-layer equations whatever fmmpc_set_bem_form set.  The
- * first call forms the tables of (1/2 I + K) and of the double layer next to the boundary; a
- * first call under stream capture, or where they do not fit, sums them directly instead.
- * Asynchronous on the handle's stream.  Errors: _INVALID. */
+ * first call allocates the tables of (1/2 I + K) and of the double layer next to the boundary and
+ * forms them on the stream; while the handle's stream is being captured, and where they do not
+ * fit, the calls sum them directly instead.  Asynchronous on the handle's stream, the first call
+ * too; a capture of another stream is left alone.  Errors: _INVALID. */
 int fmmpc_apply_bc(fmmpc_handle *h, const double *f_dev, const double *g_dev, double *u_dev, int32_t n_rhs);
 
 /* The transpose of the preconditioner, rb = P^{-T} zb: the gradient of a loss of z = P^{-1} r

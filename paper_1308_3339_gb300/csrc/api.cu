@@ -270,8 +270,12 @@ int fmmpc_apply_bc(fmmpc_handle *h, const double *f_dev, const double *g_dev, do
     } restore{h, h->bem_form};
     h->bem_form = 0;
     h->bc_g = g_dev;
-    init_bem_bc(*h);
-    init_bnd_dl(*h);
+    cudaStreamCaptureStatus cap{};
+    FMMPC_CUDA(cudaStreamIsCapturing(h->stream, &cap));
+    if (cap == cudaStreamCaptureStatusNone && !h->no_bc_tables) {
+      init_bem_bc(*h);
+      if (!init_bnd_dl(*h)) h->no_bc_tables = true;
+    }
     apply_fmm(*h, PART_BC, f_dev, u_dev, n_rhs);
     return FMMPC_OK;
   });

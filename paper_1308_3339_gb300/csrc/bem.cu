@@ -50,75 +50,50 @@ __device__ __forceinline__ double seg_log_int_d(double s1, double ell, double d)
   return v;
 }
 
-// S_mk = -(h/2pi) (int_k ln|y_m - y|_node ds_node + l ln h)  (physical units)
-__global__ void k_bem_S(int n, double h, double lnh, double *__restrict__ S) {
-  const int NG = 4 * n;
-  int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= (int64_t)NG * NG) return;
-  const int mrow = (int)(t / NG), k = (int)(t % NG);
+// Matrices in the folded form (rows m < h of the first block row [S0 | S1 | S2 | S3]):
+//  SINGLE  S_mk = -(h/2pi) (int_k ln|y_m - y|_node ds_node + l ln h)  (physical units)
+//  DOUBLE  diag I + K, K_mk = int_k dG/dn_y(y_m, y) dGamma = (1/2pi) atan2(l d, d^2 + s1 s2) with d
+//          the signed normal offset of y_m from element k's line (zero on the same side): diag =
+//          -1/2 the system (-1/2 I + K) mu = -(V r)|_Gamma of the double-layer correction, diag
+//          = 1/2 the boundary data term of Eq. e:ubound.
+enum class BemMatrix { SINGLE, DOUBLE };
+
+// entry (m, element k of side sk), the collocation point m on side 0; a, b: h and ln h, or diag and unused
+template <BemMatrix KIND>
+__device__ __forceinline__ double bem_entry(int n, int m, int sk, int k, double a, double b) {
   const double ell = (n + 1.0) / n, np1 = n + 1.0;
-  // collocation point m in node units
-  const int sm = mrow / n, km = mrow % n;
-  const double tm = (km + 0.5) * ell;
-  double x, y;
-  switch (sm) {
-    case 0: x = tm; y = 0; break;
-    case 1: x = np1; y = tm; break;
-    case 2: x = np1 - tm; y = np1; break;
-    default: x = 0; y = np1 - tm; break;
-  }
-  const int sk = k / n, kk = k % n;
+  if (KIND == BemMatrix::DOUBLE && sk == 0) return k == m ? a : 0.0;
   double u, d;
-  side_coords_d(sk, np1, x, y, u, d);
-  double I;
-  if (sk == sm) I = seg_log_int_d((kk - km - 0.5) * ell, ell, 0.0);  // same side: exact offsets
-  else I = seg_log_int_d(kk * ell - u, ell, d);
-  S[t] = -(h / (2.0 * PI)) * (I + ell * lnh);
-}
-
-// First block row of diag I + K, K_mk = int_k dG/dn_y(y_m, y) dGamma = (1/2pi) atan2(l d,
-// d^2 + s1 s2) with d the signed normal offset of y_m from element k's line (zero on the
-// same side): diag = -1/2 the system (-1/2 I + K) mu = -(V r)|_Gamma of the double-layer
-// correction, diag = 1/2 the boundary data term of Eq. e:ubound.
-__global__ void k_bem_Kdl(int n, double diag, double *__restrict__ A) {
-  const int NG = 4 * n;
-  int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= (int64_t)n * NG) return;
-  const int mrow = (int)(t / NG), k = (int)(t % NG);
-  const double ell = (n + 1.0) / n, np1 = n + 1.0;
-  const double x = (mrow + 0.5) * ell, y = 0.0;  // collocation point mrow of side 0
-  const int sk = k / n, kk = k % n;
-  double v = 0.0;
-  if (sk == 0) {
-    v = (k == mrow) ? diag : 0.0;
-  } else {
-    double u, d;
-    side_coords_d(sk, np1, x, y, u, d);
-    const double s1 = kk * ell - u, s2 = s1 + ell;
-    v = atan2(ell * d, d * d + s1 * s2) / (2.0 * PI);
+  side_coords_d(sk, np1, (m + 0.5) * ell, 0.0, u, d);
+  if (KIND == BemMatrix::SINGLE) {
+    const double I = sk == 0 ? seg_log_int_d((k - m - 0.5) * ell, ell, 0.0)  // same side: exact offsets
+                             : seg_log_int_d(k * ell - u, ell, d);
+    return -(a / (2.0 * PI)) * (I + ell * b);
   }
-  A[t] = v;
+  const double s1 = k * ell - u, s2 = s1 + ell;
+  return atan2(ell * d, d * d + s1 * s2) / (2.0 * PI);
 }
 
-// The folded form of a first block row A = [S0 | S1 | S2 | S3] (n x 4n), row m < h: T[m] (4n values).
-__global__ void k_bem_fold(int n, const double *__restrict__ A, double *__restrict__ T) {
+// Row m < h of the folded form, T[m] (4n values): thread per (m, k < h), the eight entries of columns k and
+// n - 1 - k of every side.
+template <BemMatrix KIND>
+__global__ void k_bem_fold(int n, double a, double b, double *__restrict__ T) {
   const int h = n >> 1;
   const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= (int64_t)h * h) return;
-  const int64_t m = t / h;
-  const int k = (int)(t % h);
-  const double *r = A + m * 4 * n;
+  const int m = (int)(t / h), k = (int)(t % h);
   double x[2][4];  // C^0, C^2, A, B at columns k and n - 1 - k
 #pragma unroll
   for (int j = 0; j < 2; ++j) {
-    const int c = j ? n - 1 - k : k;
-    const double s0 = r[c], s1 = r[n + c], s2 = r[2 * n + c], s3 = r[3 * n + c];
-    x[j][0] = (s0 + s2) + (s1 + s3);
-    x[j][1] = (s0 + s2) - (s1 + s3);
-    x[j][2] = s0 - s2;
-    x[j][3] = s1 - s3;
+    double s[4];
+#pragma unroll 1
+    for (int sk = 0; sk < 4; ++sk) s[sk] = bem_entry<KIND>(n, m, sk, j ? n - 1 - k : k, a, b);
+    x[j][0] = (s[0] + s[2]) + (s[1] + s[3]);
+    x[j][1] = (s[0] + s[2]) - (s[1] + s[3]);
+    x[j][2] = s[0] - s[2];
+    x[j][3] = s[1] - s[3];
   }
-  double *o = T + m * 4 * n + k;
+  double *o = T + (int64_t)m * 4 * n + k;
 #pragma unroll
   for (int q = 0; q < 3; ++q) {
     o[(2 * q) * h] = x[0][q] + x[1][q];
@@ -256,10 +231,8 @@ void init_bem(fmmpc_handle &H, DevPool &tmp) {
   const int n = g.n, N = g.NG;
   const size_t nt = (size_t)(n / 2) * N;  // the folded form
   cudaStream_t s = H.stream;
-  double *S = tmp.get<double>((size_t)n * N);  // first block row, n x 4n
-  k_bem_S<<<nblk((int64_t)n * N), 256, 0, s>>>(n, g.h, g.lnh, S);
   H.Sinv = H.pool.get<double>(nt);
-  k_bem_fold<<<nblk((int64_t)(n / 2) * (n / 2)), 256, 0, s>>>(n, S, H.Sinv);
+  k_bem_fold<BemMatrix::SINGLE><<<nblk((int64_t)(n / 2) * (n / 2)), 256, 0, s>>>(n, g.h, g.lnh, H.Sinv);
   FMMPC_LAUNCH_CHECK();
   if (!invert_folded(n, H.Sinv, s, tmp))
     throw Error(FMMPC_ERR_INVALID, "single-layer BEM matrix is singular for this domain");
@@ -307,10 +280,8 @@ void init_bem_dl(fmmpc_handle &H) {
   cudaStream_t s = H.stream;
   DevPool tmp;
   try {
-    double *A = tmp.get<double>((size_t)n * N);
-    k_bem_Kdl<<<nblk((int64_t)n * N), 256, 0, s>>>(n, -0.5, A);
     double *T = H.pool.get<double>(nt);
-    k_bem_fold<<<nblk((int64_t)(n / 2) * (n / 2)), 256, 0, s>>>(n, A, T);
+    k_bem_fold<BemMatrix::DOUBLE><<<nblk((int64_t)(n / 2) * (n / 2)), 256, 0, s>>>(n, -0.5, 0.0, T);
     FMMPC_LAUNCH_CHECK();
     if (!invert_folded(n, T, s, tmp))
       throw Error(FMMPC_ERR_INVALID, "double-layer BEM matrix is singular for this domain");
@@ -332,34 +303,24 @@ void init_bem_dl(fmmpc_handle &H) {
 }
 
 // 1/2 I + K in the folded form, the boundary data term of Eq. e:ubound, for apply_bc; formed
-// on its first call.  Summing the 16 n^2 atan2 of K g directly took 1160 us at n = 1024; the
-// 3 n^2 multiply-adds of the folded form take 9 us.  Not formed (false) while the
-// handle's stream is being captured, or without memory for it: the caller sums directly.
-bool init_bem_bc(fmmpc_handle &H) {
-  if (H.Kbc) return true;
-  cudaStreamCaptureStatus cap{};
-  if (cudaStreamIsCapturing(H.stream, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
-    cudaGetLastError();
-    return false;
-  }
+// on its first call, in the stream's order and without a wait.  Summing the 16 n^2 atan2 of K g
+// directly took 1160 us at n = 1024; the 3 n^2 multiply-adds of the folded form take 9 us.  Not
+// formed while the handle's stream is being captured (a later call forms it), nor where there is
+// no memory for it (then for good): the caller sums directly.
+void init_bem_bc(fmmpc_handle &H) {
+  if (H.Kbc || H.no_bc_tables) return;
   const int n = H.g.n;
-  const size_t nv = (size_t)H.g.NG * H.nrhs_max;
-  double *A = nullptr, *T = nullptr;
-  DevPool tmp;
-  try {
-    if (!H.bc_vt) H.bc_vt = H.pool.get<double>(nv);
-    if (!H.bc_kg) H.bc_kg = H.pool.get<double>(nv);
-    A = tmp.get<double>((size_t)n * H.g.NG);
-    T = H.pool.get<double>((size_t)(n / 2) * H.g.NG);
-  } catch (const Error &) {
-    return false;
+  const size_t nt = (size_t)(n / 2) * H.g.NG, nv = (size_t)H.g.NG * H.nrhs_max;
+  double *T = static_cast<double *>(H.pool.try_alloc(sizeof(double) * (nt + 2 * nv)));
+  if (!T) {
+    H.no_bc_tables = true;
+    return;
   }
-  k_bem_Kdl<<<nblk((int64_t)n * H.g.NG), 256, 0, H.stream>>>(n, 0.5, A);
-  k_bem_fold<<<nblk((int64_t)(n / 2) * (n / 2)), 256, 0, H.stream>>>(n, A, T);
+  k_bem_fold<BemMatrix::DOUBLE><<<nblk((int64_t)(n / 2) * (n / 2)), 256, 0, H.stream>>>(n, 0.5, 0.0, T);
   FMMPC_LAUNCH_CHECK();
-  FMMPC_CUDA(cudaStreamSynchronize(H.stream));  // A goes out of scope
+  H.bc_vt = T + nt;
+  H.bc_kg = H.bc_vt + nv;
   H.Kbc = T;
-  return true;
 }
 
 }  // namespace fmmpc

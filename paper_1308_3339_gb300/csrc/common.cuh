@@ -50,16 +50,26 @@ struct DevPool {
   DevPool(const DevPool &) = delete;
   DevPool &operator=(const DevPool &) = delete;
   ~DevPool() { release(); }
-  void *alloc(size_t nbytes) {
+  // nullptr where the memory is not there.  An allocation waits for nothing and belongs to no stream, so
+  // it is let through while some stream of the process is being captured, which it would else end.
+  void *try_alloc(size_t nbytes) {
     void *p = nullptr;
     if (nbytes == 0) nbytes = 16;
-    cudaError_t e = cudaMalloc(&p, nbytes);
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    const cudaError_t e = cudaMalloc(&p, nbytes);
+    cudaThreadExchangeStreamCaptureMode(&mode);
     if (e != cudaSuccess) {
       cudaGetLastError();
-      throw Error(FMMPC_ERR_OOM, "cudaMalloc of " + std::to_string(nbytes) + " bytes failed");
+      return nullptr;
     }
     ptrs.push_back(p);
     bytes += nbytes;
+    return p;
+  }
+  void *alloc(size_t nbytes) {
+    void *p = try_alloc(nbytes);
+    if (!p) throw Error(FMMPC_ERR_OOM, "cudaMalloc of " + std::to_string(nbytes) + " bytes failed");
     return p;
   }
   template <typename T>

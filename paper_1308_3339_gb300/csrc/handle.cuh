@@ -170,6 +170,7 @@ struct fmmpc_handle {
   double *SinvT = nullptr;    // the same for S^T (the transpose pass), made on first use
   float *Kdl_hi = nullptr, *Kdl_lo = nullptr;  // and as two FP32 words (single-precision forms)
   double *Kbc = nullptr;      // 1/2 I + K in the same form (apply_bc), made on first use
+  bool no_bc_tables = false;  // apply_bc's tables did not fit: it sums the boundary data directly
   double *bc_vt = nullptr, *bc_kg = nullptr;  // [nrhs][NG] side DFT of the boundary data, -(1/2 I + K) g
   int bem_form = 0;         // 0: single-layer correction (Eq. e:ubound), 1: second-kind double layer
   const double *bc_g = nullptr;  // boundary data of the running fmmpc_apply_bc call (else NULL)
@@ -239,7 +240,7 @@ void init_fmm_transpose(fmmpc_handle &H);
 void init_bem(fmmpc_handle &H, DevPool &tmp);
 void init_bem_dl(fmmpc_handle &H);
 void init_bem_transpose(fmmpc_handle &H);
-bool init_bem_bc(fmmpc_handle &H);
+void init_bem_bc(fmmpc_handle &H);
 bool init_bnd_dl(fmmpc_handle &H);
 void spmv5(fmmpc_handle &H, const double *x, double *y, int nrhs);
 int solve(fmmpc_handle &H, const double *f, const double *g, double *u, int nrhs,

@@ -284,3 +284,47 @@ def test_fp64_set_up_costs_no_more_than_twice_the_fp32_forms():
     fp32, fp64 = best("fp32"), best("fp64")
     print(f"set-up of 64^2: fp32 {1e3 * fp32:.2f} ms, fp64 {1e3 * fp64:.2f} ms", flush=True)
     assert fp64 < 2 * fp32
+
+
+@pytest.mark.parametrize("prec", ["fp64", "fp32"])
+def test_first_apply_bc_leaves_another_streams_capture_alone(prec):
+    # the first call allocates its tables; a capture of some other stream (in the global mode, the default)
+    # must go on, and the call on its own stream runs at once
+    from paper_1308_3339_gb300 import FmmPreconditioner
+    n = 64
+    f, g = dev(S.gaussian_mixture(n, 3)), dev(S.random_field(n, 4)[:4 * n])
+    own, other = torch.cuda.Stream(), torch.cuda.Stream()
+    P = FmmPreconditioner(n, p=8, precision=prec, stream=own)
+    u, x = torch.empty_like(f), torch.zeros(4, device="cuda")
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=other):
+        x += 1
+        P.apply_bc(f, g, out=u)
+    own.synchronize()
+    graph.replay()
+    again = P.apply_bc(f, g)
+    torch.cuda.synchronize()
+    assert x.tolist() == [1.0] * 4 and torch.equal(u, again)
+    P.close()
+
+
+def test_first_apply_bc_does_not_wait_for_its_stream():
+    from paper_1308_3339_gb300 import FmmPreconditioner
+    n = 64
+    f, g = dev(S.gaussian_mixture(n, 3)), dev(S.random_field(n, 4)[:4 * n])
+    st = torch.cuda.Stream()
+    for attempt in range(2):  # the first handle loads the kernels
+        with torch.cuda.stream(st):
+            P = FmmPreconditioner(n, p=8, precision="fp32", stream=st)
+            u = torch.empty_like(f)
+            st.synchronize()
+            before = torch.cuda.Event()
+            if attempt:
+                torch.cuda._sleep(2_000_000_000)  # about a second
+            before.record(st)
+            P.apply_bc(f, g, out=u)
+            if attempt:
+                assert not before.query()  # the call came back ahead of the work before it
+            st.synchronize()
+            P.close()
