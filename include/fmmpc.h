@@ -122,7 +122,10 @@ typedef struct {
  * translation tables, boundary elements and the FP64 inverse of the single-layer BEM
  * matrix (Sec. 4.3), workspace.  stream: a cudaStream_t (NULL = legacy default stream)
  * on which every later call of this handle runs.  On success *out owns all of it and
- * must be released with fmmpc_destroy.  Errors: _INVALID (grid/params), _OOM, _CUDA. */
+ * must be released with fmmpc_destroy.  The FP64 form's tensor-core kernels take their operands
+ * last (512 MB a right-hand side at 4096^2); where these do not fit, then or when a later
+ * allocation of the handle needs the room, its near field and M2L run on the CUDA cores.
+ * Errors: _INVALID (grid/params), _OOM, _CUDA. */
 int fmmpc_create(fmmpc_handle **out, const fmmpc_grid *g, const fmmpc_params *prm, void *stream);
 
 /* Preconditioner action z = P^{-1} r (Sec. 3.2, PCApply): for each right-hand side,

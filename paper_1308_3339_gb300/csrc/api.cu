@@ -94,10 +94,22 @@ void setup(fmmpc_handle &H, const fmmpc_grid &g, const fmmpc_params &p) {
     G.npad = n + 2 * G.pad;
     init_fmm(H);
     init_tc_p2p(H);
-    init_p2p_oz(H);
     init_tc_m2l(H, tmp);
-    init_m2l_oz(H, tmp);
     init_bem(H, tmp);
+    FMMPC_CUDA(cudaStreamSynchronize(H.stream));
+    tmp.release();
+    // the FP64 form's digit kernels last, in the memory that is left: 16 GB of operands at 4096^2 x 32
+    auto where_it_fits = [&](DevPool &pool, auto &state, auto &&init) {
+      try {
+        init();
+      } catch (const Error &e) {
+        if (e.code != FMMPC_ERR_OOM) throw;
+        pool.release();
+        state = {};
+      }
+    };
+    where_it_fits(H.ozp_pool, H.ozp, [&] { init_p2p_oz(H); });
+    where_it_fits(H.ozm_pool, H.ozm, [&] { init_m2l_oz(H, tmp); });
     FMMPC_CUDA(cudaStreamSynchronize(H.stream));
   } catch (...) {
     cudaStreamSynchronize(H.stream);
@@ -106,6 +118,27 @@ void setup(fmmpc_handle &H, const fmmpc_grid &g, const fmmpc_params &p) {
   }
   tmp.release();
   H.t_setup_ms = std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count();
+}
+
+// Gives back the operands of the FP64 form's digit kernels when an allocation of the handle fails: the
+// CUDA-core kernels take over.  False if there were none.
+bool drop_digit_kernels(fmmpc_handle &H) {
+  if (H.ozp_pool.ptrs.empty() && H.ozm_pool.ptrs.empty()) return false;
+  cudaStreamCaptureStatus cap{};
+  if (cudaStreamIsCapturing(H.stream, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone ||
+      cudaStreamSynchronize(H.stream) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  for (auto &e : H.gcache) cudaGraphExecDestroy(e.exec);  // captured graphs hold them, as do
+  H.gcache.clear();
+  clear_solve_graphs(H);
+  ++H.ws_gen;  // batch graphs kept by another handle
+  H.ozp = {};
+  H.ozm = {};
+  H.ozp_pool.release();
+  H.ozm_pool.release();
+  return true;
 }
 
 void check_rhs(const fmmpc_handle *h, int32_t n_rhs) {
@@ -138,6 +171,8 @@ void release(fmmpc_handle *h) {
     if (h->ev[k]) cudaEventDestroy(h->ev[k]);
   if (h->kw.hbuf) cudaFreeHost(h->kw.hbuf);
   h->kpool.release();
+  h->ozp_pool.release();
+  h->ozm_pool.release();
   h->pool.release();
   delete h;
 }
@@ -153,6 +188,7 @@ int create_handle(fmmpc_handle **out, const fmmpc_grid &g, const fmmpc_params &p
     return set_global_error(FMMPC_ERR_OOM, "host allocation failed");
   }
   h->stream = (cudaStream_t)stream;
+  h->pool.make_room = h->kpool.make_room = [h] { return drop_digit_kernels(*h); };
   int rc = guarded(h, [&] {
     setup(*h, g, prm);
     return FMMPC_OK;
@@ -381,7 +417,7 @@ int fmmpc_query(const fmmpc_handle *h, int32_t what, int64_t *value) {
     case 8: *value = (int64_t)h->g.n * h->g.n; break;
     case 9: *value = h->st.count; break;
     case 10: *value = h->launches; break;
-    case 11: *value = (int64_t)(h->pool.bytes + h->kpool.bytes); break;
+    case 11: *value = (int64_t)(h->pool.bytes + h->kpool.bytes + h->ozp_pool.bytes + h->ozm_pool.bytes); break;
     case 12: {  // device-side error flags of the tensor-core kernels (bounded waits that gave up)
       int e = 0, e2 = 0;
       cudaStreamSynchronize(h->stream);

@@ -11,6 +11,7 @@
 
 #include <cstdint>
 #include <cstdio>
+#include <functional>
 #include <string>
 #include <vector>
 
@@ -46,6 +47,7 @@ inline void require(bool ok, const std::string &msg) {
 struct DevPool {
   std::vector<void *> ptrs;
   size_t bytes = 0;
+  std::function<bool()> make_room;  // gives back what its owner can do without; true if there was any
   DevPool() = default;
   DevPool(const DevPool &) = delete;
   DevPool &operator=(const DevPool &) = delete;
@@ -69,6 +71,7 @@ struct DevPool {
   }
   void *alloc(size_t nbytes) {
     void *p = try_alloc(nbytes);
+    if (!p && make_room && make_room()) p = try_alloc(nbytes);
     if (!p) throw Error(FMMPC_ERR_OOM, "cudaMalloc of " + std::to_string(nbytes) + " bytes failed");
     return p;
   }

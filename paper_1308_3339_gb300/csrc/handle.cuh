@@ -162,6 +162,8 @@ struct fmmpc_handle {
   std::string err;
   fmmpc::DevPool pool;      // lifetime of the handle
   fmmpc::DevPool kpool;     // Krylov workspace (grown on demand)
+  // operands of the FP64 form's digit kernels; without the memory for them the CUDA-core kernels run
+  fmmpc::DevPool ozp_pool, ozm_pool;
   fmmpc::TreeOut tree{};
   fmmpc::Lists lists{};
   fmmpc::FmmBufs fb{};

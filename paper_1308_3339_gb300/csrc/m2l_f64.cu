@@ -568,17 +568,17 @@ void init_m2l_oz(fmmpc_handle &H, DevPool &tmp) {
     idx[q] = make_int2(o[c] < 0 ? -1 : mat_of[o[c]], o[c + 1] < 0 ? -1 : mat_of[o[c + 1]]);
   }
   const size_t ibytes = (size_t)H.nrhs_max * 4 * rows * 128, nexp = (size_t)H.nrhs_max * rows;
-  T.img = H.pool.get<unsigned char>(ibytes);
+  T.img = H.ozm_pool.get<unsigned char>(ibytes);
   FMMPC_CUDA(cudaMemsetAsync(T.img, 0, ibytes, H.stream));
-  T.lexp = H.pool.get<int2>(nexp);
+  T.lexp = H.ozm_pool.get<int2>(nexp);
   k_ozm_fill<<<nblk(nexp), 256, 0, H.stream>>>((int64_t)nexp, T.lexp);
   FMMPC_LAUNCH_CHECK();
-  T.bmat = H.pool.get<unsigned char>(shifts.size() * 4 * 2 * W * 128);
-  T.tiles = H.pool.get<int2>(tiles.size());
-  T.shifts = H.pool.get<int4>(shifts.size());
+  T.bmat = H.ozm_pool.get<unsigned char>(shifts.size() * 4 * 2 * W * 128);
+  T.tiles = H.ozm_pool.get<int2>(tiles.size());
+  T.shifts = H.ozm_pool.get<int4>(shifts.size());
   T.part_stride = (int64_t)H.nrhs_max * g.ncell * p;
-  T.Lp = H.pool.get<double>((size_t)2 * T.nparts * T.part_stride);
-  T.err = H.pool.get<int>(1);
+  T.Lp = H.ozm_pool.get<double>((size_t)2 * T.nparts * T.part_stride);
+  T.err = H.ozm_pool.get<int>(1);
   double *dmats = tmp.get<double>(mats.size());
   int2 *didx = tmp.get<int2>(idx.size());
   FMMPC_CUDA(cudaMemcpyAsync(dmats, mats.data(), sizeof(double) * mats.size(), cudaMemcpyHostToDevice, H.stream));

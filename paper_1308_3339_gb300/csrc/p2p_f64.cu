@@ -491,10 +491,10 @@ void init_p2p_oz(fmmpc_handle &H) {
     T.part_n[p] = e - b;
   }
   const size_t nimg = (size_t)H.nrhs_max * OZ_S * T.rows * 64;
-  T.img = H.pool.get<uint16_t>(nimg);
+  T.img = H.ozp_pool.get<uint16_t>(nimg);
   FMMPC_CUDA(cudaMemsetAsync(T.img, 0, sizeof(uint16_t) * nimg, H.stream));
   const size_t nexp = (size_t)H.nrhs_max * T.rows;
-  T.lexp = H.pool.get<int2>(nexp);
+  T.lexp = H.ozp_pool.get<int2>(nexp);
   k_oz_fill<<<nblk(nexp), 256, 0, H.stream>>>((int64_t)nexp, T.lexp);  // padding leaves are empty
   FMMPC_LAUNCH_CHECK();
   const double cself = -0.5 * std::log(2.0) - 1.5 + 0.25 * PI;
@@ -508,7 +508,7 @@ void init_p2p_oz(fmmpc_handle &H) {
     for (auto d : {std::pair<int, int>{0, 0}, {1, 0}, {dm, dm}}) vmax = std::max(vmax, std::fabs(value(d.first, d.second)));
     int eb = 0;
     std::frexp(vmax, &eb);  // vmax < 2^eb
-    unsigned char *dB = H.pool.get<unsigned char>((size_t)no * OZ_S * OZ_BLK);
+    unsigned char *dB = H.ozp_pool.get<unsigned char>((size_t)no * OZ_S * OZ_BLK);
     k_oz_table<<<nblk((int64_t)no * 512), 256, 0, H.stream>>>(
         rows_of(T), no, T.nrows, eb, (const double *)(variant ? H.fb.table_lnh : H.fb.table), H.fb.Rn, H.fb.table_c0,
         H.fb.table_stride, dB);
@@ -517,8 +517,8 @@ void init_p2p_oz(fmmpc_handle &H) {
     T.eb[variant] = eb;
   }
   T.part_stride = (int64_t)H.nrhs_max * g.n * g.n;
-  if (T.nparts > 1) T.near = H.pool.get<double>((size_t)T.nparts * T.part_stride);
-  T.err = H.pool.get<int>(1);
+  if (T.nparts > 1) T.near = H.ozp_pool.get<double>((size_t)T.nparts * T.part_stride);
+  T.err = H.ozp_pool.get<int>(1);
   FMMPC_CUDA(cudaMemsetAsync(T.err, 0, sizeof(int), H.stream));
   raise_smem_limit(k_p2p_oz);
   T.enabled = true;

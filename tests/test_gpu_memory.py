@@ -1,0 +1,88 @@
+"""FP64 handles where device memory is short: the tensor-core kernels' operands are only taken where
+they fit, and given back when the handle needs the room."""
+import numpy as np
+import pytest
+
+import synth_inputs as S
+from conftest import check_close
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+MB = 1 << 20
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _cuda():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+
+
+def free_memory():
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    return torch.cuda.mem_get_info()[0]
+
+
+def make(n, nrhs):
+    from paper_1308_3339_gb300 import FmmPreconditioner
+    return FmmPreconditioner(n, p=10, precision="fp64", n_rhs=nrhs)
+
+
+@pytest.mark.parametrize("missing,near_fits", [(800, True), (1200, False)])
+def test_fp64_handle_without_room_for_the_digit_operands(missing, near_fits):
+    # 1024^2 x 32: the operands take 1.6 GB, 0.5 of them the near field's.  With part of that missing the handle
+    # is still made, as it was before there were such kernels, and gives the CUDA-core kernels' values.
+    n, nrhs = 1024, 32
+    r = torch.tensor(np.stack([S.random_field(n, 5), S.gaussian_mixture(n, 6)]), dtype=torch.float64, device="cuda")
+    start = free_memory()
+    P = make(n, nrhs)
+    full = start - free_memory()
+    z, near = P.apply(r).cpu().numpy(), P.apply_part("near", r).cpu().numpy()
+    assert P.query("tc_p2p") == 1
+    P.close()
+    hog = torch.empty(free_memory() - (full - missing * MB), dtype=torch.uint8, device="cuda")
+    try:
+        Q = make(n, nrhs)
+        assert Q.query("tc_p2p") == int(near_fits)
+        check_close("fp64 apply, operands missing", Q.apply(r).cpu().numpy(), z, 1e-13, 1e-12)
+        check_close("fp64 near, operands missing", Q.apply_part("near", r).cpu().numpy(), near, 1e-14, 1e-13)
+        assert Q.query("device_errors") == 0
+        Q.close()
+    finally:
+        del hog
+        free_memory()
+
+
+@pytest.mark.parametrize("use_graphs", [1, 2])
+def test_fp64_handle_gives_the_digit_operands_back_to_a_solve(use_graphs):
+    # room for the handle, but not for its Krylov workspace beside the operands: the solve takes theirs, also
+    # where the apply's graph, which holds them, was captured before
+    n, nrhs = 1024, 16
+    f = torch.tensor(np.stack([S.gaussian_mixture(n, 10 + k) for k in range(nrhs)]), dtype=torch.float64, device="cuda")
+    f = f.reshape(nrhs, n, n)
+    out, zero = torch.empty_like(f), torch.zeros_like(f)
+    opts = dict(u0=zero, method="fgmres", restart=6, rtol=1e-9, use_graphs=use_graphs)
+    P = make(n, nrhs)
+    z = P.apply(f, out=out).cpu().numpy()
+    held = P.query("device_bytes")
+    u, info = P.solve(f, **opts)
+    workspace = P.query("device_bytes") - held
+    ref = u.cpu().numpy()
+    P.close()
+    del u
+    Q = make(n, nrhs)
+    Q.apply(f, out=out)
+    assert Q.query("tc_p2p") == 1
+    torch.cuda.synchronize()
+    room = workspace - 300 * MB  # the blocks of the tensors freed above stay cached for the solve's
+    hog = torch.empty(torch.cuda.mem_get_info()[0] - room, dtype=torch.uint8, device="cuda")
+    try:
+        v, info2 = Q.solve(f, **opts)
+        assert Q.query("tc_p2p") == 0 and info2["status"] == 0 and info2["iters"] == info["iters"]
+        check_close("solve after giving back", v.cpu().numpy(), ref, 1e-8, 1e-8)
+        check_close("apply after giving back", Q.apply(f, out=out).cpu().numpy(), z, 1e-13, 1e-12)
+        Q.close()
+    finally:
+        del hog
+        free_memory()
