@@ -328,3 +328,40 @@ def test_first_apply_bc_does_not_wait_for_its_stream():
                 assert not before.query()  # the call came back ahead of the work before it
             st.synchronize()
             P.close()
+
+
+@pytest.mark.parametrize("prec,nrhs", [("fp32", 1), ("mixed_tf32", 3), ("fp64", 2)])
+def test_folded_boundary_solve_of_two_rows(prec, nrhs):
+    # n = 4, one leaf: folded blocks of 2 x 2, whose rows hold no 16-byte column of the two-word kernel
+    test_folded_boundary_solve_matches_oracle(4, prec, nrhs)
+
+
+def test_fp64_tensor_core_m2l_in_the_far_corner_of_a_small_quadrant():
+    # weights 12 decades smaller in one quadrant: its far corner relative to its own values (FP64 form's bar)
+    from paper_1308_3339_gb300 import FmmPreconditioner
+    n = 256
+    f = S.random_field(n, 90)
+    f.reshape(n, n)[n // 2:, n // 2:] *= 1e-12
+    P = FmmPreconditioner(n, p=12, precision="fp64")
+    vr = P.apply_part("vr", dev(f)).cpu().numpy().reshape(n, n)
+    ref = O.Problem(n, p=12).apply(f, "fmm", stages=True)["vr"].reshape(n, n)
+    corner = np.s_[7 * n // 8:, 7 * n // 8:]
+    check_close("fp64 vr, far corner", vr[corner], ref[corner], 1e-12, 1e-12)
+    P.close()
+
+
+@pytest.mark.parametrize("n,theta", [(128, 0.4), (1024, 0.333)])
+@pytest.mark.parametrize("mantissa", [2 ** 53 - 1, int("11111111 011111111 011111111 011111111 011111111 011111111".replace(" ", ""), 2)])
+def test_fp64_tensor_core_near_field_of_constant_weights(n, theta, mantissa):
+    # equal weights of one sign, just below a power of two, or with every digit at 255: the largest L1 bound (61
+    # offsets in one part at theta = 0.333) and digit sums past 2^24 in the last orders.  The two engines differ
+    # by the rounding of sums of 61 x 64 terms.
+    from paper_1308_3339_gb300 import FmmPreconditioner
+    P = FmmPreconditioner(n, p=8, theta=theta, precision="fp64")
+    assert P.query("stencil") == (37 if theta == 0.4 else 61)
+    r = np.full(n * n, mantissa / 2.0 ** 53 / P.h ** 2)
+    a = P.apply_part("near", dev(r)).cpu().numpy()
+    P.set_p2p_engine("simt")
+    b = P.apply_part("near", dev(r)).cpu().numpy()
+    check_close(f"fp64 near, constant weights n={n}", a, b, 1e-14, 1e-13)
+    P.close()
