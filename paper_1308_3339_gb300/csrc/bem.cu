@@ -304,14 +304,14 @@ void init_bem_dl(fmmpc_handle &H) {
 
 // 1/2 I + K in the folded form, the boundary data term of Eq. e:ubound, for apply_bc; formed
 // on its first call, in the stream's order and without a wait.  Summing the 16 n^2 atan2 of K g
-// directly took 1160 us at n = 1024; the 3 n^2 multiply-adds of the folded form take 9 us.  Not
-// formed while the handle's stream is being captured (a later call forms it), nor where there is
-// no memory for it (then for good): the caller sums directly.
+// directly took 1160 us at n = 1024; the 3 n^2 multiply-adds of the folded form take 9 us.  The
+// handle's stream is not being captured.  Not formed where there is no memory for it (then for good):
+// the caller sums directly.
 void init_bem_bc(fmmpc_handle &H) {
   if (H.Kbc || H.no_bc_tables) return;
   const int n = H.g.n;
   const size_t nt = (size_t)(n / 2) * H.g.NG, nv = (size_t)H.g.NG * H.nrhs_max;
-  double *T = static_cast<double *>(H.pool.try_alloc(sizeof(double) * (nt + 2 * nv)));
+  double *T = static_cast<double *>(H.pool.try_alloc_beside_captures(sizeof(double) * (nt + 2 * nv)));
   if (!T) {
     H.no_bc_tables = true;
     return;

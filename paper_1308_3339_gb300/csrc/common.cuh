@@ -52,21 +52,27 @@ struct DevPool {
   DevPool(const DevPool &) = delete;
   DevPool &operator=(const DevPool &) = delete;
   ~DevPool() { release(); }
-  // nullptr where the memory is not there.  An allocation waits for nothing and belongs to no stream, so
-  // it is let through while some stream of the process is being captured, which it would else end.
+  // nullptr where the memory is not there
   void *try_alloc(size_t nbytes) {
     void *p = nullptr;
     if (nbytes == 0) nbytes = 16;
-    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
-    cudaThreadExchangeStreamCaptureMode(&mode);
     const cudaError_t e = cudaMalloc(&p, nbytes);
-    cudaThreadExchangeStreamCaptureMode(&mode);
     if (e != cudaSuccess) {
       cudaGetLastError();
       return nullptr;
     }
     ptrs.push_back(p);
     bytes += nbytes;
+    return p;
+  }
+  // The same while some other stream of the process is being captured: an allocation waits for nothing and
+  // belongs to no stream, but is refused then, and ends the capture.  For callers that know that their
+  // own stream is not being captured: set-up work must not end up in the caller's graph.
+  void *try_alloc_beside_captures(size_t nbytes) {
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    void *p = try_alloc(nbytes);
+    cudaThreadExchangeStreamCaptureMode(&mode);
     return p;
   }
   void *alloc(size_t nbytes) {

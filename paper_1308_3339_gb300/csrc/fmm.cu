@@ -2722,12 +2722,13 @@ void form_near(fmmpc_handle &H) {
 
 }  // namespace
 
-// The near double layer's operator, on first use; false where there is no memory for it.
+// The near double layer's operator, on first use, while the handle's stream is not being captured; false
+// where there is no memory for it.
 bool init_bnd_dl(fmmpc_handle &H) {
   const int64_t nent = H.lists.n_p2p_vb * (int64_t)H.g.m * H.g.m * H.g.m;
   if (H.fb.kdl || nent <= 0 || H.lists.nbnear <= 0) return true;
   const bool f64 = H.prec == FMMPC_PREC_FP64;
-  void *K = H.pool.try_alloc((f64 ? sizeof(double) : sizeof(float)) * (size_t)nent);
+  void *K = H.pool.try_alloc_beside_captures((f64 ? sizeof(double) : sizeof(float)) * (size_t)nent);
   if (!K) return false;
   if (f64)
     k_bnd_near_mat<double, 2><<<(unsigned)H.lists.nbnear, 256, 0, H.stream>>>(

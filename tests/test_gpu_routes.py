@@ -365,3 +365,43 @@ def test_fp64_tensor_core_near_field_of_constant_weights(n, theta, mantissa):
     b = P.apply_part("near", dev(r)).cpu().numpy()
     check_close(f"fp64 near, constant weights n={n}", a, b, 1e-14, 1e-13)
     P.close()
+
+
+SET_UP_UNDER_CAPTURE = """
+import torch
+from paper_1308_3339_gb300 import FmmPreconditioner, FmmpcError
+n = 64
+f = torch.rand(n * n, dtype=torch.float64, device="cuda")
+st = torch.cuda.Stream()
+with torch.cuda.stream(st):
+    P = FmmPreconditioner(n, p=8, precision="fp32", stream=st)
+    st.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    graph.capture_begin()
+    try:
+        P.set_operator("q1")
+        print("accepted")
+    except FmmpcError:
+        print("refused")
+    try:
+        graph.capture_end()
+    except RuntimeError:
+        pass
+    st.synchronize()
+    P.set_operator("q1")
+    u, _ = P.solve(f, method="cg")
+    Q = FmmPreconditioner(n, p=8, precision="fp32", stream=st)
+    Q.set_operator("q1")
+    v, _ = Q.solve(f, method="cg")
+    st.synchronize()
+    print("same" if torch.equal(u, v) else "different")
+"""
+
+
+def test_set_up_work_stays_out_of_a_capture_of_the_handles_stream():
+    # an operator's tables cannot be formed while the handle's own stream is being captured: refused, and
+    # formed when asked for afterwards (a process of its own: the capture that was ended stays behind)
+    import subprocess
+    import sys
+    out = subprocess.run([sys.executable, "-c", SET_UP_UNDER_CAPTURE], capture_output=True, text=True, timeout=120)
+    assert out.stdout.split() == ["refused", "same"], out.stdout + out.stderr[-2000:]
