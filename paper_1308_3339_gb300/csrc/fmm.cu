@@ -484,7 +484,6 @@ __device__ __forceinline__ void m2l_accum_half(cpx<R> (&H)[P / 2], const cpx<R> 
   }
 }
 
-// warp-reduce H, scale by (-1)^n/n!, then store (add = 0) or accumulate (add = 1)
 // Offset between a volume and a boundary cell centre in cell units, d * scale with
 // scale = 1 / (rho 2^(L+1)) and d an integer in those fine units.  When the scale is a power
 // of two and |d| < 2^24 the FP32 product is exact and equals the FP64 one rounded to FP32,
@@ -516,36 +515,31 @@ __device__ __forceinline__ R scaled_offset(int64_t d, const OffsetScale &o) {
   return (R)((double)d * o.s64);
 }
 
+// warp-reduce H, scale by (-1)^n/n!, store
 template <typename R, int P>
-__device__ __forceinline__ void m2l_finish(cpx<R> (&H)[P], int lane, cpx<R> *__restrict__ out, int add) {
+__device__ __forceinline__ void m2l_finish(cpx<R> (&H)[P], int lane, cpx<R> *__restrict__ out) {
   R f = 1;
 #pragma unroll
   for (int n = 0; n < P; ++n) {
     if (n > 0) f = -f / R(n);
     R re = warp_sum(H[n].re), im = warp_sum(H[n].im);
-    if (lane == 0) {
-      cpx<R> v = mk(f * re, f * im);
-      out[n] = add ? out[n] + v : v;
-    }
+    if (lane == 0) out[n] = mk(f * re, f * im);
   }
 }
 
-// Volume targets: warp per (cell, rhs).  do_vol: volume sources from the M2L list;
-// do_bnd: boundary sources from the volume-boundary list; add: accumulate into L.
-// cells (optional): only the listed cells (ntgt of them) instead of all ncell.
+// Volume targets: warp per (cell, rhs), volume sources from the M2L list.  do_bnd: boundary sources from the
+// volume-boundary list too (trees of fewer than three levels; deeper ones keep them apart, k_m2l_vbv).
 template <typename R, int P>
-__global__ void k_m2l_vol(GeoDev gd, int64_t ncell, int64_t nbcell, int nrhs, int do_vol, int do_bnd, int add,
+__global__ void k_m2l_vol(GeoDev gd, int64_t ncell, int64_t nbcell, int nrhs, int do_bnd,
                           const int32_t *__restrict__ first, const int32_t *__restrict__ src,
                           const int32_t *__restrict__ bfirst, const int32_t *__restrict__ bsrc,
                           const cpx<R> *__restrict__ Mv, const cpx<R> *__restrict__ Mb,
-                          cpx<R> *__restrict__ Lv, const int32_t *__restrict__ cells = nullptr,
-                          int64_t ntgt = 0) {
+                          cpx<R> *__restrict__ Lv) {
   const int64_t wid = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
-  const int64_t nt = cells ? ntgt : ncell;
-  if (wid >= nt * nrhs) return;
-  const int rhs = (int)(wid / nt);
-  const int64_t gidx = cells ? (int64_t)cells[wid % nt] : wid % nt;
+  if (wid >= ncell * nrhs) return;
+  const int rhs = (int)(wid / ncell);
+  const int64_t gidx = wid % ncell;
   int l = 0;
   while (level_offset(l + 1) <= gidx) ++l;
   const uint32_t c = (uint32_t)(gidx - level_offset(l));
@@ -556,14 +550,12 @@ __global__ void k_m2l_vol(GeoDev gd, int64_t ncell, int64_t nbcell, int nrhs, in
   cpx<R> H[P];
 #pragma unroll
   for (int k = 0; k < P; ++k) H[k] = mk<R>(0, 0);
-  if (do_vol) {
-    const cpx<R> *M = Mv + (int64_t)rhs * ncell * P + level_offset(l) * P;
-    for (int e = first[gidx] + lane; e < first[gidx + 1]; e += 32) {
-      const uint32_t s = (uint32_t)src[e];
-      int sx, sy;
-      morton_decode(s, sx, sy);
-      m2l_accum<R, P>(H, M + (int64_t)s * P, mk<R>((R)(tx - sx), (R)(ty - sy)), lnrho);
-    }
+  const cpx<R> *M = Mv + (int64_t)rhs * ncell * P + level_offset(l) * P;
+  for (int e = first[gidx] + lane; e < first[gidx + 1]; e += 32) {
+    const uint32_t s = (uint32_t)src[e];
+    int sx, sy;
+    morton_decode(s, sx, sy);
+    m2l_accum<R, P>(H, M + (int64_t)s * P, mk<R>((R)(tx - sx), (R)(ty - sy)), lnrho);
   }
   if (do_bnd) {
     int64_t X, Y, sw;
@@ -580,7 +572,7 @@ __global__ void k_m2l_vol(GeoDev gd, int64_t ncell, int64_t nbcell, int nrhs, in
                       mk<R>(scaled_offset<R>(X - BX, scale), scaled_offset<R>(Y - BY, scale)), lnrho);
     }
   }
-  m2l_finish<R, P>(H, lane, Lv + (int64_t)rhs * ncell * P + gidx * P, add);
+  m2l_finish<R, P>(H, lane, Lv + (int64_t)rhs * ncell * P + gidx * P);
 }
 
 // Boundary sources added to volume locals, for the cells that have them (cells[0, ntgt)):
@@ -788,29 +780,23 @@ __global__ void k_m2l_bnd(GeoDev gd, int64_t ncell, int64_t nbcell, int nrhs,
     m2l_accum<R, P>(H, M + (int64_t)v * P,
                     mk<R>(scaled_offset<R>(BX - X, scale), scaled_offset<R>(BY - Y, scale)), lnrho);
   }
-  m2l_finish<R, P>(H, lane, Lb + (int64_t)rhs * nbcell * P + gb * P, 0);
+  m2l_finish<R, P>(H, lane, Lb + (int64_t)rhs * nbcell * P + gb * P);
   // the four side roots also take the ln h part of G times the total volume weight
   if (gb < 4 && lane == 0)
     Lb[(int64_t)rhs * nbcell * P + gb * P].re += (R)(lnh * (double)Mv[(int64_t)rhs * ncell * P].re);
 }
 
 // ------------------------------------------------------------------ root constants
-// The ln h part of G times the total weight, added to the root local expansions.
-// mode 0: boundary roots += ln h W_vol (pass A); 1: volume root += ln h W_vol;
-// 2: volume root += ln h (W_vol + W_bnd).
+// The ln h part of G times the total weight (volume, and boundary with with_bnd), added to the volume root's
+// local expansion (the side roots' is added in the boundary M2L).
 template <typename R>
-__global__ void k_root_const(int p, int64_t ncell, int64_t nbcell, int nrhs, double lnh, int mode,
-                             const cpx<R> *__restrict__ Mv, const cpx<R> *__restrict__ Mb,
-                             cpx<R> *__restrict__ Lv, cpx<R> *__restrict__ Lb) {
+__global__ void k_root_const(int p, int64_t ncell, int64_t nbcell, int nrhs, double lnh, int with_bnd,
+                             const cpx<R> *__restrict__ Mv, const cpx<R> *__restrict__ Mb, cpx<R> *__restrict__ Lv) {
   for (int rhs = threadIdx.x; rhs < nrhs; rhs += blockDim.x) {
     double W = (double)Mv[(int64_t)rhs * ncell * p].re;
-    if (mode == 0) {
-      for (int s = 0; s < 4; ++s) Lb[(int64_t)rhs * nbcell * p + (int64_t)s * p].re += (R)(lnh * W);
-    } else {
-      if (mode == 2)
-        for (int s = 0; s < 4; ++s) W += (double)Mb[(int64_t)rhs * nbcell * p + (int64_t)s * p].re;
-      Lv[(int64_t)rhs * ncell * p].re += (R)(lnh * W);
-    }
+    if (with_bnd)
+      for (int s = 0; s < 4; ++s) W += (double)Mb[(int64_t)rhs * nbcell * p + (int64_t)s * p].re;
+    Lv[(int64_t)rhs * ncell * p].re += (R)(lnh * W);
   }
 }
 
@@ -1992,7 +1978,7 @@ __global__ void __launch_bounds__(256, P <= 10 && M <= 8 ? (sizeof(R) == 8 ? 3 :
 #pragma unroll
         for (int e = 0; e < NPT; ++e) o[e * rstep] = (sn[e] + far[e]) * NEG_INV_2PI;
       } else {
-        // the parts often cancel, so they are added as a two-word FP32 sum (TwoSum) and scaled by
+        // the two parts often cancel, so they are added as a two-word FP32 sum (TwoSum) and scaled by
         // -1/(2 pi) in two-word arithmetic, the far term added, and the two-word result converted
         // to FP64 with one FP64 addition (FP64 is scarce here)
         float sl[NPT];
@@ -2000,10 +1986,6 @@ __global__ void __launch_bounds__(256, P <= 10 && M <= 8 ? (sizeof(R) == 8 ? 3 :
         for (int e = 0; e < NPT; ++e) {
           sl[e] = 0.0f;
           two_sum_acc(sn[e], sl[e], sm[e]);
-        }
-        for (int q = 2; q < np; ++q) {
-#pragma unroll
-          for (int e = 0; e < NPT; ++e) two_sum_acc(sn[e], sl[e], nearp[q * nstride + off + e * rstep]);
         }
 #pragma unroll
         for (int e = 0; e < NPT; ++e) o[e * rstep] = near_far_sum(sn[e], sl[e], far[e]);
@@ -2210,7 +2192,7 @@ void run_downward(fmmpc_handle &H, double *out, int nrhs, int do_bnd, int with_b
   constexpr bool f64 = std::is_same<R, double>::value;
   const R *nearp = nullptr;
   if (tc_near) nearp = (const R *)(f64 ? (const void *)(H.ozp.nparts > 1 ? H.ozp.near : out) : (const void *)H.tcp.near);
-  const int np = f64 ? H.ozp.nparts : H.tcp.nparts;
+  const int np = f64 ? H.ozp.nparts : 2;
   const int64_t nstride = f64 ? H.ozp.part_stride : H.tcp.part_stride;
   const int32_t *vslot = sep ? H.lists.vbv_slot : nullptr;
   const cpx<R> *Lsep = (const cpx<R> *)H.fb.Lvb;
@@ -2373,8 +2355,8 @@ void apply_impl(fmmpc_handle &H, int part, const double *r, double *out, int nrh
     } else if (f64 && H.ozm.enabled) {
       launches += run_m2l_oz(H, Mv, Lv, nrhs, st);
     } else {
-      k_m2l_vol<R, P><<<nblk(g.ncell * nrhs * 32), 256, 0, st>>>(gd, g.ncell, g.nbcell, nrhs, 1,
-                                                                with_bnd && !vbv_sep ? 1 : 0, 0, Ls.m2l_first,
+      k_m2l_vol<R, P><<<nblk(g.ncell * nrhs * 32), 256, 0, st>>>(gd, g.ncell, g.nbcell, nrhs,
+                                                                with_bnd && !vbv_sep ? 1 : 0, Ls.m2l_first,
                                                                 Ls.m2l_src, Ls.vbv_first, Ls.vbv_src, Mv, Mb, Lv);
       FMMPC_LAUNCH_CHECK();
       ++launches;
@@ -2533,7 +2515,7 @@ void apply_impl(fmmpc_handle &H, int part, const double *r, double *out, int nrh
   mark(6);
   if (vbv_sep && !side) run_vbv_sep();
   if (g.L < 2) {  // else the downward kernel adds the root constant
-    k_root_const<R><<<1, 32, 0, s>>>(P, g.ncell, g.nbcell, nrhs, g.lnh, with_bnd ? 2 : 1, Mv, Mb, Lv, Lb);
+    k_root_const<R><<<1, 32, 0, s>>>(P, g.ncell, g.nbcell, nrhs, g.lnh, with_bnd ? 1 : 0, Mv, Mb, Lv);
     FMMPC_LAUNCH_CHECK();
     launches += 1;
   }

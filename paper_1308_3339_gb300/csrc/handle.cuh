@@ -58,7 +58,6 @@ struct TcP2P {
   uint16_t *ahi = nullptr, *alo = nullptr;        // FP16 weight strips (scaled), hi and lo words
   uint16_t *bmat = nullptr, *bmat_lnh = nullptr;  // FP16 kernel tables, hi and lo words
   float *near = nullptr;                     // [part][nrhs][n][n] the two parts of the near-field sum, FP32
-  int nparts = 2;
   int64_t part_stride = 0;
   float *lsc = nullptr;                      // [nrhs][NLY][NLX] 2^-e of each leaf's FP16 weights
   int *err = nullptr;

@@ -1809,13 +1809,11 @@ void build_chain(fmmpc_handle &H, cudaGraph_t G, int method, int m, int nrhs, bo
   }
   cudaStream_t cs = H.cstream;
   const int64_t N = (int64_t)H.g.n * H.g.n, NR = N * nrhs, vs = N * H.nrhs_max;
-  const double s = 1.0 / (H.g.h * H.g.h);
   const bool flexible = method == FMMPC_FGMRES;
   GmState st = gm_state(K);
   int *ctl = K.g_ctl;
   cudaGraphConditionalHandle hloop;
   FMMPC_CUDA(cudaGraphConditionalHandleCreate(&hloop, G, 0, cudaGraphCondAssignDefault));
-  Ctx c{H, N, nrhs, cs};
   const OpDev od = op_of(H);
   auto precond = [&](const double *in, double *out, double *scratch) {
     precond_op(H, in, out, scratch, nrhs, true);
@@ -1832,7 +1830,6 @@ void build_chain(fmmpc_handle &H, cudaGraph_t G, int method, int m, int nrhs, bo
   // ---- set-up
   const std::vector<cudaGraphNode_t> none;
   auto f_init = capture_into(H, cs, G, none, [&] {
-    c.s = H.stream;
     k_fold_rhs<<<nblk(NR), 256, 0, H.stream>>>(od, NR, K.fin, has_g ? K.gin : nullptr, K.b);
     k_gbnorm<<<rgrid, rth, 0, H.stream>>>(ctl, N, st, K.b, K.part, K.g_cnt);
     FMMPC_LAUNCH_CHECK();
@@ -1862,7 +1859,6 @@ void build_chain(fmmpc_handle &H, cudaGraph_t G, int method, int m, int nrhs, bo
     // condition (no IF node): z = P^{-1} r, beta, p = z + beta p, q = A p with alpha, then
     // x, r and the test
     capture_into(H, cs, step, none, [&] {
-      c.s = H.stream;
       precond(K.r, z, K.zin);
       k_cgf_rz<<<rgrid, rth, 0, H.stream>>>(N, st, K.r, z, K.part, K.g_cnt, rz_old);
       k_cg_p<<<nblk(NR), 256, 0, H.stream>>>(N, nrhs, K.g_sc, z, p);
@@ -1872,7 +1868,6 @@ void build_chain(fmmpc_handle &H, cudaGraph_t G, int method, int m, int nrhs, bo
       FMMPC_LAUNCH_CHECK();
     });
     capture_into(H, cs, body, {n_steps}, [&] {
-      c.s = H.stream;
       residual(Check{});
     });
   } else {
@@ -1882,7 +1877,6 @@ void build_chain(fmmpc_handle &H, cudaGraph_t G, int method, int m, int nrhs, bo
     });
     cudaGraphNode_t n_steps = add_conditional(body, f_begin, hsteps, cudaGraphCondTypeWhile, &step);
     capture_into(H, cs, step, none, [&] {
-      c.s = H.stream;
       precond(K.t, K.zin, K.t);  // K.t holds v_j (written with V_j by the previous step)
       // w = A z_j with the first CGS pass, the first update with the second pass, the second
       // update with |w|^2: three sweeps over the basis, each reduction finished in its grid's
@@ -1897,7 +1891,6 @@ void build_chain(fmmpc_handle &H, cudaGraph_t G, int method, int m, int nrhs, bo
       FMMPC_LAUNCH_CHECK();
     });
     capture_into(H, cs, body, {n_steps}, [&] {
-      c.s = H.stream;
       if (flexible) {
         k_gmaxpy<<<nblk(NR), 256, 0, H.stream>>>(ctl, N, nrhs, K.Z, vs, K.scal, K.x);
       } else {

@@ -22,26 +22,22 @@
 #include <complex>
 #include <vector>
 
-#include <cuda_fp16.h>
-
 #include "handle.cuh"
+#include "oz.cuh"
 #include "tc.cuh"
 
 namespace fmmpc {
 
 namespace {
 
-constexpr int OZ_S = 7;
 constexpr int OZM_WROWS = 144;  // window: 128 targets, shifts of -4 .. 4, alignment
 constexpr int OZM_WPAIR = OZM_WROWS * 128;  // one digit pair's window
 constexpr int OZM_WBYTES = 4 * OZM_WPAIR;
 constexpr int OZM_NWIN = 2;
 constexpr int OZM_TAIL = 384;   // zero rows after each sub-image
-constexpr int OZM_LSB = 56;
 constexpr int OZM_MAXPART = 4;
 constexpr int OZM_MAXSH = 255;
 constexpr int OZM_THREADS = 352;  // window producer, MMA issuer, eight epilogue warps, B producer
-constexpr int OZ_NONE = -(1 << 20), OZ_NAN = 1 << 20;
 
 template <int W>
 struct OzmShape {
@@ -69,15 +65,6 @@ struct OzmArgs {
   int p, n;
 };
 
-__host__ __device__ __forceinline__ void ozm_digits(long long X, int (&d)[OZ_S]) {
-#pragma unroll
-  for (int i = OZ_S - 1; i > 0; --i) {
-    d[i] = (int)((X + 256) & 511) - 256;
-    X = (X - d[i]) >> 9;
-  }
-  d[0] = (int)X;
-}
-
 // power-of-two scale of coefficient k
 __host__ __device__ __forceinline__ int ozm_col(int k) {
   int lg = 0;
@@ -102,25 +89,17 @@ __global__ void k_m2l_oz_pack(OzmArgs a, int nrhs, int64_t ncell_lo, int64_t nce
   for (int q = 0; q < 8; ++q) {
     const int v = 8 * (c & 3) + q;
     x[q] = v < 2 * a.p && in ? ldexp(M[v], ozm_col(v >> 1)) : 0.0;
-    mx = max(mx, (unsigned long long)__double_as_longlong(x[q]) & 0x7fffffffffffffffull);
+    mx = max(mx, oz_bits(x[q]));
   }
 #pragma unroll
   for (int o = 1; o < 4; o <<= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-  const int em = max((int)(mx >> 52), 1);
+  const int em = oz_biased(mx);
   uint32_t pk[4][4];  // [pair][two digits a word]
   float l1 = 0.0f;
 #pragma unroll
   for (int q = 0; q < 8; ++q) {
-    const unsigned long long u = (unsigned long long)__double_as_longlong(x[q]);
-    const int ex = (int)(u >> 52) & 0x7ff;
-    const long long mant = (long long)((u & 0xfffffffffffffull) | (ex ? 0x10000000000000ull : 0ull));
-    const int sh = 9 - (em - max(ex, 1));
-    long long X = sh >= 0 ? mant << sh : (sh > -60 ? (mant + (1ll << (-sh - 1))) >> -sh : 0);
-    if (em == 0x7ff) X = 0;
-    l1 += __ll2float_ru(X);
-    if (u >> 63) X = -X;
     int d[OZ_S];
-    ozm_digits(X, d);
+    oz_digits(oz_fixed(x[q], em, l1), d);
 #pragma unroll
     for (int pr = 0; pr < 4; ++pr) {
       const int dg = (c >> 2) ? (2 * pr + 1 < OZ_S ? d[2 * pr + 1 < OZ_S ? 2 * pr + 1 : 0] : 0) : d[2 * pr];
@@ -139,9 +118,7 @@ __global__ void k_m2l_oz_pack(OzmArgs a, int nrhs, int64_t ncell_lo, int64_t nce
   const int P = a.lev_P[l], q = (cx & 1) + 2 * (cy & 1);
   const int64_t f = (int64_t)((cy >> 1) + 4) * P + (cx >> 1) + 4;
   const int64_t row = a.lev_row0[l] + (int64_t)q * ((int64_t)P * P + OZM_TAIL) + f;
-  if (c == 0)
-    lexp[rhs * a.rows + row] = make_int2(mx == 0 ? OZ_NONE : (em == 0x7ff ? OZ_NAN : em - 1022),
-                                         __float_as_int(l1 * (0x1p-62f * 1.00001f)));
+  if (c == 0) lexp[rhs * a.rows + row] = oz_group(mx, em, l1);
 #pragma unroll
   for (int pr = 0; pr < 4; ++pr)
     reinterpret_cast<uint4 *>(img + ((rhs * 4 + pr) * a.rows + row) * 128)[c ^ (int)(f & 7)] =
@@ -284,12 +261,9 @@ __global__ void __launch_bounds__(OZM_THREADS, 1) k_m2l_oz(OzmArgs a) {
     for (int j = 0; j < ns; ++j) {
       const int4 g = ssh[j];
       if (!((g.w >> (1 + h)) & 1)) continue;  // not in this class's lists
-      const int2 v = __ldg(le + (int64_t)g.x * sub + g.y * P + g.z);
-      const int e = max(emax, v.x);
-      l1 = l1 * exp2f((float)max(emax - e, -200)) + __int_as_float(v.y) * exp2f((float)max(v.x - e, -200));
-      emax = e;
+      oz_bound(__ldg(le + (int64_t)g.x * sub + g.y * P + g.z), emax, l1);
     }
-    const int lsb = min(OZM_LSB, 60 - max(ilogbf(fmaxf(l1, 1.0f)), 0));
+    const int lsb = oz_unit(l1);
     long long acc[W];
 #pragma unroll
     for (int i = 0; i < W; ++i) acc[i] = 0;
@@ -298,7 +272,7 @@ __global__ void __launch_bounds__(OZM_THREADS, 1) k_m2l_oz(OzmArgs a) {
     for (int j = 0; j < ns; ++j) {
       const int4 g = ssh[j];
       const bool mine = (g.w >> (1 + h)) & 1;  // else its sums are zero
-      const int d = mine ? min(emax - __ldg(le + (int64_t)g.x * sub + g.y * P + g.z).x + OZM_LSB - lsb, 62) : 62;
+      const int d = mine ? min(emax - __ldg(le + (int64_t)g.x * sub + g.y * P + g.z).x + OZ_LSB - lsb, 62) : 62;
       const long long half = d > 0 ? 1ll << (d - 1) : 0;
       int tl[W];
       if (!__all_sync(0xffffffffu, tc::mbar_wait(&acc_full[0], j & 1, &abort_flag))) { ok = false; break; }
@@ -310,10 +284,7 @@ __global__ void __launch_bounds__(OZM_THREADS, 1) k_m2l_oz(OzmArgs a) {
         tc::tmem_ld8(tb + N * 5 + 8 * c, v5);
         tc::tmem_ld8(tb + N * 4 + 8 * c, v4);
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
-          const int s6 = __float2int_rn(v6[i]), s5 = __float2int_rn(v5[i]), s4 = __float2int_rn(v4[i]);
-          tl[8 * c + i] = s4 * 16 + ((s5 + ((s6 + 256) >> 9) + 16) >> 5);
-        }
+        for (int i = 0; i < 8; ++i) tl[8 * c + i] = oz_join_low(v4[i], v5[i], v6[i]);
       }
       tc::fence_before();
       __syncwarp();
@@ -328,14 +299,7 @@ __global__ void __launch_bounds__(OZM_THREADS, 1) k_m2l_oz(OzmArgs a) {
         tc::tmem_ld8(tb + 2 * N + 8 * c, v2);
         tc::tmem_ld8(tb + 3 * N + 8 * c, v3);
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
-          long long t = (long long)tl[8 * c + i];
-          t += (long long)__float2int_rn(v3[i]) * (1 << 13);
-          t += (long long)__float2int_rn(v2[i]) * (1 << 22);
-          t += (long long)__float2int_rn(v1[i]) * (1ll << 31);
-          t += (long long)__float2int_rn(v0[i]) * (1ll << 40);
-          acc[8 * c + i] += (t + half) >> d;
-        }
+        for (int i = 0; i < 8; ++i) acc[8 * c + i] += (oz_join(tl[8 * c + i], v0[i], v1[i], v2[i], v3[i]) + half) >> d;
       }
       tc::fence_before();
       __syncwarp();
@@ -409,7 +373,7 @@ __global__ void k_ozm_table(OzmArgs a, int ns, const int2 *__restrict__ idx, con
   for (int j = 0; j < 8; ++j) {
     const int v = 8 * vc + j;
     int d[OZ_S];
-    ozm_digits(used && v < p2 ? __double2ll_rn(ldexp(x[v], 62 - a.rb[u])) : 0, d);
+    oz_digits(used && v < p2 ? __double2ll_rn(ldexp(x[v], 62 - a.rb[u])) : 0, d);
 #pragma unroll
     for (int e = 0; e < 8; ++e) {
       const uint32_t hv = __half_as_ushort(__int2half_rn(e < OZ_S ? d[e < OZ_S ? e : 0] : 0));
@@ -421,11 +385,6 @@ __global__ void k_ozm_table(OzmArgs a, int ns, const int2 *__restrict__ idx, con
   for (int e = 0; e < 8; ++e)  // digit e: row set e / 2, columns 32 (e % 2) ..
     reinterpret_cast<uint4 *>(bmat + ((int64_t)q * 4 + e / 2) * 2 * W * 128 + row * 128)[(vc + 4 * (e & 1)) ^ (row & 7)] =
         make_uint4(pk[e][0], pk[e][1], pk[e][2], pk[e][3]);
-}
-
-__global__ void k_ozm_fill(int64_t total, int2 *__restrict__ le) {
-  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t < total) le[t] = make_int2(OZ_NONE, 0);
 }
 
 inline unsigned nblk(int64_t n, int t = 256) { return (unsigned)((n + t - 1) / t); }
@@ -571,7 +530,7 @@ void init_m2l_oz(fmmpc_handle &H, DevPool &tmp) {
   T.img = H.ozm_pool.get<unsigned char>(ibytes);
   FMMPC_CUDA(cudaMemsetAsync(T.img, 0, ibytes, H.stream));
   T.lexp = H.ozm_pool.get<int2>(nexp);
-  k_ozm_fill<<<nblk(nexp), 256, 0, H.stream>>>((int64_t)nexp, T.lexp);
+  k_oz_fill<<<nblk(nexp), 256, 0, H.stream>>>((int64_t)nexp, T.lexp);
   FMMPC_LAUNCH_CHECK();
   T.bmat = H.ozm_pool.get<unsigned char>(shifts.size() * 4 * 2 * W * 128);
   T.tiles = H.ozm_pool.get<int2>(tiles.size());

@@ -30,25 +30,21 @@
 #include <cmath>
 #include <vector>
 
-#include <cuda_fp16.h>
-
 #include "handle.cuh"
+#include "oz.cuh"
 #include "tc.cuh"
 
 namespace fmmpc {
 
 namespace {
 
-constexpr int OZ_S = 7;            // digits
 constexpr int OZ_TILE = 128;       // flattened target leaves per CTA
 constexpr int OZ_BLK = 8192;       // one digit of one offset's table: 64 x 64 FP16
 constexpr int OZ_MAXB = 12;        // table block slots at most (7 in use, the rest ahead)
-constexpr int OZ_LSB = 56;         // unit 2^-56 of an offset's sum (at most 64 of unit operands: 2^62)
-constexpr int OZ_MAXOFS = 64;      // offsets per part at most: an L1 bound of 2^12, units of 2^-49 and finer
+constexpr int OZ_MAXOFS = 64;      // offsets per part at most: an L1 bound of about 2^12, units of 2^-48 and finer
 constexpr int OZ_MAXPART = 8;
 constexpr int OZ_MAXROWS = 33;
 constexpr int OZ_THREADS = 320;    // producer, MMA issuer, eight epilogue warps
-constexpr int OZ_NONE = -(1 << 20), OZ_NAN = 1 << 20;  // exponents of an empty and of a non-finite leaf
 
 struct OzArgs {
   const uint16_t *img;        // [nrhs][OZ_S][rows][64] digits, swizzled per row
@@ -57,26 +53,15 @@ struct OzArgs {
   double *out;                // [part][nrhs][n][n] near-field sums (unscaled)
   int64_t part_stride, rows;
   int *err;
-  int n, NL, P, R, eb, nbs, sh, nparts, nsr, vec;
+  int n, NL, P, R, eb, nbs, sh, nsr, vec;
   int16_t row_oy[OZ_MAXROWS], row_ox0[OZ_MAXROWS], row_cnt[OZ_MAXROWS];
   int16_t part_r[OZ_MAXPART], part_q[OZ_MAXPART], part_n[OZ_MAXPART];
   int part_o[OZ_MAXPART];     // index of the part's first offset
 };
 
-// digits of X (|X| <= 2^62): X = sum_i d[i] 2^(9 (6 - i)), |d| <= 256
-__host__ __device__ __forceinline__ void oz_digits(long long X, int (&d)[OZ_S]) {
-#pragma unroll
-  for (int i = OZ_S - 1; i > 0; --i) {
-    d[i] = (int)((X + 256) & 511) - 256;
-    X = (X - d[i]) >> 9;
-  }
-  d[0] = (int)X;
-}
-
 // Digit rows of the weights w = h^2 r and the FP64 weight image.  Thread per (rhs, leaf, node row
-// jr of the leaf), jr fastest: the eight lanes of a leaf find its largest |w| by shuffles (the
-// bit patterns of non-negative doubles order like the values), take every weight as a
-// fixed-point number below it, and write their row's digits as the 16-byte chunk jr of the leaf's
+// jr of the leaf), jr fastest: the eight lanes of a leaf find its largest |w| by shuffles, take every weight
+// as a fixed-point number below it, and write their row's digits as the 16-byte chunk jr of the leaf's
 // swizzled row in each digit's image.
 __global__ void k_oz_strips(int n, int lgNL, int P, int R, int64_t rows, double h2, int nrhs,
                             const double *__restrict__ r, uint16_t *__restrict__ img, int2 *__restrict__ lexp,
@@ -92,26 +77,18 @@ __global__ void k_oz_strips(int n, int lgNL, int P, int R, int64_t rows, double 
 #pragma unroll
   for (int q = 0; q < 8; ++q) {
     w[q] = in ? h2 * r[rhs * (int64_t)n * n + (int64_t)j * n + i0 + q] : 0.0;
-    mx = max(mx, (unsigned long long)__double_as_longlong(w[q]) & 0x7fffffffffffffffull);
+    mx = max(mx, oz_bits(w[q]));
   }
 #pragma unroll
   for (int o = 1; o < 8; o <<= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-  const int em = max((int)(mx >> 52), 1);  // |w| < 2^(em - 1022), subnormal numbers included
+  const int em = oz_biased(mx);
   const int64_t f = (int64_t)(Yl + R) * P + Xl + R;
   uint32_t pk[OZ_S][4];
   float l1 = 0.0f;
 #pragma unroll
   for (int q = 0; q < 8; ++q) {
-    const unsigned long long u = (unsigned long long)__double_as_longlong(w[q]);
-    const int ex = (int)(u >> 52) & 0x7ff;
-    const long long mant = (long long)((u & 0xfffffffffffffull) | (ex ? 0x10000000000000ull : 0ull));
-    const int sh = 9 - (em - max(ex, 1));  // X = |w| 2^(62 - E)
-    long long X = sh >= 0 ? mant << sh : (sh > -60 ? (mant + (1ll << (-sh - 1))) >> -sh : 0);
-    if (em == 0x7ff) X = 0;
-    l1 += __ll2float_ru(X);
-    if (u >> 63) X = -X;
     int d[OZ_S];
-    oz_digits(X, d);
+    oz_digits(oz_fixed(w[q], em, l1), d);
 #pragma unroll
     for (int s = 0; s < OZ_S; ++s) {
       const uint32_t hv = __half_as_ushort(__int2half_rn(d[s]));  // exact
@@ -122,9 +99,7 @@ __global__ void k_oz_strips(int n, int lgNL, int P, int R, int64_t rows, double 
 #pragma unroll
   for (int o = 1; o < 8; o <<= 1) l1 += __shfl_xor_sync(0xffffffffu, l1, o);
   if (!in) return;
-  if (jr == 0)
-    lexp[rhs * rows + f] = make_int2(mx == 0 ? OZ_NONE : (em == 0x7ff ? OZ_NAN : em - 1022),
-                                     __float_as_int(l1 * (0x1p-62f * 1.00001f)));
+  if (jr == 0) lexp[rhs * rows + f] = oz_group(mx, em, l1);
   const int pos = jr ^ (int)(f & 7);
 #pragma unroll
   for (int s = 0; s < OZ_S; ++s)
@@ -272,15 +247,11 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_p2p_oz(OzArgs a) {
     {
       int r = rs, q = qs;
       for (int g = 0; g < ng; ++g) {
-        const int2 v = __ldg(le + (int)a.row_oy[r] * a.P + a.row_ox0[r] + q);
-        const int e = max(emax, v.x);
-        l1 = l1 * exp2f((float)max(emax - e, -200)) + __int_as_float(v.y) * exp2f((float)max(v.x - e, -200));
-        emax = e;
+        oz_bound(__ldg(le + (int)a.row_oy[r] * a.P + a.row_ox0[r] + q), emax, l1);
         if (++q == a.row_cnt[r]) q = 0, ++r;
       }
     }
-    // unit 2^-lsb: the sum of the bounds stays below 2^61 (one bit for the roundings)
-    const int lsb = min(OZ_LSB, 60 - max(ilogbf(fmaxf(l1, 1.0f)), 0));
+    const int lsb = oz_unit(l1);
     long long acc[32];
 #pragma unroll
     for (int i = 0; i < 32; ++i) acc[i] = 0;
@@ -291,7 +262,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_p2p_oz(OzArgs a) {
       const int d = min(emax - __ldg(le + (int)a.row_oy[r] * a.P + a.row_ox0[r] + q).x + OZ_LSB - lsb, 62);
       const long long half = d > 0 ? 1ll << (d - 1) : 0;
       if (++q == a.row_cnt[r]) q = 0, ++r;
-      int tl[32];  // orders 4-6 in units of 2^-56 (order 4 is in units of 2^-52)
+      int tl[32];  // orders 4-6 in units of 2^-56
       if (!__all_sync(0xffffffffu, tc::mbar_wait(&acc_full[0], g & 1, &abort_flag))) {
         ok = false;
         break;
@@ -304,10 +275,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_p2p_oz(OzArgs a) {
         tc::tmem_ld16(tb + 64 * 5 + 16 * c, v5);
         tc::tmem_ld16(tb + 64 * 4 + 16 * c, v4);
 #pragma unroll
-        for (int i = 0; i < 16; ++i) {
-          const int s6 = __float2int_rn(v6[i]), s5 = __float2int_rn(v5[i]), s4 = __float2int_rn(v4[i]);
-          tl[16 * c + i] = s4 * 16 + ((s5 + ((s6 + 256) >> 9) + 16) >> 5);
-        }
+        for (int i = 0; i < 16; ++i) tl[16 * c + i] = oz_join_low(v4[i], v5[i], v6[i]);
       }
       tc::fence_before();
       __syncwarp();
@@ -325,14 +293,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_p2p_oz(OzArgs a) {
         tc::tmem_ld16(tb + 128 + 16 * c, v2);
         tc::tmem_ld16(tb + 192 + 16 * c, v3);
 #pragma unroll
-        for (int i = 0; i < 16; ++i) {  // order s in units of 2^(-9 s - 16)
-          long long t = (long long)tl[16 * c + i];
-          t += (long long)__float2int_rn(v3[i]) * (1 << 13);
-          t += (long long)__float2int_rn(v2[i]) * (1 << 22);
-          t += (long long)__float2int_rn(v1[i]) * (1ll << 31);
-          t += (long long)__float2int_rn(v0[i]) * (1ll << 40);
-          acc[16 * c + i] += (t + half) >> d;
-        }
+        for (int i = 0; i < 16; ++i) acc[16 * c + i] += (oz_join(tl[16 * c + i], v0[i], v1[i], v2[i], v3[i]) + half) >> d;
       }
       tc::fence_before();
       __syncwarp();
@@ -408,11 +369,6 @@ __global__ void k_oz_table(OzArgs a, int no, int nrows, int eb, const double *__
   for (int s = 0; s < OZ_S; ++s)
     reinterpret_cast<uint4 *>(bmat + ((int64_t)o * OZ_S + oz_pos(s)) * OZ_BLK + t * 128)[kc ^ (t & 7)] =
         make_uint4(pk[s][0], pk[s][1], pk[s][2], pk[s][3]);
-}
-
-__global__ void k_oz_fill(int64_t total, int2 *__restrict__ le) {
-  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t < total) le[t] = make_int2(OZ_NONE, 0);
 }
 
 __global__ void k_near_combine64(int64_t total, const double *__restrict__ a, int64_t stride, int nparts,
@@ -555,7 +511,6 @@ int run_p2p_oz(fmmpc_handle &H, bool with_lnh, double *out, int nrhs, cudaStream
   a.nbs = T.nbs;
   a.sh = T.sh;
   a.nsr = T.nsr;
-  a.nparts = T.nparts;
   for (int p = 0; p < T.nparts; ++p) {
     a.part_r[p] = (int16_t)T.part_r[p];
     a.part_q[p] = (int16_t)T.part_q[p];

@@ -427,7 +427,6 @@ void init_tc_p2p(fmmpc_handle &H) {
     H.tcp.usplit = best;
   }
   H.tcp.part_stride = (int64_t)H.nrhs_max * g.n * g.n;
-  H.tcp.nparts = 2;
   H.tcp.near = H.pool.get<float>((size_t)2 * H.tcp.part_stride);
   H.tcp.lsc = H.pool.get<float>((size_t)H.nrhs_max * NL * NL);
   FMMPC_CUDA(cudaMemsetAsync(H.tcp.lsc, 0, sizeof(float) * H.nrhs_max * NL * NL, H.stream));  // padding leaves
