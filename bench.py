@@ -271,9 +271,10 @@ def load_peaks():
 
 
 def rooflines(P, stage_ms, nrhs=1):
-    """Roofline of the P2P (tensor cores) and M2L (FP32 CUDA cores) kernels from their
-    live CUDA-event times; the dominant one (larger time) is reported as `roofline`."""
+    """Roofline of the P2P and M2L kernels of the handle's form from their live CUDA-event
+    times; the dominant one (larger time) is reported as `roofline`."""
     m = P.query("leaf_side")
+    digits = P.precision == "fp64"  # tensor cores: 28 products of FP16 digits per FP64 product
     pk = load_peaks()
     out = {}
     # P2P: one FMA (2 flops) per source-target pair of the near-field lists
@@ -286,11 +287,15 @@ def rooflines(P, stage_ms, nrhs=1):
         else:
             peak, src = 1900.0, "fallback bf16 1.9 PFLOP/s (FP16 runs at the BF16 rate)"
         ach = 2.0 * pairs / (t * 1e-3) / 1e12
-        out["p2p"] = {"bound": "tensor", "kernel": "k_p2p_tc (lattice P2P, tcgen05 FP16 x3)",
+        mult = 28 if digits else 3
+        how = ("each FP64-accurate product takes 28 FP16 MMAs (pairs of 9-bit digits)" if digits else
+               "each FP32-accurate product takes 3 FP16 MMAs (hi*hi, hi*lo, lo*hi)")
+        out["p2p"] = {"bound": "tensor",
+                      "kernel": "k_p2p_oz (lattice P2P, tcgen05 FP16 digits)" if digits else
+                                "k_p2p_tc (lattice P2P, tcgen05 FP16 x3)",
                       "achieved": ach, "peak": peak, "unit": "TFLOP/s",
-                      "peak_source": src + "; each FP32-accurate product takes 3 FP16 MMAs (hi*hi, hi*lo, lo*hi), "
-                                           "so the tensor pipe executes 3x the algorithmic flops",
-                      "executed_frac": 3.0 * ach / peak,
+                      "peak_source": f"{src}; {how}, so the tensor pipe executes {mult}x the algorithmic flops",
+                      "executed_frac": mult * ach / peak,
                       "work": f"{pairs:.4e} pairs/launch x 2 flop", "launch_ms": t}
     else:
         peak = SMS * LANES * 2 * SM_MAX_MHZ * 1e6 / 1e12
@@ -302,7 +307,14 @@ def rooflines(P, stage_ms, nrhs=1):
     p = P.p
     t = stage_ms["m2l"]
     tcm = P.query("tc_m2l")
-    if tcm:
+    if digits and p <= 15:
+        pairs_m = P.query("n_m2l") * nrhs
+        peak = pk["bf16_tflops"] if pk else 1900.0
+        out["m2l"] = {"bound": "tensor", "kernel": "k_m2l_oz (+ k_m2l_oz_pack, k_m2l_oz_sum; tcgen05 FP16 digits)",
+                      "achieved": 8.0 * p * p * pairs_m / (t * 1e-3) / 1e12, "peak": peak, "unit": "TFLOP/s",
+                      "peak_source": ("measured bf16 burst" if pk else "fallback bf16") + ", 28 digit products each",
+                      "work": f"{pairs_m} pairs/launch x 8p^2 flop (p={p})", "launch_ms": t}
+    elif tcm:
         pairs_m = P.query("n_m2l") * nrhs  # volume pairs; boundary sources run in stage m2l_bnd
         if tcm == 2:
             peak = pk["bf16_tflops"] if pk else 1900.0
