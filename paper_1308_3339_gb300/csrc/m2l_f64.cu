@@ -14,8 +14,11 @@
 //
 // A CTA takes 128 flattened targets and two of the four parity classes (N = 2 W, so that seven
 // orders fit TMEM), and sweeps the shifts that hold an offset of either class.  Parts of the shifts
-// write L~ images of their own, which a last kernel adds.  Bound by the MMAs: 28 x 2 of about 48
-// cycles per shift and class pair.
+// write L~ images of their own, which a last kernel adds.
+//
+// Bound by the epilogue, as the near field (p2p_f64.cu): the tensor pipe is active 23% of the 268 us of a
+// 1024^2 grid, DRAM 1%, and a scheduler's two epilogue warps wait for TMEM reads, conversions and each
+// other's 64-bit chains.
 #include <algorithm>
 #include <array>
 #include <cmath>
@@ -416,12 +419,14 @@ void init_m2l_oz(fmmpc_handle &H, DevPool &tmp) {
   }
   T.rows = rows;
   T.ntiles = (int)tiles.size();
-  // with few tiles the shifts are split between up to four CTAs (1024^2: 104 CTAs a part); the
-  // choice depends on the geometry only
+  // a tile's two class pairs are two CTAs: where these do not fill the SMs twice, the shifts are split between
+  // four of each (1024^2: 52 tiles, 104 CTAs a part); the choice depends on the geometry and the device's
+  // SM count (152), not on the right-hand sides
   int dev = 0, nsm = 0;
   FMMPC_CUDA(cudaGetDevice(&dev));
   FMMPC_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
-  T.nparts = 2 * T.ntiles >= 2 * nsm ? 1 : OZM_MAXPART;
+  const int ctas = 2 * T.ntiles;
+  T.nparts = ctas >= 2 * nsm ? 1 : OZM_MAXPART;
   std::vector<int4> shifts;
   std::vector<int> shq;  // the shift (index of shift_ofs) of each entry
   int count[2] = {};
