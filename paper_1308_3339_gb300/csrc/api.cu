@@ -342,7 +342,8 @@ int fmmpc_set_bem_form(fmmpc_handle *h, int32_t form) {
     require(form == FMMPC_BEM_SINGLE_LAYER || form == FMMPC_BEM_DOUBLE_LAYER, "set_bem_form: unknown form");
     if (form == FMMPC_BEM_DOUBLE_LAYER) {
       init_bem_dl(*h);
-      if (!init_bnd_dl(*h)) throw Error(FMMPC_ERR_OOM, "set_bem_form: no memory for the near double layer");
+      if (!init_bnd_dl(*h) && !(drop_digit_kernels(*h) && init_bnd_dl(*h)))
+        throw Error(FMMPC_ERR_OOM, "set_bem_form: no memory for the near double layer");
     }
     if (form != h->bem_form) {
       for (auto &e : h->gcache) cudaGraphExecDestroy(e.exec);  // captured with the other form

@@ -279,13 +279,14 @@ void init_bem_dl(fmmpc_handle &H) {
   const size_t nt = (size_t)(n / 2) * N;
   cudaStream_t s = H.stream;
   DevPool tmp;
+  double *T = nullptr;
+  float *th = nullptr, *tl = nullptr;
   try {
-    double *T = H.pool.get<double>(nt);
+    T = H.pool.get<double>(nt);
     k_bem_fold<BemMatrix::DOUBLE><<<nblk((int64_t)(n / 2) * (n / 2)), 256, 0, s>>>(n, -0.5, 0.0, T);
     FMMPC_LAUNCH_CHECK();
     if (!invert_folded(n, T, s, tmp))
       throw Error(FMMPC_ERR_INVALID, "double-layer BEM matrix is singular for this domain");
-    float *th = nullptr, *tl = nullptr;
     if (H.prec != FMMPC_PREC_FP64) {
       th = H.pool.get<float>(nt);
       tl = H.pool.get<float>(nt);
@@ -296,8 +297,11 @@ void init_bem_dl(fmmpc_handle &H) {
     H.Kdl_inv = T;
     H.Kdl_hi = th;
     H.Kdl_lo = tl;
-  } catch (...) {
+  } catch (...) {  // the handle keeps nothing of it
     cudaStreamSynchronize(s);
+    H.pool.give_back(T, sizeof(double) * nt);
+    H.pool.give_back(th, sizeof(float) * nt);
+    H.pool.give_back(tl, sizeof(float) * nt);
     throw;
   }
 }

@@ -9,6 +9,7 @@
 
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cstdint>
 #include <cstdio>
 #include <functional>
@@ -84,6 +85,13 @@ struct DevPool {
   template <typename T>
   T *get(size_t count) {
     return static_cast<T *>(alloc(sizeof(T) * count));
+  }
+  void give_back(void *p, size_t nbytes) {
+    const auto it = std::find(ptrs.begin(), ptrs.end(), p);
+    if (!p || it == ptrs.end()) return;
+    cudaFree(p);
+    ptrs.erase(it);
+    bytes -= nbytes;
   }
   void release() {
     for (void *p : ptrs) cudaFree(p);

@@ -86,3 +86,26 @@ def test_fp64_handle_gives_the_digit_operands_back_to_a_solve(use_graphs):
     finally:
         del hog
         free_memory()
+
+
+def test_double_layer_form_that_does_not_fit_leaves_nothing_behind():
+    # 2048^2: the inverse takes 67 MB and its set-up and FP32 words some 200 more; with 211 MB left the form is
+    # refused, and the handle holds no more than before, however often it is asked
+    from paper_1308_3339_gb300 import FmmPreconditioner, FmmpcError
+    free_memory()
+    Q = FmmPreconditioner(2048, p=8, precision="fp32")  # the solver library's own memory is there
+    Q.set_bem_form("double_layer")
+    Q.close()
+    P = FmmPreconditioner(2048, p=8, precision="fp32")
+    held = P.query("device_bytes")
+    hog = torch.empty(free_memory() - 211 * MB, dtype=torch.uint8, device="cuda")
+    try:
+        for _ in range(2):
+            with pytest.raises(FmmpcError):
+                P.set_bem_form("double_layer")
+            assert P.query("device_bytes") == held
+    finally:
+        del hog
+        free_memory()
+    P.set_bem_form("double_layer")
+    P.close()
